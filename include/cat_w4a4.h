@@ -362,8 +362,9 @@ int32_t cat_dp_planes(int32_t bits);
  *   planes       out, device [D][n][d_in] bytes (digit planes of the codes of x').
  *   x_scale      out, device [n] float32 steps (0 for an all-zero or non-finite token).
  *   x_zero       out, device [n] int32 zero points (asymmetric only; may be NULL when symmetric).
- * x_scale and x_zero also serve as the row statistics' scratch while the call runs.  Runs on SIMT
- * cores (transform, row statistics, codes: four launches).
+ * bf16 rows on the fused tensor-core kernel: one launch (as cat_transform_quantize_act).  fp32 rows and the
+ * shapes that kernel does not take run on SIMT cores (transform, row statistics, codes: four launches);
+ * x_scale and x_zero then also serve as the row statistics' scratch while the call runs.
  */
 cat_status cat_transform_quantize_act_dp(const void* x, cat_dtype dtype, int64_t n, int64_t d_in, int32_t k,
                                          const float* T_blocks, int32_t bits, int32_t asymmetric, uint8_t* planes,

@@ -20,6 +20,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "dp_codes.cuh"
 
 namespace cat {
 namespace {
@@ -45,6 +46,19 @@ struct TcCfg {
                                     ((uint32_t)(TM >> 4) << 24);
 };
 
+// What the fused kernel writes: 4-bit codes (packed words or bytes), or the digit planes of b-bit
+// symmetric or asymmetric codes.  An asymmetric row has two extremes, max(v', 0) and max(-v', 0): both
+// are non-negative floats, so each is an integer maximum of bit patterns as the symmetric one is.
+// The b-bit modes run in the time of the 4-bit one (bound by the same MMAs and hand-over of maxima): layer
+// calls 4096 -> 6144 on 2048 tokens at 8 bits asymmetric 435 -> 270 us and 14336 -> 4096 on 1000 tokens at
+// 8 bits 455 -> 228 us against two SIMT passes over the block products (193 and 259 us, now 17 and 37).
+enum FusedMode : int { kW4 = 0, kDpSym = 1, kDpAsym = 2 };
+struct DpOut {
+  float qmax;       // symmetric: 2^(b-1) - 1; asymmetric: N = 2^b - 1
+  int planes;       // digit planes
+  int32_t* zero;    // asymmetric: zero points
+};
+
 // Shared-memory layout of the fused kernel.  A unit is (group of N output channels, 128-row tile);
 // the group's block has KD input channels (N = KD = 128 or 64; N = 64, KD = 256 for 256-blocks, whose
 // three bf16 planes would not fit whole: a group is a quarter of the block's outputs).  An x stage
@@ -54,8 +68,9 @@ struct TcCfg {
 // maxima (128 floats): in a single wave at N = KD = 128 (at most kXStages units) in the unit's x
 // stage, free once its MMAs are done; otherwise in their own room, with one x stage fewer at 128 in
 // waves, and three at KD = 256, to make room.
-template <int N, int KD, bool WAVES>
+template <int N, int KD, bool WAVES, int MODE = kW4>
 struct FusedCfg {
+  static constexpr int EXT = MODE == kDpAsym ? 2 : 1;        // extremes kept per row
   static constexpr int U = 512 / N;
   static constexpr int XH = KD > 128 ? KD / 128 : 1;
   static constexpr int XW = KD > 128 ? 128 : KD;
@@ -69,16 +84,17 @@ struct FusedCfg {
   static constexpr uint32_t BAR_BYTES = 512;
   static constexpr bool AMAX_IN_X = !WAVES && N == 128 && KD == 128;
   static constexpr uint32_t AMAX_OFF = BAR_OFF + BAR_BYTES;
-  static constexpr size_t SMEM = AMAX_OFF + (AMAX_IN_X ? 0 : U * TM * 4) + 1024;
+  static constexpr size_t SMEM = AMAX_OFF + (AMAX_IN_X ? 0 : EXT * U * TM * 4) + 1024;
   // kind::f16: D fp32 (bit 4), A = B = BF16 (format 1 at bits 7 and 10), K-major, M = 128, N
   static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
                                     ((uint32_t)(TM >> 4) << 24);
   __device__ static float* amax_slot(uint8_t* smem, int slot) {
-    return reinterpret_cast<float*>(AMAX_IN_X ? smem + X_OFF + slot * X_STAGE : smem + AMAX_OFF + slot * TM * 4);
+    return reinterpret_cast<float*>(AMAX_IN_X ? smem + X_OFF + slot * X_STAGE : smem + AMAX_OFF + slot * EXT * TM * 4);
   }
 };
 static_assert(FusedCfg<128, 128, false>::SMEM <= 227 * 1024 && FusedCfg<128, 128, true>::SMEM <= 227 * 1024 &&
-                  FusedCfg<64, 256, true>::SMEM <= 227 * 1024,
+                  FusedCfg<64, 256, true>::SMEM <= 227 * 1024 && FusedCfg<128, 128, true, kDpAsym>::SMEM <= 227 * 1024 &&
+                  FusedCfg<64, 256, true, kDpAsym>::SMEM <= 227 * 1024,
               "shared memory");
 
 struct TcBars {
@@ -312,6 +328,125 @@ __device__ __forceinline__ void quant_chunk(uint32_t taddr, const QRow& qr, uint
   }
 }
 
+// b-bit codes (digit planes).  The float32 estimate p = fl(v * inv) carries a relative error of at most
+// 3 * 2^-24 (inv has one rounding for symmetric rows, two for asymmetric ones, the product one more), so for
+// |p| <= 255 it is within 255 * 3 * 2^-24 < 2^-14 of the quotient: rint(p) is the exact code unless p lies
+// within 2^-14 of a half-integer, and there the decision is redone exactly.
+constexpr float kNearTieDp = 0.5f - 0x1p-14f;
+
+// One row's grid: symmetric (lo unused) or asymmetric.
+struct DpRow {
+  QRow q;           // symmetric
+  float hi, lo;     // asymmetric extremes (lo <= 0 <= hi)
+  float inv;        // 0: an all-zero or non-finite row, all codes 0
+  int z;
+};
+
+__device__ __noinline__ int qcode_exact_dp(float v, QRow q, float qmax) { return qcode_exact(v, q, qmax); }
+__device__ __noinline__ int asym_code_exact(float v, float hi, float lo, float N) {
+  return asym_code(v, asym_row(hi, lo, N), N);
+}
+__device__ __noinline__ int asym_zero_exact(float hi, float lo, float N) { return asym_row(hi, lo, N).z; }
+
+template <int MODE>
+__device__ __forceinline__ DpRow dp_row(float hi, float neg_lo, float qmax) {
+  DpRow r;
+  r.z = 0;
+  if (MODE == kDpSym) {
+    r.q = qrow_setup(hi, qmax);
+    r.hi = r.lo = 0.f;
+    r.inv = r.q.inv;
+    return r;
+  }
+  r.q = QRow{};
+  r.hi = hi;
+  r.lo = -neg_lo;
+  const float w = __fadd_rn(hi, neg_lo);
+  r.inv = 0.f;
+  if (isfinite(hi) && isfinite(neg_lo) && (hi > 0.f || neg_lo > 0.f)) {
+    if (isfinite(w)) r.inv = __fdiv_rn(qmax, w);
+    // z = round(N (-lo) / (hi - lo)), decided like a code
+    const float p = __fmul_rn(neg_lo, r.inv), rq = rintf(p);
+    r.z = (fabsf(p - rq) <= kNearTieDp) ? (int)rq : asym_zero_exact(r.hi, r.lo, qmax);
+  }
+  return r;
+}
+
+// The codes of the 32 values in tensor memory at taddr (this lane's row) as eight words of code bytes: two's
+// complement (symmetric) or unsigned (asymmetric); called by the whole warp.  As quant_chunk.
+template <int MODE>
+__device__ __forceinline__ void quant_chunk_dp(uint32_t taddr, const DpRow& row, float qmax, uint32_t (&out)[8]) {
+  constexpr float kMagic = 12582912.0f;
+  constexpr int kMagicBits = 0x4B400000;
+  int bq[32];
+  bool near = MODE == kDpSym && row.q.exact;
+  const int top = (int)qmax;
+  {
+    uint32_t r[32];
+    __syncwarp();
+    CAT_TMEM_LD32(taddr, r);
+    tmem_ld_wait();
+    const float scl = MODE == kDpSym ? row.q.sc : 1.f;   // rescaled rows take the exact route for every value
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      const float p = __fmul_rn(__uint_as_float(r[e]) * scl, row.inv);
+      const float rb = __fadd_rn(p, kMagic);
+      near |= !(fabsf(__fsub_rn(__fsub_rn(rb, kMagic), p)) <= kNearTieDp);
+      bq[e] = __float_as_int(rb) - kMagicBits;
+      if (MODE == kDpAsym) bq[e] = max(0, min(bq[e] + row.z, top));
+    }
+  }
+  if (__any_sync(0xFFFFFFFFu, near)) {
+    uint32_t r[32];
+    __syncwarp();
+    CAT_TMEM_LD32(taddr, r);
+    tmem_ld_wait();
+    if (near) {
+#pragma unroll
+      for (int e = 0; e < 32; ++e) {
+        const float v = __uint_as_float(r[e]);
+        const float p = __fmul_rn(v, row.inv);
+        const bool here = !(fabsf(__fsub_rn(__fsub_rn(__fadd_rn(p, kMagic), kMagic), p)) <= kNearTieDp);
+        if (MODE == kDpSym) {
+          if (row.q.exact || here) bq[e] = qcode_exact_dp(v, row.q, qmax);
+        } else if (here) {
+          bq[e] = asym_code_exact(v, row.hi, row.lo, qmax);
+        }
+      }
+    }
+  }
+  const bool zero = row.inv == 0.f;
+#pragma unroll
+  for (int g = 0; g < 8; ++g) {
+    const uint32_t w = __byte_perm(__byte_perm((uint32_t)bq[4 * g], (uint32_t)bq[4 * g + 1], 0x0040),
+                                   __byte_perm((uint32_t)bq[4 * g + 2], (uint32_t)bq[4 * g + 3], 0x0040), 0x5410);
+    out[g] = zero ? 0u : w;
+  }
+}
+
+// Four code bytes -> the E4M3 digit bytes of both planes (sign << 7 | magnitude).
+template <int MODE>
+__device__ __forceinline__ void digit_words(uint32_t w, int planes, uint32_t* d0, uint32_t* d1) {
+  if (MODE == kDpAsym) {                             // digits q mod 16 and q / 16 (one plane: q <= 15)
+    *d0 = w & 0x0F0F0F0Fu;
+    *d1 = (w >> 4) & 0x0F0F0F0Fu;
+    return;
+  }
+  if (planes == 1) {
+    *d0 = twos_to_sm(w);
+    *d1 = 0u;
+    return;
+  }
+  // q = 16 a + m with m = q mod 16 and a = floor(q / 16): the low digit is m - 16 c and the high one a + c,
+  // c = 1 where m >= 8; a + c lies in [-8, 8] and is formed as (a + 8) + c - 8, byte by byte
+  const uint32_t m = w & 0x0F0F0F0Fu;
+  const uint32_t c = (m >> 3) & 0x01010101u;
+  const uint32_t ah = (((w >> 4) & 0x0F0F0F0Fu) ^ 0x08080808u) + c;      // a + 8 + c, in [0, 16]
+  const uint32_t hi = ((ah | 0x80808080u) - 0x08080808u) ^ 0x80808080u;   // minus 8 in every byte, no borrow across
+  *d0 = twos_to_sm(m | (c * 0xF0u));
+  *d1 = twos_to_sm(hi);
+}
+
 // The four SM4x8 words of a chunk's 32 code bytes (codes 8g .. 8g+7 in word g).
 __device__ __forceinline__ uint4 sm4_words(const uint32_t (&e)[8]) {
   return make_uint4(e[0] | __funnelshift_l(e[1], e[1], 4), e[2] | __funnelshift_l(e[3], e[3], 4),
@@ -325,6 +460,17 @@ __device__ __forceinline__ uint32_t absmax_bits32(const uint32_t (&r)[32], uint3
 #pragma unroll
   for (int e = 0; e < 32; ++e) m = max(m, r[e] & 0x7FFFFFFFu);
   return m;
+}
+
+// The two extremes of asymmetric rows, max(v, 0) and max(-v, 0), as running integer maxima: a signed
+// maximum with 0 keeps the positive patterns only, and a NaN of either sign ends above the infinity in
+// one of the two.
+__device__ __forceinline__ void extremes32(const uint32_t (&r)[32], int& hi, int& lo) {
+#pragma unroll
+  for (int e = 0; e < 32; ++e) {
+    hi = max(hi, (int)r[e]);
+    lo = max(lo, (int)(r[e] ^ 0x80000000u));
+  }
 }
 
 template <int K, int PASS>
@@ -604,14 +750,14 @@ __device__ __forceinline__ bool wait_count(const uint32_t* ctr, uint32_t expecte
 // three warps share (slot (c + 1) % 3): the epilogue warp joins when its phase A is done.
 __device__ __forceinline__ int chunk_slot(int c, bool last) { return last ? (c + 1) % 3 : 1 + (c & 1); }
 
-template <int N, int KD, bool WAVES>
+template <int N, int KD, bool WAVES, int MODE>
 __device__ __forceinline__ void quantize_units(uint32_t tmem, uint8_t* smem, const FusedUnits& fu, int num_tiles,
                                                int n, int d, uint64_t* maxima_ready, uint64_t* tmem_free,
-                                               uint32_t* __restrict__ codes, int e8, volatile int* abort_flag,
-                                               int slot) {
+                                               uint32_t* __restrict__ codes, int e8, const DpOut& dp,
+                                               volatile int* abort_flag, int slot) {
   // unit j sits in tensor-memory slot j % U (phase (j / U) & 1 of the slot's barriers); with WAVES the
   // converter warps (slots 1 and 2) hand the slot back once their chunks of the unit are done
-  using F = FusedCfg<N, KD, WAVES>;
+  using F = FusedCfg<N, KD, WAVES, MODE>;
   const int lane = threadIdx.x & 31, quad = (threadIdx.x >> 5) & 3;
   const int64_t words_per_row = d / 8;
   const int nu = fu.count;
@@ -629,15 +775,32 @@ __device__ __forceinline__ void quantize_units(uint32_t tmem, uint8_t* smem, con
       fused_unit(fu, j, num_tiles, &b, &tile);
       const int t = tile * TM + quad * 32 + lane;
       const float a = F::amax_slot(smem, us)[quad * 32 + lane];
-      const QRow qr = qrow_setup(a, 7.0f);     // inv == 0: zero or non-finite row, all codes 0
+      [[maybe_unused]] QRow qr;
+      [[maybe_unused]] DpRow dr;
+      if constexpr (MODE == kW4) qr = qrow_setup(a, 7.0f);     // inv == 0: zero or non-finite row, all codes 0
+      else dr = dp_row<MODE>(a, MODE == kDpAsym ? F::amax_slot(smem, us)[TM + quad * 32 + lane] : 0.f, dp.qmax);
       tc_fence_after();
 #pragma unroll 1
       for (int c = 0; c < N / 32; ++c) {
         if (chunk_slot(c, last) != slot) continue;
         uint32_t e[8];
-        quant_chunk(tmem + ((uint32_t)(quad * 32) << 16) + us * N + c * 32, qr, e);
+        const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + us * N + c * 32;
+        if constexpr (MODE == kW4) quant_chunk(taddr, qr, e);
+        else quant_chunk_dp<MODE>(taddr, dr, dp.qmax, e);
         if (t < n) {
-          if (e8) {                            // byte codes: 32 bytes of row t
+          if constexpr (MODE != kW4) {         // digit planes: 32 bytes of row t in each
+            uint8_t* dst = reinterpret_cast<uint8_t*>(codes) + (int64_t)t * d + (int64_t)b * N + c * 32;
+            uint32_t d0[8], d1[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) digit_words<MODE>(e[g], dp.planes, &d0[g], &d1[g]);
+            reinterpret_cast<uint4*>(dst)[0] = make_uint4(d0[0], d0[1], d0[2], d0[3]);
+            reinterpret_cast<uint4*>(dst)[1] = make_uint4(d0[4], d0[5], d0[6], d0[7]);
+            if (dp.planes == 2) {
+              dst += (int64_t)n * d;
+              reinterpret_cast<uint4*>(dst)[0] = make_uint4(d1[0], d1[1], d1[2], d1[3]);
+              reinterpret_cast<uint4*>(dst)[1] = make_uint4(d1[4], d1[5], d1[6], d1[7]);
+            }
+          } else if (e8) {                     // byte codes: 32 bytes of row t
             uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(codes) + (int64_t)t * d + (int64_t)b * N +
                                                   c * 32);
             dst[0] = make_uint4(e[0], e[1], e[2], e[3]);
@@ -656,16 +819,17 @@ __device__ __forceinline__ void quantize_units(uint32_t tmem, uint8_t* smem, con
   }
 }
 
-template <int N, int KD, bool WAVES>
+template <int N, int KD, bool WAVES, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
     transform_quant_tc_fused_kernel(const __grid_constant__ CUtensorMap tmX, const float* __restrict__ A,
                                     const uint8_t* __restrict__ planes, int n, int d, int kb, float* __restrict__ scale,
-                                    uint32_t* __restrict__ codes, int e8, uint32_t* __restrict__ state,
+                                    uint32_t* __restrict__ codes, int e8, const DpOut dp, uint32_t* __restrict__ state,
                                     uint32_t* __restrict__ amax_sets, uint32_t* __restrict__ rec_sets,
                                     uint32_t* __restrict__ status) {
   // state: the slot's epoch, start counter and tiles per set; amax_sets: two sets of kAmaxRows row
-  // maxima (float bits); rec_sets: two sets of kAmaxTiles tile records
-  using F = FusedCfg<N, KD, WAVES>;
+  // maxima (float bits; asymmetric rows: max(v, 0) of all tiles, then max(-v, 0) of all tiles); rec_sets:
+  // two sets of kAmaxTiles tile records
+  using F = FusedCfg<N, KD, WAVES, MODE>;
   constexpr int U = F::U;                              // tensor-memory slots (units resident at once)
   static_assert(sizeof(TcBars) + (4 * U + 4) * sizeof(uint64_t) + 8 <= F::BAR_BYTES, "barrier room");
   static_assert(!F::AMAX_IN_X || U <= F::XS, "in one wave at k = 128 unit j's x stage holds its maxima");
@@ -843,9 +1007,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t v[TM / 32];
 #pragma unroll
       for (int i = 0; i < TM / 32; ++i) v[i] = __ldcg(&amax_bits[tile * TM + 32 * i + lane]);  // < kAmaxRows
+      [[maybe_unused]] uint32_t vl[TM / 32];                 // asymmetric: the negative extremes
+      if constexpr (MODE == kDpAsym) {
+#pragma unroll
+        for (int i = 0; i < TM / 32; ++i) vl[i] = __ldcg(&amax_bits[(num_tiles + tile) * TM + 32 * i + lane]);
+      }
       float* am = F::amax_slot(smem, j % U);
 #pragma unroll
-      for (int i = 0; i < TM / 32; ++i) am[32 * i + lane] = __uint_as_float(v[i]);
+      for (int i = 0; i < TM / 32; ++i) {
+        am[32 * i + lane] = __uint_as_float(v[i]);
+        if constexpr (MODE == kDpAsym) am[TM + 32 * i + lane] = __uint_as_float(vl[i]);
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(&maxima_ready[j % U]);
       if (b == 0) {                                      // the CTAs holding block 0 write the steps
@@ -855,10 +1027,17 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float a = __uint_as_float(v[i]);
           if (t >= n) continue;
           float sc = 0.f;
-          if (isfinite(a))
-            sc = __fdiv_rn(a, 7.0f);
-          else
+          if constexpr (MODE == kDpAsym) {
+            const float neg_lo = __uint_as_float(vl[i]);
+            const AsymRow ar = asym_row(a, -neg_lo, dp.qmax);
+            if (!(isfinite(a) && isfinite(neg_lo))) report(status, kStatusNonFinite);
+            if (ar.inv != 0.f) sc = (float)(ar.r / (double)dp.qmax);
+            dp.zero[t] = ar.z;
+          } else if (isfinite(a)) {
+            sc = __fdiv_rn(a, MODE == kW4 ? 7.0f : dp.qmax);
+          } else {
             report(status, kStatusNonFinite);
+          }
           scale[t] = sc;
         }
       }
@@ -892,7 +1071,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       __threadfence();
       if (atomicAdd(&state[1], 1u) == gridDim.x - 1) {
-        state[2 + P] = (uint32_t)num_tiles;
+        state[2 + P] = (uint32_t)(F::EXT * num_tiles);
         state[1] = 0u;
         __threadfence();
         state[0] = E + 1u;
@@ -938,8 +1117,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         ++version;
       }
     }
-    quantize_units<N, KD, WAVES>(tmem, smem, fu, num_tiles, n, d, maxima_ready, tmem_free, codes, e8, abort_flag,
-                                 1 + ((warp - kCvtWarp0) >> 2));
+    quantize_units<N, KD, WAVES, MODE>(tmem, smem, fu, num_tiles, n, d, maxima_ready, tmem_free, codes, e8, dp,
+                                       abort_flag, 1 + ((warp - kCvtWarp0) >> 2));
     tc_fence_before();
   } else if (warp >= kEpiWarp0) {
     // ---------------------------------------------------------------- phase A: one row per thread
@@ -955,6 +1134,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!__all_sync(0xFFFFFFFFu, got)) break;        // warp-uniform: TMEM loads need the whole warp
       tc_fence_after();
       uint32_t mb = 0;
+      [[maybe_unused]] int hi = 0, lo = 0;
 #pragma unroll 1
       for (int c = 0; c < N / 32; c += 2) {            // two loads in flight
         uint32_t r0[32], r1[32];
@@ -962,19 +1142,32 @@ __global__ void __launch_bounds__(kThreads, 1)
         CAT_TMEM_LD32(tmem + ((uint32_t)(quad * 32) << 16) + (j % U) * N + c * 32, r0);
         CAT_TMEM_LD32(tmem + ((uint32_t)(quad * 32) << 16) + (j % U) * N + (c + 1) * 32, r1);
         tmem_ld_wait();
-        mb = absmax_bits32(r1, absmax_bits32(r0, mb));
+        if constexpr (MODE == kDpAsym) {
+          extremes32(r0, hi, lo);
+          extremes32(r1, hi, lo);
+        } else {
+          mb = absmax_bits32(r1, absmax_bits32(r0, mb));
+        }
       }
+      if constexpr (MODE == kDpAsym) mb = max((uint32_t)hi, (uint32_t)lo);
       const bool row_finite = mb < 0x7F800000u;
       finite &= row_finite;
       // a non-finite value makes the row's maximum the largest NaN pattern: its codes and step become 0
-      if (t < n) atomicMax(&amax_bits[t], row_finite ? mb : 0x7FFFFFFFu);
+      if constexpr (MODE == kDpAsym) {
+        if (t < n) {
+          atomicMax(&amax_bits[t], row_finite ? (uint32_t)hi : 0x7FFFFFFFu);
+          atomicMax(&amax_bits[num_tiles * TM + t], (uint32_t)lo);
+        }
+      } else if (t < n) {
+        atomicMax(&amax_bits[t], row_finite ? mb : 0x7FFFFFFFu);
+      }
       __syncwarp();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&epi_done[j % U]);
     }
     if (!finite) report(status, kStatusNonFinite);
-    quantize_units<N, KD, WAVES>(tmem, smem, fu, num_tiles, n, d, maxima_ready, tmem_free, codes, e8, abort_flag, 0);
+    quantize_units<N, KD, WAVES, MODE>(tmem, smem, fu, num_tiles, n, d, maxima_ready, tmem_free, codes, e8, dp, abort_flag, 0);
     tc_fence_before();
   }
 
@@ -1108,9 +1301,12 @@ bool cooperative_ok() {
   return cudaDeviceGetAttribute(&v, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && v != 0;
 }
 
-template <int N, int KD>
+template <int N, int KD, int MODE>
 cudaError_t launch_fused_k(const __nv_bfloat16* x, int64_t n, int64_t d, int kb, const float* A, const uint8_t* planes,
-                           uint32_t* amax, uint32_t* words, int e8, uint32_t* status, cudaStream_t stream) {
+                           uint32_t* amax, uint32_t* words, int e8, const DpOut& dp, uint32_t* status,
+                           cudaStream_t stream) {
+  using F0 = FusedCfg<N, KD, false, MODE>;
+  using F1 = FusedCfg<N, KD, true, MODE>;
   const int nb = (int)(d / N);                         // groups of N output channels
   const int tiles = (int)((n + TM - 1) / TM);
   const int64_t units = (int64_t)nb * tiles;
@@ -1131,7 +1327,7 @@ cudaError_t launch_fused_k(const __nv_bfloat16* x, int64_t n, int64_t d, int kb,
   if (!cooperative_ok()) return cudaErrorNotSupported;
   EncodeTiledFn fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
-  if (n > kAmaxRows) return cudaErrorNotSupported;
+  if (n > kAmaxRows / F0::EXT) return cudaErrorNotSupported;
   cudaError_t e;
   const TqScratch* sc = tq_scratch(&e);
   if (!sc) return e;
@@ -1152,18 +1348,18 @@ cudaError_t launch_fused_k(const __nv_bfloat16* x, int64_t n, int64_t d, int kb,
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(transform_quant_tc_fused_kernel<N, KD, false>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedCfg<N, KD, false>::SMEM);
+    attr = cudaFuncSetAttribute(transform_quant_tc_fused_kernel<N, KD, false, MODE>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F0::SMEM);
     if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(transform_quant_tc_fused_kernel<N, KD, true>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FusedCfg<N, KD, true>::SMEM);
+      attr = cudaFuncSetAttribute(transform_quant_tc_fused_kernel<N, KD, true, MODE>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F1::SMEM);
   });
   if (attr != cudaSuccess) return attr;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = waves ? FusedCfg<N, KD, true>::SMEM : FusedCfg<N, KD, false>::SMEM;
+  cfg.dynamicSmemBytes = waves ? F1::SMEM : F0::SMEM;
   cfg.stream = stream;
   // not a programmatic dependent launch: measured, one cost the c2 step ~4 us (the kernel still
   // releases its dependents early, so a programmatic GEMM launch after it gets going sooner)
@@ -1174,10 +1370,10 @@ cudaError_t launch_fused_k(const __nv_bfloat16* x, int64_t n, int64_t d, int kb,
   cfg.numAttrs = 1;
   note_launch();
   if (waves)
-    return cudaLaunchKernelEx(&cfg, transform_quant_tc_fused_kernel<N, KD, true>, map, A, planes, (int)n, (int)d, kb,
-                              reinterpret_cast<float*>(amax), words, e8, state, amax_sets, rec_sets, status);
-  return cudaLaunchKernelEx(&cfg, transform_quant_tc_fused_kernel<N, KD, false>, map, A, planes, (int)n, (int)d, kb,
-                            reinterpret_cast<float*>(amax), words, e8, state, amax_sets, rec_sets, status);
+    return cudaLaunchKernelEx(&cfg, transform_quant_tc_fused_kernel<N, KD, true, MODE>, map, A, planes, (int)n, (int)d,
+                              kb, reinterpret_cast<float*>(amax), words, e8, dp, state, amax_sets, rec_sets, status);
+  return cudaLaunchKernelEx(&cfg, transform_quant_tc_fused_kernel<N, KD, false, MODE>, map, A, planes, (int)n, (int)d,
+                            kb, reinterpret_cast<float*>(amax), words, e8, dp, state, amax_sets, rec_sets, status);
 }
 
 }  // namespace
@@ -1234,9 +1430,36 @@ cudaError_t launch_transform_quantize_tc_fused(const void* x, int64_t n, int64_t
                                                uint32_t* status, cudaStream_t stream) {
   const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(x);
   const int KD = transform_tc_group(k, d);
-  if (KD == 64) return launch_fused_k<64, 64>(xb, n, d, k, A, planes, amax, words, e8, status, stream);
-  if (KD == 128) return launch_fused_k<128, 128>(xb, n, d, k, A, planes, amax, words, e8, status, stream);
-  if (KD == 256) return launch_fused_k<64, 256>(xb, n, d, k, A, planes, amax, words, e8, status, stream);
+  const DpOut none = {7.0f, 1, nullptr};
+  if (KD == 64) return launch_fused_k<64, 64, kW4>(xb, n, d, k, A, planes, amax, words, e8, none, status, stream);
+  if (KD == 128) return launch_fused_k<128, 128, kW4>(xb, n, d, k, A, planes, amax, words, e8, none, status, stream);
+  if (KD == 256) return launch_fused_k<64, 256, kW4>(xb, n, d, k, A, planes, amax, words, e8, none, status, stream);
   return cudaErrorNotSupported;
+}
+
+template <int MODE>
+static cudaError_t launch_fused_dp(const __nv_bfloat16* x, int64_t n, int64_t d, int k, const float* A, uint8_t* planes,
+                                   float* scale, const DpOut& dp, uint32_t* status, cudaStream_t stream) {
+  const int KD = transform_tc_group(k, d);
+  uint32_t* amax = reinterpret_cast<uint32_t*>(scale);
+  uint32_t* out = reinterpret_cast<uint32_t*>(planes);
+  if (KD == 64) return launch_fused_k<64, 64, MODE>(x, n, d, k, A, nullptr, amax, out, 0, dp, status, stream);
+  if (KD == 128) return launch_fused_k<128, 128, MODE>(x, n, d, k, A, nullptr, amax, out, 0, dp, status, stream);
+  if (KD == 256) return launch_fused_k<64, 256, MODE>(x, n, d, k, A, nullptr, amax, out, 0, dp, status, stream);
+  return cudaErrorNotSupported;
+}
+
+// bf16 activations at b bits: transform, row extremes, codes and digit planes in the fused launch;
+// cudaErrorNotSupported (nothing launched) where it does not apply, as for the 4-bit codes.
+cudaError_t launch_transform_quantize_dp_fused(const void* x, int64_t n, int64_t d, int k, const float* A, int bits,
+                                               int asym, uint8_t* planes, float* scale, int32_t* zero, uint32_t* status,
+                                               cudaStream_t stream) {
+  if (!transform_quantize_tc_supported(1, k, n, d)) return cudaErrorNotSupported;
+  const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(x);
+  const int D = bits <= 4 ? 1 : 2;
+  if (asym)
+    return launch_fused_dp<kDpAsym>(xb, n, d, k, A, planes, scale, DpOut{(float)((1 << bits) - 1), D, zero}, status, stream);
+  return launch_fused_dp<kDpSym>(xb, n, d, k, A, planes, scale, DpOut{(float)((1 << (bits - 1)) - 1), D, nullptr}, status,
+                                 stream);
 }
 }  // namespace cat

@@ -18,6 +18,8 @@
 // Asymmetric: D = 1 for b <= 4 (d0 = q in [0, 15]), else d0 = q mod 16, d1 = q / 16.  Plane p of an
 // [R][d] code matrix is the byte matrix at planes + p * R * d.
 //
+// bf16 activations run on the fused tensor-core kernel (act_quant_tc.cu, modes kDpSym and kDpAsym); the SIMT
+// kernels here serve fp32 rows, the shapes that kernel refuses, and weights (range search, code sums).
 // The row statistics span every block of a row while a CTA holds one block, so the work runs in
 // passes over the same tiles (64 rows x OC channels of one block, the block slab and the input rows
 // staged transposed in shared memory, each thread 4 rows x 8 channels):
@@ -29,6 +31,7 @@
 //   pass 1: the codes (and, optionally, each row's code sum), written as digit planes;
 //   finalize: steps s (and zero points).
 #include "common.cuh"
+#include "dp_codes.cuh"
 
 namespace cat {
 namespace {
@@ -45,68 +48,6 @@ struct DpCfg {
   static constexpr int XS_LD = kRows + 4;
   static constexpr size_t SMEM = (size_t)(K * AS_LD + K * XS_LD) * sizeof(float);
 };
-
-struct DpMode {
-  int bits;      // 2..8
-  int asym;      // 0: symmetric, 1: asymmetric
-  int planes;    // digit planes D
-  float qmax;    // symmetric: 2^(b-1) - 1; asymmetric: N = 2^b - 1
-};
-
-// Order-preserving key of a float (max of keys = key of the max), for signed min / max atomics.
-__device__ __forceinline__ uint32_t fkey(float f) {
-  const uint32_t b = __float_as_uint(f);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float fkey_inv(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
-}
-
-__device__ __forceinline__ uint32_t e4m3_digit(int d) { return (d < 0 ? 0x80u : 0u) | (uint32_t)(d < 0 ? -d : d); }
-
-// The digits' E4M3 bytes of one code.
-__device__ __forceinline__ void code_digits(int q, const DpMode& m, uint32_t* b0, uint32_t* b1) {
-  if (m.planes == 1) {
-    *b0 = e4m3_digit(q);
-    *b1 = 0u;
-  } else if (m.asym) {
-    *b0 = (uint32_t)(q & 15);
-    *b1 = (uint32_t)(q >> 4);
-  } else {
-    const int lo = ((q + 8) & 15) - 8;
-    *b0 = e4m3_digit(lo);
-    *b1 = e4m3_digit((q - lo) / 16);
-  }
-}
-
-// Per-row asymmetric grid: float32 estimate inputs and the float64 operands of the exact route.
-struct AsymRow {
-  float inv;      // fl(N / fl(hi - lo)); 0 for a zero or non-finite row
-  double lo, r;   // lo and hi - lo in float64
-  int z;
-};
-
-__device__ __forceinline__ AsymRow asym_row(float hi, float lo, float N) {
-  AsymRow a;
-  a.lo = lo;
-  a.r = (double)hi - (double)lo;
-  a.inv = 0.f;
-  a.z = 0;
-  if (!(isfinite(hi) && isfinite(lo)) || !(a.r > 0.0)) return a;
-  a.inv = __fdiv_rn(N, __fsub_rn(hi, lo));
-  a.z = (int)rint(((double)N * -a.lo) / a.r);
-  return a;
-}
-
-__device__ __forceinline__ int asym_code(float v, const AsymRow& a, float N) {
-  if (a.inv == 0.f || !isfinite(v)) return a.inv == 0.f ? 0 : a.z;
-  const float p = __fmul_rn(v, a.inv);
-  float rq = rintf(p);
-  if (fabsf(p - rq) > 0.5f - 0x1p-12f) rq = (float)rint(((double)N * (double)v) / a.r);  // exact route
-  int q = (int)rq + a.z;
-  const int top = (int)N;
-  return q < 0 ? 0 : (q > top ? top : q);
-}
 
 // Symmetric code on a shrunk range a_i = a (100 - i) / 100 (the L_2.4 choice): the float32 estimate
 // v * fl(qmax / fl(a_i)), redone as (100 qmax v) / (a (100 - i)) in float64 -- two exact operands,
@@ -431,6 +372,10 @@ int dp_planes(int bits, int asym) {
 // Workspace of the L_2.4 range search (weights): row ranges and the candidates' scores.
 size_t dp_l24_work_bytes(int64_t n) { return (size_t)n * 8 + 16 + (size_t)n * kL24Cands * sizeof(double); }
 
+cudaError_t launch_transform_quantize_dp_fused(const void* x, int64_t n, int64_t d, int k, const float* A, int bits,
+                                               int asym, uint8_t* planes, float* scale, int32_t* zero, uint32_t* status,
+                                               cudaStream_t stream);
+
 // scale [n] and, for asymmetric rows, zero [n] hold the row keys until the last launch writes the
 // steps and zero points there.  With l24 the workspace (dp_l24_work_bytes) must be zero on entry.
 cudaError_t launch_transform_quantize_dp(const void* x, int dtype, int64_t n, int64_t d, int k, const float* A, int bits,
@@ -442,6 +387,10 @@ cudaError_t launch_transform_quantize_dp(const void* x, int dtype, int64_t n, in
   m.asym = asym;
   m.planes = dp_planes(bits, asym);
   m.qmax = asym ? (float)((1 << bits) - 1) : (float)((1 << (bits - 1)) - 1);
+  if (dtype == 1 && !l24 && !rowsum) {   // bf16 rows without a range search or code sums: one tensor-core launch
+    const cudaError_t e = launch_transform_quantize_dp_fused(x, n, d, k, A, bits, asym, planes, scale, zero, status, stream);
+    if (e != cudaErrorNotSupported) return e;
+  }
   if (dtype == 0) return launch_dp_t(static_cast<const float*>(x), n, d, k, A, m, l24, planes, scale, zero, rowsum, work,
                                      status, stream);
   return launch_dp_t(static_cast<const __nv_bfloat16*>(x), n, d, k, A, m, l24, planes, scale, zero, rowsum, work, status,

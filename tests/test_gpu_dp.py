@@ -286,3 +286,42 @@ def test_dp_w4a4_equals_packed_path():
     wp = torch.from_numpy(dp_planes.encode(qw, 4, False)).to(DEV)
     y_dp = cat.cat_linear_dp(xp, 4, sx, wp, 4, sw)
     assert torch.equal(y_dp, y_packed)
+
+
+# ------------------------------------------------------------------------------------------
+# bf16 activations on tensor cores: the edges of the tiles and waves
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n,d,k,bits,asym", [(1, 256, 128, 8, True), (129, 192, 64, 6, True), (128, 192, 64, 8, False),
+                                             (257, 512, 256, 8, False), (140, 768, 256, 5, True),
+                                             (2600, 4096, 128, 8, True), (2561, 4096, 32, 8, False)])
+def test_dp_transform_tensor_core_edges(n, d, k, bits, asym):
+    """One row, ragged row tiles, 64-wide and 256-deep groups, and more units than tensor memory holds
+    (n = 2561 and 2600); a row with an infinity has step 0 and codes 0."""
+    rng = np.random.default_rng(n + d + bits)
+    X = rng.standard_normal((n, d)) * rng.lognormal(0, 1.0, d) + (0.3 if asym else 0.0)
+    bad = n // 2
+    Xt = WL.cast(X, "bf16")
+    T32 = (rng.standard_normal((d // k, k, k)) / np.sqrt(k)).astype(np.float32)
+    x = to_dev(Xt)
+    if n > 1:
+        x[bad, d - 3] = float("inf")
+    planes, sx, zx = cat.cat_transform_quantize_act_dp(x, torch.from_numpy(T32).to(DEV), k, bits, asym)
+    q = dp_planes.decode(planes.cpu().numpy())
+    keep = np.arange(n) != (bad if n > 1 else -1)
+    ref = O.transform_quantize_act(Xt.values[keep], T32.astype(np.float64), bits=bits, asymmetric=asym)
+    # codes up to 255: x' moves by up to ~1e-6 of the row's range in float32 sums of 256 terms, so a code lies
+    # within ~255e-6 of the oracle's boundary; four times that, and 1e-3 of the codes at most
+    diff = np.asarray(q[keep]) - ref.qx
+    assert np.abs(diff).max() <= 1
+    off = np.abs(ref.pre_x[diff != 0])
+    assert np.all(np.abs(off - np.floor(off) - 0.5) <= 1e-3)
+    assert np.mean(diff != 0) <= 1e-3
+    np.testing.assert_allclose(sx.cpu().numpy().astype(np.float64)[keep], ref.sx, rtol=1e-5)
+    if asym:
+        assert np.sum(zx.cpu().numpy()[keep] != ref.zx) <= max(1, 1e-3 * n)
+    if n > 1:
+        assert sx[bad].item() == 0.0 and np.all(q[bad] == 0)
+        assert cat.cat_device_status()[0] == 4
+    else:
+        assert cat.cat_device_status()[0] == 0
