@@ -12,43 +12,71 @@
 // an integer and adds them in int32; asymmetric activations then subtract z[t] times the weight row's
 // code sum (the zero-point correction), and the product is scaled by the two steps in fp32.
 //
-// Tile: 128 tokens (MMA M) x 128 output channels (MMA N) per CTA, K steps of 128 codes (one 128-byte
-// swizzle atom per row and plane).  One TMA producer thread loads, per K step, every digit plane of
-// the token tile and of the weight tile through a ring of stages (full / empty mbarriers); one thread
-// issues the MMAs (four of K = 32 per digit pair); four epilogue warps (thread = token row = TMEM
-// lane) read the accumulators, combine, scale and store y.  Every wait is bounded.
+// Tiles: 256 tokens (MMA M) x NB output channels per CTA pair (tcgen05.mma.cta_group::2): each CTA holds 128
+// token rows and NB / 2 channel rows, every digit plane of both, so a channel row loaded once serves 256
+// tokens.  A stage is KS codes of every plane (128, or 256 with one plane on either side): at the widest NB
+// 64 KB or 48 KB a CTA, for 1024 cycles of MMAs, i.e. 48-64 B per cycle from L2; one CTA with a 128 x 128
+// tile needed 64-96 and was held by that.  Persistent pairs, tiles in bands (tile_coords):
+//   warps 0, 2   TMA producers of the token and the channel planes (one thread each)
+//   warps 1, 3   even CTA: MMA issuers; odd CTA: forward its stages' readiness to the even CTA
+//   warps 4..11  epilogue: two warps per TMEM lane quadrant, half of the tile's channels each
+// The accumulators (one of NB columns per digit weight) are double-buffered where they fit twice in tensor
+// memory.  Where they don't, the epilogue adds them up into registers first (int32, NB / 2 a thread) and
+// gives tensor memory back before it scales and stores, so the next tile's MMAs wait for the loads only.
+// Measured (8-bit asymmetric activations x 4-bit weights, 2048 x 4096 -> 6144; 8 x 8 bits, 1000 x 14336
+// -> 4096): 230 and 185 us with one CTA per 128 x 128 tile and scalar stores, now 72 and 132 us; with one MMA
+// issuer instead of two the second takes 154 us.
+// Every wait is bounded.
 #include <cstring>
 #include <mutex>
 
 #include "common.cuh"
+#include "gemm_pair.cuh"
 
 namespace cat {
 namespace {
 
-constexpr int BM = 128, BN = 128, KB = 128;          // tokens, channels, codes (bytes) per K step
-constexpr uint32_t kTile = BM * KB;                  // 16 KiB per plane and operand (BN == BM)
-constexpr int kThreads = 192;                        // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
-constexpr int kEpiWarp0 = 2;
-constexpr size_t kSmemBudget = 200 * 1024;
+constexpr int BM = 128;                              // token rows per CTA (256 per pair)
+constexpr int KB = 128;                              // codes (bytes) of one 128-byte swizzle atom
+constexpr int kThreads = 384;
+constexpr int kEpiWarp0 = 4, kEpiWarps = 8;
+constexpr uint32_t kAtomA = BM * KB;                 // 16 KiB: one plane's atom of the token rows
+constexpr uint32_t kEpiStage = 32 * 32 * 4;          // y staging buffer of an epilogue warp
+constexpr int kMaxStages = 8;
 
-template <int DX, int DW>
+struct DpBars {
+  uint64_t full[kMaxStages], ready[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], mma_done;
+  uint32_t fwd_word[kMaxStages];                     // even CTA: targets of the odd CTA's st.async per stage
+  uint32_t tmem_addr;
+  int abort;
+};
+
+// DX, DW digit planes; NB channels per pair tile.
+template <int DX, int DW, int NB>
 struct DpGemmCfg {
-  static constexpr int G = DX + DW - 1;                                   // accumulators (digit weights)
-  static constexpr uint32_t STAGE = (uint32_t)(DX + DW) * kTile;
-  static constexpr int S = (int)(kSmemBudget / STAGE) < 8 ? (int)(kSmemBudget / STAGE) : 8;
-  static constexpr uint32_t TMEM_COLS = G * BN <= 128 ? 128 : (G * BN <= 256 ? 256 : 512);
-  static constexpr size_t SMEM = 1024 + (size_t)S * STAGE + 256;
-  static_assert(S >= 2, "stages");
+  // accumulators: one per digit weight; with one plane on either side one per atom of a stage, so that the
+  // two MMA issuers always have their own
+  static constexpr int G = DX + DW == 2 ? 2 : DX + DW - 1;
+  static constexpr int SHIFT = DX + DW == 2 ? 0 : 4;               // accumulator g stands for (1 << SHIFT g)
+  static constexpr int NACC = 2 * G * NB <= 512 ? 2 : 1;           // copies of them in tensor memory
+  static constexpr int AT = DX + DW == 2 ? 2 : 1;                  // atoms of codes per stage
+  static constexpr int KS = AT * KB;                               // codes per stage
+  static constexpr uint32_t ATOM_B = (uint32_t)(NB / 2) * KB;
+  static constexpr uint32_t A_BYTES = (uint32_t)(DX * AT) * kAtomA, B_BYTES = (uint32_t)(DW * AT) * ATOM_B;
+  static constexpr uint32_t STAGE = A_BYTES + B_BYTES;
+  static constexpr uint32_t EPI_OFF_MAX = 192 * 1024;
+  static constexpr int S = (int)(EPI_OFF_MAX / STAGE) < kMaxStages ? (int)(EPI_OFF_MAX / STAGE) : kMaxStages;
+  static constexpr uint32_t EPI_OFF = S * STAGE;
+  static constexpr uint32_t BAR_OFF = EPI_OFF + kEpiWarps * kEpiStage;
+  static constexpr size_t SMEM = BAR_OFF + 512 + 1024;
+  static constexpr uint32_t TMEM_COLS = NACC * G * NB <= 128 ? 128 : (NACC * G * NB <= 256 ? 256 : 512);
+  static constexpr int CH = NB / 64;                               // 32-column chunks per epilogue warp
+  static_assert(S >= 3 && SMEM <= 227 * 1024, "shared memory");
+  static_assert(sizeof(DpBars) <= 512 && STAGE % 1024 == 0 && G * NB <= 512, "layout");
 };
 
 // Bound of the pipeline waits (ns); kWaitLimitNs unless a test shortens it (cat_set_wait_limit_ns).
 __device__ uint64_t g_dp_wait_limit = kWaitLimitNs;
-
-struct DpBars {
-  uint64_t full[8], empty[8], acc_full, mma_done;
-  uint32_t tmem_addr;
-  int abort;
-};
 
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, int32_t x, int32_t y, int32_t z,
                                             uint64_t* bar) {
@@ -59,147 +87,244 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
-__device__ __forceinline__ void mma_ss_f8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{ .reg .pred p; setp.ne.b32 p, %4, 0; "
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p; }" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-template <int DX, int DW>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int DX, int DW, int NB>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     dp_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
-                   const float* __restrict__ sx, const int32_t* __restrict__ zx, const float* __restrict__ sw,
-                   const int32_t* __restrict__ w_rowsum, int n, int d_in, int d_out, float* __restrict__ y,
-                   int32_t* __restrict__ acc_out, uint32_t* __restrict__ status) {
-  using C = DpGemmCfg<DX, DW>;
+                   const __grid_constant__ CUtensorMap tmY, const float* __restrict__ sx, const int32_t* __restrict__ zx,
+                   const float* __restrict__ sw, const int32_t* __restrict__ w_rowsum, int n, int d_in, int d_out,
+                   float* __restrict__ y, int32_t* __restrict__ acc_out, int use_tma_store,
+                   uint32_t* __restrict__ status) {
+  using C = DpGemmCfg<DX, DW, NB>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  DpBars* bars = reinterpret_cast<DpBars*>(smem + (size_t)C::S * C::STAGE);
+  DpBars* bars = reinterpret_cast<DpBars*>(smem + C::BAR_OFF);
   volatile int* abort_flag = &bars->abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int o0 = blockIdx.x * BN, t0 = blockIdx.y * BM;
-  const int num_k = (d_in + KB - 1) / KB;
-  const uint64_t lim = g_dp_wait_limit;
+  const uint32_t rank = cluster_rank();               // 0: the pair's MMA issuer
+  const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+  const int num_m = (n + 2 * BM - 1) / (2 * BM), num_n = (d_out + NB - 1) / NB;
+  const int num_tiles = num_m * num_n;
+  const int num_k = (d_in + C::KS - 1) / C::KS;
 
   if (tid == 0) {
     for (int s = 0; s < C::S; ++s) {
-      mbar_init(&bars->full[s], 1);
-      mbar_init(&bars->empty[s], 1);
+      mbar_init(&bars->full[s], 2);                   // the two producers (+ 4 bytes from the odd CTA)
+      mbar_init(&bars->ready[s], 2);
+      mbar_init(&bars->empty[s], 2);                  // both MMA issuers' multicast commits
     }
-    mbar_init(&bars->acc_full, 1);
-    mbar_init(&bars->mma_done, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&bars->acc_full[b], 2);
+      mbar_init(&bars->acc_empty[b], 2 * kEpiWarps);  // the epilogue warps of both CTAs (even CTA)
+    }
+    mbar_init(&bars->mma_done, 2);
     bars->abort = 0;
     fence_mbar_init();
   }
-  pdl_wait_then_release();
-  if (warp == 1) tmem_alloc(&bars->tmem_addr, C::TMEM_COLS);
+  __syncwarp();
+  pdl_wait_then_release();                            // nothing global or in tensor memory before this
+  const uint64_t lim = g_dp_wait_limit;
+  if (warp == 0) tmem_alloc_pair(&bars->tmem_addr, C::TMEM_COLS);
   tc_fence_before();
-  __syncthreads();
+  cluster_sync();                                     // both CTAs' barriers are initialized before any remote arrive
   tc_fence_after();
   const uint32_t tmem = bars->tmem_addr;
 
-  if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer
+  if (warp == 0 || warp == 2) {
+    // ------------------------------------------------------------------ TMA producers (warp 0: tokens, warp 2: channels)
     if (lane == 0) {
-      prefetch_tensormap(&tmX);
-      prefetch_tensormap(&tmW);
-      int kb = 0;
-      for (; kb < num_k; ++kb) {
-        const int s = kb % C::S;
-        if (kb >= C::S && !mbar_wait_bounded(&bars->empty[s], ((kb / C::S) - 1) & 1, abort_flag, __LINE__, lim)) break;
-        uint8_t* st = smem + (size_t)s * C::STAGE;
-        mbar_arrive_expect_tx(&bars->full[s], C::STAGE);
+      const bool is_a = warp == 0;
+      const CUtensorMap* map = is_a ? &tmX : &tmW;
+      prefetch_tensormap(map);
+      uint32_t it = 0;
+      bool ok = true;
+      for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
+        int m, nn;
+        tile_coords(tile, num_m, num_n, &m, &nn);
+        const int row = is_a ? m * 2 * BM + (int)rank * BM : nn * NB + (int)rank * (NB / 2);
+        for (int ks = 0; ks < num_k; ++ks, ++it) {
+          const uint32_t s = it % C::S, use = it / C::S;
+          if (use > 0 && !(ok = mbar_wait_bounded(&bars->empty[s], (use - 1) & 1, abort_flag, __LINE__, lim))) break;
+          uint8_t* dst = smem + s * C::STAGE + (is_a ? 0u : C::A_BYTES);
+          uint64_t* fb = rank == 0 ? &bars->full[s] : &bars->ready[s];
+          mbar_arrive_expect_tx(fb, is_a ? C::A_BYTES + (rank == 0 ? 4u : 0u) : C::B_BYTES);
+          const int planes = is_a ? DX : DW;
+          const uint32_t atom = is_a ? kAtomA : C::ATOM_B;
+          for (int p = 0; p < planes; ++p)
 #pragma unroll
-        for (int p = 0; p < DX; ++p) tma_load_3d(st + p * kTile, &tmX, kb * KB, t0, p, &bars->full[s]);
-#pragma unroll
-        for (int p = 0; p < DW; ++p) tma_load_3d(st + (DX + p) * kTile, &tmW, kb * KB, o0, p, &bars->full[s]);
+            for (int at = 0; at < C::AT; ++at)
+              tma_load_3d(dst + (p * C::AT + at) * atom, map, ks * C::KS + at * KB, row, p, fb);
+        }
       }
-      // loads in flight land before the CTA exits (their stages were never waited for by the MMA
-      // thread if it gave up)
+      // the copies in flight land before the CTA exits (they have, unless a wait gave up)
       volatile int no_abort = 0;
-      for (int q = kb > C::S ? kb - C::S : 0; q < kb; ++q) mbar_wait_bounded(&bars->full[q % C::S], (q / C::S) & 1, &no_abort);
+      for (uint32_t j = it > (uint32_t)C::S ? it - C::S : 0; j < it; ++j)
+        mbar_wait_bounded(rank == 0 ? &bars->full[j % C::S] : &bars->ready[j % C::S], (j / C::S) & 1, &no_abort);
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
+  } else if ((warp == 1 || warp == 3) && rank == 1) {
+    // ------------------------------------------------------------------ odd CTA: forward stage readiness
+    // Each forwarder takes the stages of one parity, so that every barrier's phases are waited for in order
+    // by one thread, whatever the number of stages.
     if (lane == 0) {
-      constexpr uint32_t kIdesc = idesc_e4m3_f32(BM, BN);
-      bool started[C::G];
-#pragma unroll
-      for (int g = 0; g < C::G; ++g) started[g] = false;
-      for (int kb = 0; kb < num_k; ++kb) {
-        const int s = kb % C::S;
-        if (!mbar_wait_bounded(&bars->full[s], (kb / C::S) & 1, abort_flag, __LINE__, lim)) break;
+      const uint32_t grp = warp == 1 ? 0u : 1u;
+      uint32_t it = 0;
+      bool ok = true;
+      for (int tile = pair; tile < num_tiles && ok; tile += num_pairs)
+        for (int ks = 0; ks < num_k; ++ks, ++it) {
+          const uint32_t s = it % C::S;
+          if ((s & 1u) != grp) continue;
+          if (!(ok = mbar_wait_bounded(&bars->ready[s], (it / C::S) & 1, abort_flag, __LINE__, lim))) break;
+          tc_fence_after();
+          st_async_signal(&bars->fwd_word[s], &bars->full[s], 0);
+        }
+    }
+  } else if (warp == 1 || warp == 3) {
+    // ------------------------------------------------------------------ MMA issuers (even CTA)
+    // Two threads, each with accumulators of its own: a thread's wait for a stage returns only once its
+    // earlier MMAs have been handed on, and meanwhile the other's keep the tensor core busy.  Digit weights
+    // go to issuer g & 1 (equal work: weight 1 has two products where there are three); with one plane on
+    // either side each issuer takes one atom of the stage.
+    if (lane == 0) {
+      constexpr uint32_t kIdesc = idesc_e4m3_f32(2 * BM, NB);
+      const int me = warp == 1 ? 0 : 1;
+      uint32_t it = 0, tcount = 0;
+      bool ok = true;
+      for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++tcount) {
+        const uint32_t ab = tcount % C::NACC, use = tcount / C::NACC;
+        if (use > 0 && !(ok = mbar_wait_bounded(&bars->acc_empty[ab], (use - 1) & 1, abort_flag, __LINE__, lim))) break;
         tc_fence_after();
-        const uint32_t base = smem_u32(smem + (size_t)s * C::STAGE);
+        const uint32_t acc = tmem + ab * C::G * NB;
+        for (int ks = 0; ks < num_k; ++ks, ++it) {
+          const uint32_t s = it % C::S;
+          if (!(ok = mbar_wait_bounded(&bars->full[s], (it / C::S) & 1, abort_flag, __LINE__, lim))) break;
+          tc_fence_after();
+          const uint32_t abase = smem_u32(smem + s * C::STAGE), bbase = abase + C::A_BYTES;
 #pragma unroll
-        for (int a = 0; a < DX; ++a)
+          for (int a = 0; a < DX; ++a)
 #pragma unroll
-          for (int b = 0; b < DW; ++b) {
-            const int g = a + b;
-            const uint64_t da = sdesc_kmajor_sw128(base + a * kTile);
-            const uint64_t db = sdesc_kmajor_sw128(base + (DX + b) * kTile);
+            for (int b = 0; b < DW; ++b)
 #pragma unroll
-            for (int kk = 0; kk < KB / 32; ++kk) {   // K = 32 bytes (E4M3) per MMA: +32 B in the atom
-              mma_ss_f8(tmem + g * BN, da + 2 * kk, db + 2 * kk, kIdesc, started[g] ? 1u : 0u);
-              started[g] = true;
-            }
-          }
-        mma_commit(&bars->empty[s]);
+              for (int at = 0; at < C::AT; ++at) {
+                const int g = DX + DW == 2 ? at : a + b;
+                if ((g & 1) != me) continue;
+                // the pair (a, b) is the first one of its weight when a = 0 or b is the last plane
+                const bool first = a == 0 || b == DW - 1;
+#pragma unroll
+                for (int kk = 0; kk < KB / 32; ++kk) {    // K = 32 codes per MMA: +32 B within an atom
+                  const uint64_t da = sdesc_kmajor_sw128(abase + (uint32_t)(a * C::AT + at) * kAtomA) + 2 * kk;
+                  const uint64_t db = sdesc_kmajor_sw128(bbase + (uint32_t)(b * C::AT + at) * C::ATOM_B) + 2 * kk;
+                  mma_pair_ss(acc + g * NB, da, db, kIdesc, (ks != 0 || kk != 0 || !first) ? 1u : 0u);
+                }
+              }
+          mma_commit_pair(&bars->empty[s]);
+        }
+        if (ok) mma_commit_pair(&bars->acc_full[ab]);
       }
-      mma_commit(&bars->acc_full);
-      mma_commit(&bars->mma_done);
+      mma_commit_pair(&bars->mma_done);                // all MMAs complete before TMEM is released
       volatile int no_abort = 0;
       mbar_wait_bounded(&bars->mma_done, 0, &no_abort);
     }
-  } else {
+  } else if (warp >= kEpiWarp0) {
     // ------------------------------------------------------------------ epilogue: token row = TMEM lane
-    const int quad = warp & 3;
-    const int t = t0 + quad * 32 + lane;
-    const bool t_ok = t < n;
-    const float sxt = t_ok ? sx[t] : 0.f;
-    const int zt = (t_ok && zx) ? zx[t] : 0;
-    if (mbar_wait_bounded(&bars->acc_full, 0, abort_flag, __LINE__, lim)) {
+    const int quad = warp & 3, half = (warp - kEpiWarp0) >> 2;
+    uint8_t* buf = smem + C::EPI_OFF + (warp - kEpiWarp0) * kEpiStage;
+    uint32_t tcount = 0;
+    for (int tile = pair; tile < num_tiles; tile += num_pairs, ++tcount) {
+      const uint32_t ab = tcount % C::NACC;
+      int m, nn;
+      tile_coords(tile, num_m, num_n, &m, &nn);
+      const int row0 = m * 2 * BM + (int)rank * BM + quad * 32, t = row0 + lane;
+      const int col0 = nn * NB + half * (NB / 2);
+      const float sxt = t < n ? sx[t] : 0.f;
+      const uint32_t zt = (t < n && zx) ? (uint32_t)zx[t] : 0u;
+      if (!mbar_wait_bounded(&bars->acc_full[ab], (tcount / C::NACC) & 1, abort_flag, __LINE__, lim)) break;
       __syncwarp();
       tc_fence_after();
-#pragma unroll 1
-      for (int c = 0; c < BN / 32; ++c) {
-        int acc[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) acc[j] = 0;
+      const uint32_t tcol = tmem + ((uint32_t)(quad * 32) << 16) + ab * C::G * NB + half * (NB / 2);
+      auto gather = [&](int c, uint32_t (&acc)[32]) {  // chunk c: sum over the digit weights, int32
 #pragma unroll
         for (int g = 0; g < C::G; ++g) {
           uint32_t r[32];
           __syncwarp();
-          CAT_TMEM_LD32(tmem + ((uint32_t)(quad * 32) << 16) + g * BN + c * 32, r);
+          CAT_TMEM_LD32(tcol + g * NB + c * 32, r);
           tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) acc[j] += __float2int_rn(__uint_as_float(r[j]) * kAccScale) * (1 << (4 * g));
+          for (int j = 0; j < 32; ++j) {
+            const uint32_t v = (uint32_t)__float2int_rn(__uint_as_float(r[j]) * kAccScale) << (C::SHIFT * g);
+            acc[j] = g == 0 ? v : acc[j] + v;
+          }
         }
-        if (!t_ok) continue;
-        const int ob = o0 + c * 32;
-        float* yrow = y + (int64_t)t * d_out;
+      };
+      auto release = [&] {                             // the accumulators are read: the MMAs may have them back
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(&bars->acc_empty[ab], 0);
+      };
+      auto finish = [&](int c, uint32_t (&acc)[32]) {
+        const int o0 = col0 + c * 32;
+        if (o0 >= d_out || row0 >= n) return;          // warp-uniform: nothing of this chunk is in range
+        const bool in = o0 + lane < d_out;             // the chunk's 32 channel steps and code sums, one per lane
+        const float swl = in ? __ldg(sw + o0 + lane) : 0.f;
+        if (zx) {
+          // zero points: the result fits int32, so the difference may be taken modulo 2^32
+          const uint32_t rsl = in ? (uint32_t)__ldg(w_rowsum + o0 + lane) : 0u;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int o = ob + j;
-          if (o >= d_out) break;
-          // the zero-point correction in 64 bits: both terms fit int32, their difference too
-          const int a = (int)((long long)acc[j] - (zx ? (long long)zt * w_rowsum[o] : 0ll));
-          yrow[o] = (float)a * sxt * sw[o];
-          if (acc_out) acc_out[(int64_t)t * d_out + o] = a;
+          for (int j = 0; j < 32; ++j) acc[j] -= zt * __shfl_sync(0xFFFFFFFFu, rsl, j);
         }
+        if (acc_out && t < n) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (o0 + j < d_out) acc_out[(int64_t)t * d_out + o0 + j] = (int32_t)acc[j];
+        }
+        float v[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = (float)(int32_t)acc[j] * sxt * __shfl_sync(0xFFFFFFFFu, swl, j);
+        if (use_tma_store) {
+          if (lane == 0) bulk_wait_read_all();         // the store before has read the buffer
+          __syncwarp();
+#pragma unroll
+          for (int q = 0; q < 8; ++q)                  // row `lane`, 16-byte chunk q at q ^ (lane % 8)
+            *reinterpret_cast<float4*>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+                make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_2d(&tmY, buf, o0, row0);
+            bulk_commit();
+          }
+        } else if (t < n) {
+          float* yrow = y + (int64_t)t * d_out;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (o0 + j < d_out) yrow[o0 + j] = v[j];
+        }
+      };
+      if constexpr (C::NACC == 2) {                    // the other copy takes the next tile meanwhile
+#pragma unroll 1
+        for (int c = 0; c < C::CH; ++c) {
+          uint32_t acc[32];
+          gather(c, acc);
+          if (c == C::CH - 1) release();
+          finish(c, acc);
+        }
+      } else {
+        uint32_t acc[C::CH][32];
+#pragma unroll
+        for (int c = 0; c < C::CH; ++c) gather(c, acc[c]);
+        release();
+#pragma unroll
+        for (int c = 0; c < C::CH; ++c) finish(c, acc[c]);
       }
     }
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
   }
 
   tc_fence_before();
-  __syncthreads();
+  cluster_sync();                                     // the pair's MMAs and both epilogues are done with TMEM
   if (bars->abort && tid == 0) report(status, timeout_bits(kWhereGemmDp, bars->abort));
-  if (warp == 1) {
+  if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem, C::TMEM_COLS);
+    tmem_dealloc_pair(tmem, C::TMEM_COLS);
   }
 }
 
@@ -220,46 +345,107 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// Tensor map of D digit planes [D][rows][d_in] bytes: box 128 codes x 128 rows x 1 plane, 128B swizzle;
+// Tensor map of D digit planes [D][rows][d_in] bytes: box 128 codes x box_rows rows x 1 plane, 128B swizzle;
 // rows past the end read as zero.
-bool plane_map(CUtensorMap* map, const uint8_t* planes, int64_t rows, int64_t d_in, int D) {
+bool plane_map(CUtensorMap* map, const uint8_t* planes, int64_t rows, int64_t d_in, int D, int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   memset(map, 0, sizeof(*map));
   cuuint64_t dims[3] = {(cuuint64_t)d_in, (cuuint64_t)rows, (cuuint64_t)D};
   cuuint64_t strides[2] = {(cuuint64_t)d_in, (cuuint64_t)(rows * d_in)};
-  cuuint32_t box[3] = {(cuuint32_t)KB, (cuuint32_t)BM, 1};
+  cuuint32_t box[3] = {(cuuint32_t)KB, (cuuint32_t)box_rows, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(planes), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int DX, int DW>
-cudaError_t launch_dx_dw(const CUtensorMap& mx, const CUtensorMap& mw, const float* sx, const int32_t* zx,
-                         const float* sw, const int32_t* rowsum, int64_t n, int64_t d_in, int64_t d_out, float* y,
-                         int32_t* acc_out, uint32_t* status, cudaStream_t stream) {
-  using C = DpGemmCfg<DX, DW>;
+// y [n][d_out] float32, box 32 x 32, 128-byte swizzle (the epilogue's staging layout).
+bool output_map(CUtensorMap* map, float* y, int64_t n, int64_t d_out) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)d_out, (cuuint64_t)n};
+  cuuint64_t strides[1] = {(cuuint64_t)d_out * sizeof(float)};
+  cuuint32_t box[2] = {32, 32};
+  cuuint32_t estr[2] = {1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+         CUDA_SUCCESS;
+}
+
+int num_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 148;
+  return sms;
+}
+
+struct DpCall {
+  const uint8_t* x_planes;
+  const float* sx;
+  const int32_t* zx;
+  const uint8_t* w_planes;
+  const float* sw;
+  const int32_t* w_rowsum;
+  int64_t n, d_in, d_out;
+  float* y;
+  int32_t* acc_out;
+  uint32_t* status;
+  cudaStream_t stream;
+};
+
+template <int DX, int DW, int NB>
+cudaError_t launch_nb(const DpCall& c) {
+  using C = DpGemmCfg<DX, DW, NB>;
+  CUtensorMap mx, mw, my;
+  memset(&my, 0, sizeof(my));
+  if (!plane_map(&mx, c.x_planes, c.n, c.d_in, DX, BM) || !plane_map(&mw, c.w_planes, c.d_out, c.d_in, DW, NB / 2))
+    return cudaErrorInvalidValue;
+  const int use_tma = (c.d_out % 4 == 0 && output_map(&my, c.y, c.n, c.d_out)) ? 1 : 0;
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(dp_gemm_kernel<DX, DW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    attr = cudaFuncSetAttribute(dp_gemm_kernel<DX, DW, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
   });
   if (attr != cudaSuccess) return attr;
-  const int64_t gx = (d_out + BN - 1) / BN, gy = (n + BM - 1) / BM;
-  if (gx > 0x7FFFFFFF || gy > 65535) return cudaErrorInvalidValue;
+  const int64_t tiles = ((c.n + 2 * BM - 1) / (2 * BM)) * ((c.d_out + NB - 1) / NB);
+  if (tiles > 0x3FFFFFFF) return cudaErrorInvalidValue;
+  const int64_t pairs = num_sms() / 2;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)gx, (unsigned)gy, 1);
+  cfg.gridDim = dim3((unsigned)(2 * (tiles < pairs ? tiles : pairs)), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = C::SMEM;
-  cfg.stream = stream;
+  cfg.stream = c.stream;
   cudaLaunchAttribute attrs[1] = {pdl_attr()};
   cfg.attrs = attrs;
   cfg.numAttrs = 1;
   note_launch();
-  return cudaLaunchKernelEx(&cfg, dp_gemm_kernel<DX, DW>, mx, mw, sx, zx, sw, rowsum, (int)n, (int)d_in, (int)d_out, y,
-                            acc_out, status);
+  return cudaLaunchKernelEx(&cfg, dp_gemm_kernel<DX, DW, NB>, mx, mw, my, c.sx, c.zx, c.sw, c.w_rowsum, (int)c.n,
+                            (int)c.d_in, (int)c.d_out, c.y, c.acc_out, use_tma, c.status);
+}
+
+// The cycles a launch with NB-wide tiles should take: whole waves of tiles, each its stages (the MMAs of a
+// stage plus the ~200 cycles its barrier wait idles the tensor core, or the stage's loads at ~55 B per cycle
+// and SM) and an epilogue of ~8 cycles per column and accumulator.
+template <int DX, int DW, int NB>
+double tile_model(int64_t n, int64_t d_in, int64_t d_out, int64_t pairs) {
+  using C = DpGemmCfg<DX, DW, NB>;
+  const int64_t tiles = ((n + 2 * BM - 1) / (2 * BM)) * ((d_out + NB - 1) / NB);
+  const double mma = (double)DX * DW * (C::KS / 32) * (NB / 2) + 200.0, load = C::STAGE / 55.0;
+  const double stages = (double)((d_in + C::KS - 1) / C::KS);
+  return (double)((tiles + pairs - 1) / pairs) * (stages * (mma > load ? mma : load) + 8.0 * C::G * NB / C::NACC);
+}
+
+// Wide tiles load the token planes less often and have more MMA work behind each wait; narrow ones spread
+// a small call over more pairs.
+template <int DX, int DW>
+cudaError_t launch_dx_dw(const DpCall& c) {
+  constexpr int WIDE = DX + DW == 4 ? 128 : 256;     // G accumulators of WIDE columns fit tensor memory
+  const int64_t pairs = num_sms() / 2;
+  const double w0 = tile_model<DX, DW, WIDE>(c.n, c.d_in, c.d_out, pairs);
+  const double w1 = tile_model<DX, DW, WIDE / 2>(c.n, c.d_in, c.d_out, pairs);
+  return w1 < w0 ? launch_nb<DX, DW, WIDE / 2>(c) : launch_nb<DX, DW, WIDE>(c);
 }
 
 }  // namespace
@@ -272,12 +458,11 @@ cudaError_t launch_dp_gemm(const uint8_t* x_planes, int DX, const float* sx, con
                            int DW, const float* sw, const int32_t* w_rowsum, int64_t n, int64_t d_in, int64_t d_out,
                            float* y, int32_t* acc_out, uint32_t* status, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  CUtensorMap mx, mw;
-  if (!plane_map(&mx, x_planes, n, d_in, DX) || !plane_map(&mw, w_planes, d_out, d_in, DW)) return cudaErrorInvalidValue;
-  if (DX == 1 && DW == 1) return launch_dx_dw<1, 1>(mx, mw, sx, zx, sw, w_rowsum, n, d_in, d_out, y, acc_out, status, stream);
-  if (DX == 2 && DW == 1) return launch_dx_dw<2, 1>(mx, mw, sx, zx, sw, w_rowsum, n, d_in, d_out, y, acc_out, status, stream);
-  if (DX == 1 && DW == 2) return launch_dx_dw<1, 2>(mx, mw, sx, zx, sw, w_rowsum, n, d_in, d_out, y, acc_out, status, stream);
-  if (DX == 2 && DW == 2) return launch_dx_dw<2, 2>(mx, mw, sx, zx, sw, w_rowsum, n, d_in, d_out, y, acc_out, status, stream);
+  const DpCall c = {x_planes, sx, zx, w_planes, sw, w_rowsum, n, d_in, d_out, y, acc_out, status, stream};
+  if (DX == 1 && DW == 1) return launch_dx_dw<1, 1>(c);
+  if (DX == 2 && DW == 1) return launch_dx_dw<2, 1>(c);
+  if (DX == 1 && DW == 2) return launch_dx_dw<1, 2>(c);
+  if (DX == 2 && DW == 2) return launch_dx_dw<2, 2>(c);
   return cudaErrorInvalidValue;
 }
 

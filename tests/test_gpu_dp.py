@@ -325,3 +325,27 @@ def test_dp_transform_tensor_core_edges(n, d, k, bits, asym):
         assert cat.cat_device_status()[0] == 4
     else:
         assert cat.cat_device_status()[0] == 0
+
+
+@pytest.mark.parametrize("n,d_in,d_out,bx,bw,asym", [
+    (1, 32, 1, 8, 8, True), (255, 160, 258, 8, 4, True), (256, 128, 256, 4, 8, False), (513, 416, 1028, 4, 4, True),
+    (2300, 544, 9000, 8, 8, False), (2300, 544, 9001, 8, 4, True), (4600, 288, 9004, 4, 4, False)])
+def test_dp_linear_tile_edges(n, d_in, d_out, bx, bw, asym):
+    """Pair tiles with one row or one channel over, both tile widths and several tiles per pair: accumulators
+    equal to float64 products of the codes (exact), y = acc s_x s_w."""
+    rng = np.random.default_rng(n + d_in + d_out)
+    qx, qw = _rand_codes(rng, (n, d_in), bx, asym), _rand_codes(rng, (d_out, d_in), bw, False)
+    zx = rng.integers(0, 2 ** bx, n) if asym else np.zeros(n, dtype=np.int64)
+    sx = torch.from_numpy(rng.uniform(0.01, 2.0, n).astype(np.float32)).to(DEV)
+    sw = torch.from_numpy(rng.uniform(0.001, 0.1, d_out).astype(np.float32)).to(DEV)
+    kw = {}
+    if asym:
+        kw = dict(x_zero=torch.from_numpy(zx.astype(np.int32)).to(DEV),
+                  w_rowsum=torch.from_numpy(qw.sum(axis=1).astype(np.int32)).to(DEV))
+    acc = torch.full((n, d_out), -1, dtype=torch.int32, device=DEV)
+    y = cat.cat_linear_dp(torch.from_numpy(dp_planes.encode(qx, bx, asym)).to(DEV), bx, sx,
+                          torch.from_numpy(dp_planes.encode(qw, bw, False)).to(DEV), bw, sw, acc_out=acc, **kw)
+    ref = torch.from_numpy(qx - zx[:, None]).to(DEV).double() @ torch.from_numpy(qw).to(DEV).double().T
+    assert torch.equal(acc.double(), ref)
+    assert torch.equal(y, acc.float() * sx[:, None] * sw[None, :])
+    assert cat.cat_device_status()[0] == 0
