@@ -329,10 +329,10 @@ __device__ __forceinline__ void quant_chunk(uint32_t taddr, const QRow& qr, uint
 }
 
 // b-bit codes (digit planes).  The float32 estimate p = fl(v * inv) carries a relative error of at most
-// 3 * 2^-24 (inv has one rounding for symmetric rows, two for asymmetric ones, the product one more), so for
-// |p| <= 255 it is within 255 * 3 * 2^-24 < 2^-14 of the quotient: rint(p) is the exact code unless p lies
-// within 2^-14 of a half-integer, and there the decision is redone exactly.
-constexpr float kNearTieDp = 0.5f - 0x1p-14f;
+// 3 * 2^-24 (inv has one rounding for symmetric rows, two for asymmetric ones, the product one more), so with
+// |p| <= qmax it is within qmax * 2^-22 of the quotient: rint(p) is the exact code unless p lies that near a
+// half-integer, and there the decision is redone exactly.
+__device__ __forceinline__ float near_tie_dp(float qmax) { return 0.5f - qmax * 0x1p-22f; }
 
 // One row's grid: symmetric (lo unused) or asymmetric.
 struct DpRow {
@@ -367,9 +367,20 @@ __device__ __forceinline__ DpRow dp_row(float hi, float neg_lo, float qmax) {
     if (isfinite(w)) r.inv = __fdiv_rn(qmax, w);
     // z = round(N (-lo) / (hi - lo)), decided like a code
     const float p = __fmul_rn(neg_lo, r.inv), rq = rintf(p);
-    r.z = (fabsf(p - rq) <= kNearTieDp) ? (int)rq : asym_zero_exact(r.hi, r.lo, qmax);
+    r.z = (fabsf(p - rq) <= near_tie_dp(qmax)) ? (int)rq : asym_zero_exact(r.hi, r.lo, qmax);
   }
   return r;
+}
+
+// s = (hi - lo) / N of an asymmetric row: the sum's rounding error (two-sum) and the quotient's remainder (an
+// exact fma) correct one float32 division.  In float64 the watcher's divisions held the CTAs of block 0 (this
+// GPU's FP64 pipe is ~60 times slower): 4096 channels x 2048 tokens 31.9 us at 8 bits, now 23.6.
+__device__ __forceinline__ float asym_step(float hi, float neg_lo, float N) {
+  const float w = __fadd_rn(hi, neg_lo);
+  const float b = __fsub_rn(w, hi);
+  const float werr = __fadd_rn(__fsub_rn(hi, __fsub_rn(w, b)), __fsub_rn(neg_lo, b));
+  const float q = __fdiv_rn(w, N);
+  return __fadd_rn(q, __fdiv_rn(__fadd_rn(__fmaf_rn(-q, N, w), werr), N));
 }
 
 // The codes of the 32 values in tensor memory at taddr (this lane's row) as eight words of code bytes: two's
@@ -379,21 +390,33 @@ __device__ __forceinline__ void quant_chunk_dp(uint32_t taddr, const DpRow& row,
   constexpr float kMagic = 12582912.0f;
   constexpr int kMagicBits = 0x4B400000;
   int bq[32];
-  bool near = MODE == kDpSym && row.q.exact;
-  const int top = (int)qmax;
+  bool near = MODE == kDpSym && row.q.exact;   // rescaled rows take the exact route for every value
+  const float thr = near_tie_dp(qmax);
+  [[maybe_unused]] const int top = (int)qmax, zoff = row.z - kMagicBits;   // symmetric: the low byte is the code
   {
     uint32_t r[32];
     __syncwarp();
     CAT_TMEM_LD32(taddr, r);
     tmem_ld_wait();
-    const float scl = MODE == kDpSym ? row.q.sc : 1.f;   // rescaled rows take the exact route for every value
+    uint64_t inv2, mg2;                      // products and sums as f32x2 pairs, rounded as the scalar operations
+    asm("mov.b64 %0, {%1, %1};" : "=l"(inv2) : "f"(row.inv));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(mg2) : "f"(kMagic));
 #pragma unroll
-    for (int e = 0; e < 32; ++e) {
-      const float p = __fmul_rn(__uint_as_float(r[e]) * scl, row.inv);
-      const float rb = __fadd_rn(p, kMagic);
-      near |= !(fabsf(__fsub_rn(__fsub_rn(rb, kMagic), p)) <= kNearTieDp);
-      bq[e] = __float_as_int(rb) - kMagicBits;
-      if (MODE == kDpAsym) bq[e] = max(0, min(bq[e] + row.z, top));
+    for (int e = 0; e < 32; e += 2) {
+      uint64_t v2, p2, rb2, d2;
+      asm("mov.b64 %0, {%1, %2};" : "=l"(v2) : "r"(r[e]), "r"(r[e + 1]));
+      asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(p2) : "l"(v2), "l"(inv2));
+      asm("add.rn.f32x2 %0, %1, %2;" : "=l"(rb2) : "l"(p2), "l"(mg2));
+      asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d2) : "l"(rb2), "l"(mg2));
+      asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d2) : "l"(d2), "l"(p2));
+      float d0, d1;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(d2));
+      asm("mov.b64 {%0, %1}, %2;" : "=r"(bq[e]), "=r"(bq[e + 1]) : "l"(rb2));
+      near |= !(fabsf(d0) <= thr) || !(fabsf(d1) <= thr);
+      if (MODE == kDpAsym) {
+        bq[e] = max(0, min(bq[e] + zoff, top));
+        bq[e + 1] = max(0, min(bq[e + 1] + zoff, top));
+      }
     }
   }
   if (__any_sync(0xFFFFFFFFu, near)) {
@@ -406,7 +429,7 @@ __device__ __forceinline__ void quant_chunk_dp(uint32_t taddr, const DpRow& row,
       for (int e = 0; e < 32; ++e) {
         const float v = __uint_as_float(r[e]);
         const float p = __fmul_rn(v, row.inv);
-        const bool here = !(fabsf(__fsub_rn(__fsub_rn(__fadd_rn(p, kMagic), kMagic), p)) <= kNearTieDp);
+        const bool here = !(fabsf(__fsub_rn(__fsub_rn(__fadd_rn(p, kMagic), kMagic), p)) <= thr);
         if (MODE == kDpSym) {
           if (row.q.exact || here) bq[e] = qcode_exact_dp(v, row.q, qmax);
         } else if (here) {
@@ -959,7 +982,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc_fence_after();
           const uint32_t xbase = smem_u32(xs + st * F::X_STAGE);
 #pragma unroll
-          for (int sp = 0; sp < 3; ++sp) {
+          for (int i = 0; i < 3; ++i) {
+            // b-bit codes are finer: their planes go smallest first, so that the M and L sums round at their
+            // own size (measured against float64, layer outputs at 8 bits are as exact as the SIMT kernel's)
+            const int sp = MODE == kW4 ? i : 2 - i;
             if (own_planes && q == 0) {                 // later stages find every plane in place
               if (!(ok = mbar_wait_bounded(&plane_full[sp], 0, abort_flag, __LINE__))) break;
               tc_fence_after();
@@ -970,7 +996,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const uint32_t a_off = (kk >> 2) * (TM * 128) + (kk & 3) * 32;
               const uint32_t b_off = (kg >> 2) * (N * 128) + (kg & 3) * 32;
               mma_bf16(dcol, sdesc_kmajor_sw128(xbase + a_off), sdesc_kmajor_sw128(tbase + sp * F::SPLIT + b_off),
-                       F::IDESC, (h | kk | sp) != 0);
+                       F::IDESC, (h | kk | i) != 0);
             }
           }
           if (!ok) break;
@@ -1029,9 +1055,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           float sc = 0.f;
           if constexpr (MODE == kDpAsym) {
             const float neg_lo = __uint_as_float(vl[i]);
-            const AsymRow ar = asym_row(a, -neg_lo, dp.qmax);
+            const DpRow ar = dp_row<kDpAsym>(a, neg_lo, dp.qmax);
             if (!(isfinite(a) && isfinite(neg_lo))) report(status, kStatusNonFinite);
-            if (ar.inv != 0.f) sc = (float)(ar.r / (double)dp.qmax);
+            if (ar.inv != 0.f) sc = asym_step(a, neg_lo, dp.qmax);
             dp.zero[t] = ar.z;
           } else if (isfinite(a)) {
             sc = __fdiv_rn(a, MODE == kW4 ? 7.0f : dp.qmax);
