@@ -122,9 +122,10 @@ cat_status cat_calib_cov(const void* x, cat_dtype dtype, int64_t n, int64_t d, i
  *   T_blocks       out, device [d_in/k][k][k] float32: the online activation transform T.
  *   Wq             out, device [d_out][d_in/2] bytes: SM4x8 codes of W T^{-1}.
  *   w_scale        out, device [d_out] float32: per-output-channel step s_w = max_i |W'_{o,i}| / 7.
- * Synchronous: it reads the calibration sums back, builds T and T^{-1} in float64 on the host
- * (per block, in parallel over host threads), uploads them, and runs the weight kernels; it
- * returns after the outputs are written.  It allocates and frees its own temporaries.
+ * Synchronous: it returns after the outputs are written.  CAT and CAT_HD blocks of k <= 128 are built
+ * on the device in float64; the other kinds, k = 256, and a layer with a block whose condition number
+ * may exceed 1e11 or that is not positive definite are built on the host in float64 (per block, in
+ * parallel over host threads) from the sums read back.  It allocates and frees its own temporaries.
  * Returns CAT_ERR_NUMERIC if a Sigma_x or Sigma_w block is not positive definite.
  */
 cat_status cat_quantize_weights(const void* W, cat_dtype dtype, int64_t d_out, int64_t d_in, int32_t k,
@@ -137,7 +138,7 @@ cat_status cat_quantize_weights(const void* W, cat_dtype dtype, int64_t d_out, i
  * in the paper: it exists for callers that cannot take new device memory mid-run, e.g. a process
  * that has handed all free device memory to its own pool and re-quantizes a layer later (after
  * re-calibration), where a new allocation would fail or evict that pool.
- * Same arguments, steps and results as cat_quantize_weights.  Its two temporaries (the float64
+ * Same arguments and results as cat_quantize_weights (T is always built on the host).  Its two temporaries (the float64
  * Sigma_w blocks and the float32 blocks (T_b^{-1})^T, 12 bytes per element of d_in * k) live in a
  * fixed 12 MiB scratch area that the library reserves statically on every device it is loaded on.
  *   Limit: d_in * k <= CAT_PREP_NOALLOC_MAX_DK; a larger call returns CAT_ERR_SHAPE before any

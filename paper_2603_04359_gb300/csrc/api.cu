@@ -27,6 +27,10 @@ cudaError_t launch_codes_to_e4m3(const uint8_t* codes, int64_t rows, int64_t d, 
 cudaError_t launch_block_row_stats(const void* V, int dtype, int64_t rows, int64_t d, int k, const float* M,
                                    int transpose, float* row_sumsq, float* row_amax, double* out3,
                                    cudaStream_t stream);
+bool transform_dev_supported(int k, int64_t nb);
+size_t transform_dev_bytes(int k, int64_t nb);
+cudaError_t launch_build_transform(int k, int64_t nb, const double* sx, int64_t n_calib, const double* sw, int with_h,
+                                   float* T, float* Aw, void* work, const int** flags, cudaStream_t s);
 int dp_planes(int bits, int asym);
 cudaError_t launch_block_transform(const void* V, int dtype, int64_t rows, int64_t d, int k, const float* M,
                                    int transpose, float* Vt, cudaStream_t stream);
@@ -255,6 +259,67 @@ cat_status cat_build_transform_host(cat_tkind kind, int64_t d_in, int32_t k, con
   return ok();
 }
 
+// The layer's T (to T_blocks) and A_w = (T^{-1})^T (to aw_d), both float32 [d_in/k][k][k] on the device: A_w maps
+// a weight row w to its (W T^{-1}) row.  Synchronizes the stream; on an error T_blocks is untouched.
+// CAT and CAT_HD with k <= 128 are built on the device (transform_dev.cu); the kinds without calibration, the
+// diagonal one, k = 256, and a layer with a block that the device build does not decide (not positive definite,
+// or too near it) are built on the host in float64, which also gives that layer's error.
+static cat_status build_layer_transform(const void* W, cat_dtype dtype, int64_t d_out, int64_t d_in, int32_t k,
+                                        cat_tkind kind, const double* sigma_x_blocks, int64_t n_calib,
+                                        const float* rht_signs, float* T_blocks, float* aw_d, uint32_t* status,
+                                        cudaStream_t s) {
+  const int64_t nb = d_in / k;
+  const size_t kk = (size_t)k * k, nblk = (size_t)nb * kk;
+  std::vector<double> sx_h, sw_h;
+  cudaError_t e;
+  if (kind == CAT_T_CAT || kind == CAT_T_DIAG || kind == CAT_T_CAT_HD) {
+    double* sw_d = nullptr;
+    if ((e = cudaMallocAsync((void**)&sw_d, nblk * sizeof(double), s)) != cudaSuccess) return cuda_fail(e, "cudaMallocAsync");
+    e = cat::launch_calib_cov(W, (int)dtype, d_out, d_in, k, sw_d, 0, status, s);  // Sigma_w = W^T W blocks
+    void* work = nullptr;
+    if (e == cudaSuccess && kind != CAT_T_DIAG && cat::transform_dev_supported(k, nb) &&
+        cudaMallocAsync(&work, cat::transform_dev_bytes(k, nb), s) == cudaSuccess) {
+      const int* flags = nullptr;
+      int raised[3] = {1, 1, 1};
+      e = cat::launch_build_transform(k, nb, sigma_x_blocks, n_calib, sw_d, kind == CAT_T_CAT ? 1 : 0, T_blocks, aw_d,
+                                      work, &flags, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(raised, flags, sizeof(raised), cudaMemcpyDeviceToHost, s);
+      cudaFreeAsync(work, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess || !(raised[0] | raised[1] | raised[2])) {
+        cudaFreeAsync(sw_d, s);
+        return e == cudaSuccess ? CAT_OK : cuda_fail(e, "device transform build");
+      }
+    } else {
+      cudaGetLastError();   // no scratch for the device build: the host one needs none
+    }
+    sx_h.resize(nblk);
+    sw_h.resize(nblk);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sx_h.data(), sigma_x_blocks, nblk * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sw_h.data(), sw_d, nblk * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFreeAsync(sw_d, s);
+    if (e != cudaSuccess) return cuda_fail(e, "Sigma_w / Sigma_x readback");
+  }
+  std::vector<double> T(nblk), Ti(nblk);
+  cat_status st = cat_build_transform_host(kind, d_in, k, sx_h.empty() ? nullptr : sx_h.data(), n_calib,
+                                           sw_h.empty() ? nullptr : sw_h.data(), rht_signs, T.data(), Ti.data());
+  if (st != CAT_OK) return st;
+  std::vector<float> Tf(nblk), Awf(nblk);
+  for (int64_t b = 0; b < nb; ++b)
+    for (int i = 0; i < k; ++i)
+      for (int j = 0; j < k; ++j) {
+        Tf[b * kk + (size_t)i * k + j] = (float)T[b * kk + (size_t)i * k + j];
+        Awf[b * kk + (size_t)i * k + j] = (float)Ti[b * kk + (size_t)j * k + i];
+      }
+  e = cudaMemcpyAsync(T_blocks, Tf.data(), nblk * sizeof(float), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(aw_d, Awf.data(), nblk * sizeof(float), cudaMemcpyHostToDevice, s);
+  cudaError_t e2 = cudaStreamSynchronize(s);  // host buffers above must outlive the copies
+  if (e != cudaSuccess) return cuda_fail(e, "transform upload");
+  if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamSynchronize");
+  return CAT_OK;
+}
+
 cat_status cat_quantize_weights(const void* W, cat_dtype dtype, int64_t d_out, int64_t d_in, int32_t k,
                                 cat_tkind kind, const double* sigma_x_blocks, int64_t n_calib,
                                 const float* rht_signs, float* T_blocks, uint8_t* Wq, float* w_scale,
@@ -279,51 +344,26 @@ cat_status cat_quantize_weights(const void* W, cat_dtype dtype, int64_t d_out, i
   if ((st = check_device()) != CAT_OK) return st;
 
   cudaStream_t s = (cudaStream_t)stream;
-  const int64_t nb = d_in / k;
-  const size_t kk = (size_t)k * k, nblk = (size_t)nb * kk;
-  std::vector<double> sx_h, sw_h;
+  const size_t nblk = (size_t)d_in * k;
   cudaError_t e;
-  if (cat_like) {
-    double* sw_d = nullptr;
-    if ((e = cudaMallocAsync((void**)&sw_d, nblk * sizeof(double), s)) != cudaSuccess) return cuda_fail(e, "cudaMallocAsync");
-    uint32_t* st_word = status_word(&e);
-    if (!st_word) return cuda_fail(e, "status word");
-    e = cat::launch_calib_cov(W, (int)dtype, d_out, d_in, k, sw_d, 0, st_word, s);  // Sigma_w = W^T W blocks
-    sx_h.resize(nblk);
-    sw_h.resize(nblk);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sx_h.data(), sigma_x_blocks, nblk * sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sw_h.data(), sw_d, nblk * sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(sw_d, s);
-    if (e != cudaSuccess) return cuda_fail(e, "Sigma_w / Sigma_x readback");
-  }
-  std::vector<double> T(nblk), Ti(nblk);
-  st = cat_build_transform_host(kind, d_in, k, sx_h.empty() ? nullptr : sx_h.data(), n_calib,
-                                sw_h.empty() ? nullptr : sw_h.data(), rht_signs, T.data(), Ti.data());
-  if (st != CAT_OK) return st;
-  // Upload T (online transform) and A_w = (T^{-1})^T, which maps a weight row w to (W T^{-1}) row.
-  std::vector<float> Tf(nblk), Awf(nblk);
-  for (int64_t b = 0; b < nb; ++b)
-    for (int i = 0; i < k; ++i)
-      for (int j = 0; j < k; ++j) {
-        Tf[b * kk + (size_t)i * k + j] = (float)T[b * kk + (size_t)i * k + j];
-        Awf[b * kk + (size_t)i * k + j] = (float)Ti[b * kk + (size_t)j * k + i];
-      }
-  float* aw_d = nullptr;
   uint32_t* status = status_word(&e);
   if (!status) return cuda_fail(e, "status word");
+  float* aw_d = nullptr;
   if ((e = cudaMallocAsync((void**)&aw_d, nblk * sizeof(float), s)) != cudaSuccess) return cuda_fail(e, "cudaMallocAsync");
-  e = cudaMemcpyAsync(T_blocks, Tf.data(), nblk * sizeof(float), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(aw_d, Awf.data(), nblk * sizeof(float), cudaMemcpyHostToDevice, s);
+  st = build_layer_transform(W, dtype, d_out, d_in, k, kind, sigma_x_blocks, n_calib, rht_signs, T_blocks, aw_d, status, s);
+  if (st != CAT_OK) {
+    cudaFreeAsync(aw_d, s);
+    return st;
+  }
   if (kind == CAT_T_CAT_HD) {
     // W' = W M^{-1} H_d: the rows through the blocks (M_b^{-1})^T, the full-size Hadamard, then the
     // codes of the float32 rows (identity blocks)
-    if (e == cudaSuccess) e = transform_fwht_quantize(W, (int)dtype, d_out, d_in, k, aw_d, 1, Wq, w_scale, status, s);
-  } else if (e == cudaSuccess) {
+    e = transform_fwht_quantize(W, (int)dtype, d_out, d_in, k, aw_d, 1, Wq, w_scale, status, s);
+  } else {
     e = cat::launch_transform_quantize(W, (int)dtype, d_out, d_in, k, aw_d, Wq, w_scale, status, s);
   }
   cudaFreeAsync(aw_d, s);
-  cudaError_t e2 = cudaStreamSynchronize(s);  // host buffers above must outlive the copies
+  cudaError_t e2 = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "weight quantization");
   if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamSynchronize");
   return ok();
@@ -453,48 +493,24 @@ cat_status cat_quantize_weights_dp(const void* W, cat_dtype dtype, int64_t d_out
   if ((st = check_device()) != CAT_OK) return st;
 
   cudaStream_t s = (cudaStream_t)stream;
-  const int64_t nb = d_in / k;
-  const size_t kk = (size_t)k * k, nblk = (size_t)nb * kk;
-  std::vector<double> sx_h, sw_h;
+  const size_t nblk = (size_t)d_in * k;
   cudaError_t e;
-  if (kind == CAT_T_CAT) {
-    double* sw_d = nullptr;
-    if ((e = cudaMallocAsync((void**)&sw_d, nblk * sizeof(double), s)) != cudaSuccess) return cuda_fail(e, "cudaMallocAsync");
-    uint32_t* st_word = status_word(&e);
-    if (!st_word) return cuda_fail(e, "status word");
-    e = cat::launch_calib_cov(W, (int)dtype, d_out, d_in, k, sw_d, 0, st_word, s);  // Sigma_w = W^T W blocks
-    sx_h.resize(nblk);
-    sw_h.resize(nblk);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sx_h.data(), sigma_x_blocks, nblk * sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sw_h.data(), sw_d, nblk * sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(sw_d, s);
-    if (e != cudaSuccess) return cuda_fail(e, "Sigma_w / Sigma_x readback");
-  }
-  std::vector<double> T(nblk), Ti(nblk);
-  st = cat_build_transform_host(kind, d_in, k, sx_h.empty() ? nullptr : sx_h.data(), n_calib,
-                                sw_h.empty() ? nullptr : sw_h.data(), rht_signs, T.data(), Ti.data());
-  if (st != CAT_OK) return st;
-  std::vector<float> Tf(nblk), Awf(nblk);
-  for (int64_t b = 0; b < nb; ++b)
-    for (int i = 0; i < k; ++i)
-      for (int j = 0; j < k; ++j) {
-        Tf[b * kk + (size_t)i * k + j] = (float)T[b * kk + (size_t)i * k + j];
-        Awf[b * kk + (size_t)i * k + j] = (float)Ti[b * kk + (size_t)j * k + i];
-      }
   uint32_t* status = status_word(&e);
   if (!status) return cuda_fail(e, "status word");
   float* aw_d = nullptr;
   void* work = nullptr;
   const size_t work_bytes = l24_range ? cat::dp_l24_work_bytes(d_out) : 0;
   if ((e = cudaMallocAsync((void**)&aw_d, nblk * sizeof(float), s)) != cudaSuccess) return cuda_fail(e, "cudaMallocAsync");
+  st = build_layer_transform(W, dtype, d_out, d_in, k, kind, sigma_x_blocks, n_calib, rht_signs, T_blocks, aw_d, status, s);
+  if (st != CAT_OK) {
+    cudaFreeAsync(aw_d, s);
+    return st;
+  }
   if (work_bytes && (e = cudaMallocAsync(&work, work_bytes, s)) != cudaSuccess) {
     cudaFreeAsync(aw_d, s);
     return cuda_fail(e, "cudaMallocAsync");
   }
   if (work_bytes) e = cudaMemsetAsync(work, 0, work_bytes, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(T_blocks, Tf.data(), nblk * sizeof(float), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(aw_d, Awf.data(), nblk * sizeof(float), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cat::launch_transform_quantize_dp(W, (int)dtype, d_out, d_in, k, aw_d, bits, 0, l24_range, planes, w_scale,
                                           nullptr, w_rowsum, work, status, s);

@@ -508,3 +508,37 @@ def test_gemm_f32(m, n, kd):
     C = cat.cat_gemm_f32(torch.from_numpy(A).to(DEV), torch.from_numpy(B).to(DEV)).cpu().numpy()
     ref = A.astype(np.float64) @ B.astype(np.float64).T
     assert np.max(np.abs(C - ref)) <= 1e-5 * np.sqrt(kd) * np.max(np.abs(ref)) + 1e-6
+
+
+# ------------------------------------------------------------------------------------------
+# The transform built on the device
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("d,k,spread", [(32, 16, 1.0), (96, 32, 30.0), (64, 64, 1.0), (1280, 128, 100.0), (256, 128, 3e5)])
+def test_device_transform_matches_host(d, k, spread):
+    """T from cat_quantize_weights against the host builder's float64 T on the same statistics (float32 inputs: the
+    autocorrelations are exact to ~1e-12).  Both are good to ~1e-15 x the blocks' condition (1e11 at most on the
+    device, 3e5^2 and more go to the host), far below float32: T agrees to one float32 rounding."""
+    rng = np.random.default_rng(d + k)
+    X = rng.standard_normal((4 * k, d)) @ (np.eye(d) + 0.5 * rng.standard_normal((d, d)) / np.sqrt(d))
+    X[:, :: max(2, d // 5)] *= spread
+    W = 0.02 * rng.standard_normal((2 * d + 40, d)) * rng.lognormal(0, 0.5, (2 * d + 40, 1))
+    x, w = (torch.from_numpy(a.astype(np.float32)).cuda() for a in (X, W))
+    sig = cat.cat_calib_cov(x, k)
+    T, _, _ = cat.cat_quantize_weights(w, k, "cat", sigma_x=sig, n_calib=4 * k)
+    ref, _ = cat.cat_build_transform_host("cat", d, k, sig.cpu().numpy(), 4 * k, cat.cat_calib_cov(w, k).cpu().numpy())
+    got = T.cpu().numpy().astype(np.float64)
+    scale = np.abs(ref).max(axis=(1, 2), keepdims=True)
+    assert np.all(np.abs(got - ref) <= 2.0 ** -23 * np.abs(ref) + 1e-9 * scale)
+
+
+def test_device_transform_refuses_singular_blocks():
+    """One block without full rank (fewer tokens than channels) is refused as before: CAT_ERR_NUMERIC."""
+    rng = np.random.default_rng(5)
+    x = torch.from_numpy(rng.standard_normal((40, 128)).astype(np.float32)).cuda()
+    w = torch.from_numpy(rng.standard_normal((300, 128)).astype(np.float32)).cuda()
+    with pytest.raises(cat.CatError) as err:
+        cat.cat_quantize_weights(w, 64, "cat", sigma_x=cat.cat_calib_cov(x, 64), n_calib=40)
+    assert err.value.status == 4
+    T, _, _ = cat.cat_quantize_weights(w, 32, "cat", sigma_x=cat.cat_calib_cov(x, 32), n_calib=40)   # 40 tokens: full rank
+    assert torch.isfinite(T).all()
