@@ -10,30 +10,42 @@
 //   * two producer warps stream 16 KiB packed weight tiles (128 rows x 128 bytes = 256 codes,
 //     128-byte swizzle) through a TMA ring -- two issuers, because one issuer's TMA rate is below
 //     the per-SM share of HBM bandwidth;
-//   * sixteen decode warps, in four groups taking every fourth K step (the decode of a step is a
-//     latency chain), turn each tile into E4M3 in tensor memory (thread = weight row = TMEM lane,
-//     the whole 256 codes);
-//   * one thread issues tcgen05.mma (A from tensor memory, B from shared memory), accumulating the
-//     exact products q_x q_w 2^-18 in fp32 (|acc| <= 49 d_in < 2^24);
-//   * four epilogue warps read the double-buffered accumulator (thread = output channel) and write
+//   * twelve decode warps, in three groups taking every third K step, turn each tile into E4M3 in
+//     tensor memory (thread = weight row = TMEM lane, the whole 256 codes).  Six stages of 64 columns,
+//     two a group, so a group decodes its next step while the MMAs of its last one run;
+//   * two threads issue tcgen05.mma (A from tensor memory, B from shared memory), on alternate K steps
+//     into accumulators of their own, the exact products q_x q_w 2^-18 in fp32 (|acc| <= 49 d_in < 2^24).
+//     One thread issues an MMA about every 55 cycles whatever N is; a decode warp that issued them
+//     itself stood still meanwhile (a step took its group ~1.5 us, and four K steps per group were the
+//     kernel's time at 4096 channels);
+//   * four epilogue warps read the double-buffered accumulators (thread = output channel) and write
 //     y[t][o] with consecutive o across a warp; y_ref, when given, is loaded while the MMAs run.
-// Work split (stream-K): the (unit, K step) sequence -- unit-major, num_units x num_ks steps of
-// 16 KiB -- is cut into one contiguous, equal range per CTA, one CTA per SM, so every SM streams
-// the same number of weight bytes whatever the number of units (with 128-row units alone, 112 units
-// at d_out = 14336 left 40 of 152 SMs idle).  A unit whose steps fall into one CTA's range is
-// finished there.  A unit cut between CTAs is owned by the CTA holding its first step, where it is
-// the last segment of the range; every other part is the first segment of its CTA's range, so it
-// is done early: it stores its raw accumulators (integers times 2^-18, exact in fp32) to its CTA's
-// slice of device scratch and bumps the unit's per-warp counter.  The owner waits (bounded) for the
-// counter while its own MMAs run, loads the other slices, adds them (an exact sum in any order),
-// writes y and resets the counter.  The launch is cooperative, so all parts are resident while the
-// owners wait.  Every mbarrier wait is bounded; a wait that gives up raises the device status word
+// Work split, three forms, chosen by pick_parts:
+//   * whole 128-row units, one contiguous range of units per CTA (parts = 1);
+//   * fewer units than SMs, or rows too long for a CTA's shared memory: a unit's K steps are cut over a
+//     cluster of 2, 4 or 8 CTAs, which exchange their accumulators through distributed shared memory;
+//     each finishes 128 / parts of the unit's channels (no global scratch, no waiting beyond the
+//     cluster's barrier).  A CTA then keeps only its own K steps of the tokens in shared memory, so rows up
+//     to eight times as long run here: 27 tokens through 14336 -> 4096 took 25 us on the mma.sync
+//     kernel, 14.6 now, one token through 4096 -> 6144 10.4, now 8.1 (cluster of 2);
+//   * more units than SMs (stream-K): the (unit, K step) sequence -- unit-major, num_units x num_ks steps
+//     of 16 KiB -- is cut into one contiguous, equal range per CTA, one CTA per SM, so every SM streams
+//     the same number of weight bytes.  A unit whose steps fall into one CTA's range is
+//     finished there.  A unit cut between CTAs is owned by the CTA holding its first step, where it is
+//     the last segment of the range; every other part is the first segment of its CTA's range, so it
+//     is done early: it stores its raw accumulators (integers times 2^-18, exact in fp32) to its CTA's
+//     slice of device scratch and bumps the unit's per-warp counter.  The owner waits (bounded) for the
+//     counter while its own MMAs run, loads the other slices, adds them (an exact sum in any order),
+//     writes y and resets the counter.  The launch is cooperative, so all parts are resident while the
+//     owners wait.
+// Every mbarrier wait is bounded; a wait that gives up raises the device status word
 // and all roles drain and exit.
 #include <atomic>
 #include <cstring>
 #include <mutex>
 
 #include "common.cuh"
+#include "gemm_pair.cuh"
 #include "sqnr_slot.cuh"
 
 namespace cat {
@@ -42,28 +54,23 @@ namespace {
 constexpr int UM = 128;                      // weight rows per unit (MMA M)
 constexpr int KSB = 128;                     // packed bytes per row per K step (256 codes)
 constexpr uint32_t kPkStage = UM * KSB;      // 16 KiB packed tile
-constexpr int kMaxSP = 8;                    // packed stages (runtime count <= this)
-constexpr int kMaxSE = 8;                    // decoded A stages in tensor memory, 64 columns each
-constexpr int kThreads = 768;
-constexpr int kProd0 = 0, kProd1 = 2;
-constexpr int kStageWarp0 = 3;               // warps 3.. stage the token operand at the start
-constexpr int kDecWarp0 = 4, kDecWarps = 16, kDecGroups = 4;
-constexpr int kEpiWarp0 = 20, kEpiWarps = 4;
-constexpr int kTokLoads = 4;                 // token loads in flight per staging thread
-constexpr int kGroupBar0 = 4;                // named barriers 4..7: the four warps of a decode group
+constexpr int kMaxSP = 9;                    // packed stages (runtime count <= this)
+constexpr int kSE = 6;                       // decoded A stages in tensor memory, 64 columns each
+constexpr int kThreads = 640;
+constexpr int kProd0 = 0, kIss0 = 1, kProd1 = 2, kIss1 = 3;
+constexpr int kDecWarp0 = 4, kDecWarps = 12, kDecGroups = 3;
+constexpr int kIssuers = 2;
+constexpr int kEpiWarp0 = 16, kEpiWarps = 4;
+constexpr int kStageWarp0 = 4;               // warps 4.. stage the token operand at the start
+constexpr int kMaxParts = 8;                 // CTAs of a cluster sharing a unit
 
-// Tensor memory: accumulator (group g, buffer b) at column (b * kDecGroups + g) * NTOK, then the
-// decoded A stages of 64 columns.  Stage s is only ever used by group s % kDecGroups, and packed
-// stage ps only by group ps % kDecGroups (both counts are multiples of the group count): every
-// mbarrier phase a group waits for is then the one after the phase it last saw.
+// Tensor memory: accumulator (issuer i, buffer b) at column (b * kIssuers + i) * NTOK, then the decoded A
+// stages.  Packed stage ps is only ever used by group ps % kDecGroups and producer ps % 2, decoded stage s by
+// group s % kDecGroups and issuer s % 2 (both counts are multiples of the group count, kSE of the issuers):
+// every mbarrier phase a role waits for is then the one after the phase it last saw.
 template <int NTOK>
-struct TmemPlan {
-  static constexpr uint32_t kAccCols = 2u * kDecGroups * NTOK;
-  // two stages per group where they fit (a group decodes its next step while the MMAs of the last
-  // one run), else one
-  static constexpr int kSE = kAccCols + 64u * 2 * kDecGroups <= 512u ? 2 * kDecGroups : kDecGroups;
-  static_assert(kAccCols + 64u * kSE <= 512u && kSE <= kMaxSE, "tensor memory plan");
-};
+__host__ __device__ constexpr uint32_t acc_cols() { return 2u * kIssuers * NTOK; }
+static_assert(acc_cols<32>() + 64u * kSE <= 512u && kSE % kDecGroups == 0 && kSE % kIssuers == 0, "tensor memory plan");
 constexpr uint32_t kTmemCols = 512;
 constexpr size_t kSmemBudget = 220 * 1024;
 
@@ -97,8 +104,8 @@ __device__ __forceinline__ int cta_of_step(int s, int g, int total) {
 }
 
 struct DecBars {
-  uint64_t p_full[kMaxSP], p_empty[kMaxSP], empty[kMaxSE], acc_full[2], acc_empty[2], tok_ready, mma_done;
-  f32x2 sums[4][2];                            // SQNR sums of the four epilogue warps
+  uint64_t p_full[kMaxSP], p_empty[kMaxSP], ready[kSE], empty[kSE], acc_full[2], acc_empty[2], tok_ready, mma_done;
+  f32x2 sums[kThreads / 32][2];                // SQNR sums of the warps that write y
   uint32_t tmem_addr;
   int abort;
 };
@@ -120,16 +127,6 @@ struct DecBars {
 
 __device__ __forceinline__ void dec_tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Named barrier over the 128 threads of a decode group; true on every thread if pred is true on any.
-__device__ __forceinline__ bool group_barrier_any(int id, bool pred) {
-  uint32_t r;
-  asm volatile("{ .reg .pred q, p; setp.ne.u32 q, %1, 0; bar.red.or.pred p, %2, 128, q; selp.u32 %0, 1, 0, p; }"
-               : "=r"(r)
-               : "r"((uint32_t)pred), "r"(id)
-               : "memory");
-  return r != 0;
-}
-
 __device__ __forceinline__ void dec_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                            uint32_t accumulate) {
   asm volatile(
@@ -139,29 +136,53 @@ __device__ __forceinline__ void dec_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uin
       : "memory");
 }
 
-// Bytes of the resident token operand: one [NTOK rows x 128 B] block per 128-code slab.
-__host__ __device__ constexpr size_t tok_bytes(int ntok, int num_ks) { return (size_t)num_ks * 2 * ntok * 128; }
+// Bytes of the resident token operand, nk K steps: one [NTOK rows x 128 B] block per 128-code slab.
+__host__ __device__ constexpr size_t tok_bytes(int ntok, int nk) { return (size_t)nk * 2 * ntok * 128; }
+// Bytes of the cluster exchange: [part][token][128 / parts channels] float accumulators.
+__host__ __device__ constexpr size_t xch_bytes(int ntok, int parts) { return parts > 1 ? (size_t)ntok * UM * 4 : 0; }
+
+// The two halves of a cluster barrier.  A CTA's shared memory may be written by its peers once it runs: every
+// thread arrives at the start, and waits before the first remote store or the final barrier.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ void st_cluster_f32(float* p, uint32_t rank, float v) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
+}
 
 template <int NTOK, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
     w4a4_gemm_decode_tc_kernel(const __grid_constant__ CUtensorMap tmW, const uint8_t* __restrict__ xq,
                                const float* __restrict__ sx, const float* __restrict__ sw, int n, int d_in, int d_out,
-                               int sp, float* __restrict__ y, int32_t* __restrict__ acc_out,
+                               int sp, int parts, int nk, float* __restrict__ y, int32_t* __restrict__ acc_out,
                                const float* __restrict__ y_ref, double* __restrict__ sums3, int sqnr_slot,
                                int part_slot, uint32_t* __restrict__ status) {
+  // parts > 1 (never with SPLIT): the cluster's size; nk: K steps of the tokens that fit the resident operand
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int row_bytes = d_in / 2;
   const int num_ks = (row_bytes + KSB - 1) / KSB;
   const int num_units = (d_out + UM - 1) / UM;
   const int total = num_units * num_ks;
-  const int s0 = range_begin(blockIdx.x, gridDim.x, num_units, num_ks, SPLIT);
-  const int s1 = range_begin(blockIdx.x + 1, gridDim.x, num_units, num_ks, SPLIT);
-  constexpr int kSE = TmemPlan<NTOK>::kSE;
-  constexpr uint32_t kAStage0 = TmemPlan<NTOK>::kAccCols;
+  int s0, s1, ks_lo = 0, ks_n = num_ks;                           // the range, and the K steps it touches
+  if (!SPLIT && parts > 1) {                                      // this CTA's part of one unit
+    const int u = blockIdx.x / parts, p = blockIdx.x % parts;     // p: rank in the cluster
+    ks_lo = p * num_ks / parts;
+    ks_n = (p + 1) * num_ks / parts - ks_lo;                      // <= nk
+    s0 = u * num_ks + ks_lo;
+    s1 = s0 + ks_n;
+  } else {
+    s0 = range_begin(blockIdx.x, gridDim.x, num_units, num_ks, SPLIT);
+    s1 = range_begin(blockIdx.x + 1, gridDim.x, num_units, num_ks, SPLIT);
+  }
+  constexpr uint32_t kAStage0 = acc_cols<NTOK>();
+  constexpr int kTokLoads = NTOK / 4;                             // token loads in flight per staging thread
   uint8_t* bst = smem;                                            // tokens, E4M3
-  uint8_t* pk = smem + tok_bytes(NTOK, num_ks);                   // sp x 16 KiB packed weight tiles
-  DecBars* bars = reinterpret_cast<DecBars*>(pk + (size_t)sp * kPkStage);
+  uint8_t* pk = smem + tok_bytes(NTOK, nk);                       // sp x 16 KiB packed weight tiles
+  float* xch = reinterpret_cast<float*>(pk + (size_t)sp * kPkStage);
+  DecBars* bars = reinterpret_cast<DecBars*>(reinterpret_cast<uint8_t*>(xch) + xch_bytes(NTOK, parts));
   float* sxs = reinterpret_cast<float*>(bars + 1);                // NTOK token steps
   volatile int* abort_flag = &bars->abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -172,16 +193,22 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&bars->p_full[s], 1);
       mbar_init(&bars->p_empty[s], kDecWarps / kDecGroups);   // the decode group of that K step
     }
-    for (int s = 0; s < kSE; ++s) mbar_init(&bars->empty[s], 1);
+    for (int s = 0; s < kSE; ++s) {
+      mbar_init(&bars->ready[s], kDecWarps / kDecGroups);
+      mbar_init(&bars->empty[s], 1);
+    }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(&bars->acc_full[b], kDecGroups);  // every group commits once per segment
+      mbar_init(&bars->acc_full[b], kIssuers);    // every issuer commits once per segment
       mbar_init(&bars->acc_empty[b], kEpiWarps);
     }
     mbar_init(&bars->tok_ready, kThreads / 32 - kStageWarp0);
-    mbar_init(&bars->mma_done, kDecGroups);
+    mbar_init(&bars->mma_done, kIssuers);
     bars->abort = 0;
     fence_mbar_init();
   }
+  const bool clustered = !SPLIT && parts > 1;
+  __syncwarp();
+  if (clustered) cluster_arrive();
   pdl_wait_then_release();                        // nothing global or in tensor memory before this
   if (warp == 0) tmem_alloc(&bars->tmem_addr, kTmemCols);
   tc_fence_before();
@@ -190,26 +217,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = bars->tmem_addr;
 
   if (warp >= kStageWarp0) {
-    // resident token operand, staged by warps 3.. while the weight tiles start to stream (all of a
+    // resident token operand, staged by warps 4.. while the weight tiles start to stream (all of a
     // thread's loads in flight at once: the first MMA waits for the whole operand): slab a (codes
-    // 128a .. 128a+127) of token t at a*NTOK*128 + t*128, 16-byte chunk c at c ^ (t % 8); tokens >= n
-    // and codes >= d_in are zero
-    // Only the K steps of this CTA's range are staged: with fewer steps than a row has, they are the
-    // num_ks-periodic run starting at s0 % num_ks.  Item e = 16-byte chunk c of token t's packed row
-    // (e = t * row_chunks + c); (t, c) advance incrementally, with no division inside the loops.
-    const int span = s1 - s0, ks_lo = s0 % num_ks;
-    const int row_chunks = 8 * num_ks;                            // 16-byte chunks per (padded) packed row
+    // 128a .. 128a+127 of the range's K steps) of token t at a*NTOK*128 + t*128, 16-byte chunk c at
+    // c ^ (t % 8); tokens >= n and codes >= d_in are zero
+    // Item e = 16-byte chunk c of token t's packed row (e = t * row_chunks + c, from the range's first K
+    // step on); (t, c) advance incrementally, with no division inside the loops.
+    const int row_chunks = 8 * ks_n;                              // 16-byte chunks per (padded) row piece
     const int st = tid - kStageWarp0 * 32, nst = kThreads - kStageWarp0 * 32;
     const float sx_pre = (st < NTOK && st < n) ? sx[st] * kAccScale : 0.f;   // loaded beside the token rows
     const int items = NTOK * row_chunks;
     const int step_t = nst / row_chunks, step_c = nst % row_chunks;
     int t_cur = st / row_chunks, c_cur = st % row_chunks;
-    auto needed = [&](int c) {
-      if (!SPLIT) return true;
-      int dk = (c >> 3) - ks_lo;
-      if (dk < 0) dk += num_ks;
-      return span >= num_ks || dk < span;
-    };
     for (int e0 = st; e0 < items; e0 += kTokLoads * nst) {
       uint4 w[kTokLoads];
       int tc[kTokLoads];                                          // t << 16 | c of each item, -1 past the end
@@ -218,9 +237,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int e = e0 + q * nst;
         const int t = t_cur, c = c_cur;
         tc[q] = e < items ? (t << 16 | c) : -1;
-        const int off = c * 16;                                   // packed byte offset in the row
+        const int off = ks_lo * KSB + c * 16;                     // packed byte offset in the row
         w[q] = make_uint4(0u, 0u, 0u, 0u);
-        if (e < items && t < n && off < row_bytes && needed(c))
+        if (e < items && t < n && off < row_bytes)
           w[q] = *reinterpret_cast<const uint4*>(xq + (int64_t)t * row_bytes + off);
         c_cur += step_c;
         t_cur += step_t;
@@ -233,7 +252,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int q = 0; q < kTokLoads; ++q) {
         if (tc[q] < 0) break;
         const int t = tc[q] >> 16, c = tc[q] & 0xFFFF;
-        if (!needed(c)) continue;
         const int a = c >> 2, j = c & 3;                          // 64-byte slab a, 16-byte chunk j in it
         uint8_t* dst = bst + (size_t)a * NTOK * 128 + t * 128;
         const int swz = t & 7;
@@ -250,17 +268,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   if (warp == kProd0 || warp == kProd1) {
-    // ---------------------------------------------------------------- TMA producers (alternate K steps)
+    // ---------------------------------------------------------------- TMA producers (a stage's parity each)
     if (lane == 0) {
       const uint32_t me = warp == kProd0 ? 0u : 1u;
       if (me == 0) prefetch_tensormap(&tmW);
       // it = the CTA-local step index (step s0 + it of the (unit, K step) sequence)
-      uint32_t it = 0, issued_end = 0;                  // this producer issued every K step of its parity below issued_end
+      uint32_t it = 0, issued_end = 0;                  // this producer issued every K step of its stages below issued_end
       bool ok = true;
       for (int sg = s0; sg < s1 && ok; ++sg, ++it) {
-        if ((it & 1u) != me) continue;
-        const int u = sg / num_ks, ks = sg % num_ks;
         const uint32_t s = it % sp, use = it / sp;
+        if ((s & 1u) != me) continue;
+        const int u = sg / num_ks, ks = sg % num_ks;
         if (use > 0 && !(ok = mbar_wait_bounded(&bars->p_empty[s], (use - 1) & 1, abort_flag, __LINE__, lim))) break;
         mbar_arrive_expect_tx(&bars->p_full[s], kPkStage);
         tma_load_2d(pk + s * kPkStage, &tmW, ks * KSB, u * UM, &bars->p_full[s]);
@@ -271,70 +289,34 @@ __global__ void __launch_bounds__(kThreads, 1)
       // to wait for; this producer waits for the ones it issued
       volatile int no_abort = 0;
       for (uint32_t q = it > (uint32_t)sp ? it - sp : 0; q < it && q < issued_end; ++q)
-        if ((q & 1u) == me) mbar_wait_bounded(&bars->p_full[q % sp], (q / sp) & 1, &no_abort);
+        if (((q % sp) & 1u) == me) mbar_wait_bounded(&bars->p_full[q % sp], (q / sp) & 1, &no_abort);
     }
-  } else if (warp >= kDecWarp0 && warp < kDecWarp0 + kDecWarps) {
-    // ---------------------------------------------------------------- decode + MMA: weight row = TMEM lane
-    // Four groups of four warps (one per TMEM lane quadrant) take every fourth step of the CTA's
-    // range (group = local step index mod 4, so every stage has one consumer).  A thread decodes its
-    // whole 128-byte row (256 codes, 64 TMEM columns); then the group's leader thread issues the
-    // step's eight MMAs into the group's own accumulator.  One thread issues an MMA about every 55
-    // cycles whatever N is, so four issuers keep the tensor core fed at N = 16; the partial
-    // accumulators of a segment (the range's steps of one unit) are added in the epilogue (integers
-    // times 2^-18: exact).  Every group commits the segment's accumulator barrier once, with or
-    // without steps in it, after waiting for that buffer to be drained.
-    const int quad = warp & 3, grp = (warp - kDecWarp0) >> 2;
-    const bool leader = quad == 0 && lane == 0;
-    const int r = quad * 32 + lane;
-    constexpr uint32_t kIdesc = idesc_e4m3_f32(UM, NTOK);
-    const uint32_t bbase = smem_u32(bst);
-    bool stop = false;
-    if (leader) {
-      mbar_wait_bounded(&bars->tok_ready, 0, abort_flag, __LINE__, lim);
+  } else if (warp == kIss0 || warp == kIss1) {
+    // ---------------------------------------------------------------- MMA issuers (alternate K steps)
+    // Every issuer commits a segment's accumulator barrier once (a segment: the range's steps of one unit),
+    // with or without steps in it, after waiting for that buffer to be drained, so its arrivals can never run
+    // a phase ahead.
+    if (lane == 0) {
+      const uint32_t me = warp == kIss0 ? 0u : 1u;
+      constexpr uint32_t kIdesc = idesc_e4m3_f32(UM, NTOK);
+      const uint32_t bbase = smem_u32(bst);
+      bool ok = mbar_wait_bounded(&bars->tok_ready, 0, abort_flag, __LINE__, lim);
       tc_fence_after();
-    }
-    uint32_t seg = 0;
-    for (int sb = s0; sb < s1 && !stop; ++seg) {
-      const int u = sb / num_ks;
-      const int se = min(s1, (u + 1) * num_ks);        // segment [sb, se): the range's steps of unit u
-      const uint32_t ab = seg & 1;
-      const uint32_t d_acc = tmem + (ab * kDecGroups + grp) * NTOK;
-      bool first = true;                                 // the group's first step of the segment
-      for (int sg = sb + ((grp - (sb - s0)) % kDecGroups + kDecGroups) % kDecGroups; sg < se; sg += kDecGroups) {
-        const uint32_t it = (uint32_t)(sg - s0);         // it % kDecGroups == grp
-        const int ks = sg % num_ks;
-        const uint32_t ps = it % sp, sa = it % kSE;
-        const bool good = mbar_wait_bounded(&bars->p_full[ps], (it / sp) & 1, abort_flag, __LINE__, lim) &&
-                          (it < (uint32_t)kSE || mbar_wait_bounded(&bars->empty[sa], ((it / kSE) - 1) & 1, abort_flag, __LINE__, lim));
-        if (good) {
-          tc_fence_after();
-          const uint8_t* prow = pk + ps * kPkStage + r * 128;
-#pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            uint32_t av[32];
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {  // 16-byte chunk j of the 128-byte row, at j ^ (r % 8)
-              const int j = 4 * half + jj;
-              const uint4 w = *reinterpret_cast<const uint4*>(prow + ((j ^ (r & 7)) << 4));
-              av[8 * jj + 0] = sm4_lo(w.x); av[8 * jj + 1] = sm4_hi(w.x);
-              av[8 * jj + 2] = sm4_lo(w.y); av[8 * jj + 3] = sm4_hi(w.y);
-              av[8 * jj + 4] = sm4_lo(w.z); av[8 * jj + 5] = sm4_hi(w.z);
-              av[8 * jj + 6] = sm4_lo(w.w); av[8 * jj + 7] = sm4_hi(w.w);
-            }
-            __syncwarp();
-            DEC_TMEM_ST32(tmem + ((uint32_t)(quad * 32) << 16) + kAStage0 + 64u * sa + 32u * half, av);
-          }
-          dec_tmem_st_wait();
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0 && good) mbar_arrive(&bars->p_empty[ps]);
-        // the group's four warps have stored the stage (and agree on whether to go on)
-        stop = group_barrier_any(kGroupBar0 + grp, *abort_flag != 0);
-        if (stop) break;
-        if (leader) {
-          tc_fence_after();
-          if (first && seg >= 2) mbar_wait_bounded(&bars->acc_empty[ab], ((seg >> 1) - 1) & 1, abort_flag, __LINE__, lim);
+      uint32_t seg = 0;
+      for (int sb = s0; sb < s1 && ok; ++seg) {
+        const int u = sb / num_ks;
+        const int se = min(s1, (u + 1) * num_ks);      // segment [sb, se): the range's steps of unit u
+        const uint32_t ab = seg & 1;
+        const uint32_t d_acc = tmem + (ab * kIssuers + me) * NTOK;
+        if (seg >= 2 && !(ok = mbar_wait_bounded(&bars->acc_empty[ab], ((seg >> 1) - 1) & 1, abort_flag, __LINE__, lim))) break;
+        tc_fence_after();
+        bool first = true;
+        for (int sg = sb; sg < se; ++sg) {
+          const uint32_t it = (uint32_t)(sg - s0);
+          if ((it & 1u) != me) continue;
+          const int ks = sg - u * num_ks - ks_lo;      // K step within the resident tokens
+          const uint32_t sa = it % kSE;
+          if (!(ok = mbar_wait_bounded(&bars->ready[sa], (it / kSE) & 1, abort_flag, __LINE__, lim))) break;
           tc_fence_after();
           const uint32_t ta = tmem + kAStage0 + 64u * sa;
 #pragma unroll
@@ -342,28 +324,59 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint64_t db = sdesc_kmajor_sw128(bbase + (uint32_t)((2 * ks + (kk >> 2)) * NTOK * 128)) + 2 * (kk & 3);
             dec_mma_ts(d_acc, ta + 8u * kk, db, kIdesc, (first && kk == 0) ? 0u : 1u);
           }
+          first = false;
           mma_commit(&bars->empty[sa]);
         }
-        first = false;
-      }
-      if (stop) break;
-      if (leader) {
-        // a group without steps in this segment still waits for the buffer to be drained before it
-        // commits, so its arrivals can never run a phase ahead
-        if (first && seg >= 2) mbar_wait_bounded(&bars->acc_empty[ab], ((seg >> 1) - 1) & 1, abort_flag, __LINE__, lim);
+        if (!ok) break;
         mma_commit(&bars->acc_full[ab]);
+        sb = se;
       }
-      sb = se;
-    }
-    if (leader) {
       mma_commit(&bars->mma_done);  // all MMAs complete before tensor memory is released
       volatile int no_abort = 0;
       mbar_wait_bounded(&bars->mma_done, 0, &no_abort);
+    }
+  } else if (warp >= kDecWarp0 && warp < kDecWarp0 + kDecWarps) {
+    // ---------------------------------------------------------------- decode: weight row = TMEM lane
+    // Three groups of four warps (one per TMEM lane quadrant) take every third step of the CTA's range.  A
+    // thread decodes its whole 128-byte row (256 codes, 64 TMEM columns).
+    const int quad = warp & 3, grp = (warp - kDecWarp0) >> 2;
+    const int r = quad * 32 + lane;
+    for (uint32_t it = (uint32_t)grp; it < (uint32_t)(s1 - s0); it += kDecGroups) {
+      const uint32_t ps = it % sp, sa = it % kSE;
+      const bool good = mbar_wait_bounded(&bars->p_full[ps], (it / sp) & 1, abort_flag, __LINE__, lim) &&
+                        (it < (uint32_t)kSE || mbar_wait_bounded(&bars->empty[sa], ((it / kSE) - 1) & 1, abort_flag, __LINE__, lim));
+      if (!__all_sync(0xFFFFFFFFu, good)) break;       // warp-uniform: TMEM stores need the whole warp
+      tc_fence_after();
+      const uint8_t* prow = pk + ps * kPkStage + r * 128;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        uint32_t av[32];
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {  // 16-byte chunk j of the 128-byte row, at j ^ (r % 8)
+          const int j = 4 * half + jj;
+          const uint4 w = *reinterpret_cast<const uint4*>(prow + ((j ^ (r & 7)) << 4));
+          av[8 * jj + 0] = sm4_lo(w.x); av[8 * jj + 1] = sm4_hi(w.x);
+          av[8 * jj + 2] = sm4_lo(w.y); av[8 * jj + 3] = sm4_hi(w.y);
+          av[8 * jj + 4] = sm4_lo(w.z); av[8 * jj + 5] = sm4_hi(w.z);
+          av[8 * jj + 6] = sm4_lo(w.w); av[8 * jj + 7] = sm4_hi(w.w);
+        }
+        __syncwarp();
+        DEC_TMEM_ST32(tmem + ((uint32_t)(quad * 32) << 16) + kAStage0 + 64u * sa + 32u * half, av);
+      }
+      fence_proxy_async_smem();                        // the row is read: TMA may refill the stage
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->p_empty[ps]);
+      dec_tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->ready[sa]);
     }
   } else if (warp >= kEpiWarp0) {
     // ---------------------------------------------------------------- epilogue: output channel = TMEM lane
     const int quad = warp & 3;
     const int ch = quad * 32 + lane;                 // channel within the unit
+    __syncwarp();
+    if (clustered) cluster_wait();                   // the peers run: their shared memory may be written
     bool ok = true;
     f32x2 sig = {0.f, 0.f}, err = {0.f, 0.f};      // SQNR sums (Sec. 2, Eq. 1) when y_ref is given
     uint32_t seg = 0;
@@ -379,15 +392,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int cl = whole ? (int)blockIdx.x : cta_of_step((u + 1) * num_ks - 1, gridDim.x, total);
       const bool owner = cf == (int)blockIdx.x;       // writes the unit's outputs
       // y_ref in flight while the MMAs of the segment run, where this CTA writes the unit
-      const bool pre = y_ref && o_ok && owner;
+      const bool pre = y_ref && o_ok && owner && !clustered;
       float yr[NTOK];
 #pragma unroll
       for (int t = 0; t < NTOK; ++t) yr[t] = (pre && t < n) ? __ldcs(y_ref + (int64_t)t * d_out + o) : 0.f;
       if (!(ok = mbar_wait_bounded(&bars->acc_full[ab], (seg >> 1) & 1, abort_flag, __LINE__, lim))) break;
       __syncwarp();
       tc_fence_after();
-      // the groups with steps in the segment: local steps sb - s0 .. se - s0 - 1, group = step % 4
-      const int nact = se - sb < kDecGroups ? se - sb : kDecGroups;
+      // the issuers with steps in the segment: local steps sb - s0 .. se - s0 - 1, issuer = step % 2
+      const int nact = se - sb < kIssuers ? se - sb : kIssuers;
       uint32_t* cnt = &g_dec_cnt[part_slot][u][quad];
       float s_run = 0.f, e_run = 0.f;
       auto emit = [&](int t, float a) {                // y (and acc_out, SQNR terms) of token t
@@ -442,9 +455,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int j = 0; j < 16; ++j) acc[j] = 0.f;
         for (int i = 0; i < nact; ++i) {
-          const int g = (sb - s0 + i) % kDecGroups;
+          const int g = (sb - s0 + i) % kIssuers;
           uint32_t part[16];
-          DEC_TMEM_LD16(tmem + ((uint32_t)(quad * 32) << 16) + (ab * kDecGroups + g) * NTOK + 16u * c, part);
+          DEC_TMEM_LD16(tmem + ((uint32_t)(quad * 32) << 16) + (ab * kIssuers + g) * NTOK + 16u * c, part);
           tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < 16; ++j) acc[j] += __uint_as_float(part[j]);  // integers times 2^-18: exact
@@ -454,7 +467,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(&bars->acc_empty[ab]);
         }
-        if (owner) {
+        if (clustered) {
+          // channel ch goes to the cluster's CTA ch / (128 / parts): [part][token][channel] there
+          const int cps = UM / parts, f = ch / cps;
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (16 * c + j < n)
+              st_cluster_f32(xch + ((size_t)(blockIdx.x % parts) * NTOK + 16 * c + j) * cps + ch % cps, (uint32_t)f, acc[j]);
+        } else if (owner) {
           if (!whole) {
             if constexpr (kEarly) {
 #pragma unroll
@@ -486,7 +506,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       err = f2_add(err, e_run);
       sb = se;
     }
-    if (y_ref) {
+    if (y_ref && !clustered) {
       // the four warps' sums meet in shared memory; one warp hands the CTA's pair to the slot
       sig = f2_warp_sum(sig);
       err = f2_warp_sum(err);
@@ -503,6 +523,46 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
 
+  __syncwarp();
+  tc_fence_before();
+  if (clustered) {
+    if (warp < kEpiWarp0) cluster_wait();             // the phase of the arrival at the start
+    // every part's accumulators are in the CTAs that finish them; no CTA writes to another after this
+    cluster_sync();
+    const int u = blockIdx.x / parts, cps = UM / parts, o0 = u * UM + (int)(blockIdx.x % parts) * cps;
+    f32x2 sig = {0.f, 0.f}, err = {0.f, 0.f};
+    for (int i = tid; i < n * cps; i += kThreads) {   // n <= 32: at most four outputs a thread
+      const int t = i / cps, c = i % cps, o = o0 + c;
+      if (o >= d_out) continue;
+      float a = 0.f;
+      for (int p = 0; p < parts; ++p) a += xch[((size_t)p * NTOK + t) * cps + c];   // integers times 2^-18: exact
+      const float v = a * sxs[t] * sw[o];
+      y[(int64_t)t * d_out + o] = v;
+      if (acc_out) acc_out[(int64_t)t * d_out + o] = __float2int_rn(a * kAccScale);
+      if (y_ref) {
+        const float r = __ldcs(y_ref + (int64_t)t * d_out + o), e = r - v;
+        sig = f2_add(sig, r * r);
+        err = f2_add(err, e * e);
+      }
+    }
+    if (y_ref) {
+      __syncwarp();
+      sig = f2_warp_sum(sig);
+      err = f2_warp_sum(err);
+      if (lane == 0) {
+        bars->sums[warp][0] = sig;
+        bars->sums[warp][1] = err;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        for (int w = 1; w < kThreads / 32; ++w) {
+          sig = f2_add(w == 1 ? bars->sums[0][0] : sig, bars->sums[w][0]);
+          err = f2_add(w == 1 ? bars->sums[0][1] : err, bars->sums[w][1]);
+        }
+        sqnr_cta_done(sqnr_slot, sig, err, sums3);
+      }
+    }
+  }
   __syncthreads();
   if (bars->abort && tid == 0) report(status, timeout_bits(kWhereGemmDecode, bars->abort));
   if (warp == 0) {
@@ -535,8 +595,40 @@ int num_sms() {
   return sms;
 }
 
-size_t smem_bytes(int ntok, int num_ks, int sp) {
-  return 1024 + tok_bytes(ntok, num_ks) + (size_t)sp * kPkStage + sizeof(DecBars) + 32 * sizeof(float);
+size_t smem_bytes(int ntok, int nk, int sp, int parts) {
+  return 1024 + tok_bytes(ntok, nk) + (size_t)sp * kPkStage + xch_bytes(ntok, parts) + sizeof(DecBars) + 32 * sizeof(float);
+}
+
+// Packed stages that fit beside nk K steps of resident tokens: a multiple of the decode groups, 0 if none do.
+int stages_for(int ntok, int nk, int parts) {
+  const size_t fixed = smem_bytes(ntok, nk, 0, parts);
+  if (fixed >= kSmemBudget) return 0;
+  int sp = (int)((kSmemBudget - fixed) / kPkStage);
+  if (sp > kMaxSP) sp = kMaxSP;
+  return sp - sp % kDecGroups;
+}
+
+// CTAs per unit (the cluster's size; 1: whole units or stream-K), 0 when the tokens fit in no form.  A CTA
+// takes about kStart + its K steps, in units of one K step (start-up, token staging and the last outputs
+// ~4.5 us against ~0.28 us a step); clusters beyond what is resident run in waves, stream-K does not.
+constexpr int kStart = 16;
+int pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms) {
+  const int ntok = n <= 16 ? 16 : 32;
+  const int64_t num_ks = (d_in / 2 + KSB - 1) / KSB, units = (d_out + UM - 1) / UM;
+  int best = 0;
+  int64_t least = 0;
+  for (int parts = 1; parts <= kMaxParts && parts <= num_ks; parts *= 2) {
+    const int64_t nk = (num_ks + parts - 1) / parts;
+    if (stages_for(ntok, (int)nk, parts) == 0) continue;
+    const int64_t resident = sms / parts * parts;
+    int64_t cost = parts == 1 && units > sms ? kStart + (units * num_ks + sms - 1) / sms
+                                             : ((units * parts + resident - 1) / resident) * (kStart + nk);
+    if (best == 0 || cost < least) {
+      best = parts;
+      least = cost;
+    }
+  }
+  return best;
 }
 
 // Whether one CTA per SM of the kernel is resident at once on this device under a cooperative launch
@@ -564,7 +656,7 @@ bool coop_fits(size_t smem) {
 template <int NTOK>
 cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw, int64_t n,
                         int64_t d_in, int64_t d_out, float* y, int32_t* acc_out, const float* y_ref, double* sums3,
-                        uint32_t* status, int sp, cudaStream_t stream) {
+                        uint32_t* status, int parts, cudaStream_t stream) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
   const int64_t row_bytes = d_in / 2;
@@ -579,7 +671,9 @@ cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, c
          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
   const int num_ks = (int)((row_bytes + KSB - 1) / KSB);
-  const size_t smem = smem_bytes(NTOK, num_ks, sp);
+  const int nk = (num_ks + parts - 1) / parts, sp = stages_for(NTOK, nk, parts);
+  if (sp == 0) return cudaErrorInvalidValue;
+  const size_t smem = smem_bytes(NTOK, nk, sp, parts);
   static std::mutex mu;
   static size_t configured = 0;
   {
@@ -601,11 +695,11 @@ cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, c
   // than the owner's is the head of its CTA's range, done early.  With fewer units than SMs a range
   // would be shorter than a unit; CTAs inside a unit finish together with the unit's owner, and the
   // exchange through global memory then sits on the tail (measured at 16 tokens, 4096 -> 14336:
-  // 15.8 us on 152 CTAs against 12.8 us for whole units on 112).  Whole units per CTA in that case.
-  const int split = units > sms && units <= kDecMaxUnits && coop_fits<NTOK>(smem) ? 1 : 0;
-  const int64_t work = split ? units * num_ks : units;
-  const unsigned grid = (unsigned)(work < sms ? work : sms);
-  if (grid > (unsigned)kSqnrMaxCtas) return cudaErrorInvalidConfiguration;
+  // 15.8 us on 152 CTAs against 12.8 us for whole units on 112).
+  const int split = parts == 1 && units > sms && units <= kDecMaxUnits && coop_fits<NTOK>(smem) ? 1 : 0;
+  const int64_t ctas = parts > 1 ? units * parts : (units < sms ? units : sms);
+  if (ctas > 0x7FFFFFFF || (y_ref && ctas > kSqnrMaxCtas)) return cudaErrorInvalidConfiguration;
+  const unsigned grid = (unsigned)ctas;
   const int slot = y_ref ? next_sqnr_slot() : 0;
   static std::atomic<unsigned> next_part{0};
   const int part_slot = split ? (int)(next_part.fetch_add(1, std::memory_order_relaxed) % kDecSlots) : 0;
@@ -617,15 +711,21 @@ cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, c
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attrs[2] = {pdl_attr(), {}};
-  attrs[1].id = cudaLaunchAttributeCooperative;       // the owners of cut units wait for the other parts
-  attrs[1].val.cooperative = 1;
+  if (split) {
+    attrs[1].id = cudaLaunchAttributeCooperative;     // the owners of cut units wait for the other parts
+    attrs[1].val.cooperative = 1;
+  } else {
+    attrs[1].id = cudaLaunchAttributeClusterDimension;
+    attrs[1].val.clusterDim.x = (unsigned)parts;
+    attrs[1].val.clusterDim.y = attrs[1].val.clusterDim.z = 1;
+  }
   cfg.attrs = attrs;
-  cfg.numAttrs = split ? 2 : 1;
+  cfg.numAttrs = split || parts > 1 ? 2 : 1;
   if (split)
     return cudaLaunchKernelEx(&cfg, w4a4_gemm_decode_tc_kernel<NTOK, true>, map, xq, sx, sw, (int)n, (int)d_in,
-                              (int)d_out, sp, y, acc_out, y_ref, sums3, slot, part_slot, status);
+                              (int)d_out, sp, parts, nk, y, acc_out, y_ref, sums3, slot, part_slot, status);
   return cudaLaunchKernelEx(&cfg, w4a4_gemm_decode_tc_kernel<NTOK, false>, map, xq, sx, sw, (int)n, (int)d_in,
-                            (int)d_out, sp, y, acc_out, y_ref, sums3, slot, part_slot, status);
+                            (int)d_out, sp, parts, nk, y, acc_out, y_ref, sums3, slot, part_slot, status);
 }
 
 }  // namespace
@@ -634,17 +734,13 @@ cudaError_t set_decode_wait_limit(uint64_t ns) {
   return cudaMemcpyToSymbol(g_dec_wait_limit, &ns, sizeof(ns));
 }
 
-// Packed stages that fit beside the resident tokens; 0 when this kernel does not apply.
-int decode_tc_stages(int64_t n, int64_t d_in) {
-  if (n < 1 || n > 32) return 0;
-  const int ntok = n <= 16 ? 16 : 32;
-  const int num_ks = (int)((d_in / 2 + KSB - 1) / KSB);
-  const size_t fixed = smem_bytes(ntok, num_ks, 0);
-  if (fixed >= kSmemBudget) return 0;
-  int sp = (int)((kSmemBudget - fixed) / kPkStage);
-  if (sp > kMaxSP) sp = kMaxSP;
-  sp -= sp % kDecGroups;                      // a multiple of the decode groups (see TmemPlan)
-  return sp >= kDecGroups ? sp : 0;
+// Whether this kernel takes n tokens of d_in codes (else the mma.sync kernel does): clusters may not be many
+// enough to overflow the SQNR slot's rows.
+bool decode_tc_applies(int64_t n, int64_t d_in, int64_t d_out, bool with_sqnr) {
+  if (n < 1 || n > 32) return false;
+  const int parts = pick_parts(n, d_in, d_out, num_sms());
+  if (parts == 0) return false;
+  return !with_sqnr || parts == 1 || (d_out + UM - 1) / UM * parts <= kSqnrMaxCtas;
 }
 
 // y_ref != nullptr: the epilogue also forms the SQNR sums of y against y_ref and writes
@@ -652,10 +748,10 @@ int decode_tc_stages(int64_t n, int64_t d_in) {
 cudaError_t launch_w4a4_gemm_decode_tc(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw,
                                        int64_t n, int64_t d_in, int64_t d_out, float* y, int32_t* acc_out,
                                        const float* y_ref, double* sums3, uint32_t* status, cudaStream_t stream) {
-  const int sp = decode_tc_stages(n, d_in);
-  if (sp == 0) return cudaErrorInvalidValue;
-  if (n <= 16) return launch_ntok<16>(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, sp, stream);
-  return launch_ntok<32>(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, sp, stream);
+  const int parts = pick_parts(n, d_in, d_out, num_sms());
+  if (parts == 0) return cudaErrorInvalidValue;
+  if (n <= 16) return launch_ntok<16>(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, parts, stream);
+  return launch_ntok<32>(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, parts, stream);
 }
 
 }  // namespace cat

@@ -542,3 +542,31 @@ def test_device_transform_refuses_singular_blocks():
     assert err.value.status == 4
     T, _, _ = cat.cat_quantize_weights(w, 32, "cat", sigma_x=cat.cat_calib_cov(x, 32), n_calib=40)   # 40 tokens: full rank
     assert torch.isfinite(T).all()
+
+
+# ------------------------------------------------------------------------------------------
+# Decode GEMM: the work splits (whole units, clusters of 2, 4 and 8, stream-K)
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n,d_in,d_out", [(1, 32, 1), (1, 4096, 6144), (16, 4096, 14336), (17, 544, 130), (27, 14336, 4096),
+                                          (32, 4064, 1000), (5, 20000, 129), (32, 32768, 260), (16, 1024, 24001),
+                                          (32, 8192, 20480), (9, 262144, 128)])
+def test_decode_gemm_splits(n, d_in, d_out):
+    """Accumulators equal to float64 products of the codes (exact), y = acc s_x s_w, and the SQNR sums."""
+    rng = np.random.default_rng(n + d_in + d_out)
+    qx, qw = WL.random_codes(rng, (n, d_in)), WL.random_codes(rng, (d_out, d_in))
+    sx = torch.from_numpy(rng.uniform(0.01, 2.0, n).astype(np.float32)).cuda()
+    sw = torch.from_numpy(rng.uniform(0.001, 0.1, d_out).astype(np.float32)).cuda()
+    xq, wq = torch.from_numpy(sm4x8.pack(qx)).cuda(), torch.from_numpy(sm4x8.pack(qw)).cuda()
+    acc = torch.full((n, d_out), -1, dtype=torch.int32, device="cuda")
+    y = cat.cat_w4a4_linear(xq, sx, wq, sw, acc_out=acc)
+    ref = torch.from_numpy(qx).cuda().double() @ torch.from_numpy(qw).cuda().double().T
+    assert torch.equal(acc.double(), ref)
+    y64 = ref * sx[:, None].double() * sw[None, :].double()
+    assert ((y.double() - y64).abs() <= 2.0 ** -22 * y64.abs()).all()          # two float32 roundings and the steps' product
+    y_ref = (y64 + 0.1 * y64.std() * torch.randn(n, d_out, device="cuda", dtype=torch.float64)).float() if n * d_out > 1 else 2 * y + 1
+    y2, out = cat.cat_w4a4_linear_sqnr(xq, sx, wq, sw, y_ref)
+    assert torch.equal(y2, y)
+    sums = torch.stack([y_ref.double().square().sum(), (y_ref.double() - y.double()).square().sum()])
+    assert ((out[:2] - sums).abs() <= 1e-5 * sums).all()
+    assert cat.cat_device_status()[0] == 0
