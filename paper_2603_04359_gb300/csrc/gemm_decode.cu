@@ -1,6 +1,6 @@
 // W4A4 GEMM for a few tokens (decode) on the legacy mma.sync path: the fallback of the tcgen05
 // weight-streaming kernel (gemm_decode_tc.cu) for token operands too large for its shared memory
-// (d_in beyond ~10k codes at 16 tokens).  The packed weight stream is read once from HBM.
+// (d_in beyond ~82k codes at 16 tokens, ~39k at 32).  The packed weight stream is read once from HBM.
 //
 //   acc[t, o] = sum_i q_x[t, i] q_w[o, i],   y[t, o] = acc * s_x[t] * s_w[o]   (Sec. 3, Eq. 5)
 //
