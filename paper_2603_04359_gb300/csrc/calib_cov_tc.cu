@@ -20,9 +20,12 @@
 // consecutive doubles (256 bytes) -- the written blocks are D^T, equal to D up to the rounding of
 // the accumulation order.
 // Warps: 0 TMA producer + TMEM allocator, 1 MMA issuer, 2..9 epilogue (a TMEM lane quadrant and a
-// 32-column half of the slice each).  Tokens arrive in 64-row chunks of 64-channel, 128B-swizzled
-// boxes; with up to kStages chunks in flight, the 512-token calibration split of the configurations
-// is read in one go.
+// 32-column half of the slice each).  Tokens arrive in chunks of 64-channel, 128B-swizzled boxes.  Short
+// runs take 64-token chunks, eight in flight: the 512-token calibration split of the configurations is read
+// in one go and the first MMA starts on 16 KB.  Runs of kLongRun tokens or more per CTA are bound by the
+// rate at which the producer thread can issue boxes (~300 cycles each, whatever their size up to 32 KB), so
+// they take the longest chunks that leave three or four in flight: 256 tokens, 128 at k = 256.  16384 tokens x
+// 4096 channels: 41.5 us with 64-token chunks, 33.5 now.
 #include <cstring>
 #include <mutex>
 
@@ -31,8 +34,9 @@
 namespace cat {
 namespace {
 
-constexpr int kChunk = 64;      // tokens per stage
-constexpr int kStages = 8;      // 512 tokens in flight at once
+constexpr int kChunk = 64;      // tokens per stage, short runs
+constexpr int kStages = 8;      // 512 tokens in flight at once (the most stages there are)
+constexpr int kLongRun = 1024;  // tokens per CTA from which on the chunks are long
 constexpr int kThreads = 320;         // producer, MMA issuer, 8 epilogue warps
 constexpr uint32_t kBox = kChunk * 128;  // one 64-token x 64-channel bf16 box, 8 KiB
 constexpr int NACC = 8;                  // round-robin accumulators: all 512 TMEM columns
@@ -48,13 +52,15 @@ struct CovCfg {
   // when k <= 128), and at k = 256 the column slice's own box
   static constexpr int BOXES = G2 == 1 ? 2 : 3;
   static constexpr uint32_t STAGE = BOXES * kBox;
-  static constexpr uint32_t BAR_OFF = kStages * STAGE;
+  // long runs: LONG times the chunk and the stage, LONG_S stages
+  static constexpr int LONG = G2 == 1 ? 4 : 2, LONG_S = G2 == 1 ? 3 : 4;
+  static constexpr uint32_t BAR_OFF = kStages * STAGE > LONG_S * LONG * STAGE ? kStages * STAGE : LONG_S * LONG * STAGE;
   static constexpr size_t SMEM = BAR_OFF + 256 + 1024;
   // kind::f16, D fp32, A = B = BF16, both MN-major (bits 15, 16), M = 128, N = 64
   static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
                                     ((uint32_t)(kSliceN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 };
-static_assert(CovCfg<2>::SMEM <= 227 * 1024, "shared memory budget");
+static_assert(CovCfg<1>::SMEM <= 227 * 1024 && CovCfg<2>::SMEM <= 227 * 1024, "shared memory budget");
 
 struct CovBars {
   uint64_t full[kStages], empty[kStages], acc_full, mma_done;
@@ -119,8 +125,9 @@ __device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, ui
 template <int G2>
 __global__ void __launch_bounds__(kThreads, 1)
     calib_cov_tc_kernel(const __grid_constant__ CUtensorMap tmX, int n, int d, int k, int tok_per_split,
-                        double* __restrict__ sigma, int mode /* 0 store, 1 add, 2 atomic add */,
+                        int chunk, double* __restrict__ sigma, int mode /* 0 store, 1 add, 2 atomic add */,
                         uint32_t* __restrict__ status) {
+  // chunk: tokens per stage, kChunk or LONG kChunk (the tensor map's box has as many rows)
   using C = CovCfg<G2>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -133,8 +140,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int c0 = g * C::G;                            // first channel of the group
   const int t_begin = blockIdx.y * tok_per_split;
   const int t_end = min(n, t_begin + tok_per_split);
-  const int chunks = (t_end - t_begin + kChunk - 1) / kChunk;
-  const int total_steps = chunks * (kChunk / 16);
+  const int chunks = (t_end - t_begin + chunk - 1) / chunk;
+  const int stages = chunk == kChunk ? kStages : C::LONG_S;
+  const uint32_t box = (uint32_t)chunk * 128, stage = C::BOXES * box;
+  // 16-token MMA steps, counted as in 64-token chunks (the steps past the run's end are zero rows)
+  const int total_steps = (t_end - t_begin + kChunk - 1) / kChunk * (kChunk / 16);
   // accumulators in use: 4 (16 MMA steps each at most) for short runs, 8 beyond -- fewer
   // accumulators are fewer tensor-memory reads in the epilogue, more keep each one's sum short
   const int nacc = total_steps > 4 * 16 ? NACC : NACC / 2;
@@ -165,33 +175,34 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool ok = true;
       int c = 0;
       for (; c < chunks && ok; ++c) {
-        const uint32_t s = c % kStages;
-        if (c >= kStages && !(ok = mbar_wait_bounded(&bars->empty[s], ((c / kStages) - 1) & 1, abort_flag, __LINE__))) break;
-        mbar_arrive_expect_tx(&bars->full[s], C::STAGE);
-        const int t0 = t_begin + c * kChunk;
+        const uint32_t s = c % stages;
+        if (c >= stages && !(ok = mbar_wait_bounded(&bars->empty[s], ((c / stages) - 1) & 1, abort_flag, __LINE__))) break;
+        mbar_arrive_expect_tx(&bars->full[s], stage);
+        const int t0 = t_begin + c * chunk;
         for (int bx = 0; bx < 2; ++bx)            // the CTA's 128 rows
-          tma_load_2d(smem + s * C::STAGE + bx * kBox, &tmX, c0 + ih * 128 + 64 * bx, t0, &bars->full[s]);
+          tma_load_2d(smem + s * stage + bx * box, &tmX, c0 + ih * 128 + 64 * bx, t0, &bars->full[s]);
         if (G2 == 2)                              // the column slice's box
-          tma_load_2d(smem + s * C::STAGE + 2 * kBox, &tmX, c0 + kSliceN * h, t0, &bars->full[s]);
+          tma_load_2d(smem + s * stage + 2 * box, &tmX, c0 + kSliceN * h, t0, &bars->full[s]);
       }
-      const int first = c > kStages ? c - kStages : 0;
+      const int first = c > stages ? c - stages : 0;
       volatile int no_abort = 0;
-      for (int q = first; q < c; ++q) mbar_wait_bounded(&bars->full[q % kStages], (q / kStages) & 1, &no_abort);
+      for (int q = first; q < c; ++q) mbar_wait_bounded(&bars->full[q % stages], (q / stages) & 1, &no_abort);
     }
   } else if (warp == 1) {
     if (lane == 0) {
       bool ok = true;
       for (int c = 0; c < chunks && ok; ++c) {
-        const uint32_t s = c % kStages;
-        if (!(ok = mbar_wait_bounded(&bars->full[s], (c / kStages) & 1, abort_flag, __LINE__))) break;
+        const uint32_t s = c % stages;
+        if (!(ok = mbar_wait_bounded(&bars->full[s], (c / stages) & 1, abort_flag, __LINE__))) break;
         tc_fence_after();
-        const uint32_t base = smem_u32(smem + s * C::STAGE);
-#pragma unroll
-        for (int kk = 0; kk < kChunk / 16; ++kk) {  // 16 tokens per MMA: 16 rows of 128 B
-          const int step = c * (kChunk / 16) + kk;
-          const uint64_t da = sdesc_mnmajor_sw128(base + kk * 2048, kBox);
-          const uint64_t db = sdesc_mnmajor_sw128(base + b_box * kBox + kk * 2048, kBox);
-          mma_bf16_ss(tmem + (step % nacc) * kSliceN, da, db, C::IDESC, step >= nacc);
+        const uint32_t base = smem_u32(smem + s * stage);
+        const int step0 = c * (chunk / 16), steps = min(chunk / 16, total_steps - step0);
+#pragma unroll 4
+        for (int kk = 0; kk < steps; ++kk) {      // 16 tokens per MMA: 16 rows of 128 B
+          const int step = step0 + kk;
+          const uint64_t da = sdesc_mnmajor_sw128(base + kk * 2048, box);
+          const uint64_t db = sdesc_mnmajor_sw128(base + b_box * box + kk * 2048, box);
+          mma_bf16_ss(tmem + (step & (nacc - 1)) * kSliceN, da, db, C::IDESC, step >= nacc);
         }
         mma_commit(&bars->empty[s]);
       }
@@ -313,11 +324,21 @@ cudaError_t launch_g(const void* x, int64_t n, int64_t d, int k, double* sigma, 
   using C = CovCfg<G2>;
   EncodeTiledFn fn = encode_fn();
   if (!fn) return cudaErrorNotSupported;
+  const int64_t groups = (d + C::G - 1) / C::G;
+  const int64_t chunks = (n + kChunk - 1) / kChunk;
+  const int sms = num_sms();
+  // token splits (their CTAs add with float64 atomics) only for long calibration runs: >= 2048 tokens
+  // per CTA, within one wave
+  int64_t ysplits = sms / (groups * C::CTAS);
+  if (ysplits > chunks / 32) ysplits = chunks / 32;
+  if (ysplits < 1) ysplits = 1;
+  const int64_t tps = ((chunks + ysplits - 1) / ysplits) * kChunk;
+  const int chunk = tps >= kLongRun ? C::LONG * kChunk : kChunk;
   CUtensorMap map;
   memset(&map, 0, sizeof(map));
   cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)n};
   cuuint64_t strides[1] = {(cuuint64_t)d * 2};
-  cuuint32_t box[2] = {64, kChunk};
+  cuuint32_t box[2] = {64, (cuuint32_t)chunk};
   cuuint32_t estr[2] = {1, 1};
   if (fn(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr,
          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -329,15 +350,6 @@ cudaError_t launch_g(const void* x, int64_t n, int64_t d, int k, double* sigma, 
     attr = cudaFuncSetAttribute(calib_cov_tc_kernel<G2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
   });
   if (attr != cudaSuccess) return attr;
-  const int64_t groups = (d + C::G - 1) / C::G;
-  const int64_t chunks = (n + kChunk - 1) / kChunk;
-  const int sms = num_sms();
-  // token splits (their CTAs add with float64 atomics) only for long calibration runs: >= 2048 tokens
-  // per CTA, within one wave
-  int64_t ysplits = sms / (groups * C::CTAS);
-  if (ysplits > chunks / 32) ysplits = chunks / 32;
-  if (ysplits < 1) ysplits = 1;
-  const int64_t tps = ((chunks + ysplits - 1) / ysplits) * kChunk;
   int mode = accumulate ? 1 : 0;
   if (ysplits > 1) {
     mode = 2;
@@ -355,7 +367,7 @@ cudaError_t launch_g(const void* x, int64_t n, int64_t d, int k, double* sigma, 
   // not a programmatic dependent launch: measured, one gained ~0.4 us per c4 step and lost ~0.7 us per
   // c2 step (the kernel still releases its dependents early)
   note_launch();
-  cudaError_t e = cudaLaunchKernelEx(&cfg, calib_cov_tc_kernel<G2>, map, (int)n, (int)d, k, (int)tps, sigma, mode,
+  cudaError_t e = cudaLaunchKernelEx(&cfg, calib_cov_tc_kernel<G2>, map, (int)n, (int)d, k, (int)tps, chunk, sigma, mode,
                                      status);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

@@ -570,3 +570,24 @@ def test_decode_gemm_splits(n, d_in, d_out):
     sums = torch.stack([y_ref.double().square().sum(), (y_ref.double() - y.double()).square().sum()])
     assert ((out[:2] - sums).abs() <= 1e-5 * sums).all()
     assert cat.cat_device_status()[0] == 0
+
+
+# ------------------------------------------------------------------------------------------
+# Calibration: long runs (long chunks, token splits)
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n,d,k", [(1023, 128, 128), (1024, 256, 64), (1281, 128, 16), (4097, 256, 128), (2100, 512, 256),
+                                   (9001, 256, 256)])
+def test_calib_cov_long_runs(n, d, k):
+    """Around the chunk sizes and the token splits, against float64 sums.  A 16-token step's fp32 addition is off by at
+    most 2^-23 of its accumulator; an accumulator takes at most n / 64 of them (8 accumulators beyond 1024 tokens,
+    16 tokens a step, four of them added): n / 64 * 2^-23 of the norm is the bound, 1e-6 where that is less."""
+    x = torch.randn(n, d, device="cuda").to(torch.bfloat16) * torch.linspace(0.1, 30.0, d, device="cuda").to(torch.bfloat16)
+    v = x.double().view(n, d // k, k).transpose(0, 1)
+    ref = v.transpose(1, 2) @ v
+    S = cat.cat_calib_cov(x, k)
+    tol = max(1e-6, n / 64 * 2.0 ** -23)
+    assert float((S - ref).norm() / ref.norm()) < tol
+    twice = cat.cat_calib_cov(x, k, out=S.clone(), accumulate=True)
+    assert float((twice - 2 * ref).norm() / ref.norm()) < 2 * tol
+    assert cat.cat_device_status()[0] == 0
