@@ -168,11 +168,13 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // order of magnitude slower), waits until all S parts of the tile have arrived (bounded; the launch
 // is cooperative, so all parts are resident), and then finishes NB / S of the tile's channels:
 // the sum over the parts (exact in any order: integer multiples of 2^-18 below 2^6 in magnitude),
-// the scaling, y, acc_out and the SQNR sums.  Counters are per (tile, CTA, epilogue warp); the last
+// the scaling, y, acc_out and the SQNR sums.  The scratch has room for a 256-wide part on every pair, so a
+// tail of up to half a wave is always split: 14336 -> 4096 on 4096 tokens (3.37 waves) 149 -> 136 us against
+// room for half as many, when its 28 tail tiles took a fourth wave.  Counters are per (tile, CTA, epilogue warp); the last
 // part to finish sets them back to zero.  Slots of this scratch are handed out round robin per launch.
 constexpr int kSplitSlots = 2;
 constexpr int kMaxSplitTiles = 38;            // half a wave of 76 pairs
-constexpr int kMaxSplitUnits = 80;            // tail tiles x parts x NB / 128 <= pairs
+constexpr int kMaxSplitUnits = 160;           // tail tiles x parts x NB / 128: up to a part per pair, 256 wide
 constexpr int kMaxSplit = 16;
 // Per slot: [part][channel/4][row] float4 slices of NB / 4 x 2 BM, room for kMaxSplitUnits 128-wide parts
 // (half as many 256-wide ones).
