@@ -15,6 +15,11 @@
 // Tile: 64 rows x OC output channels of one block (OC = min(k, 128)), the block slab A_b[c0:c0+OC, :]
 // and the 64 input rows are staged transposed in shared memory; each thread owns 4 rows x 8
 // consecutive channels (32 fp32 accumulators), which is exactly one packed word per row.
+//
+// Small transforms (transform_quant_rows_kernel): where all of T is small, a CTA takes 16 whole rows through every
+// block, so the row maximum never leaves it: one launch and one pass instead of a memset, two passes and a
+// finalize launch, with the same sums in the same order.  512 float32 rows of 256 channels at k = 32: 19 us
+// and four launches before, 8.6 us now.
 #include "common.cuh"
 
 namespace cat {
@@ -116,6 +121,159 @@ __global__ void __launch_bounds__(ActCfg<K>::THREADS) transform_quant_kernel(
   }
 }
 
+// ---- small transforms: 16 whole rows per CTA -------------------------------------------------
+// Thread: output channel c of a slab, RPT rows.  The rows lie in shared memory, all loaded at the start, and a
+// block's x' replaces its x there; the transposed slabs of A arrive by cp.async one ahead (two buffers), so a
+// block costs its sums and two barriers, not a trip to L2.
+// Every CTA reads all of A (from L2), so A is bounded: kRowsMaxT elements (256 KB).
+constexpr int kWholeRows = 16;
+constexpr int kRowsThreads = 256;
+constexpr int64_t kRowsMaxT = 65536;
+constexpr size_t kRowsMaxSmem = 220 * 1024;
+
+template <int K>
+struct RowsCfg {
+  static constexpr int OC = K < 128 ? K : 128, SLABS = K / OC;
+  static constexpr int AS_LD = OC + 1;
+  static constexpr int BUFS = K <= 128 ? 2 : 1;                   // two slabs of 256 inputs would not fit
+  static constexpr int RPT = kWholeRows * OC / kRowsThreads;      // rows per thread
+  static constexpr size_t smem(int64_t d) {
+    return (size_t)kWholeRows * (d + 4) * sizeof(float) + (size_t)BUFS * K * AS_LD * sizeof(float);
+  }
+};
+
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+template <typename Tin, int K>
+__global__ void __launch_bounds__(kRowsThreads) transform_quant_rows_kernel(
+    const Tin* __restrict__ x, int64_t n, int d, const float* __restrict__ A, uint8_t* __restrict__ codes, int e8,
+    float* __restrict__ scale, uint32_t* __restrict__ status) {
+  using C = RowsCfg<K>;
+  extern __shared__ __align__(16) float smem[];
+  float* V = smem;                                   // [16][d + 4]: x, then x'
+  float* As = V + kWholeRows * (d + 4);              // BUFS x [K][AS_LD], transposed slabs
+  __shared__ uint32_t red[kWholeRows];
+  const int tid = threadIdx.x, c = tid % C::OC, r0 = tid / C::OC * C::RPT, ld = d + 4;
+  const int64_t t0 = (int64_t)blockIdx.x * kWholeRows;
+  const int slabs = d / K * C::SLABS;
+  auto load_slab = [&](int s) {                      // slab s: rows s OC .. of the stacked blocks
+    float* dst = As + (s % C::BUFS) * K * C::AS_LD;
+    const float* src = A + (size_t)s * C::OC * K;
+    for (int e = tid; e < C::OC * K; e += kRowsThreads) cp_async4(dst + e % K * C::AS_LD + e / K, src + e);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  load_slab(0);
+  if (tid < kWholeRows) red[tid] = 0u;
+  for (int e = tid; e < kWholeRows * d; e += kRowsThreads) {
+    const int r = e / d, j = e % d;
+    V[r * ld + j] = (t0 + r < n) ? to_f32(x[t0 * d + e]) : 0.f;   // rows past n read as zero
+  }
+  bool finite = true;
+  float m[C::RPT];
+#pragma unroll
+  for (int r = 0; r < C::RPT; ++r) m[r] = 0.f;
+  for (int b = 0; b < d / K; ++b) {
+    float acc[C::SLABS][C::RPT];
+#pragma unroll
+    for (int h = 0; h < C::SLABS; ++h) {
+      const int s = b * C::SLABS + h;
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();                               // slab s (and at first the rows) are in; the slab before is done with
+      if (C::BUFS == 2 && s + 1 < slabs) load_slab(s + 1);
+      const float* a = As + (s % C::BUFS) * K * C::AS_LD + c;
+      const float* v = V + r0 * ld + b * K;
+#pragma unroll
+      for (int r = 0; r < C::RPT; ++r) acc[h][r] = 0.f;
+#pragma unroll 4
+      for (int j = 0; j < K; j += 4) {
+        const float a0 = a[j * C::AS_LD], a1 = a[(j + 1) * C::AS_LD], a2 = a[(j + 2) * C::AS_LD], a3 = a[(j + 3) * C::AS_LD];
+#pragma unroll
+        for (int r = 0; r < C::RPT; ++r) {           // inputs in ascending order, as the tiled kernels add them
+          const float4 xv = *reinterpret_cast<const float4*>(v + r * ld + j);
+          acc[h][r] = fmaf(a3, xv.w, fmaf(a2, xv.z, fmaf(a1, xv.y, fmaf(a0, xv.x, acc[h][r]))));
+        }
+      }
+      if (C::BUFS == 1) {
+        __syncthreads();
+        if (s + 1 < slabs) load_slab(s + 1);
+      }
+    }
+    __syncthreads();                                 // the block's x has been read
+#pragma unroll
+    for (int h = 0; h < C::SLABS; ++h)
+#pragma unroll
+      for (int r = 0; r < C::RPT; ++r) {
+        finite &= isfinite(acc[h][r]);
+        m[r] = fmaxf(m[r], fabsf(acc[h][r]));
+        V[(r0 + r) * ld + b * K + h * C::OC + c] = acc[h][r];
+      }
+  }
+#pragma unroll
+  for (int r = 0; r < C::RPT; ++r) atomicMax(&red[r0 + r], __float_as_uint(m[r]));
+  if (!finite) report(status, kStatusNonFinite);
+  __syncthreads();
+  for (int w = tid; w < kWholeRows * (d / 8); w += kRowsThreads) {
+    const int r = w / (d / 8), i = w % (d / 8);
+    if (t0 + r >= n) break;                          // rows ascend with w
+    const QRow qr = qrow_setup(__uint_as_float(red[r]), 7.0f);
+    const float4 v0 = *reinterpret_cast<const float4*>(V + r * ld + 8 * i);
+    const float4 v1 = *reinterpret_cast<const float4*>(V + r * ld + 8 * i + 4);
+    const float v[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+    int q[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) q[e] = qcode_exact(v[e], qr, 7.0f);
+    if (e8) {
+      uint2 o;
+      o.x = e4m3_code_byte(q[0]) | e4m3_code_byte(q[1]) << 8 | e4m3_code_byte(q[2]) << 16 | e4m3_code_byte(q[3]) << 24;
+      o.y = e4m3_code_byte(q[4]) | e4m3_code_byte(q[5]) << 8 | e4m3_code_byte(q[6]) << 16 | e4m3_code_byte(q[7]) << 24;
+      *reinterpret_cast<uint2*>(codes + (t0 + r) * d + 8 * i) = o;
+    } else {
+      *reinterpret_cast<uint32_t*>(codes + (t0 + r) * (d / 2) + 4 * i) = sm4_pack(q);
+    }
+  }
+  if (tid < kWholeRows && t0 + tid < n) {
+    const float a = __uint_as_float(red[tid]);
+    float s = 0.f;
+    if (isfinite(a))
+      s = __fdiv_rn(a, 7.0f);
+    else
+      report(status, kStatusNonFinite);
+    scale[t0 + tid] = s;
+  }
+}
+
+template <typename Tin, int K>
+cudaError_t launch_rows_k(const Tin* x, int64_t n, int64_t d, const float* A, uint8_t* codes, int e8, float* scale,
+                          uint32_t* status, cudaStream_t stream) {
+  const size_t smem = RowsCfg<K>::smem(d);
+  const int64_t ctas = (n + kWholeRows - 1) / kWholeRows;
+  if (d * K > kRowsMaxT || smem > kRowsMaxSmem || ctas > 0x7FFFFFFF) return cudaErrorNotSupported;
+  // always the same limit: calls from other threads may set it in between
+  cudaError_t e = cudaFuncSetAttribute(transform_quant_rows_kernel<Tin, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kRowsMaxSmem);
+  if (e != cudaSuccess) return e;
+  note_launch();
+  transform_quant_rows_kernel<Tin, K><<<(unsigned)ctas, kRowsThreads, smem, stream>>>(x, n, (int)d, A, codes, e8, scale,
+                                                                                    status);
+  return cudaGetLastError();
+}
+
+// cudaErrorNotSupported (nothing launched): T or the rows are too large, the tiled kernels take the call.
+template <typename Tin>
+cudaError_t launch_rows(const Tin* x, int64_t n, int64_t d, int k, const float* A, uint8_t* codes, int e8, float* scale,
+                        uint32_t* status, cudaStream_t stream) {
+  switch (k) {
+    case 16: return launch_rows_k<Tin, 16>(x, n, d, A, codes, e8, scale, status, stream);
+    case 32: return launch_rows_k<Tin, 32>(x, n, d, A, codes, e8, scale, status, stream);
+    case 64: return launch_rows_k<Tin, 64>(x, n, d, A, codes, e8, scale, status, stream);
+    case 128: return launch_rows_k<Tin, 128>(x, n, d, A, codes, e8, scale, status, stream);
+    case 256: return launch_rows_k<Tin, 256>(x, n, d, A, codes, e8, scale, status, stream);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 // scale[t] = max|v'_t| / 7 (in place).  Non-finite maxima become 0 and raise the status bit.
 __global__ void finalize_scale_kernel(uint32_t* __restrict__ amax_bits, int64_t n, uint32_t* __restrict__ status) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -208,19 +366,25 @@ cudaError_t launch_transform_quantize(const void* x, int dtype, int64_t n, int64
     // k = 256 beyond the fused kernel (more 64-output groups than SMs, more rows than its scratch):
     // the SIMT kernel below
   }
+  const cudaError_t er =
+      dtype == 0 ? launch_rows(static_cast<const float*>(x), n, d, k, A, codes, 0, scale, status, stream)
+                 : launch_rows(static_cast<const __nv_bfloat16*>(x), n, d, k, A, codes, 0, scale, status, stream);
+  if (er != cudaErrorNotSupported) return er;
   if (dtype == 0) return launch_t(static_cast<const float*>(x), n, d, k, A, codes, scale, status, stream);
   return launch_t(static_cast<const __nv_bfloat16*>(x), n, d, k, A, codes, scale, status, stream);
 }
 
 // The same codes as byte codes ([n][d], one E4M3 byte per code), written by the fused tensor-core
-// kernel; cudaErrorNotSupported (nothing launched) where that kernel does not apply.
+// kernel or the whole-row kernel; cudaErrorNotSupported (nothing launched) where neither applies.
 cudaError_t launch_transform_quantize_e8(const void* x, int dtype, int64_t n, int64_t d, int k, const float* A,
                                          uint8_t* codes8, float* scale, uint32_t* status, cudaStream_t stream,
                                          const uint8_t* planes) {
   if (n == 0) return cudaSuccess;
-  if (!transform_quantize_tc_supported(dtype, k, n, d)) return cudaErrorNotSupported;
-  return launch_transform_quantize_tc_fused(x, n, d, k, A, planes, reinterpret_cast<uint32_t*>(scale),
-                                            reinterpret_cast<uint32_t*>(codes8), 1, status, stream);
+  if (transform_quantize_tc_supported(dtype, k, n, d))
+    return launch_transform_quantize_tc_fused(x, n, d, k, A, planes, reinterpret_cast<uint32_t*>(scale),
+                                              reinterpret_cast<uint32_t*>(codes8), 1, status, stream);
+  if (dtype == 0) return launch_rows(static_cast<const float*>(x), n, d, k, A, codes8, 1, scale, status, stream);
+  return launch_rows(static_cast<const __nv_bfloat16*>(x), n, d, k, A, codes8, 1, scale, status, stream);
 }
 
 }  // namespace cat

@@ -591,3 +591,42 @@ def test_calib_cov_long_runs(n, d, k):
     twice = cat.cat_calib_cov(x, k, out=S.clone(), accumulate=True)
     assert float((twice - 2 * ref).norm() / ref.norm()) < 2 * tol
     assert cat.cat_device_status()[0] == 0
+
+
+# ------------------------------------------------------------------------------------------
+# Small transforms: 16 whole rows per CTA
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n,d,k,dtype", [(1, 32, 16, "f32"), (15, 96, 32, "bf16"), (16, 256, 32, "f32"), (17, 128, 128, "f32"),
+                                         (33, 256, 256, "f32"), (50, 2048, 32, "f32"), (40, 512, 128, "f32"), (65, 1024, 64, "f32"),
+                                         (20, 640, 128, "f32")])
+def test_small_transform_whole_rows(n, d, k, dtype):
+    """The whole-row kernel (T up to 65536 elements; 640 x 128 is past it) against the oracle, the packed and the byte
+    form alike; float32 rows of a wider layer whose first blocks are these (the tiled kernels, with zero
+    columns added) get the same codes and steps: the same sums in the same order."""
+    rng = np.random.default_rng(n + d + k)
+    X = rng.standard_normal((n, d)) * rng.lognormal(0, 1.0, d)
+    X[n // 2] = 0.0
+    Xt = WL.cast(X, dtype)
+    T32 = (rng.standard_normal((d // k, k, k)) / np.sqrt(k)).astype(np.float32)
+    x, T = to_dev(Xt), torch.from_numpy(T32).cuda()
+    xq, sx = cat.cat_transform_quantize_act(x, T, k)
+    xq8, sx8 = cat.cat_transform_quantize_act_e8(x, T, None, k)
+    assert torch.equal(sx, sx8) and torch.equal(cat.cat_codes_to_e4m3(xq), xq8)
+    ref = O.transform_quantize_act(Xt.values, T32.astype(np.float64))
+    check_codes(sm4x8.unpack(xq.cpu().numpy()), ref.qx, ref.pre_x)
+    np.testing.assert_allclose(sx.cpu().numpy().astype(np.float64), ref.sx, rtol=1e-5)
+    if dtype == "f32":
+        wide = 128 * 1024 // k                               # T of 131072 elements
+        xw = torch.zeros((n, wide), device="cuda")
+        xw[:, :d] = x
+        Tw = torch.zeros((wide // k, k, k), device="cuda")
+        Tw[: d // k] = T
+        q2, s2 = cat.cat_transform_quantize_act(xw, Tw, k)
+        assert torch.equal(s2, sx) and torch.equal(q2[:, : d // 2], xq)
+    bad = x.clone()
+    bad[n - 1, 1] = float("inf")
+    assert cat.cat_device_status()[0] == 0
+    xq, sx = cat.cat_transform_quantize_act(bad, T, k)
+    assert sx[n - 1].item() == 0.0 and not xq[n - 1].any()
+    assert cat.cat_device_status()[0] == 4
