@@ -24,7 +24,7 @@
 // memory.  Where they don't, the epilogue adds them up into registers first (int32, NB / 2 a thread) and
 // gives tensor memory back before it scales and stores, so the next tile's MMAs wait for the loads only.
 // Measured (8-bit asymmetric activations x 4-bit weights, 2048 x 4096 -> 6144; 8 x 8 bits, 1000 x 14336
-// -> 4096): 230 and 185 us with one CTA per 128 x 128 tile and scalar stores, now 72 and 132 us; with one MMA
+// -> 4096): 230 and 185 us with one CTA per 128 x 128 tile and scalar stores, now 65 and 131 us; with one MMA
 // issuer instead of two the second takes 154 us.
 // Every wait is bounded.
 #include <cstring>
@@ -70,9 +70,11 @@ struct DpGemmCfg {
   static constexpr uint32_t BAR_OFF = EPI_OFF + kEpiWarps * kEpiStage;
   static constexpr size_t SMEM = BAR_OFF + 512 + 1024;
   static constexpr uint32_t TMEM_COLS = NACC * G * NB <= 128 ? 128 : (NACC * G * NB <= 256 ? 256 : 512);
-  static constexpr int CH = NB / 64;                               // 32-column chunks per epilogue warp
+  static constexpr int CHUNKS = NB / 32;                           // 32-column chunks of the tile
+  static constexpr int CH = (CHUNKS + 1) / 2;                      // a quadrant's first epilogue warp takes these, the second the rest
   static_assert(S >= 3 && SMEM <= 227 * 1024, "shared memory");
-  static_assert(sizeof(DpBars) <= 512 && STAGE % 1024 == 0 && G * NB <= 512, "layout");
+  static_assert(sizeof(DpBars) <= 512 && STAGE % 1024 == 0 && ATOM_B % 1024 == 0 && G * NB <= 512, "layout");
+  static_assert(NB % 32 == 0, "pair MMAs have N in steps of 32");
 };
 
 // Bound of the pipeline waits (ns); kWaitLimitNs unless a test shortens it (cat_set_wait_limit_ns).
@@ -233,13 +235,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       int m, nn;
       tile_coords(tile, num_m, num_n, &m, &nn);
       const int row0 = m * 2 * BM + (int)rank * BM + quad * 32, t = row0 + lane;
-      const int col0 = nn * NB + half * (NB / 2);
+      const int col0 = nn * NB + half * C::CH * 32, chunks = half == 0 ? C::CH : C::CHUNKS - C::CH;
       const float sxt = t < n ? sx[t] : 0.f;
       const uint32_t zt = (t < n && zx) ? (uint32_t)zx[t] : 0u;
       if (!mbar_wait_bounded(&bars->acc_full[ab], (tcount / C::NACC) & 1, abort_flag, __LINE__, lim)) break;
       __syncwarp();
       tc_fence_after();
-      const uint32_t tcol = tmem + ((uint32_t)(quad * 32) << 16) + ab * C::G * NB + half * (NB / 2);
+      const uint32_t tcol = tmem + ((uint32_t)(quad * 32) << 16) + ab * C::G * NB + half * C::CH * 32;
       auto gather = [&](int c, uint32_t (&acc)[32]) {  // chunk c: sum over the digit weights, int32
 #pragma unroll
         for (int g = 0; g < C::G; ++g) {
@@ -300,19 +302,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       };
       if constexpr (C::NACC == 2) {                    // the other copy takes the next tile meanwhile
 #pragma unroll 1
-        for (int c = 0; c < C::CH; ++c) {
+        for (int c = 0; c < chunks; ++c) {
           uint32_t acc[32];
           gather(c, acc);
-          if (c == C::CH - 1) release();
+          if (c == chunks - 1) release();
           finish(c, acc);
         }
       } else {
         uint32_t acc[C::CH][32];
 #pragma unroll
-        for (int c = 0; c < C::CH; ++c) gather(c, acc[c]);
+        for (int c = 0; c < C::CH; ++c)
+          if (c < chunks) gather(c, acc[c]);
         release();
 #pragma unroll
-        for (int c = 0; c < C::CH; ++c) finish(c, acc[c]);
+        for (int c = 0; c < C::CH; ++c)
+          if (c < chunks) finish(c, acc[c]);
       }
     }
     if (lane == 0) bulk_wait_all();
@@ -438,14 +442,26 @@ double tile_model(int64_t n, int64_t d_in, int64_t d_out, int64_t pairs) {
 }
 
 // Wide tiles load the token planes less often and have more MMA work behind each wait; narrow ones spread
-// a small call over more pairs.
+// a small call over more pairs, and the widths between fill the last wave (2048 tokens -> 6144 channels: 192
+// tiles of 256 are 2.53 waves, 224 of 224 are 2.95, of seven eighths the work: 71.4 -> 65.3 us at 8 x 4 bits).
 template <int DX, int DW>
 cudaError_t launch_dx_dw(const DpCall& c) {
-  constexpr int WIDE = DX + DW == 4 ? 128 : 256;     // G accumulators of WIDE columns fit tensor memory
+  constexpr int WIDE = DX + DW == 4 ? 128 : 256;         // G accumulators of WIDE columns fit tensor memory
+  constexpr int MID1 = WIDE - 32, MID2 = WIDE == 256 ? 192 : WIDE / 2;   // 224 and 192; 96
   const int64_t pairs = num_sms() / 2;
-  const double w0 = tile_model<DX, DW, WIDE>(c.n, c.d_in, c.d_out, pairs);
-  const double w1 = tile_model<DX, DW, WIDE / 2>(c.n, c.d_in, c.d_out, pairs);
-  return w1 < w0 ? launch_nb<DX, DW, WIDE / 2>(c) : launch_nb<DX, DW, WIDE>(c);
+  const double cost[4] = {tile_model<DX, DW, WIDE>(c.n, c.d_in, c.d_out, pairs),
+                          tile_model<DX, DW, MID1>(c.n, c.d_in, c.d_out, pairs),
+                          tile_model<DX, DW, MID2>(c.n, c.d_in, c.d_out, pairs),
+                          tile_model<DX, DW, WIDE / 2>(c.n, c.d_in, c.d_out, pairs)};
+  int best = 0;
+  for (int i = 1; i < 4; ++i)
+    if (cost[i] < cost[best]) best = i;
+  switch (best) {
+    case 0: return launch_nb<DX, DW, WIDE>(c);
+    case 1: return launch_nb<DX, DW, MID1>(c);
+    case 2: return launch_nb<DX, DW, MID2>(c);
+    default: return launch_nb<DX, DW, WIDE / 2>(c);
+  }
 }
 
 }  // namespace
