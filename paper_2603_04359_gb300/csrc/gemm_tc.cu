@@ -11,8 +11,8 @@
 // Two operand formats share this kernel (template parameter E8):
 //   * byte codes (E8): the codes are stored one E4M3 byte each, so TMA loads them into 128B-swizzled
 //     shared memory as they are and the pair MMAs read both operands there -- no decode warps.  Tiles
-//     are 256 x 128 (four 48 KB stages) or 256 x 256 (NB = 256: three 64 KB stages, the two
-//     accumulators filling tensor memory), chosen per shape by e8_wide_tiles;
+//     are 256 x 128 (four 48 KB stages) or 256 x 256, 224 or 192 (three stages of 64 KB and less, the two
+//     accumulators taking up to all of tensor memory), chosen per shape by e8_tile_width;
 //   * SM4x8 codes: the packed codes are decoded in the kernel, as described below (tiles 256 x 128).
 // Both walk the tiles in bands of kBandM token tiles, and both split a last wave that is at most half
 // full along K.
@@ -100,10 +100,13 @@ constexpr int kEpiBufs8 = 1;                // byte codes: y and y_ref staging b
 // Shared memory and tensor memory of the two operand formats.  The byte-code stages leave room for
 // one y and one y_ref staging buffer per epilogue warp, and the output-channel steps of a chunk go
 // through registers instead of shared memory.
+// Parts a tail tile of nb channels may be split into: the finishing warp takes nb / 4 / parts channel groups, in
+// whole batches.
+__host__ __device__ constexpr int max_parts(int nb) { return nb == 224 ? 2 : 16; }
 template <bool E8, int NB = BN>
 struct GemmLayout {
-  // byte codes at NB = 256: three 64 KB stages; NB = 128: kStages8 stages of 48 KB
-  static constexpr int S = E8 ? (NB == 256 ? 3 : kStages8) : SE;   // operand stages the MMA consumes
+  // byte codes at NB = 256, 224, 192: three stages of 64, 60, 56 KB; NB = 128: kStages8 stages of 48 KB
+  static constexpr int S = E8 ? (NB > 128 ? 3 : kStages8) : SE;   // operand stages the MMA consumes
   static constexpr uint32_t kStageOp = kStageA8 + (uint32_t)(NB / 2) * BK;
   static constexpr int EB = E8 ? kEpiBufs8 : kEpiBufs;   // y staging buffers per epilogue warp
   static constexpr int RB = E8 ? kEpiBufs8 : kEpiBufs;   // y_ref staging buffers per epilogue warp
@@ -114,11 +117,12 @@ struct GemmLayout {
   static constexpr uint32_t kBarOffset = kScaleOffset + (E8 ? 0u : kEpiWarps * NB * 4);
   static constexpr uint32_t kBarRoom = E8 ? 512u : kBarBytes;
   static constexpr size_t kSmemBytes = kBarOffset + kBarRoom + 1024;  // + barriers + alignment slack
-  static constexpr uint32_t kTmem = E8 ? 2 * NB : kTmemCols;   // E8: the two accumulators
+  static constexpr uint32_t kTmem = E8 && NB == 128 ? 256 : kTmemCols;   // E8: the two accumulators (a power of two)
+  static constexpr int kMaxParts = max_parts(NB);        // parts a tail tile may be split into
   static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
   static_assert(S <= SE && EB <= kEpiBufs && RB <= kEpiBufs, "barrier arrays");
   static_assert(E8 || S % kDecGroups == 0, "a decode group's steps keep to the stages of one parity");
-  static_assert((E8 && (NB == 128 || NB == 256)) || NB == BN, "tile widths");
+  static_assert((E8 && (NB == 128 || NB == 192 || NB == 224 || NB == 256)) || NB == BN, "tile widths");
   static_assert(kStageOp % 1024 == 0, "128B-swizzle alignment");
 };
 static_assert(kAccCols + SE * 64 <= kTmemCols, "tensor memory budget");
@@ -137,7 +141,7 @@ struct Bars {
 };
 static_assert(sizeof(Bars) <= GemmLayout<false>::kBarRoom && sizeof(Bars) <= GemmLayout<true>::kBarRoom &&
                   sizeof(Bars) <= GemmLayout<true, 256>::kBarRoom,
-              "barrier block must fit its reserved room");
+              "barrier block must fit its reserved room");  // (the room does not depend on the width)
 
 // ---- tensor-memory stores and the TMA store path -------------------------------------------
 #define CAT_TMEM_ST32(taddr, v)                                                                                 \
@@ -175,7 +179,6 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 constexpr int kSplitSlots = 2;
 constexpr int kMaxSplitTiles = 38;            // half a wave of 76 pairs
 constexpr int kMaxSplitUnits = 160;           // tail tiles x parts x NB / 128: up to a part per pair, 256 wide
-constexpr int kMaxSplit = 16;
 // Per slot: [part][channel/4][row] float4 slices of NB / 4 x 2 BM, room for kMaxSplitUnits 128-wide parts
 // (half as many 256-wide ones).
 constexpr size_t kSplitSlotF4 = (size_t)kMaxSplitUnits * (BN / 4) * (2 * BM);
@@ -492,6 +495,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           constexpr int S = decltype(split_c)::value;
           constexpr int L = S >= 4 ? 16 : 8;      // loads of parts per batch
           constexpr int G = NB / 4 / S, PB = L / S;   // groups of the share, groups per batch
+          static_assert(G % PB == 0, "whole batches");
           const int g0 = w.part * G;
 #pragma unroll 1
           for (int b = 0; b < G; b += PB) {
@@ -542,11 +546,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
           }
         };
-        switch (split) {
-          case 2: fixup(std::integral_constant<int, 2>{}); break;
-          case 4: fixup(std::integral_constant<int, 4>{}); break;
-          case 8: fixup(std::integral_constant<int, 8>{}); break;
-          default: fixup(std::integral_constant<int, 16>{}); break;
+        if constexpr (GemmLayout<E8, NB>::kMaxParts == 2) {
+          fixup(std::integral_constant<int, 2>{});
+        } else {
+          switch (split) {
+            case 2: fixup(std::integral_constant<int, 2>{}); break;
+            case 4: fixup(std::integral_constant<int, 4>{}); break;
+            case 8: fixup(std::integral_constant<int, 8>{}); break;
+            default: fixup(std::integral_constant<int, 16>{}); break;
+          }
         }
         if (with_ref) {
           sig = f2_add(sig, s_run);
@@ -862,6 +870,21 @@ bool split_launch_ok(int64_t pairs) {
   return ok == 1;
 }
 
+// Parts that the tiles of the last wave (of nb channels each) are split into along K: a power of two, when that
+// wave is at most half full; 1: not split.
+int split_parts(int64_t tiles, int64_t num_k, int nb, int64_t pairs) {
+  const int64_t tail = tiles >= pairs ? tiles % pairs : tiles;
+  int split = 1;
+  if (tail > 0 && tail <= kMaxSplitTiles && 2 * tail <= pairs)
+    while (2 * split <= max_parts(nb) && 2 * split * tail <= pairs && 2 * split <= num_k &&
+           2 * split * tail * nb <= (int64_t)kMaxSplitUnits * BN)
+      split *= 2;
+  // a single partial wave has no whole tiles to hide the parts' exchange behind: split it only
+  // when that saves ten K steps or more
+  if (split > 1 && tiles < pairs && num_k - num_k / split < 10) split = 1;
+  return split;
+}
+
 // y_ref != nullptr: the epilogue also forms the SQNR sums of y against y_ref and writes
 // sums3 = {sum y_ref^2, sum (y_ref - y)^2, dB} (sums3 needs no zeroing).  Needs d_out % 4 == 0
 // (TMA row pitch).  E8: xq and wq hold one code per byte, else SM4x8 (two per byte).  NB: channels per
@@ -893,21 +916,12 @@ cudaError_t launch_gemm_tc(const uint8_t* xq, const float* sx, const uint8_t* wq
   const int64_t tiles = ((n + 2 * BM - 1) / (2 * BM)) * ((d_out + NB - 1) / NB);
   const int64_t num_k = (d_in + BK - 1) / BK;
   const int64_t pairs_max = num_sms() / 2;
-  // the last wave's tiles, split along K into a power-of-two number of parts when that wave is at
-  // most half full (the parts wait for one another: only with a cooperative launch)
+  int split = split_parts(tiles, num_k, NB, pairs_max);   // the parts wait for one another: only with a cooperative launch
+  if (split > 1 && !split_launch_ok<E8, NB>(pairs_max)) split = 1;
   const int64_t tail = tiles >= pairs_max ? tiles % pairs_max : tiles;
-  int split = 1;
-  constexpr int64_t kWide = NB / BN;             // a part's scratch, in 128-wide parts
-  if (tail > 0 && tail <= kMaxSplitTiles && 2 * tail <= pairs_max && split_launch_ok<E8, NB>(pairs_max))
-    while (2 * split <= kMaxSplit && 2 * split * tail <= pairs_max && 2 * split <= num_k &&
-           2 * split * tail * kWide <= kMaxSplitUnits)
-      split *= 2;
-  // a single partial wave has no whole tiles to hide the parts' exchange behind: split it only
-  // when that saves ten K steps or more
-  if (split > 1 && tiles < pairs_max && num_k - num_k / split < 10) split = 1;
   const int64_t num_full = split > 1 ? tiles - tail : tiles;
   const int64_t units = num_full + (tiles - num_full) * split;
-  if (split > 1 && ((units - num_full) * kWide > kMaxSplitUnits || num_full % pairs_max != 0))
+  if (split > 1 && ((units - num_full) * NB > kMaxSplitUnits * BN || num_full % pairs_max != 0))
     return cudaErrorInvalidConfiguration;
   const int grid = 2 * (int)(units < pairs_max ? units : pairs_max);  // CTA pairs (cluster of 2)
   if (grid > kSqnrMaxCtas) return cudaErrorInvalidConfiguration;
@@ -933,24 +947,28 @@ cudaError_t launch_gemm_tc(const uint8_t* xq, const float* sx, const uint8_t* wq
                             status);
 }
 
-// Byte codes: 256-channel pair tiles where they take less time than 128-channel ones.  The MMA thread's
-// wait for each stage idles the tensor core for ~200-300 cycles, whatever the tile width, so a 256-wide
-// tile (twice the MMA work per stage) costs kWideTileCost of two 128-wide tiles (measured: 0.78 on the
-// 8192 x 8192 x 28672 and 4096 x 14336 x 4096 layers); but there are half as many tiles to spread over
-// the pairs, and the last wave is not split along K.
-constexpr double kWideTileCost = 0.78;
-bool e8_wide_tiles(int64_t n, int64_t d_out) {
-  const int64_t pairs = num_sms() / 2, m_tiles = (n + 2 * BM - 1) / (2 * BM);
-  const int64_t t128 = m_tiles * ((d_out + BN - 1) / BN), t256 = m_tiles * ((d_out + 255) / 256);
-  // a last wave at most half full is split along K over the idle pairs (in about that proportion),
-  // when the scratch holds at least two parts of each of its tiles (as the launcher decides)
-  auto waves = [&](int64_t tiles, int64_t wide) {
-    const int64_t tail = tiles % pairs;
-    const bool split = tail > 0 && 2 * tail <= pairs && tail <= kMaxSplitTiles && 2 * tail * wide <= kMaxSplitUnits;
-    return split ? (double)tiles / pairs : (double)((tiles + pairs - 1) / pairs);
-  };
-  const double w128 = waves(t128, 1), w256 = 2.0 * kWideTileCost * waves(t256, 2);
-  return w256 < w128;
+// Byte codes: the width of the pair tiles.  The MMA thread's wait for each stage idles the tensor core for
+// ~200-300 cycles, whatever the tile width, so a tile costs kTileBase + its width's share: a 256-wide tile 1.56 of a
+// 128-wide one (measured on the 8192 x 8192 x 28672 and 4096 x 14336 x 4096 layers), the widths between on the
+// line through the two.  Against that stands the last wave: 224 and 192 channels fill it where 256 leave it half
+// empty (2048 tokens, 4096 -> 6144: 2.53 waves of 256, 2.95 of 224: 41.5 -> 39.8 us,
+// with the SQNR sums 57.0 -> 52.2).
+constexpr double kTileBase = 0.44;
+int e8_tile_width(int64_t n, int64_t d_in, int64_t d_out) {
+  const int64_t pairs = num_sms() / 2, m_tiles = (n + 2 * BM - 1) / (2 * BM), num_k = (d_in + BK - 1) / BK;
+  int best = 0;
+  double least = 0.0;
+  for (int nb : {256, 224, 192, 128}) {
+    const int64_t tiles = m_tiles * ((d_out + nb - 1) / nb);
+    const int split = split_parts(tiles, num_k, nb, pairs);   // a tail of split tiles takes 1 / split of a wave
+    const double waves = (double)(tiles / pairs) + (tiles % pairs == 0 ? 0.0 : 1.0 / split);
+    const double cost = waves * (kTileBase + (1.0 - kTileBase) * nb / 128.0);
+    if (best == 0 || cost < least) {
+      best = nb;
+      least = cost;
+    }
+  }
+  return best;
 }
 
 }  // namespace
@@ -964,8 +982,15 @@ cudaError_t launch_w4a4_gemm_tc(const uint8_t* xq, const float* sx, const uint8_
 cudaError_t launch_w4a4_gemm_tc_e8(const uint8_t* xq8, const float* sx, const uint8_t* wq8, const float* sw, int64_t n,
                                    int64_t d_in, int64_t d_out, float* y, int32_t* acc_out, const float* y_ref,
                                    double* sums3, uint32_t* status, cudaStream_t stream) {
-  if (e8_wide_tiles(n, d_out))
-    return launch_gemm_tc<true, 256>(xq8, sx, wq8, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, stream);
+  switch (e8_tile_width(n, d_in, d_out)) {
+    case 256:
+      return launch_gemm_tc<true, 256>(xq8, sx, wq8, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, stream);
+    case 224:
+      return launch_gemm_tc<true, 224>(xq8, sx, wq8, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, stream);
+    case 192:
+      return launch_gemm_tc<true, 192>(xq8, sx, wq8, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, stream);
+    default: break;
+  }
   return launch_gemm_tc<true, BN>(xq8, sx, wq8, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, stream);
 }
 

@@ -148,3 +148,27 @@ def test_transform_quantize_act_e8(n, d, k, dtype):
         b = xq8.cpu().numpy().astype(np.int64)
         check_codes(np.where(b & 0x80, -(b & 0x7F), b & 0x7F), ref.qx, ref.pre_x)
     assert cat.cat_device_status()[0] == 0
+
+
+@pytest.mark.parametrize("n,d_in,d_out", [(2048, 512, 6144), (2047, 300 * 32, 6145), (4096, 1024, 3600), (1100, 4096, 5312),
+                                          (256, 8192, 3000), (201, 4096, 6144), (4096, 14336, 1088)])
+def test_w4a4_linear_e8_tile_widths(n, d_in, d_out):
+    """Shapes whose tiles are 256, 224, 192 and 128 channels wide, whole and split along K: accumulators equal to float64
+    products of the codes (exact), y = acc s_x s_w; the SQNR call writes the same y."""
+    g = torch.Generator(device=DEV).manual_seed(n + d_in + d_out)
+    qx, qw = (torch.randint(-7, 8, s, device=DEV, generator=g) for s in ((n, d_in), (d_out, d_in)))
+    b = lambda q: ((q < 0).to(torch.uint8) << 7) | q.abs().to(torch.uint8)  # noqa: E731
+    sx, sw = torch.rand(n, device=DEV, generator=g), torch.rand(d_out, device=DEV, generator=g)
+    acc = torch.full((n, d_out), -1, dtype=torch.int32, device=DEV)
+    y = cat.cat_w4a4_linear_e8(b(qx), sx, b(qw), sw, acc_out=acc)
+    for i in range(0, n, 1024):
+        assert torch.equal(acc[i:i + 1024].double(), qx[i:i + 1024].double() @ qw.double().T)
+    y64 = acc.double() * sx[:, None].double() * sw.double()
+    assert ((y.double() - y64).abs() <= 2.0 ** -22 * y64.abs()).all()          # two float32 roundings and the steps' product
+    y_ref = torch.randn(n, d_out, device=DEV, generator=g)
+    for _ in range(2):                                                         # the counters and slots are clean again
+        y2, out = cat.cat_w4a4_linear_sqnr_e8(b(qx), sx, b(qw), sw, y_ref)
+        assert torch.equal(y2, y)
+        sums = torch.stack([y_ref.double().square().sum(), (y_ref.double() - y.double()).square().sum()])
+        assert ((out[:2] - sums).abs() <= 1e-5 * sums).all()
+    assert cat.cat_device_status()[0] == 0
