@@ -339,11 +339,16 @@ cudaError_t launch_transform_quantize_tc_fused(const void* x, int64_t n, int64_t
                                                const uint8_t* planes, uint32_t* amax, uint32_t* words, int e8,
                                                uint32_t* status, cudaStream_t stream);
 
+cudaError_t launch_transform_quantize_few(const void* x, int dtype, int64_t n, int64_t d, int k, const float* T,
+                                          uint8_t* codes, int e8, float* scale, uint32_t* status, cudaStream_t stream);
+
 // planes (optional): T's pre-split bf16 planes (cat_split_transform), used by the tensor-core path.
 cudaError_t launch_transform_quantize(const void* x, int dtype, int64_t n, int64_t d, int k, const float* A,
                                       uint8_t* codes, float* scale, uint32_t* status, cudaStream_t stream,
                                       const uint8_t* planes) {
   if (n == 0) return cudaSuccess;
+  const cudaError_t e1 = launch_transform_quantize_few(x, dtype, n, d, k, A, codes, 0, scale, status, stream);
+  if (e1 != cudaErrorNotSupported) return e1;             // a few rows
   if (transform_quantize_tc_supported(dtype, k, n, d)) {  // bf16 rows: tensor-core path
     uint32_t* amax = reinterpret_cast<uint32_t*>(scale);
     const cudaError_t ef = launch_transform_quantize_tc_fused(x, n, d, k, A, planes, amax,
@@ -380,6 +385,8 @@ cudaError_t launch_transform_quantize_e8(const void* x, int dtype, int64_t n, in
                                          uint8_t* codes8, float* scale, uint32_t* status, cudaStream_t stream,
                                          const uint8_t* planes) {
   if (n == 0) return cudaSuccess;
+  const cudaError_t e1 = launch_transform_quantize_few(x, dtype, n, d, k, A, codes8, 1, scale, status, stream);
+  if (e1 != cudaErrorNotSupported) return e1;
   if (transform_quantize_tc_supported(dtype, k, n, d))
     return launch_transform_quantize_tc_fused(x, n, d, k, A, planes, reinterpret_cast<uint32_t*>(scale),
                                               reinterpret_cast<uint32_t*>(codes8), 1, status, stream);

@@ -630,3 +630,35 @@ def test_small_transform_whole_rows(n, d, k, dtype):
     xq, sx = cat.cat_transform_quantize_act(bad, T, k)
     assert sx[n - 1].item() == 0.0 and not xq[n - 1].any()
     assert cat.cat_device_status()[0] == 4
+
+
+# ------------------------------------------------------------------------------------------
+# Transform of a few rows (clusters)
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n,d,k,dtype", [(1, 32, 32, "bf16"), (1, 4096, 128, "bf16"), (7, 160, 32, "f32"), (8, 2048, 64, "bf16"),
+                                         (9, 4096, 256, "bf16"), (25, 8192, 128, "bf16"), (31, 1088, 64, "f32"),
+                                         (32, 3968, 128, "f32"), (32, 4096, 32, "bf16"), (3, 7168, 256, "f32")])
+def test_transform_few_rows(n, d, k, dtype):
+    """n <= 32 rows against the oracle: one row to four per cluster, ragged shares of the outputs, the packed and the
+    byte form alike, an all-zero and a non-finite row."""
+    rng = np.random.default_rng(n + d + k)
+    X = rng.standard_normal((n, d)) * rng.lognormal(0, 1.0, d)
+    if n > 2:
+        X[n // 2] = 0.0
+    Xt = WL.cast(X, dtype)
+    T32 = (rng.standard_normal((d // k, k, k)) / np.sqrt(k)).astype(np.float32)
+    x, T = to_dev(Xt), torch.from_numpy(T32).cuda()
+    xq, sx = cat.cat_transform_quantize_act(x, T, k)
+    xq8, sx8 = cat.cat_transform_quantize_act_e8(x, T, None, k)
+    assert torch.equal(sx, sx8) and torch.equal(cat.cat_codes_to_e4m3(xq), xq8)
+    ref = O.transform_quantize_act(Xt.values, T32.astype(np.float64))
+    check_codes(sm4x8.unpack(xq.cpu().numpy()), ref.qx, ref.pre_x)
+    # the largest |x'|: 4 sums in order and a tree of 5 round 9 times, 2^-24 each, of sums at most ~3 of its size
+    np.testing.assert_allclose(sx.cpu().numpy().astype(np.float64), ref.sx, rtol=2e-6)
+    assert cat.cat_device_status()[0] == 0
+    bad = x.clone()
+    bad[n - 1, d - 1] = float("inf")
+    q2, s2 = cat.cat_transform_quantize_act(bad, T, k)
+    assert s2[n - 1].item() == 0.0 and not q2[n - 1].any() and torch.equal(q2[: n - 1], xq[: n - 1])
+    assert cat.cat_device_status()[0] == 4
