@@ -608,21 +608,61 @@ int stages_for(int ntok, int nk, int parts) {
   return sp - sp % kDecGroups;
 }
 
+cudaLaunchAttribute cluster_of(int ctas) {
+  cudaLaunchAttribute a;
+  memset(&a, 0, sizeof(a));
+  a.id = cudaLaunchAttributeClusterDimension;
+  a.val.clusterDim.x = (unsigned)ctas;
+  a.val.clusterDim.y = a.val.clusterDim.z = 1;
+  return a;
+}
+
+// CTAs that are resident at once as clusters of 1, 2, 4 and 8 (asked once per process and token count; clusters
+// stay within a group of SMs: 8s fill 120 of 152 here, 4s 144).
+template <int NTOK>
+int resident_ctas(int log2_parts) {
+  static std::once_flag once;
+  static int ctas[4];
+  std::call_once(once, [] {
+    for (int i = 0; i < 4; ++i) {
+      ctas[i] = i == 0 ? num_sms() : 0;
+      cudaLaunchConfig_t cfg;
+      memset(&cfg, 0, sizeof(cfg));
+      cfg.gridDim = dim3(1u << i, 1, 1);
+      cfg.blockDim = dim3(kThreads, 1, 1);
+      cfg.dynamicSmemBytes = kSmemBudget + 4096;
+      cudaLaunchAttribute attr = cluster_of(1 << i);
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      int found = 0;
+      if (i > 0 &&
+          cudaFuncSetAttribute(w4a4_gemm_decode_tc_kernel<NTOK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kSmemBudget + 4096) == cudaSuccess &&
+          cudaOccupancyMaxActiveClusters(&found, w4a4_gemm_decode_tc_kernel<NTOK, false>, &cfg) == cudaSuccess)
+        ctas[i] = found << i;
+    }
+    cudaGetLastError();
+  });
+  return ctas[log2_parts];
+}
+
 // CTAs per unit (the cluster's size; 1: whole units or stream-K), 0 when the tokens fit in no form.  A CTA
 // takes about kStart + its K steps, in units of one K step (start-up, token staging and the last outputs
-// ~4.5 us against ~0.28 us a step); clusters beyond what is resident run in waves, stream-K does not.
-constexpr int kStart = 16;
+// ~4.5 us against ~0.28 us a step), a cluster kExchange more; clusters beyond what is resident run in waves,
+// stream-K does not.
+constexpr int kStart = 16, kExchange = 2;
 int pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms) {
   const int ntok = n <= 16 ? 16 : 32;
   const int64_t num_ks = (d_in / 2 + KSB - 1) / KSB, units = (d_out + UM - 1) / UM;
   int best = 0;
   int64_t least = 0;
-  for (int parts = 1; parts <= kMaxParts && parts <= num_ks; parts *= 2) {
+  for (int i = 0, parts = 1; parts <= kMaxParts && parts <= num_ks; ++i, parts *= 2) {
     const int64_t nk = (num_ks + parts - 1) / parts;
-    if (stages_for(ntok, (int)nk, parts) == 0) continue;
-    const int64_t resident = sms / parts * parts;
-    int64_t cost = parts == 1 && units > sms ? kStart + (units * num_ks + sms - 1) / sms
-                                             : ((units * parts + resident - 1) / resident) * (kStart + nk);
+    const int64_t resident = ntok == 16 ? resident_ctas<16>(i) : resident_ctas<32>(i);
+    if (stages_for(ntok, (int)nk, parts) == 0 || resident < parts) continue;
+    const int64_t cost = parts == 1 && units > sms
+                             ? kStart + (units * num_ks + sms - 1) / sms
+                             : ((units * parts + resident - 1) / resident) * (kStart + nk + (parts > 1 ? kExchange : 0));
     if (best == 0 || cost < least) {
       best = parts;
       least = cost;
@@ -715,9 +755,7 @@ cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, c
     attrs[1].id = cudaLaunchAttributeCooperative;     // the owners of cut units wait for the other parts
     attrs[1].val.cooperative = 1;
   } else {
-    attrs[1].id = cudaLaunchAttributeClusterDimension;
-    attrs[1].val.clusterDim.x = (unsigned)parts;
-    attrs[1].val.clusterDim.y = attrs[1].val.clusterDim.z = 1;
+    attrs[1] = cluster_of(parts);
   }
   cfg.attrs = attrs;
   cfg.numAttrs = split || parts > 1 ? 2 : 1;
