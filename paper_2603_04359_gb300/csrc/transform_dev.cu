@@ -15,9 +15,10 @@
 // operations; the columns' scales are kept apart and folded in once a sweep), their angles in float32 (a
 // sweep is repeated until the columns are orthogonal; each rotation is made orthogonal in float64).  A
 // block's rows are split over a cluster of four CTAs, which exchange k / 2 partial inner products a round,
-// so that 32 blocks keep 128 SMs busy.  Measured, 4096 channels at k = 128: 11.6 ms (rotations 6.0 and 4.1 in
-// 12 and 8 sweeps of ~0.5, Cholesky 0.9, products 0.6) against 271 ms for the host's Jacobi on 16 cores.  A
-// round takes ~3.9 us, ~1.5 of them fmas: the rest is the exchange, the barriers and the angles' latency.
+// so that 32 blocks keep 128 SMs busy.  Measured, 4096 channels at k = 128: 9.9 ms (rotations 5.1 and 3.4 in
+// 11 and 7 sweeps of ~0.47, Cholesky 0.8, products 0.6) against 271 ms for the host's Jacobi on 16 cores.  A
+// round takes ~3.6 us, ~1.5 of them fmas; the rest is the exchange across the cluster (four CTAs are the best: two
+// double the fmas, eight do not fit the SMs).
 //
 // The host path (transform_host.cpp) stays for what this one does not decide: k = 256, the diagonal kind,
 // and any layer with a block whose condition numbers may exceed 1e11 (a bound from the traces of a block
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(kThreads)
   const double f = which ? 1.0 : inv_n;
   if (tid == 0) {
     double tr = 0.0;
+#pragma unroll 16
     for (int i = 0; i < K; ++i) tr += in[i * K + i] * f;
     s_tr = tr;
     s_bad = !(tr > 1e-280 && tr < 1e280);
@@ -83,9 +85,13 @@ __global__ void __launch_bounds__(kThreads)
         s_bad = 1;
         d = 1.0;
       }
-      const double p = sqrt(d);
-      S[j * LD + j] = p;
-      dinv[j] = 1.0 / p;
+      // d^{-1/2} by Newton steps from float32 (d is at most the scaled trace; tiny pivots by the library)
+      double r = (double)rsqrtf((float)d);
+      r = r * (1.5 - 0.5 * d * r * r);
+      r = r * (1.5 - 0.5 * d * r * r);
+      if (!(d > 1e-30)) r = 1.0 / sqrt(d);
+      S[j * LD + j] = d * r;
+      dinv[j] = r;
     }
     __syncthreads();
     if (s_bad) break;             // uniform: read after the barrier, set before it
@@ -106,17 +112,15 @@ __global__ void __launch_bounds__(kThreads)
     const int c = tid;
     double sq = dinv[c] * dinv[c];
     for (int i = 1; i < K; ++i) {
-      double s0 = 0.0, s1 = 0.0;
-      for (int j = 0; j < i; j += 2) {
-        const double x0 = j < c ? 0.0 : (j == c ? dinv[c] : S[c * LD + j]);
-        s0 += S[i * LD + j] * x0;
-        if (j + 1 < i) {
-          const double x1 = j + 1 < c ? 0.0 : (j + 1 == c ? dinv[c] : S[c * LD + j + 1]);
-          s1 += S[i * LD + j + 1] * x1;
+      double s4[4] = {0.0, 0.0, 0.0, 0.0};         // four chains: the sums are a matter of latency
+      for (int j0 = 0; j0 < i; j0 += 4)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int j = j0 + e;
+          if (j < i) s4[e] += S[i * LD + j] * (j < c ? 0.0 : (j == c ? dinv[c] : S[c * LD + j]));
         }
-      }
       if (i > c) {
-        const double x = -(s0 + s1) * dinv[i];
+        const double x = -((s4[0] + s4[1]) + (s4[2] + s4[3])) * dinv[i];
         S[c * LD + i] = x;
         sq += x * x;
       }
@@ -184,19 +188,31 @@ __device__ __forceinline__ void st_cluster(double* p, uint32_t rank, double v) {
 
 // One-sided Jacobi rotations of the columns of X[b] (K x K, in place) until they are orthogonal; sig2 gets
 // the squared norms.  Cluster of four CTAs per block, K / 4 rows each.  A round rotates K / 2 disjoint
-// column pairs (round robin): lane = pair, a warp's rows are its row group's.  Every CTA adds up the same
-// partial inner products in the same order, so all four take the same decisions.
+// column pairs (round robin).  Eight warps hold the rows (a warp its own, lane = pair): inner products, then the
+// rotations.  Two more warps (thread = pair) add up the partial inner products, exchange them and find the
+// angles; what an angle needs besides the inner product is worked out before the exchange, and the scales and
+// norms are updated while the others rotate, so a round's chain of float64 latencies is short.  Every CTA adds
+// up the same partial inner products in the same order, so all four take the same decisions.
 template <int K>
-__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads)
+struct JacCfg {
+  static constexpr int RPC = K / kCluster, PAIRS = K / 2;
+  static constexpr int NW = RPC < 8 ? RPC : 8, RW = RPC / NW;   // warps with rows, rows per warp
+  static constexpr int PL = PAIRS > 32 ? PAIRS / 32 : 1;        // pairs per lane
+  static constexpr int WARPS = 8 + PL;
+  static constexpr size_t SMEM =
+      (size_t)(RPC * K + NW * PAIRS + 2 * kCluster * PAIRS + kCluster * K + 3 * K + 2 * PAIRS) * sizeof(double);
+};
+
+template <int K>
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(JacCfg<K>::WARPS * 32)
     jacobi_kernel(double* __restrict__ X, double* __restrict__ sig2, const int* __restrict__ skip_if, int n_skip,
                   int* __restrict__ flag) {
-  constexpr int RPC = K / kCluster, PAIRS = K / 2;
-  constexpr int PG = (PAIRS + 31) / 32;                       // warps across the pairs
-  constexpr int RG = 8 / PG < RPC ? 8 / PG : RPC;             // row groups
+  using C = JacCfg<K>;
+  constexpr int RPC = C::RPC, PAIRS = C::PAIRS, NW = C::NW, RW = C::RW, PL = C::PL, NT = C::WARPS * 32;
   extern __shared__ double sm[];
   double* xs = sm;                                // [RPC][K]
-  double* part = xs + RPC * K;                    // [RG][PAIRS]
-  double* inbox = part + RG * PAIRS;              // [2][kCluster][PAIRS]
+  double* part = xs + RPC * K;                    // [NW][PAIRS]
+  double* inbox = part + NW * PAIRS;              // [2][kCluster][PAIRS]
   double* inbox_n = inbox + 2 * kCluster * PAIRS; // [kCluster][K]
   double* nrm = inbox_n + kCluster * K;           // squared norms of the (scaled) columns
   double* scl = nrm + K;                          // column scales and their reciprocals
@@ -209,18 +225,21 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads)
   for (int i = 0; i < n_skip; ++i)
     if (skip_if[i]) return;                       // raised by earlier launches: the same for the whole grid
   double* Xb = X + (size_t)b * K * K + (size_t)rank * RPC * K;
-  for (int q = tid; q < RPC * K; q += kThreads) xs[q] = Xb[q];
-  for (int c = tid; c < K; c += kThreads) scl[c] = isc[c] = 1.0;
+  for (int q = tid; q < RPC * K; q += NT) xs[q] = Xb[q];
+  for (int c = tid; c < K; c += NT) scl[c] = isc[c] = 1.0;
   if (tid == 0) s_big = 0;
   cluster_sync();
-  const int pair = (warp % PG) * 32 + lane, rg = warp / PG;
-  const bool work = pair < PAIRS && rg < RG;
+  // the round's pair i: column K - 1 with r for i = 0, r + i with r - i modulo K - 1 for the others
+  auto pair_of = [](int i, int r, int* p, int* q) {
+    *p = i == 0 ? K - 1 : r + i - (r + i >= K - 1 ? K - 1 : 0);
+    *q = i == 0 ? r : r - i + (r - i < 0 ? K - 1 : 0);
+  };
   bool done = false;
   uint32_t round = 0;
   auto fold = [&] {                               // the scales into the columns, and the columns' norms
-    for (int q = tid; q < RPC * K; q += kThreads) xs[q] *= scl[q % K];
+    for (int q = tid; q < RPC * K; q += NT) xs[q] *= scl[q % K];
     __syncthreads();
-    for (int c = tid; c < K; c += kThreads) {
+    for (int c = tid; c < K; c += NT) {
       double s = 0.0;
 #pragma unroll 4
       for (int r = 0; r < RPC; ++r) s += xs[r * K + c] * xs[r * K + c];
@@ -228,86 +247,108 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads)
       scl[c] = isc[c] = 1.0;
     }
     cluster_sync();
-    for (int c = tid; c < K; c += kThreads)
+    for (int c = tid; c < K; c += NT)
       nrm[c] = ((inbox_n[c] + inbox_n[K + c]) + inbox_n[2 * K + c]) + inbox_n[3 * K + c];
     __syncthreads();
   };
   for (int sweep = 0; sweep < kMaxSweeps && !done; ++sweep) {
     fold();
-    for (int r = 0; r < K - 1; ++r, ++round) {
-      // the round's pair: column K - 1 with r, the others r + i with r - i modulo K - 1
-      int p, q;
-      if (pair == 0) {
-        p = K - 1;
-        q = r;
-      } else {
-        p = r + pair;
-        if (p >= K - 1) p -= K - 1;
-        q = r - pair;
-        if (q < 0) q += K - 1;
-      }
-      if (work) {
-        double s = 0.0;
-#pragma unroll 4
-        for (int row = rg; row < RPC; row += RG) s += xs[row * K + p] * xs[row * K + q];
-        part[rg * PAIRS + pair] = s;
-      }
-      __syncthreads();
-      double* in = inbox + (round & 1u) * (kCluster * PAIRS);
-      if (tid < PAIRS) {                          // pair == tid there: warps below PG have row group 0
-        double s = part[tid];
-        for (int g = 1; g < RG; ++g) s += part[g * PAIRS + tid];
-        for (uint32_t c = 0; c < kCluster; ++c) st_cluster(&in[rank * PAIRS + tid], c, s);
-      }
-      cluster_sync();                             // round r + 2 writes this inbox only after round r + 1's barrier
-      if (tid < PAIRS) {
-        const double dot = ((in[tid] + in[PAIRS + tid]) + in[2 * PAIRS + tid]) + in[3 * PAIRS + tid];
-        const double sp = scl[p], sq = scl[q], aa = nrm[p], bb = nrm[q];
-        const double ab = dot * sp * sq, ab2 = ab * ab, prod = aa * bb;
-        double u1 = 0.0, u2 = 0.0;
-        if (!(ab2 <= 1e-32 * prod)) {
-          if (!(ab2 <= 1e-28 * prod)) s_big = 1;
-          // tan of the angle in float32, scaled so that its operands are near 1
-          const double big = aa > bb ? aa : bb;
-          const int ex = (int)((__double_as_longlong(big) >> 52) & 0x7FF) - 1023;
-          const double rs = pow2(-ex);
-          const float zeta = (float)((bb - aa) * rs) / (2.0f * (float)(ab * rs));
-          const float t32 = copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
-          const double t = (double)t32;
-          if (t != 0.0 && isfinite(t32)) {
-            // c = (1 + t^2)^{-1/2} by Newton steps from float32, 1 / c = (1 + t^2) c
-            const double x = 1.0 + t * t;
-            double c = (double)rsqrtf((float)x);
-            c = c * (1.5 - 0.5 * x * c * c);
-            c = c * (1.5 - 0.5 * x * c * c);
-            const double ci = x * c;
-            u1 = t * sq * isc[p];
-            u2 = t * sp * isc[q];
-            scl[p] = sp * c;
-            scl[q] = sq * c;
-            isc[p] *= ci;
-            isc[q] *= ci;
-            nrm[p] = aa - t * ab;
-            nrm[q] = bb + t * ab;
+    if (warp < 8) {
+      // ---------------------------------------------------------------- rows: warp w holds w RW .. w RW + RW - 1
+      const bool work = warp < NW && (PAIRS >= 32 || lane < PAIRS);
+      double* xw = xs + (work ? warp * RW * K : 0);
+      for (int r = 0; r < K - 1; ++r, ++round) {
+        int p[PL], q[PL];
+        double x[PL][RW], y[PL][RW];
+#pragma unroll
+        for (int u = 0; u < PL; ++u) {
+          pair_of((lane + 32 * u) % PAIRS, r, &p[u], &q[u]);
+          double s = 0.0;
+#pragma unroll
+          for (int i = 0; i < RW; ++i) {
+            x[u][i] = xw[i * K + p[u]];
+            y[u][i] = xw[i * K + q[u]];
+            s += x[u][i] * y[u][i];
+          }
+          if (work) part[warp * PAIRS + lane + 32 * u] = s;
+        }
+        __syncthreads();
+        cluster_sync();
+        __syncthreads();                          // the multipliers are there
+        if (work) {
+#pragma unroll
+          for (int u = 0; u < PL; ++u) {
+            const double u1 = m1[lane + 32 * u], u2 = m2[lane + 32 * u];
+#pragma unroll
+            for (int i = 0; i < RW; ++i) {
+              xw[i * K + p[u]] = x[u][i] - u1 * y[u][i];
+              xw[i * K + q[u]] = y[u][i] + u2 * x[u][i];
+            }
           }
         }
-        m1[tid] = u1;
-        m2[tid] = u2;
+        __syncwarp();                             // the next round's pairs lie in other lanes of this warp
       }
-      __syncthreads();
-      if (work) {
-        const double u1 = m1[pair], u2 = m2[pair];
-        if (u1 != 0.0 || u2 != 0.0) {
-#pragma unroll 4
-          for (int row = rg; row < RPC; row += RG) {
-            const double x = xs[row * K + p], y = xs[row * K + q];
-            xs[row * K + p] = x - u1 * y;
-            xs[row * K + q] = y + u2 * x;
+    } else {
+      // ---------------------------------------------------------------- angles: thread = pair
+      const int pr = tid - 256;
+      const bool work = pr < PAIRS;
+      for (int r = 0; r < K - 1; ++r, ++round) {
+        int p, q;
+        pair_of(work ? pr : 0, r, &p, &q);
+        __syncthreads();                          // the partial inner products, and the last round's scales and norms
+        double* in = inbox + (round & 1u) * (kCluster * PAIRS);
+        if (work) {
+          double s[NW];
+#pragma unroll
+          for (int g = 0; g < NW; ++g) s[g] = part[g * PAIRS + pr];
+#pragma unroll
+          for (int w = NW / 2; w > 0; w /= 2)
+#pragma unroll
+            for (int g = 0; g < w; ++g) s[g] += s[g + w];
+          for (uint32_t c = 0; c < kCluster; ++c) st_cluster(&in[rank * PAIRS + pr], c, s[0]);
+        }
+        // what the angle needs besides the inner product; rs scales its operands to about 1
+        const double sp = scl[p], sq = scl[q], ip = isc[p], iq = isc[q], aa = nrm[p], bb = nrm[q];
+        const double big = aa > bb ? aa : bb;
+        const double rs = pow2(1023 - (int)((__double_as_longlong(big) >> 52) & 0x7FF));
+        const double ss = sp * sq, sr = ss * rs, k1 = sq * ip, k2 = sp * iq;
+        const float df = (float)((bb - aa) * rs), root = sqrtf((float)(aa * rs)) * sqrtf((float)(bb * rs));
+        __syncwarp();
+        cluster_sync();                           // round r + 2 writes this inbox only after round r + 1's barrier
+        double t = 0.0, ab = 0.0;
+        if (work) {
+          const double dot = (in[pr] + in[PAIRS + pr]) + (in[2 * PAIRS + pr] + in[3 * PAIRS + pr]);
+          const float abf = (float)(dot * sr);
+          if (!(fabsf(abf) <= 1e-16f * root)) {
+            // the columns are orthogonal to 1e-8 of their norms at every rotation of the last sweep: what that sweep
+            // leaves is the square of it
+            if (!(fabsf(abf) <= 1e-8f * root)) s_big = 1;
+            const float zeta = df / (2.0f * abf);
+            const float t32 = copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
+            if (isfinite(t32)) t = (double)t32;
+            ab = dot * ss;
           }
+          m1[pr] = t * k1;
+          m2[pr] = t * k2;
+        }
+        __syncthreads();                          // the others rotate; meanwhile:
+        if (work && t != 0.0) {
+          // c = (1 + t^2)^{-1/2} by Newton steps from float32, 1 / c = (1 + t^2) c
+          const double x = 1.0 + t * t;
+          double c = (double)rsqrtf((float)x);
+          c = c * (1.5 - 0.5 * x * c * c);
+          c = c * (1.5 - 0.5 * x * c * c);
+          const double ci = x * c;
+          scl[p] = sp * c;
+          scl[q] = sq * c;
+          isc[p] = ip * ci;
+          isc[q] = iq * ci;
+          nrm[p] = aa - t * ab;
+          nrm[q] = bb + t * ab;
         }
       }
-      __syncthreads();
     }
+    __syncthreads();
     done = s_big == 0;
     __syncthreads();
     if (tid == 0) s_big = 0;
@@ -324,9 +365,9 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads)
     for (int c = 0; c < K; ++c) sum += nrm[c];     // a NaN anywhere
     if (!done || !(lo > 0.0) || !(hi <= kMaxCond * lo) || !(sum < 1e300)) raise(flag);
   }
-  for (int q = tid; q < RPC * K; q += kThreads) Xb[q] = xs[q];
+  for (int q = tid; q < RPC * K; q += NT) Xb[q] = xs[q];
   if (rank == 0)
-    for (int c = tid; c < K; c += kThreads) sig2[(size_t)b * K + c] = nrm[c];
+    for (int c = tid; c < K; c += NT) sig2[(size_t)b * K + c] = nrm[c];
   cluster_sync();                                 // no CTA leaves while another may still write to it
 }
 
@@ -408,8 +449,8 @@ template <int K>
 cudaError_t build_k(int64_t nb, const double* sx, int64_t n_calib, const double* sw, int with_h, float* T, float* Aw,
                     double* work, int* ints, cudaStream_t s) {
   constexpr size_t kChol = (size_t)(K * (K + 1) + 2 * K) * 8;
-  constexpr int RPC = K / kCluster, PAIRS = K / 2, PG = (PAIRS + 31) / 32, RG = 8 / PG < RPC ? 8 / PG : RPC;
-  constexpr size_t kJac = (size_t)(RPC * K + RG * PAIRS + 2 * kCluster * PAIRS + kCluster * K + 3 * K + 2 * PAIRS) * 8;
+  constexpr size_t kJac = JacCfg<K>::SMEM;
+  constexpr int kJacThreads = JacCfg<K>::WARPS * 32;
   constexpr int PW = K < 32 ? K : 32;
   constexpr size_t kComp = (size_t)(2 * K * PW + K * 17 + 32) * 8;
   cudaError_t e;
@@ -429,11 +470,11 @@ cudaError_t build_k(int64_t nb, const double* sx, int64_t n_calib, const double*
   if ((e = launched()) != cudaSuccess) return e;
   tn_kernel<<<dim3(g, tl, tl), kThreads, 0, s>>>(b0, b1, nullptr, K, b3);            // X = L^T R
   if ((e = launched()) != cudaSuccess) return e;
-  jacobi_kernel<K><<<kCluster * g, kThreads, kJac, s>>>(b3, sig, flags, 1, flags + 1);
+  jacobi_kernel<K><<<kCluster * g, kJacThreads, kJac, s>>>(b3, sig, flags, 1, flags + 1);
   if ((e = launched()) != cudaSuccess) return e;
   tn_kernel<<<dim3(g, tl, tl), kThreads, 0, s>>>(b2, b3, sig, K, b0);                // Y = L^{-T} W sigma^{-1/2}
   if ((e = launched()) != cudaSuccess) return e;
-  jacobi_kernel<K><<<kCluster * g, kThreads, kJac, s>>>(b0, sig, flags, 2, flags + 2);
+  jacobi_kernel<K><<<kCluster * g, kJacThreads, kJac, s>>>(b0, sig, flags, 2, flags + 2);
   if ((e = launched()) != cudaSuccess) return e;
   compose_kernel<K><<<dim3(g, K / PW), kThreads, kComp, s>>>(b0, sig, exps, with_h, T, Aw, flags);
   return launched();
