@@ -30,6 +30,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "gemm_pair.cuh"
 
 namespace cat {
 namespace {
@@ -54,13 +55,14 @@ struct CovCfg {
   static constexpr uint32_t STAGE = BOXES * kBox;
   // long runs: LONG times the chunk and the stage, LONG_S stages
   static constexpr int LONG = G2 == 1 ? 4 : 2, LONG_S = G2 == 1 ? 3 : 4;
-  static constexpr uint32_t BAR_OFF = kStages * STAGE > LONG_S * LONG * STAGE ? kStages * STAGE : LONG_S * LONG * STAGE;
-  static constexpr size_t SMEM = BAR_OFF + 256 + 1024;
+  static constexpr uint32_t BAR_OFF0 = kStages * STAGE, BAR_OFF1 = LONG_S * LONG * STAGE;
+  static constexpr size_t SMEM0 = BAR_OFF0 + 256 + 1024, SMEM1 = BAR_OFF1 + 256 + 1024;
   // kind::f16, D fp32, A = B = BF16, both MN-major (bits 15, 16), M = 128, N = 64
   static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
                                     ((uint32_t)(kSliceN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 };
-static_assert(CovCfg<1>::SMEM <= 227 * 1024 && CovCfg<2>::SMEM <= 227 * 1024, "shared memory budget");
+static_assert(CovCfg<2>::SMEM0 <= 227 * 1024 && CovCfg<1>::SMEM1 <= 227 * 1024 && CovCfg<2>::SMEM1 <= 227 * 1024,
+              "shared memory budget");
 
 struct CovBars {
   uint64_t full[kStages], empty[kStages], acc_full, mma_done;
@@ -122,16 +124,15 @@ __device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, ui
       : "memory");
 }
 
-template <int G2>
+template <int G2, bool LONGRUN>
 __global__ void __launch_bounds__(kThreads, 1)
     calib_cov_tc_kernel(const __grid_constant__ CUtensorMap tmX, int n, int d, int k, int tok_per_split,
-                        int chunk, double* __restrict__ sigma, int mode /* 0 store, 1 add, 2 atomic add */,
+                        double* __restrict__ sigma, int mode /* 0 store, 1 add, 2 atomic add */,
                         uint32_t* __restrict__ status) {
-  // chunk: tokens per stage, kChunk or LONG kChunk (the tensor map's box has as many rows)
   using C = CovCfg<G2>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  CovBars* bars = reinterpret_cast<CovBars*>(smem + C::BAR_OFF);
+  CovBars* bars = reinterpret_cast<CovBars*>(smem + (LONGRUN ? C::BAR_OFF1 : C::BAR_OFF0));
   volatile int* abort_flag = &bars->abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = blockIdx.x / C::CTAS;                 // channel group
@@ -140,9 +141,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int c0 = g * C::G;                            // first channel of the group
   const int t_begin = blockIdx.y * tok_per_split;
   const int t_end = min(n, t_begin + tok_per_split);
+  constexpr int chunk = LONGRUN ? C::LONG * kChunk : kChunk;   // tokens per stage (rows of the tensor map's box)
   const int chunks = (t_end - t_begin + chunk - 1) / chunk;
-  const int stages = chunk == kChunk ? kStages : C::LONG_S;
-  const uint32_t box = (uint32_t)chunk * 128, stage = C::BOXES * box;
+  constexpr int stages = LONGRUN ? C::LONG_S : kStages;
+  constexpr uint32_t box = (uint32_t)chunk * 128, stage = C::BOXES * box;
   // 16-token MMA steps, counted as in 64-token chunks (the steps past the run's end are zero rows)
   const int total_steps = (t_end - t_begin + kChunk - 1) / kChunk * (kChunk / 16);
   // accumulators in use: 4 (16 MMA steps each at most) for short runs, 8 beyond -- fewer
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!(ok = mbar_wait_bounded(&bars->full[s], (c / stages) & 1, abort_flag, __LINE__))) break;
         tc_fence_after();
         const uint32_t base = smem_u32(smem + s * stage);
-        const int step0 = c * (chunk / 16), steps = min(chunk / 16, total_steps - step0);
+        const int step0 = c * (chunk / 16), steps = LONGRUN ? min(chunk / 16, total_steps - step0) : chunk / 16;
 #pragma unroll 4
         for (int kk = 0; kk < steps; ++kk) {      // 16 tokens per MMA: 16 rows of 128 B
           const int step = step0 + kk;
@@ -294,6 +296,174 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+// ---- long runs, k <= 128: the token splits of a channel group as a cluster ---------------------------
+//
+// CTA = (group of 128 channels, token split): D = X^T X over its tokens, M = N = 128, so a tile is loaded once
+// instead of once per column slice, four round-robin accumulators filling tensor memory.  The cluster's
+// CTAs (the splits of one group) exchange their float32 sums through distributed shared memory, each adds up
+// 128 / S columns as float pairs (exact to ~48 bits), widens them and writes them: no memset of sigma, no
+// float64 atomics.  Used where the splits are at least twice those of the sliced kernel, so that an
+// accumulator (four here, eight there) takes no more steps than it does there: the error is no larger.
+// 16384 x 4096 (bound by HBM, 20 us at its rate): memset, gap and sliced kernel 39.3 us, now 34.8; at 1024 and 2048 tokens the
+// exchange costs more than it saves (15.3 against 8.6 us, 17.2 against 12.2): kWideRun.
+constexpr int kWideChunk = 128, kWideStages = 4, kWideAcc = 4;
+constexpr int kWideRun = 4096;   // tokens per sliced CTA from which on the exchange (~6 us) is worth it
+constexpr uint32_t kWideBox = kWideChunk * 128, kWideStage = 2 * kWideBox;
+// the exchange: [S][128 rows][128 / S columns + 4] float (rows 16 bytes apart modulo 128: float4 accesses of eight rows
+// lie in different banks); a remote store costs the same at 4 and at 16 bytes a lane
+constexpr uint32_t kWideXch = kWideStages * kWideStage;
+constexpr uint32_t kWideBars = kWideXch + (128 + 4 * 8) * 128 * 4;
+constexpr size_t kWideSmem = kWideBars + 256 + 1024;
+constexpr uint32_t kWideIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(128 >> 3) << 17) |
+                                ((uint32_t)(128 >> 4) << 24);
+static_assert(kWideSmem <= 227 * 1024, "shared memory budget");
+
+__device__ __forceinline__ void st_cluster_f32x4(float* p, uint32_t rank, float a, float b, float c, float d) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(remote), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+    calib_cov_wide_kernel(const __grid_constant__ CUtensorMap tmX, int n, int d, int k, int S, int tok_per_split,
+                          double* __restrict__ sigma, int add, uint32_t* __restrict__ status) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  float* xch = reinterpret_cast<float*>(smem + kWideXch);
+  CovBars* bars = reinterpret_cast<CovBars*>(smem + kWideBars);
+  volatile int* abort_flag = &bars->abort;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int part = blockIdx.x % S, c0 = blockIdx.x / S * 128;    // rank in the cluster, first channel of the group
+  const int t_begin = (int)min((int64_t)n, (int64_t)part * tok_per_split);
+  const int t_end = (int)min((int64_t)n, (int64_t)t_begin + tok_per_split);
+  const int chunks = (t_end - t_begin + kWideChunk - 1) / kWideChunk;
+  const int total_steps = (t_end - t_begin + 15) / 16;
+  const int CW = 128 / S;                                         // columns this CTA finishes
+
+  if (tid == 0) {
+    for (int s = 0; s < kWideStages; ++s) {
+      mbar_init(&bars->full[s], 1);
+      mbar_init(&bars->empty[s], 1);
+    }
+    mbar_init(&bars->acc_full, 1);
+    mbar_init(&bars->mma_done, 1);
+    bars->abort = 0;
+    fence_mbar_init();
+  }
+  __syncwarp();
+  pdl_wait_then_release();                        // nothing global or in tensor memory before this
+  if (warp == 0) tmem_alloc(&bars->tmem_addr, kTmemCols);
+  tc_fence_before();
+  cluster_sync();                                 // the peers run: their shared memory may be written
+  tc_fence_after();
+  const uint32_t tmem = bars->tmem_addr;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      prefetch_tensormap(&tmX);
+      int c = 0;
+      for (; c < chunks; ++c) {
+        const uint32_t s = c % kWideStages;
+        if (c >= kWideStages && !mbar_wait_bounded(&bars->empty[s], ((c / kWideStages) - 1) & 1, abort_flag, __LINE__)) break;
+        mbar_arrive_expect_tx(&bars->full[s], kWideStage);
+        for (int bx = 0; bx < 2; ++bx)
+          tma_load_2d(smem + s * kWideStage + bx * kWideBox, &tmX, c0 + 64 * bx, t_begin + c * kWideChunk, &bars->full[s]);
+      }
+      volatile int no_abort = 0;
+      for (int q = c > kWideStages ? c - kWideStages : 0; q < c; ++q)
+        mbar_wait_bounded(&bars->full[q % kWideStages], (q / kWideStages) & 1, &no_abort);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      bool ok = true;
+      for (int c = 0; c < chunks && ok; ++c) {
+        const uint32_t s = c % kWideStages;
+        if (!(ok = mbar_wait_bounded(&bars->full[s], (c / kWideStages) & 1, abort_flag, __LINE__))) break;
+        tc_fence_after();
+        const uint32_t base = smem_u32(smem + s * kWideStage);
+        const int step0 = c * (kWideChunk / 16), steps = min(kWideChunk / 16, total_steps - step0);
+        for (int kk = 0; kk < steps; ++kk) {      // both operands are the tile: rows past the run's end are not reached,
+          const int step = step0 + kk;            // a step's last tokens past n read as zero
+          const uint64_t desc = sdesc_mnmajor_sw128(base + kk * 2048, kWideBox);
+          mma_bf16_ss(tmem + (step % kWideAcc) * 128, desc, desc, kWideIdesc, step >= kWideAcc);
+        }
+        mma_commit(&bars->empty[s]);
+      }
+      if (ok && chunks > 0) mma_commit(&bars->acc_full);
+      mma_commit(&bars->mma_done);
+      volatile int no_abort = 0;
+      mbar_wait_bounded(&bars->mma_done, 0, &no_abort);
+    }
+  } else {
+    // ---------------------------------------------------------------- this split's sums to the CTAs that finish them
+    const int quad = warp & 3, half = (warp - 2) >> 2;
+    const bool live = chunks > 0 && mbar_wait_bounded(&bars->acc_full, 0, abort_flag, __LINE__);
+    const bool have = __all_sync(0xFFFFFFFFu, live);  // warp-uniform: TMEM loads need the whole warp
+    if (have) tc_fence_after();
+    const int used = total_steps < kWideAcc ? total_steps : kWideAcc;
+#pragma unroll 1
+    for (int cc = 2 * half; cc < 2 * half + 2; ++cc) {
+      float v[32];
+#pragma unroll
+      for (int e = 0; e < 32; ++e) v[e] = 0.f;
+      for (int a = 0; have && a < used; ++a) {
+        uint32_t r[32];
+        __syncwarp();
+        CAT_TMEM_LD32(tmem + ((uint32_t)(quad * 32) << 16) + a * 128 + 32 * cc, r);
+        tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] += __uint_as_float(r[e]);
+      }
+#pragma unroll
+      for (int e = 0; e < 32; e += 4) {           // columns 32 cc + e .. + 3, of CTA (column / CW): this split's part
+        const int col = 32 * cc + e;
+        st_cluster_f32x4(xch + ((size_t)part * 128 + quad * 32 + lane) * (CW + 4) + col % CW, (uint32_t)(col / CW), v[e],
+                         v[e + 1], v[e + 2], v[e + 3]);
+      }
+    }
+    tc_fence_before();
+  }
+
+  __syncwarp();
+  cluster_sync();                                 // every split's sums are in; no remote access after this
+  const int lk = 31 - __clz(k);
+  if (tid < 256) {                                // thread: row r of D, every second four of the CTA's columns
+    const int r = tid & 127, row = c0 + r;
+    // entry (row, col) of D is entry (col, row) of the block (the symmetry): lanes write consecutive doubles
+    double* base = sigma + ((int64_t)(row >> lk) << (2 * lk)) + (row & (k - 1));
+    for (int c = 4 * (tid >> 7); c < CW; c += 8) {
+      float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};   // the splits' sums as float pairs
+      for (int p = 0; p < S; ++p) {
+        const float4 x4 = *reinterpret_cast<const float4*>(xch + ((size_t)p * 128 + r) * (CW + 4) + c);
+        const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float t = __fadd_rn(hi[e], x[e]), bb = __fsub_rn(t, hi[e]);
+          lo[e] = __fadd_rn(lo[e], __fadd_rn(__fsub_rn(hi[e], __fsub_rn(t, bb)), __fsub_rn(x[e], bb)));
+          hi[e] = t;
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int col = c0 + part * CW + c + e;
+        double w = f32_to_f64_fast(hi[e]) + f32_to_f64_fast(lo[e]);
+        if (f32_widen_rare(hi[e]) || f32_widen_rare(lo[e]))
+          w = isfinite(hi[e]) ? f32_to_f64_exact(hi[e]) + f32_to_f64_exact(lo[e]) : f32_to_f64_exact(hi[e]);
+        if (row < d && col < d && row >> lk == col >> lk) {
+          double* dst = base + ((int64_t)(col & (k - 1)) << lk);
+          *dst = add ? *dst + w : w;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (bars->abort && tid == 0) report(status, timeout_bits(kWhereCalib, bars->abort));
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kTmemCols);
+  }
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -318,6 +488,48 @@ int num_sms() {
   return sms;
 }
 
+cudaLaunchAttribute cluster_of(int ctas) {
+  cudaLaunchAttribute a;
+  memset(&a, 0, sizeof(a));
+  a.id = cudaLaunchAttributeClusterDimension;
+  a.val.clusterDim.x = (unsigned)ctas;
+  a.val.clusterDim.y = a.val.clusterDim.z = 1;
+  return a;
+}
+
+// Clusters of 2, 4 and 8 CTAs of the wide kernel that are resident at once (asked once per process).
+int wide_resident(int S) {
+  static std::once_flag once;
+  static int found[4];
+  std::call_once(once, [] {
+    const bool ok = cudaFuncSetAttribute(calib_cov_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kWideSmem) == cudaSuccess;
+    for (int i = 1; i < 4; ++i) {
+      cudaLaunchConfig_t cfg;
+      memset(&cfg, 0, sizeof(cfg));
+      cfg.gridDim = dim3(1u << i, 1, 1);
+      cfg.blockDim = dim3(kThreads, 1, 1);
+      cfg.dynamicSmemBytes = kWideSmem;
+      cudaLaunchAttribute attr = cluster_of(1 << i);
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      if (!ok || cudaOccupancyMaxActiveClusters(&found[i], calib_cov_wide_kernel, &cfg) != cudaSuccess) found[i] = 0;
+    }
+    cudaGetLastError();
+  });
+  return S == 2 ? found[1] : (S == 4 ? found[2] : found[3]);
+}
+
+// The wide kernel's token splits for a run the sliced kernel would cut into `sliced` (0: not for it): the first
+// power of two of at least twice as many, when its clusters take no more waves than the sliced kernel's CTAs.
+int wide_splits(int64_t groups, int64_t sliced, int64_t sms) {
+  int S = 2;
+  while (S < 2 * sliced) S *= 2;
+  if (S > 8 || wide_resident(S) < 1) return 0;
+  const int64_t waves = (groups + wide_resident(S) - 1) / wide_resident(S);
+  return waves <= (2 * groups * sliced + sms - 1) / sms ? S : 0;
+}
+
 template <int G2>
 cudaError_t launch_g(const void* x, int64_t n, int64_t d, int k, double* sigma, int accumulate, uint32_t* status,
                      cudaStream_t stream) {
@@ -333,7 +545,8 @@ cudaError_t launch_g(const void* x, int64_t n, int64_t d, int k, double* sigma, 
   if (ysplits > chunks / 32) ysplits = chunks / 32;
   if (ysplits < 1) ysplits = 1;
   const int64_t tps = ((chunks + ysplits - 1) / ysplits) * kChunk;
-  const int chunk = tps >= kLongRun ? C::LONG * kChunk : kChunk;
+  const int wide = G2 == 1 && tps >= kWideRun ? wide_splits(groups, ysplits, sms) : 0;
+  const int chunk = wide ? kWideChunk : (tps >= kLongRun ? C::LONG * kChunk : kChunk);
   CUtensorMap map;
   memset(&map, 0, sizeof(map));
   cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)n};
@@ -347,9 +560,26 @@ cudaError_t launch_g(const void* x, int64_t n, int64_t d, int k, double* sigma, 
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(calib_cov_tc_kernel<G2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    attr = cudaFuncSetAttribute(calib_cov_tc_kernel<G2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM0);
+    if (attr == cudaSuccess)
+      attr = cudaFuncSetAttribute(calib_cov_tc_kernel<G2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM1);
   });
   if (attr != cudaSuccess) return attr;
+  if (wide) {
+    const int64_t wide_chunks = (n + kWideChunk - 1) / kWideChunk;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(groups * wide), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = kWideSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr1 = cluster_of(wide);
+    cfg.attrs = &attr1;
+    cfg.numAttrs = 1;
+    note_launch();
+    return cudaLaunchKernelEx(&cfg, calib_cov_wide_kernel, map, (int)n, (int)d, k, wide,
+                              (int)((wide_chunks + wide - 1) / wide * kWideChunk), sigma, accumulate ? 1 : 0, status);
+  }
   int mode = accumulate ? 1 : 0;
   if (ysplits > 1) {
     mode = 2;
@@ -362,13 +592,14 @@ cudaError_t launch_g(const void* x, int64_t n, int64_t d, int k, double* sigma, 
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)(groups * C::CTAS), (unsigned)ysplits, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = C::SMEM;
+  const bool long_run = chunk != kChunk;
+  cfg.dynamicSmemBytes = long_run ? C::SMEM1 : C::SMEM0;
   cfg.stream = stream;
   // not a programmatic dependent launch: measured, one gained ~0.4 us per c4 step and lost ~0.7 us per
   // c2 step (the kernel still releases its dependents early)
   note_launch();
-  cudaError_t e = cudaLaunchKernelEx(&cfg, calib_cov_tc_kernel<G2>, map, (int)n, (int)d, k, (int)tps, chunk, sigma, mode,
-                                     status);
+  auto kernel = long_run ? calib_cov_tc_kernel<G2, true> : calib_cov_tc_kernel<G2, false>;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, map, (int)n, (int)d, k, (int)tps, sigma, mode, status);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

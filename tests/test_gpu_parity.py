@@ -577,7 +577,7 @@ def test_decode_gemm_splits(n, d_in, d_out):
 # ------------------------------------------------------------------------------------------
 
 @pytest.mark.parametrize("n,d,k", [(1023, 128, 128), (1024, 256, 64), (1281, 128, 16), (4097, 256, 128), (2100, 512, 256),
-                                   (9001, 256, 256)])
+                                   (9001, 256, 256), (5000, 4096, 64), (3000, 160, 32), (16400, 1024, 128)])
 def test_calib_cov_long_runs(n, d, k):
     """Around the chunk sizes and the token splits, against float64 sums.  A 16-token step's fp32 addition is off by at
     most 2^-23 of its accumulator; an accumulator takes at most n / 64 of them (8 accumulators beyond 1024 tokens,
