@@ -975,17 +975,38 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (WAVES && j >= U && !(ok = mbar_wait_bounded(&tmem_free[j % U], ((j / U) - 1) & 1, abort_flag, __LINE__))) break;
         const uint32_t dcol = tmem + (j % U) * N;
         const uint32_t tbase = smem_u32(ts);
-        for (int h = 0; h < F::XH && ok; ++h) {       // the unit's x stages (two K halves at KD = 256)
+        if constexpr (MODE != kW4) {
+          // b-bit codes are finer: the planes go smallest first, over all of the unit's inputs, so that the L and M
+          // sums round at their own size (measured against float64: layer outputs at 8 bits are as exact as
+          // the SIMT kernel's or better)
+          for (int h = 0; h < F::XH && ok; ++h)
+            ok = mbar_wait_bounded(&bars->x_full[(j * F::XH + h) % F::XS], ((j * F::XH + h) / F::XS) & 1, abort_flag, __LINE__);
+          if (!ok) break;
+          tc_fence_after();
+#pragma unroll
+          for (int sp = 2; sp >= 0; --sp)
+#pragma unroll
+            for (int h = 0; h < F::XH; ++h) {
+              const uint32_t xbase = smem_u32(xs + (j * F::XH + h) % F::XS * F::X_STAGE);
+#pragma unroll
+              for (int kk = 0; kk < F::XW / 16; ++kk) {
+                const int kg = h * (F::XW / 16) + kk;     // the K step within the group's KD inputs
+                const uint32_t a_off = (kk >> 2) * (TM * 128) + (kk & 3) * 32;
+                const uint32_t b_off = (kg >> 2) * (N * 128) + (kg & 3) * 32;
+                mma_bf16(dcol, sdesc_kmajor_sw128(xbase + a_off), sdesc_kmajor_sw128(tbase + sp * F::SPLIT + b_off),
+                         F::IDESC, sp != 2 || (h | kk) != 0);
+              }
+            }
+          for (int h = 0; h < F::XH; ++h) mma_commit(&bars->x_empty[(j * F::XH + h) % F::XS]);
+        }
+        for (int h = 0; MODE == kW4 && h < F::XH && ok; ++h) {   // the unit's x stages (two K halves at KD = 256)
           const int q = j * F::XH + h;
           const uint32_t st = q % F::XS;
           if (!(ok = mbar_wait_bounded(&bars->x_full[st], (q / F::XS) & 1, abort_flag, __LINE__))) break;
           tc_fence_after();
           const uint32_t xbase = smem_u32(xs + st * F::X_STAGE);
 #pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            // b-bit codes are finer: their planes go smallest first, so that the M and L sums round at their
-            // own size (measured against float64, layer outputs at 8 bits are as exact as the SIMT kernel's)
-            const int sp = MODE == kW4 ? i : 2 - i;
+          for (int sp = 0; sp < 3; ++sp) {
             if (own_planes && q == 0) {                 // later stages find every plane in place
               if (!(ok = mbar_wait_bounded(&plane_full[sp], 0, abort_flag, __LINE__))) break;
               tc_fence_after();
@@ -996,7 +1017,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const uint32_t a_off = (kk >> 2) * (TM * 128) + (kk & 3) * 32;
               const uint32_t b_off = (kg >> 2) * (N * 128) + (kg & 3) * 32;
               mma_bf16(dcol, sdesc_kmajor_sw128(xbase + a_off), sdesc_kmajor_sw128(tbase + sp * F::SPLIT + b_off),
-                       F::IDESC, (h | kk | i) != 0);
+                       F::IDESC, (h | kk | sp) != 0);
             }
           }
           if (!ok) break;
