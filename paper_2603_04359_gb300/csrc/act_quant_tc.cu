@@ -375,6 +375,9 @@ __device__ __noinline__ int asym_code_exact(float v, float hi, float lo, float N
   return asym_code(v, asym_row(hi, lo, N), N);
 }
 __device__ __noinline__ int asym_zero_exact(float hi, float lo, float N) { return asym_row(hi, lo, N).z; }
+__device__ __noinline__ float asym_step_exact(float hi, float neg_lo, float N) {
+  return (float)(((double)hi + (double)neg_lo) / (double)N);
+}
 
 template <int MODE>
 __device__ __forceinline__ DpRow dp_row(float hi, float neg_lo, float qmax) {
@@ -393,18 +396,20 @@ __device__ __forceinline__ DpRow dp_row(float hi, float neg_lo, float qmax) {
   r.inv = 0.f;
   if (isfinite(hi) && isfinite(neg_lo) && (hi > 0.f || neg_lo > 0.f)) {
     if (isfinite(w)) r.inv = __fdiv_rn(qmax, w);
-    // z = round(N (-lo) / (hi - lo)), decided like a code
+    // z = round(N (-lo) / (hi - lo)), decided like a code; a range beyond float32 (inv = 0: step and codes 0) keeps its z
     const float p = __fmul_rn(neg_lo, r.inv), rq = rintf(p);
-    r.z = (fabsf(p - rq) <= near_tie_dp(qmax)) ? (int)rq : asym_zero_exact(r.hi, r.lo, qmax);
+    r.z = (isfinite(w) && fabsf(p - rq) <= near_tie_dp(qmax)) ? (int)rq : asym_zero_exact(r.hi, r.lo, qmax);
   }
   return r;
 }
 
 // s = (hi - lo) / N of an asymmetric row: the sum's rounding error (two-sum) and the quotient's remainder (an
 // exact fma) correct one float32 division.  In float64 the watcher's divisions held the CTAs of block 0 (this
-// GPU's FP64 pipe is ~60 times slower): 4096 channels x 2048 tokens 31.9 us at 8 bits, now 23.6.
+// GPU's FP64 pipe is ~60 times slower): 4096 channels x 2048 tokens 31.9 us at 8 bits, now 23.6.  Steps near the
+// subnormals, where the remainder would lose bits, keep the float64 route.
 __device__ __forceinline__ float asym_step(float hi, float neg_lo, float N) {
   const float w = __fadd_rn(hi, neg_lo);
+  if (w < 0x1p-90f) return asym_step_exact(hi, neg_lo, N);
   const float b = __fsub_rn(w, hi);
   const float werr = __fadd_rn(__fsub_rn(hi, __fsub_rn(w, b)), __fsub_rn(neg_lo, b));
   const float q = __fdiv_rn(w, N);
