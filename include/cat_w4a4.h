@@ -102,7 +102,7 @@ unsigned long long cat_kernel_launches(void);
  *                accumulate == 0 the buffer is overwritten, otherwise the sums are added to it, so
  *                calibration sets larger than one batch can be streamed through.
  * bf16 rows run on tensor cores: products are exact and tokens accumulate in fp32 (relative error
- * ~1e-7, which moves the block transform by ~1e-7).  fp32 rows accumulate products and their FMA
+ * ~1e-7 at a few hundred tokens, below 1e-6 at many thousand).  fp32 rows accumulate products and their FMA
  * errors in compensated (double-float) fp32 arithmetic, matching float64 to ~1e-12.  Sums are
  * stored as float64.
  */
@@ -236,8 +236,8 @@ cat_status cat_w4a4_linear(const uint8_t* xq, const float* x_scale, const uint8_
  *   out3   out, device [3] float64: { sum y_ref^2, sum (y_ref - y)^2, 10 log10(ratio) dB }, as cat_sqnr.
  * y is written exactly as cat_w4a4_linear writes it.  The sums are formed in the GEMM's epilogue while
  * y is produced (y is not read back) -- for n > 32 when d_out % 4 == 0, for n <= 32 when the decoded
- * tokens fit in the weight-streaming kernel's shared memory; otherwise the GEMM is followed by the
- * cat_sqnr reduction.  Squares are summed in fp32 over runs of at most 32 outputs, the runs as float pairs
+ * tokens fit in the weight-streaming kernel's shared memory (a cluster of up to eight CTAs shares a row: d_in to
+ * ~80,000 at n <= 16, ~39,000 above); otherwise the GEMM is followed by the cat_sqnr reduction.  Squares are summed in fp32 over runs of at most 32 outputs, the runs as float pairs
  * (hi + lo, ~48 significant bits); the result does not depend on CTA timing.
  */
 cat_status cat_w4a4_linear_sqnr(const uint8_t* xq, const float* x_scale, const uint8_t* Wq, const float* w_scale,
@@ -268,8 +268,9 @@ cat_status cat_codes_to_e4m3(const uint8_t* codes, int64_t rows, int64_t d, uint
  *   Arguments as cat_transform_quantize_act_split, except
  *   xq8  out, device [n][d_in] bytes: the codes of x' as byte codes.
  *   x_scale and the codes are those cat_transform_quantize_act_split writes (the same code decisions).
- *   bf16 rows on the fused tensor-core kernel write the bytes directly; elsewhere the SM4x8 codes go
- *   to stream-ordered scratch (n * d_in / 2 bytes, cudaMallocAsync) and are converted.
+ *   bf16 rows on the fused tensor-core kernel, a few rows (n <= 32) and small fp32 transforms write the bytes
+ *   directly; elsewhere the SM4x8 codes go to stream-ordered scratch (n * d_in / 2 bytes, cudaMallocAsync) and
+ *   are converted.
  */
 cat_status cat_transform_quantize_act_e8(const void* x, cat_dtype dtype, int64_t n, int64_t d_in, int32_t k,
                                          const float* T_blocks, const uint8_t* T_planes, uint8_t* xq8, float* x_scale,
@@ -279,8 +280,8 @@ cat_status cat_transform_quantize_act_e8(const void* x, cat_dtype dtype, int64_t
  * cat_w4a4_linear_e8 -- cat_w4a4_linear on byte codes (Sec. 3 Eq. 5).
  *   xq8 [n][d_in], Wq8 [d_out][d_in] byte codes; x_scale, w_scale, y, acc_out as cat_w4a4_linear.
  *   Same results as cat_w4a4_linear on the SM4x8 form of the same codes, for every n >= 1 (it
- *   always runs the 256 x 128 tile kernel: for n <= 32 the SM4x8 weight-streaming kernel reads half
- *   the bytes).  Asynchronous on stream; errors as cat_w4a4_linear.
+ *   always runs the tile kernel, 256 tokens by 128 to 256 channels: for n <= 32 the SM4x8 weight-streaming
+ *   kernel reads half the bytes).  Asynchronous on stream; errors as cat_w4a4_linear.
  */
 cat_status cat_w4a4_linear_e8(const uint8_t* xq8, const float* x_scale, const uint8_t* Wq8, const float* w_scale,
                               int64_t n, int64_t d_in, int64_t d_out, float* y, int32_t* acc_out, cat_stream_t stream);

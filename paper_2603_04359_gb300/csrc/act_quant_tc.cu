@@ -49,9 +49,9 @@ struct TcCfg {
 // What the fused kernel writes: 4-bit codes (packed words or bytes), or the digit planes of b-bit
 // symmetric or asymmetric codes.  An asymmetric row has two extremes, max(v', 0) and max(-v', 0): both
 // are non-negative floats, so each is an integer maximum of bit patterns as the symmetric one is.
-// The b-bit modes run in the time of the 4-bit one (bound by the same MMAs and hand-over of maxima): layer
-// calls 4096 -> 6144 on 2048 tokens at 8 bits asymmetric 435 -> 270 us and 14336 -> 4096 on 1000 tokens at
-// 8 bits 455 -> 228 us against two SIMT passes over the block products (193 and 259 us, now 17 and 37).
+// The b-bit modes are bound as the 4-bit one (the MMAs, the hand-over of maxima, the quantizer's instructions):
+// 2048 x 4096 at 8 bits asymmetric 193 us with two SIMT passes over the block products, now 23.8 (symmetric 20.1);
+// 1000 x 14336 at 8 bits symmetric 259 us, now 30.0.
 enum FusedMode : int { kW4 = 0, kDpSym = 1, kDpAsym = 2 };
 struct DpOut {
   float qmax;       // symmetric: 2^(b-1) - 1; asymmetric: N = 2^b - 1
@@ -405,7 +405,7 @@ __device__ __forceinline__ DpRow dp_row(float hi, float neg_lo, float qmax) {
 
 // s = (hi - lo) / N of an asymmetric row: the sum's rounding error (two-sum) and the quotient's remainder (an
 // exact fma) correct one float32 division.  In float64 the watcher's divisions held the CTAs of block 0 (this
-// GPU's FP64 pipe is ~60 times slower): 4096 channels x 2048 tokens 31.9 us at 8 bits, now 23.6.  Steps near the
+// GPU's FP64 pipe is ~60 times slower): 4096 channels x 2048 tokens 31.9 us at 8 bits, now 23.8.  Steps near the
 // subnormals, where the remainder would lose bits, keep the float64 route.
 __device__ __forceinline__ float asym_step(float hi, float neg_lo, float N) {
   const float w = __fadd_rn(hi, neg_lo);
