@@ -24,9 +24,12 @@
 // memory.  Where they don't, the epilogue adds them up into registers first (int32, NB / 2 a thread) and
 // gives tensor memory back before it scales and stores, so the next tile's MMAs wait for the loads only.
 // Measured (8-bit asymmetric activations x 4-bit weights, 2048 x 4096 -> 6144; 8 x 8 bits, 1000 x 14336
-// -> 4096): 230 and 185 us with one CTA per 128 x 128 tile and scalar stores, now 65 and 131 us; with one MMA
-// issuer instead of two the second takes 154 us.
+// -> 4096): 230 and 185 us with one CTA per 128 x 128 tile and scalar stores, now 63 and 118 us; with one MMA
+// issuer instead of two (and whole tiles) the second took 154 us, with two 130.
+// Where whole tiles leave the last wave short, the last one to two waves are cut into equal ranges of (tile, stage) steps,
+// one per pair (the stream part below): 8 x 8 bits, 1000 x 14336 -> 4096, 128 tiles on 76 pairs, 129.6 -> 117.5 us.
 // Every wait is bounded.
+#include <atomic>
 #include <cstring>
 #include <mutex>
 
@@ -80,6 +83,69 @@ struct DpGemmCfg {
 // Bound of the pipeline waits (ns); kWaitLimitNs unless a test shortens it (cat_set_wait_limit_ns).
 __device__ uint64_t g_dp_wait_limit = kWaitLimitNs;
 
+// ---- the stream part: the last tiles as equal ranges of stages ---------------------------------
+// Tiles [0, num_full) are whole, num_full / pairs per pair.  The others go in columns of `lanes` tiles (all token tiles of
+// some channels, or single tiles): the steps (column, stage) are cut into one contiguous range per group of `lanes`
+// pairs, and each pair of a group walks one tile of the column, so that a group reads its channel rows once, at the same time
+// (1000 x 14336 -> 4096 at 8 x 8 bits with single tiles instead: 126.1 against 117.5 us).  A tile cut between groups is finished by the pair with its
+// first step (its
+// owner, whose range ends in it); the other pairs begin with their part of it, so the parts are on their way early: each
+// epilogue warp sums its accumulators to int32, stores them to the pair's slice of device scratch and sets the
+// pair's flag for that warp; the owner's same warp waits for it (bounded; the launch is cooperative, so all pairs are
+// resident, and only owners wait) and adds.  Integer sums: exact in any order.  Flags hold the launch's number on its
+// slot of scratch, counted on the device (the last warp to start moves it on), so nothing has to be reset, also after
+// a launch that gave up, and graph replays count as launches.
+constexpr int kStreamSlots = 2;               // launches that may overlap; one fills the device
+constexpr int kStreamCtas = 160;
+constexpr int kStreamWarpInt4 = 4 * 8 * 32;   // a warp's part: up to four chunks of 32 columns x 32 rows
+__device__ int4 g_dp_part[kStreamSlots][kStreamCtas][kEpiWarps][kStreamWarpInt4];
+__device__ uint32_t g_dp_flag[kStreamSlots][kStreamCtas][kEpiWarps];
+__device__ uint32_t g_dp_epoch[kStreamSlots][2];   // launches so far; epilogue warps started
+
+__device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// A pair's work: whole tiles, then its range of the stream part, tile by tile.
+struct DpWork {
+  int tile, k0, k1;                                // stages [k0, k1) of the tile
+};
+template <bool STREAM>
+struct DpWalk {                                    // (not STREAM: whole tiles only)
+  int next_full, num_full, pairs, num_k;
+  int lanes, lane, group, groups, steps, g, g1;    // g: next step of the stream part
+  __device__ DpWalk(int pair, int pairs_, int num_full_, int num_tiles, int num_k_, int lanes_)
+      : next_full(pair), num_full(num_full_), pairs(pairs_), num_k(num_k_) {
+    if constexpr (STREAM) {
+      lanes = lanes_;
+      lane = pair % lanes;
+      group = pair / lanes;
+      groups = pairs / lanes;
+      steps = (num_tiles - num_full) / lanes * num_k;
+      g = group < groups ? begin(group) : 0;
+      g1 = group < groups ? begin(group + 1) : 0;
+    }
+  }
+  __device__ int begin(int q) const { return (int)((int64_t)q * steps / groups); }
+  __device__ bool next(DpWork* w) {
+    if (next_full < num_full) {
+      *w = {next_full, 0, num_k};
+      next_full += pairs;
+      return true;
+    }
+    if constexpr (STREAM) {
+      if (g >= g1) return false;
+      const int k0 = g % num_k, k1 = min(num_k, k0 + g1 - g);
+      *w = {num_full + g / num_k * lanes + lane, k0, k1};
+      g += k1 - k0;
+      return true;
+    }
+    return false;
+  }
+};
+
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, int32_t x, int32_t y, int32_t z,
                                             uint64_t* bar) {
   asm volatile(
@@ -89,13 +155,13 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
-template <int DX, int DW, int NB>
+template <int DX, int DW, int NB, bool STREAM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     dp_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                    const __grid_constant__ CUtensorMap tmY, const float* __restrict__ sx, const int32_t* __restrict__ zx,
                    const float* __restrict__ sw, const int32_t* __restrict__ w_rowsum, int n, int d_in, int d_out,
-                   float* __restrict__ y, int32_t* __restrict__ acc_out, int use_tma_store,
-                   uint32_t* __restrict__ status) {
+                   float* __restrict__ y, int32_t* __restrict__ acc_out, int use_tma_store, int num_full,
+                   int stream_lanes, int stream_slot, uint32_t* __restrict__ status) {
   using C = DpGemmCfg<DX, DW, NB>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -139,11 +205,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       prefetch_tensormap(map);
       uint32_t it = 0;
       bool ok = true;
-      for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
+      DpWalk<STREAM> walk(pair, num_pairs, num_full, num_tiles, num_k, stream_lanes);
+      for (DpWork w; ok && walk.next(&w);) {
         int m, nn;
-        tile_coords(tile, num_m, num_n, &m, &nn);
+        tile_coords(w.tile, num_m, num_n, &m, &nn);
         const int row = is_a ? m * 2 * BM + (int)rank * BM : nn * NB + (int)rank * (NB / 2);
-        for (int ks = 0; ks < num_k; ++ks, ++it) {
+        for (int ks = STREAM ? w.k0 : 0; ks < (STREAM ? w.k1 : num_k); ++ks, ++it) {
           const uint32_t s = it % C::S, use = it / C::S;
           if (use > 0 && !(ok = mbar_wait_bounded(&bars->empty[s], (use - 1) & 1, abort_flag, __LINE__, lim))) break;
           uint8_t* dst = smem + s * C::STAGE + (is_a ? 0u : C::A_BYTES);
@@ -170,8 +237,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const uint32_t grp = warp == 1 ? 0u : 1u;
       uint32_t it = 0;
       bool ok = true;
-      for (int tile = pair; tile < num_tiles && ok; tile += num_pairs)
-        for (int ks = 0; ks < num_k; ++ks, ++it) {
+      DpWalk<STREAM> walk(pair, num_pairs, num_full, num_tiles, num_k, stream_lanes);
+      for (DpWork w; ok && walk.next(&w);)
+        for (int ks = STREAM ? w.k0 : 0; ks < (STREAM ? w.k1 : num_k); ++ks, ++it) {
           const uint32_t s = it % C::S;
           if ((s & 1u) != grp) continue;
           if (!(ok = mbar_wait_bounded(&bars->ready[s], (it / C::S) & 1, abort_flag, __LINE__, lim))) break;
@@ -190,12 +258,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const int me = warp == 1 ? 0 : 1;
       uint32_t it = 0, tcount = 0;
       bool ok = true;
-      for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++tcount) {
+      DpWalk<STREAM> walk(pair, num_pairs, num_full, num_tiles, num_k, stream_lanes);
+      for (DpWork w; ok && walk.next(&w); ++tcount) {
         const uint32_t ab = tcount % C::NACC, use = tcount / C::NACC;
         if (use > 0 && !(ok = mbar_wait_bounded(&bars->acc_empty[ab], (use - 1) & 1, abort_flag, __LINE__, lim))) break;
         tc_fence_after();
         const uint32_t acc = tmem + ab * C::G * NB;
-        for (int ks = 0; ks < num_k; ++ks, ++it) {
+        for (int ks = STREAM ? w.k0 : 0; ks < (STREAM ? w.k1 : num_k); ++ks, ++it) {
           const uint32_t s = it % C::S;
           if (!(ok = mbar_wait_bounded(&bars->full[s], (it / C::S) & 1, abort_flag, __LINE__, lim))) break;
           tc_fence_after();
@@ -214,7 +283,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 for (int kk = 0; kk < KB / 32; ++kk) {    // K = 32 codes per MMA: +32 B within an atom
                   const uint64_t da = sdesc_kmajor_sw128(abase + (uint32_t)(a * C::AT + at) * kAtomA) + 2 * kk;
                   const uint64_t db = sdesc_kmajor_sw128(bbase + (uint32_t)(b * C::AT + at) * C::ATOM_B) + 2 * kk;
-                  mma_pair_ss(acc + g * NB, da, db, kIdesc, (ks != 0 || kk != 0 || !first) ? 1u : 0u);
+                  mma_pair_ss(acc + g * NB, da, db, kIdesc, (ks != (STREAM ? w.k0 : 0) || kk != 0 || !first) ? 1u : 0u);
                 }
               }
           mma_commit_pair(&bars->empty[s]);
@@ -229,11 +298,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------------------ epilogue: token row = TMEM lane
     const int quad = warp & 3, half = (warp - kEpiWarp0) >> 2;
     uint8_t* buf = smem + C::EPI_OFF + (warp - kEpiWarp0) * kEpiStage;
+    const int ew = warp - kEpiWarp0;
+    [[maybe_unused]] uint32_t mark = 0;                // this launch's number on its slot
+    if constexpr (STREAM) {
+      if (lane == 0) {
+        uint32_t* epoch = g_dp_epoch[stream_slot];
+        const uint32_t e = ld_acquire_gpu(&epoch[0]);
+        mark = e + 1u;
+        __threadfence();
+        if (atomicAdd(&epoch[1], 1u) == gridDim.x * kEpiWarps - 1u) {   // every warp has read the number
+          epoch[1] = 0u;
+          __threadfence();
+          epoch[0] = e + 1u;
+        }
+      }
+      mark = __shfl_sync(0xFFFFFFFFu, mark, 0);
+    }
     uint32_t tcount = 0;
-    for (int tile = pair; tile < num_tiles; tile += num_pairs, ++tcount) {
+    DpWalk<STREAM> walk(pair, num_pairs, num_full, num_tiles, num_k, stream_lanes);
+    bool ok = true;
+    for (DpWork w; ok && walk.next(&w); ++tcount) {
       const uint32_t ab = tcount % C::NACC;
+      const bool is_part = STREAM && w.k0 > 0, is_owner = STREAM && w.k0 == 0 && w.k1 < num_k;
       int m, nn;
-      tile_coords(tile, num_m, num_n, &m, &nn);
+      tile_coords(w.tile, num_m, num_n, &m, &nn);
       const int row0 = m * 2 * BM + (int)rank * BM + quad * 32, t = row0 + lane;
       const int col0 = nn * NB + half * C::CH * 32, chunks = half == 0 ? C::CH : C::CHUNKS - C::CH;
       const float sxt = t < n ? sx[t] : 0.f;
@@ -260,6 +348,60 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(&bars->acc_empty[ab], 0);
+      };
+      auto put_part = [&](int c, const uint32_t (&acc)[32]) {
+        int4* dst = g_dp_part[stream_slot][blockIdx.x][ew] + c * 8 * 32 + lane;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          __stcg(dst + q * 32, make_int4((int)acc[4 * q], (int)acc[4 * q + 1], (int)acc[4 * q + 2], (int)acc[4 * q + 3]));
+      };
+      auto set_flag = [&] {
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) atomicExch(&g_dp_flag[stream_slot][blockIdx.x][ew], mark);
+      };
+      // the owner: the groups after this one whose ranges begin before the tile ends
+      auto parts = [&](auto&& f) {
+        const int tile_end = ((w.tile - num_full) / walk.lanes + 1) * num_k;
+        for (int q = walk.group + 1; q < walk.groups && walk.begin(q) < tile_end; ++q)
+          if (walk.begin(q) < walk.begin(q + 1)) f(2 * (q * walk.lanes + walk.lane) + (int)rank);
+      };
+      auto wait_parts = [&] {
+        bool got = true;
+        parts([&](int cta) {
+          const uint32_t* flag = &g_dp_flag[stream_slot][cta][ew];
+          if (got && lane == 0 && ld_acquire_gpu(flag) != mark) {
+            const uint64_t t0 = globaltimer_ns();
+            for (uint32_t i = 1; got && ld_acquire_gpu(flag) != mark; ++i) {
+              __nanosleep(64);
+              if ((i & 63u) == 0u && (*abort_flag || globaltimer_ns() - t0 > lim)) {
+                if (*abort_flag == 0) *abort_flag = __LINE__;
+                got = false;
+              }
+            }
+          }
+          got = __shfl_sync(0xFFFFFFFFu, (int)got, 0);
+        });
+        return got;
+      };
+      auto add_parts = [&](int c, uint32_t (&acc)[32]) {
+        parts([&](int cta) {
+          const int4* src = g_dp_part[stream_slot][cta][ew] + c * 8 * 32 + lane;
+          constexpr int B = C::NACC == 2 ? 8 : 2;      // loads in flight: the registers left beside the accumulators
+#pragma unroll
+          for (int i0 = 0; i0 < 8; i0 += B) {
+            int4 v[B];
+#pragma unroll
+            for (int i = 0; i < B; ++i) v[i] = __ldcg(src + (i0 + i) * 32);
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+              acc[4 * (i0 + i)] += (uint32_t)v[i].x;
+              acc[4 * (i0 + i) + 1] += (uint32_t)v[i].y;
+              acc[4 * (i0 + i) + 2] += (uint32_t)v[i].z;
+              acc[4 * (i0 + i) + 3] += (uint32_t)v[i].w;
+            }
+          }
+        });
       };
       auto finish = [&](int c, uint32_t (&acc)[32]) {
         const int o0 = col0 + c * 32;
@@ -301,19 +443,45 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
       };
       if constexpr (C::NACC == 2) {                    // the other copy takes the next tile meanwhile
+        if constexpr (STREAM)
+          if (is_owner && !(ok = wait_parts())) break;
 #pragma unroll 1
         for (int c = 0; c < chunks; ++c) {
           uint32_t acc[32];
           gather(c, acc);
           if (c == chunks - 1) release();
+          if constexpr (STREAM) {
+            if (is_part) {
+              put_part(c, acc);
+              continue;
+            }
+            if (is_owner) add_parts(c, acc);
+          }
           finish(c, acc);
         }
+        if constexpr (STREAM)
+          if (is_part) set_flag();
       } else {
         uint32_t acc[C::CH][32];
 #pragma unroll
         for (int c = 0; c < C::CH; ++c)
           if (c < chunks) gather(c, acc[c]);
         release();
+        if constexpr (STREAM) {
+          if (is_part) {
+#pragma unroll
+            for (int c = 0; c < C::CH; ++c)
+              if (c < chunks) put_part(c, acc[c]);
+            set_flag();
+            continue;
+          }
+          if (is_owner) {
+            if (!(ok = wait_parts())) break;
+#pragma unroll
+            for (int c = 0; c < C::CH; ++c)
+              if (c < chunks) add_parts(c, acc[c]);
+          }
+        }
 #pragma unroll
         for (int c = 0; c < C::CH; ++c)
           if (c < chunks) finish(c, acc[c]);
@@ -384,6 +552,16 @@ int num_sms() {
   return sms;
 }
 
+// Whole tiles of a launch with a stream part: all but the last one to two waves (tiles >= pairs).
+int64_t stream_full(int64_t tiles, int64_t pairs) { return (tiles / pairs - 1) * pairs; }
+// Tiles of a column of the stream part: all token tiles, where they are one band (tile_coords), whole columns remain
+// and few pairs are left over; else single tiles.
+int stream_lanes(int64_t n, int64_t tiles, int64_t pairs) {
+  const int64_t num_m = (n + 2 * BM - 1) / (2 * BM);
+  const bool fits = num_m <= kBandM && stream_full(tiles, pairs) % num_m == 0 && 16 * (pairs % num_m) <= pairs;
+  return fits ? (int)num_m : 1;
+}
+
 struct DpCall {
   const uint8_t* x_planes;
   const float* sx;
@@ -398,9 +576,39 @@ struct DpCall {
   cudaStream_t stream;
 };
 
+// Whether a cooperative launch of `pairs` CTA pairs fits on this device (checked once per process, on the first
+// device asked).
 template <int DX, int DW, int NB>
+bool stream_launch_ok(int64_t pairs) {
+  using C = DpGemmCfg<DX, DW, NB>;
+  constexpr bool STREAM = true;
+  static int ok = -1;
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  if (ok < 0) {
+    int dev = 0, coop = 0, clusters = 0;
+    ok = 0;
+    if (2 * pairs <= kStreamCtas && cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+        cudaFuncSetAttribute(dp_gemm_kernel<DX, DW, NB, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) ==
+            cudaSuccess) {
+      cudaLaunchConfig_t cfg;
+      memset(&cfg, 0, sizeof(cfg));
+      cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
+      cfg.blockDim = dim3(kThreads, 1, 1);
+      cfg.dynamicSmemBytes = C::SMEM;
+      if (cudaOccupancyMaxActiveClusters(&clusters, dp_gemm_kernel<DX, DW, NB, STREAM>, &cfg) == cudaSuccess && clusters >= pairs)
+        ok = 1;
+    }
+    cudaGetLastError();
+  }
+  return ok == 1;
+}
+
+template <int DX, int DW, int NB, bool STREAM = false>
 cudaError_t launch_nb(const DpCall& c) {
   using C = DpGemmCfg<DX, DW, NB>;
+  static_assert(C::CH * 8 * 32 <= kStreamWarpInt4, "a warp's part");
   CUtensorMap mx, mw, my;
   memset(&my, 0, sizeof(my));
   if (!plane_map(&mx, c.x_planes, c.n, c.d_in, DX, BM) || !plane_map(&mw, c.w_planes, c.d_out, c.d_in, DW, NB / 2))
@@ -409,36 +617,50 @@ cudaError_t launch_nb(const DpCall& c) {
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(dp_gemm_kernel<DX, DW, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    attr = cudaFuncSetAttribute(dp_gemm_kernel<DX, DW, NB, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
   });
   if (attr != cudaSuccess) return attr;
   const int64_t tiles = ((c.n + 2 * BM - 1) / (2 * BM)) * ((c.d_out + NB - 1) / NB);
   if (tiles > 0x3FFFFFFF) return cudaErrorInvalidValue;
   const int64_t pairs = num_sms() / 2;
+  const int64_t num_full = STREAM ? stream_full(tiles, pairs) : tiles;
+  const int lanes = STREAM ? stream_lanes(c.n, tiles, pairs) : 1;
+  static std::atomic<unsigned> next_slot{0};
+  const int slot = STREAM ? (int)(next_slot.fetch_add(1, std::memory_order_relaxed) % kStreamSlots) : 0;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)(2 * (tiles < pairs ? tiles : pairs)), 1, 1);
+  cfg.gridDim = dim3((unsigned)(2 * (STREAM || tiles > pairs ? pairs : tiles)), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = c.stream;
-  cudaLaunchAttribute attrs[1] = {pdl_attr()};
+  cudaLaunchAttribute attrs[2];
+  attrs[0] = pdl_attr();
+  attrs[1].id = cudaLaunchAttributeCooperative;   // owners wait for their tiles' other parts
+  attrs[1].val.cooperative = 1;
   cfg.attrs = attrs;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = STREAM ? 2 : 1;
   note_launch();
-  return cudaLaunchKernelEx(&cfg, dp_gemm_kernel<DX, DW, NB>, mx, mw, my, c.sx, c.zx, c.sw, c.w_rowsum, (int)c.n,
-                            (int)c.d_in, (int)c.d_out, c.y, c.acc_out, use_tma, c.status);
+  return cudaLaunchKernelEx(&cfg, dp_gemm_kernel<DX, DW, NB, STREAM>, mx, mw, my, c.sx, c.zx, c.sw, c.w_rowsum, (int)c.n,
+                            (int)c.d_in, (int)c.d_out, c.y, c.acc_out, use_tma, (int)num_full, lanes, slot, c.status);
 }
 
 // The cycles a launch with NB-wide tiles should take: whole waves of tiles, each its stages (the MMAs of a
 // stage plus the ~200 cycles its barrier wait idles the tensor core, or the stage's loads at ~55 B per cycle
-// and SM) and an epilogue of ~8 cycles per column and accumulator.
+// and SM) and an epilogue of ~8 cycles per column and accumulator.  With a stream part (from one whole wave on) the
+// stages spread evenly over the pairs of whole groups, for one epilogue and the exchange of the parts more.
+constexpr double kStreamExchange = 16000.0;   // measured 13 to 20 thousand, the loss of L2 sharing included
 template <int DX, int DW, int NB>
-double tile_model(int64_t n, int64_t d_in, int64_t d_out, int64_t pairs) {
+double tile_model(int64_t n, int64_t d_in, int64_t d_out, int64_t pairs, bool stream = false) {
   using C = DpGemmCfg<DX, DW, NB>;
   const int64_t tiles = ((n + 2 * BM - 1) / (2 * BM)) * ((d_out + NB - 1) / NB);
   const double mma = (double)DX * DW * (C::KS / 32) * (NB / 2) + 200.0, load = C::STAGE / 55.0;
-  const double stages = (double)((d_in + C::KS - 1) / C::KS);
-  return (double)((tiles + pairs - 1) / pairs) * (stages * (mma > load ? mma : load) + 8.0 * C::G * NB / C::NACC);
+  const int64_t num_k = (d_in + C::KS - 1) / C::KS;
+  const double stage = mma > load ? mma : load, epi = 8.0 * C::G * NB / C::NACC;
+  if (!stream) return (double)((tiles + pairs - 1) / pairs) * (num_k * stage + epi);
+  if (tiles <= pairs || tiles % pairs == 0) return 1e30;
+  const int64_t full = stream_full(tiles, pairs), lanes = stream_lanes(n, tiles, pairs);
+  const double waves = (double)(full / pairs) + (double)(tiles - full) / (double)(pairs / lanes * lanes);
+  return waves * num_k * stage + (waves + 1.0) * epi + kStreamExchange;
 }
 
 // Wide tiles load the token planes less often and have more MMA work behind each wait; narrow ones spread
@@ -456,6 +678,15 @@ cudaError_t launch_dx_dw(const DpCall& c) {
   int best = 0;
   for (int i = 1; i < 4; ++i)
     if (cost[i] < cost[best]) best = i;
+  // The stream part where the model sees 3.5 % in it (what it is wrong by); 96-wide tiles take a tenth longer than
+  // modelled.  8 x 8 bits: 1000 x 14336 -> 4096 (1.68 waves) 129.6 -> 117.5 us, 2048 x 4096 -> 6144 (5.05, then 96 wide)
+  // 125.7 -> 112.9, 3000 x 4096 -> 4096 126.1 -> 113.0, 512 x 8192 -> 8192 80.0 -> 75.9; below the line 4096 x 4096 -> 4096
+  // (6.74 waves) 144.7 -> 147.6, at 8 x 4 bits 5000 x 4096 -> 6144 (6.3) 151.0 -> 155.9, and tiles for less than a wave,
+  // where nothing hides the exchange, 256 x 8192 -> 8192 43.5 -> 52.3.
+  const double whole = cost[best] * ((best == 1 && MID1 == 96) ? 1.1 : 1.0);
+  if (tile_model<DX, DW, WIDE>(c.n, c.d_in, c.d_out, pairs, true) < 0.965 * whole &&
+      stream_launch_ok<DX, DW, WIDE>(pairs))
+    return launch_nb<DX, DW, WIDE, true>(c);
   switch (best) {
     case 0: return launch_nb<DX, DW, WIDE>(c);
     case 1: return launch_nb<DX, DW, MID1>(c);

@@ -379,3 +379,47 @@ def test_dp_linear_tile_edges(n, d_in, d_out, bx, bw, asym):
     assert torch.equal(acc.double(), ref)
     assert torch.equal(y, acc.float() * sx[:, None] * sw[None, :])
     assert cat.cat_device_status()[0] == 0
+
+
+@pytest.mark.parametrize("n,d_in,d_out,bx,bw,asym", [
+    (300, 3072, 4990, 8, 8, True), (2500, 6144, 1030, 8, 8, False), (1500, 6144, 3396, 6, 8, False),
+    (1000, 6144, 4990, 8, 6, True), (300, 6144, 9980, 8, 4, True)])
+def test_dp_linear_cut_tiles(n, d_in, d_out, bx, bw, asym):
+    """A little over one or two waves of tiles, the last of them cut along K between pairs (in columns of all token tiles
+    or tile by tile), launches after one another and replays of a graph: accumulators equal to float64 products of the
+    codes (exact), y = acc s_x s_w."""
+    rng = np.random.default_rng(n + d_in + d_out)
+    qx, qw = _rand_codes(rng, (n, d_in), bx, asym), _rand_codes(rng, (d_out, d_in), bw, False)
+    zx = rng.integers(0, 2 ** bx, n) if asym else np.zeros(n, dtype=np.int64)
+    sx = torch.from_numpy(rng.uniform(0.01, 2.0, n).astype(np.float32)).to(DEV)
+    sw = torch.from_numpy(rng.uniform(0.001, 0.1, d_out).astype(np.float32)).to(DEV)
+    kw = {}
+    if asym:
+        kw = dict(x_zero=torch.from_numpy(zx.astype(np.int32)).to(DEV),
+                  w_rowsum=torch.from_numpy(qw.sum(axis=1).astype(np.int32)).to(DEV))
+    xp = torch.from_numpy(dp_planes.encode(qx, bx, asym)).to(DEV)
+    wp = torch.from_numpy(dp_planes.encode(qw, bw, False)).to(DEV)
+    ref = torch.from_numpy(qx - zx[:, None]).to(DEV).double() @ torch.from_numpy(qw).to(DEV).double().T
+    acc = torch.empty(n, d_out, dtype=torch.int32, device=DEV)
+    y = torch.empty(n, d_out, dtype=torch.float32, device=DEV)
+
+    def run():
+        cat.cat_linear_dp(xp, bx, sx, wp, bw, sw, y=y, acc_out=acc, **kw)
+
+    def check():
+        assert torch.equal(acc.double(), ref)
+        assert torch.equal(y, acc.float() * sx[:, None] * sw[None, :])
+        assert cat.cat_device_status()[0] == 0
+        acc.fill_(-1)
+        y.fill_(float("nan"))
+
+    for _ in range(3):
+        run()
+        check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+        run()
+    for _ in range(2):
+        graph.replay()
+        check()
