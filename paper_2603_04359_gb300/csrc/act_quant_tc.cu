@@ -320,8 +320,8 @@ __device__ __forceinline__ void load_chunk(uint32_t taddr, uint32_t (&r)[32]) {
 // (qcode_exact): the values are not kept live across that rare branch, which leaves the fast route
 // its registers, and the branch costs about one exact decision rather than 32.
 // qr.inv == 0 (an all-zero or non-finite row): all codes 0.
-// The instructions here and in the maxima pace the kernel in waves (most go to the half-rate integer pipe; a unit's
-// quantization took 1.15 of its ~1.9 us): fma instead of multiply and add, three-operand maxima and a shorter
+// In waves a unit's quantization (1.15 of ~1.9 us) and the hand-over of its maxima pace the kernel; most instructions
+// here go to the half-rate integer pipe.  Fma instead of multiply and add, three-operand maxima and a shorter
 // sign-magnitude step take 8192 x 8192 from 63.8 to 61.1 us (byte codes 66.7 -> 63.8, 8 bits symmetric 98.7 -> 91.0,
 // asymmetric 116.8 -> 111.1), 4096 x 14336 from 64.7 to 62.0, 2048 x 4096 from 14.1 to 13.7.
 __device__ __forceinline__ void quant_chunk(uint32_t (&r)[32], uint32_t taddr, const QRow& qr, uint32_t (&out)[8]) {
