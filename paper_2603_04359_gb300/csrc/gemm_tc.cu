@@ -172,8 +172,8 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // order of magnitude slower), waits until all S parts of the tile have arrived (bounded; the launch
 // is cooperative, so all parts are resident), and then finishes NB / S of the tile's channels:
 // the sum over the parts (exact in any order: integer multiples of 2^-18 below 2^6 in magnitude),
-// the scaling, y, acc_out and the SQNR sums.  The scratch has room for a 256-wide part on every pair, so a
-// tail of up to half a wave is always split: 14336 -> 4096 on 4096 tokens (3.37 waves) 149 -> 136 us against
+// the scaling, y, acc_out and the SQNR sums.  The scratch has room for a 256-wide part on every pair (split_parts
+// says when it is worth it): 14336 -> 4096 on 4096 tokens (3.37 waves) 149 -> 136 us against
 // room for half as many, when its 28 tail tiles took a fourth wave.  Counters are per (tile, CTA, epilogue warp); the last
 // part to finish sets them back to zero.  Slots of this scratch are handed out round robin per launch.
 constexpr int kSplitSlots = 2;
@@ -871,13 +871,17 @@ bool split_launch_ok(int64_t pairs) {
 }
 
 // Parts that the tiles of the last wave (of nb channels each) are split into along K: a power of two, when that
-// wave is at most half full; 1: not split.
+// wave is at most half full; 1: not split.  More than kFreeSplitUnits parts (128 channels each) only where that saves
+// kMinSaved K steps: many wide parts take 6 to 12 us to exchange (26 tail tiles of 256 in two: 454 x 4096 -> 22560 with the
+// SQNR sums 57.5 -> 63.7 us, 28 of them over 56 K steps, 4096 x 14336 -> 4096, 159.6 -> 147.8).
+constexpr int kFreeSplitUnits = 80, kMinSaved = 20;
 int split_parts(int64_t tiles, int64_t num_k, int nb, int64_t pairs) {
   const int64_t tail = tiles >= pairs ? tiles % pairs : tiles;
   int split = 1;
   if (tail > 0 && tail <= kMaxSplitTiles && 2 * tail <= pairs)
     while (2 * split <= max_parts(nb) && 2 * split * tail <= pairs && 2 * split <= num_k &&
-           2 * split * tail * nb <= (int64_t)kMaxSplitUnits * BN)
+           2 * split * tail * nb <= (int64_t)kMaxSplitUnits * BN &&
+           (2 * split * tail * nb <= (int64_t)kFreeSplitUnits * BN || num_k - num_k / (2 * split) >= kMinSaved))
       split *= 2;
   // a single partial wave has no whole tiles to hide the parts' exchange behind: split it only
   // when that saves ten K steps or more
