@@ -957,7 +957,9 @@ cudaError_t launch_gemm_tc(const uint8_t* xq, const float* sx, const uint8_t* wq
 // line through the two.  Against that stands the last wave: 224 and 192 channels fill it where 256 leave it half
 // empty (2048 tokens, 4096 -> 6144: 2.53 waves of 256, 2.95 of 224: 41.5 -> 39.8 us,
 // with the SQNR sums 57.0 -> 52.2).
-constexpr double kTileBase = 0.44;
+// A split adds its exchange, ~3 us or kSplitSteps K steps of a 128-wide tile: 600 x 4096 -> 15000 on 192 wide with a split
+// tail 42.1 us (53.4 with the SQNR sums), on 224 without 39.9 (49.7).
+constexpr double kTileBase = 0.44, kSplitSteps = 6.4;
 int e8_tile_width(int64_t n, int64_t d_in, int64_t d_out) {
   const int64_t pairs = num_sms() / 2, m_tiles = (n + 2 * BM - 1) / (2 * BM), num_k = (d_in + BK - 1) / BK;
   int best = 0;
@@ -966,7 +968,7 @@ int e8_tile_width(int64_t n, int64_t d_in, int64_t d_out) {
     const int64_t tiles = m_tiles * ((d_out + nb - 1) / nb);
     const int split = split_parts(tiles, num_k, nb, pairs);   // a tail of split tiles takes 1 / split of a wave
     const double waves = (double)(tiles / pairs) + (tiles % pairs == 0 ? 0.0 : 1.0 / split);
-    const double cost = waves * (kTileBase + (1.0 - kTileBase) * nb / 128.0);
+    const double cost = waves * (kTileBase + (1.0 - kTileBase) * nb / 128.0) + (split > 1 ? kSplitSteps / num_k : 0.0);
     if (best == 0 || cost < least) {
       best = nb;
       least = cost;
