@@ -61,7 +61,8 @@ __device__ __forceinline__ int asym_code(float v, const AsymRow& a, float N) {
   if (a.inv == 0.f || !isfinite(v)) return a.inv == 0.f ? 0 : a.z;
   const float p = __fmul_rn(v, a.inv);
   float rq = rintf(p);
-  if (fabsf(p - rq) > 0.5f - 0x1p-12f) rq = (float)rint(((double)N * (double)v) / a.r);  // exact route
+  // exact route; also where 1 / step overflowed (hi - lo below N / FLT_MAX): p - rq is then NaN
+  if (!(fabsf(p - rq) <= 0.5f - 0x1p-12f)) rq = (float)rint(((double)N * (double)v) / a.r);
   int q = (int)rq + a.z;
   const int top = (int)N;
   return q < 0 ? 0 : (q > top ? top : q);

@@ -289,28 +289,29 @@ def test_dp_w4a4_equals_packed_path():
 
 
 @pytest.mark.parametrize("bits,asym", [(8, False), (5, True), (8, True)])
-@pytest.mark.parametrize("n,d,k", [(40, 512, 128), (40, 192, 64), (2561, 4096, 128)])
-def test_dp_code_decision_at_the_ends_of_the_range(bits, asym, n, d, k):
-    """T = I, rows from the smallest bf16 subnormals (asymmetric: from where N / (hi - lo) is finite) to near the largest
-    value: the codes are the definition's, exactly.  A step is the float64 quotient rounded once: half a unit in the
-    last place, 2^-24 relative or 2^-150.  A range hi - lo beyond float32 has step 0 and codes 0, and keeps its zero
-    point."""
+@pytest.mark.parametrize("n,d,k,dtype", [(40, 512, 128, "bf16"), (40, 192, 64, "bf16"), (2561, 4096, 128, "bf16"),
+                                         (40, 512, 128, "f32")])
+def test_dp_code_decision_at_the_ends_of_the_range(bits, asym, n, d, k, dtype):
+    """T = I, rows from the smallest bf16 subnormals (where N / (hi - lo) overflows) to near the largest value: the codes
+    are the definition's, exactly, on the tensor-core (bf16) and the SIMT kernel (f32).  A step is the float64 quotient
+    rounded once: half a unit in the last place, 2^-24 relative or 2^-150.  A range hi - lo beyond float32 has step 0 and
+    codes 0, and keeps its zero point."""
     rng = np.random.default_rng(bits + asym + n)
     X = rng.integers(-120, 121, (n, d)) / 64.0
-    for i, e in enumerate([-119, -116, -110] if asym else [-127, -126, -120]):
+    for i, e in enumerate([-127, -126, -120, -119, -116, -110]):
         X[3 + i] *= 2.0 ** e
     for i, e in enumerate([-100, 60, 100, 124]):
-        X[6 + i] *= 2.0 ** e
+        X[9 + i] *= 2.0 ** e
     if asym:
-        X[10] *= 2.0 ** 127
-    Xt = WL.cast(X, "bf16")
+        X[13] *= 2.0 ** 127
+    Xt = WL.cast(X, dtype)
     assert np.array_equal(Xt.values, X)
     T = np.tile(np.eye(k, dtype=np.float32), (d // k, 1, 1))
     planes, sx, zx = cat.cat_transform_quantize_act_dp(to_dev(Xt), torch.from_numpy(T).to(DEV), k, bits, asym)
     if asym:
         q, s, z, _ = O.quantize_rows_asymmetric(Xt.values, bits)
         np.testing.assert_array_equal(zx.cpu().numpy(), z)
-        q[10], s[10] = 0, 0.0
+        q[13], s[13] = 0, 0.0
     else:
         q, s, _ = O.quantize_rows_symmetric(Xt.values, bits)
     np.testing.assert_array_equal(dp_planes.decode(planes.cpu().numpy()), q)
