@@ -447,8 +447,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int e = 0; e < 4; ++e) {
         const int col = c0 + part * CW + c + e;
         double w = f32_to_f64_fast(hi[e]) + f32_to_f64_fast(lo[e]);
-        if (f32_widen_rare(hi[e]) || f32_widen_rare(lo[e]))
-          w = isfinite(hi[e]) ? f32_to_f64_exact(hi[e]) + f32_to_f64_exact(lo[e]) : f32_to_f64_exact(hi[e]);
+        if (f32_widen_rare(hi[e]) || f32_widen_rare(lo[e])) {
+          if (isfinite(hi[e])) {
+            w = f32_to_f64_exact(hi[e]) + f32_to_f64_exact(lo[e]);
+          } else {                                // a sum beyond float32, or a split that is not finite: in float64
+            w = 0.0;
+            for (int p = 0; p < S; ++p) w += f32_to_f64_exact(xch[((size_t)p * 128 + r) * (CW + 4) + c + e]);
+          }
+        }
         if (row < d && col < d && row >> lk == col >> lk) {
           double* dst = base + ((int64_t)(col & (k - 1)) << lk);
           *dst = add ? *dst + w : w;

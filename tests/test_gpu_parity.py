@@ -593,6 +593,24 @@ def test_calib_cov_long_runs(n, d, k):
     assert cat.cat_device_status()[0] == 0
 
 
+def test_calib_cov_long_run_beyond_float32():
+    """Sums past the largest float32 whose token splits are within it (16384 x 4096 at k = 128: four splits a channel group)
+    are the float64 sums, not infinities; an infinity stays in its own entries."""
+    n, d, k = 16384, 4096, 128
+    x = torch.full((n, d), 2.0 ** 57, device="cuda", dtype=torch.bfloat16)   # 4096 tokens: 2^126, all of them 2^128
+    x[::2, 64:] *= -1
+    v = x.double().view(n, d // k, k).transpose(0, 1)
+    ref = v.transpose(1, 2) @ v
+    assert ref.abs().max() > torch.finfo(torch.float32).max
+    S = cat.cat_calib_cov(x, k)
+    assert torch.equal(S, ref)                           # powers of two: no sum rounds
+    x[5, 3] = x[9000, 3] = float("inf")                  # times channels 64..127: +inf in the first split, -inf in the third
+    S = cat.cat_calib_cov(x, k)
+    ref[0, 3, :] = ref[0, :, 3] = float("inf")
+    ref[0, 3, 64:] = ref[0, 64:, 3] = float("nan")
+    assert torch.equal(S.isnan(), ref.isnan()) and torch.equal(S.nan_to_num(7.0), ref.nan_to_num(7.0))
+
+
 # ------------------------------------------------------------------------------------------
 # Small transforms: 16 whole rows per CTA
 # ------------------------------------------------------------------------------------------
