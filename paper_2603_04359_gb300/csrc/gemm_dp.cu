@@ -382,6 +382,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
           got = __shfl_sync(0xFFFFFFFFu, (int)got, 0);
         });
+        __threadfence();                               // the parts' stores are seen by every lane, not by the polling one alone
         return got;
       };
       auto add_parts = [&](int c, uint32_t (&acc)[32]) {
