@@ -27,8 +27,18 @@
  *    16, 32, 64, 128, 256 and divides d_in; n, d_out >= 1 (n == 0 is accepted and does nothing).
  *  - Thread safety: calls keep no host state between calls except the error message of the
  *    calling thread and, per device, the cached device addresses of the library's static device
- *    scratch (looked up once under a lock).  Exception: cat_quantize_weights_noalloc uses one
- *    shared device scratch area per device, so its calls must be serialized by the caller.
+ *    scratch (looked up once under a lock) and whose turn it is on that scratch.  Exception:
+ *    cat_quantize_weights_noalloc uses one shared device scratch area per device, so its calls
+ *    must be serialized by the caller.
+ *  - Calls that overlap on a device (several streams): the transforms, the SQNR sums and the GEMMs
+ *    whose last tiles are cut along d_in exchange row maxima or partial sums through static device
+ *    scratch.  A call is handed its share when it is made, in turn, and keeps it: eight shares for
+ *    the transforms, eight for the SQNR sums of a kernel, twice what the device can run at once for
+ *    the GEMMs' partial sums.  Calls made one after another may overlap on any number of streams;
+ *    but a call that is held back (behind other work of its stream, or captured in a graph, which
+ *    keeps its share for every replay) must not run at the same time as a call that was handed the
+ *    same share after it.  So order the replays of two graphs of these calls, or of a graph and
+ *    calls beside it, rather than run them at the same time on two streams.
  *
  * INT4 code format ("SM4x8")
  * --------------------------

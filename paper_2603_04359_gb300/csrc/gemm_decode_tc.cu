@@ -693,6 +693,12 @@ bool coop_fits(size_t smem) {
   return ok == 1;
 }
 
+// One turn for both token counts: they share the slots.
+int next_part_slot() {
+  static std::atomic<unsigned> next{0};
+  return (int)(next.fetch_add(1, std::memory_order_relaxed) % kDecSlots);
+}
+
 template <int NTOK>
 cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw, int64_t n,
                         int64_t d_in, int64_t d_out, float* y, int32_t* acc_out, const float* y_ref, double* sums3,
@@ -741,8 +747,7 @@ cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, c
   if (ctas > 0x7FFFFFFF || (y_ref && ctas > kSqnrMaxCtas)) return cudaErrorInvalidConfiguration;
   const unsigned grid = (unsigned)ctas;
   const int slot = y_ref ? next_sqnr_slot() : 0;
-  static std::atomic<unsigned> next_part{0};
-  const int part_slot = split ? (int)(next_part.fetch_add(1, std::memory_order_relaxed) % kDecSlots) : 0;
+  const int part_slot = split ? next_part_slot() : 0;
   note_launch();
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));

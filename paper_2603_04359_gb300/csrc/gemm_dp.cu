@@ -95,7 +95,9 @@ __device__ uint64_t g_dp_wait_limit = kWaitLimitNs;
 // resident, and only owners wait) and adds.  Integer sums: exact in any order.  Flags hold the launch's number on its
 // slot of scratch, counted on the device (the last warp to start moves it on), so nothing has to be reset, also after
 // a launch that gave up, and graph replays count as launches.
-constexpr int kStreamSlots = 2;               // launches that may overlap; one fills the device
+// A launch takes every SM and is cooperative (all its CTAs are resident at once), so of two the later one begins when
+// the earlier one ends; slots are handed out in turn all the same, for the edges of the two.  42 MB.
+constexpr int kStreamSlots = 2;
 constexpr int kStreamCtas = 160;
 constexpr int kStreamWarpInt4 = 4 * 8 * 32;   // a warp's part: up to four chunks of 32 columns x 32 rows
 __device__ int4 g_dp_part[kStreamSlots][kStreamCtas][kEpiWarps][kStreamWarpInt4];
@@ -606,6 +608,12 @@ bool stream_launch_ok(int64_t pairs) {
   return ok == 1;
 }
 
+// One turn for every kind of this kernel: they share the slots.
+int next_stream_slot() {
+  static std::atomic<unsigned> next{0};
+  return (int)(next.fetch_add(1, std::memory_order_relaxed) % kStreamSlots);
+}
+
 template <int DX, int DW, int NB, bool STREAM = false>
 cudaError_t launch_nb(const DpCall& c) {
   using C = DpGemmCfg<DX, DW, NB>;
@@ -626,8 +634,7 @@ cudaError_t launch_nb(const DpCall& c) {
   const int64_t pairs = num_sms() / 2;
   const int64_t num_full = STREAM ? stream_full(tiles, pairs) : tiles;
   const int lanes = STREAM ? stream_lanes(c.n, tiles, pairs) : 1;
-  static std::atomic<unsigned> next_slot{0};
-  const int slot = STREAM ? (int)(next_slot.fetch_add(1, std::memory_order_relaxed) % kStreamSlots) : 0;
+  const int slot = STREAM ? next_stream_slot() : 0;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)(2 * (STREAM || tiles > pairs ? pairs : tiles)), 1, 1);

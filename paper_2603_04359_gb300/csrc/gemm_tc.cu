@@ -175,15 +175,17 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // the scaling, y, acc_out and the SQNR sums.  The scratch has room for a 256-wide part on every pair (split_parts
 // says when it is worth it): 14336 -> 4096 on 4096 tokens (3.37 waves) 149 -> 136 us against
 // room for half as many, when its 28 tail tiles took a fourth wave.  Counters are per (tile, CTA, epilogue warp); the last
-// part to finish sets them back to zero.  Slots of this scratch are handed out round robin per launch.
-constexpr int kSplitSlots = 2;
+// part to finish sets them back to zero.  A launch takes as much of the scratch as its parts need, in turn with all other
+// launches (take_split_units): the parts of the CTAs that are resident at once fit twice.
+constexpr int kSplitTurns = 2;
 constexpr int kMaxSplitTiles = 38;            // half a wave of 76 pairs
 constexpr int kMaxSplitUnits = 160;           // tail tiles x parts x NB / 128: up to a part per pair, 256 wide
-// Per slot: [part][channel/4][row] float4 slices of NB / 4 x 2 BM, room for kMaxSplitUnits 128-wide parts
-// (half as many 256-wide ones).
-constexpr size_t kSplitSlotF4 = (size_t)kMaxSplitUnits * (BN / 4) * (2 * BM);
-__device__ float4 g_split_part[kSplitSlots * kSplitSlotF4];
-__device__ uint32_t g_split_cnt[kSplitSlots][kMaxSplitTiles][2][kEpiWarps][2];   // arrived, finished
+// From a launch's first unit on: [part][channel/4][row] float4 slices of NB / 4 x 2 BM; its tail tile j counts at that
+// unit + j (a tile has at least two parts).  42 MB.
+constexpr int kSplitUnits = kSplitTurns * kMaxSplitUnits;
+constexpr size_t kSplitUnitF4 = (size_t)(BN / 4) * (2 * BM);
+__device__ float4 g_split_part[kSplitUnits * kSplitUnitF4];
+__device__ uint32_t g_split_cnt[kSplitUnits][2][kEpiWarps][2];   // arrived, finished
 
 __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
   uint32_t v;
@@ -212,7 +214,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                         const float* __restrict__ y_ref, double* __restrict__ sums3, int sqnr_slot,
                         const float* __restrict__ sx,
                         const float* __restrict__ sw, int n, int d_in, int d_out, float* __restrict__ y,
-                        int32_t* __restrict__ acc_out, int use_tma_store, int num_full, int split, int split_slot,
+                        int32_t* __restrict__ acc_out, int use_tma_store, int num_full, int split, int split_unit0,
                         uint32_t* __restrict__ status) {
   using L = GemmLayout<E8, NB>;
   // the pair tile: 256 tokens x NB channels; each CTA holds NB / 2 rows of B
@@ -448,9 +450,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const int my_row = (int)rank * BM + quad * 32 + lane;
     // part j's partial accumulators of channel group g (4 channels), this lane's row
     auto split_at = [&](int j, int g) {
-      return g_split_part + (size_t)split_slot * kSplitSlotF4 + ((size_t)j * (NB / 4) + g) * (2 * BM) + my_row;
+      return g_split_part + (size_t)split_unit0 * kSplitUnitF4 + ((size_t)j * (NB / 4) + g) * (2 * BM) + my_row;
     };
-    auto cnt_of = [&](int tj, int which) { return &g_split_cnt[split_slot][tj][rank][ew][which]; };
+    auto cnt_of = [&](int tj, int which) { return &g_split_cnt[split_unit0 + tj][rank][ew][which]; };
     auto arrive_part = [&](int tj) {                // after this lane's partial stores
       __threadfence();
       __syncwarp();
@@ -889,6 +891,15 @@ int split_parts(int64_t tiles, int64_t num_k, int nb, int64_t pairs) {
   return split;
 }
 
+// The first of `need` units of the split tail's scratch, one turn for every kind of this kernel: they share the array.
+int take_split_units(int need) {
+  static std::atomic<int> next{0};
+  int at = next.load(std::memory_order_relaxed), first;
+  do first = at + need <= kSplitUnits ? at : 0;
+  while (!next.compare_exchange_weak(at, first + need, std::memory_order_relaxed));
+  return first;
+}
+
 // y_ref != nullptr: the epilogue also forms the SQNR sums of y against y_ref and writes
 // sums3 = {sum y_ref^2, sum (y_ref - y)^2, dB} (sums3 needs no zeroing).  Needs d_out % 4 == 0
 // (TMA row pitch).  E8: xq and wq hold one code per byte, else SM4x8 (two per byte).  NB: channels per
@@ -929,8 +940,7 @@ cudaError_t launch_gemm_tc(const uint8_t* xq, const float* sx, const uint8_t* wq
     return cudaErrorInvalidConfiguration;
   const int grid = 2 * (int)(units < pairs_max ? units : pairs_max);  // CTA pairs (cluster of 2)
   if (grid > kSqnrMaxCtas) return cudaErrorInvalidConfiguration;
-  static std::atomic<unsigned> next_split{0};
-  const int split_slot = split > 1 ? (int)(next_split.fetch_add(1, std::memory_order_relaxed) % kSplitSlots) : 0;
+  const int split_unit0 = split > 1 ? take_split_units((int)(((units - num_full) * NB + BN - 1) / BN)) : 0;
   const int slot = y_ref ? next_sqnr_slot() : 0;
   const double* sums = y_ref ? sums3 : nullptr;
   note_launch();
@@ -947,7 +957,7 @@ cudaError_t launch_gemm_tc(const uint8_t* xq, const float* sx, const uint8_t* wq
   cfg.attrs = attrs;
   cfg.numAttrs = split > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, w4a4_gemm_tc_kernel<E8, NB>, ty, ta, tb, tr, y_ref, const_cast<double*>(sums), slot, sx,
-                            sw, (int)n, (int)d_in, (int)d_out, y, acc_out, use_tma, (int)num_full, split, split_slot,
+                            sw, (int)n, (int)d_in, (int)d_out, y, acc_out, use_tma, (int)num_full, split, split_unit0,
                             status);
 }
 
