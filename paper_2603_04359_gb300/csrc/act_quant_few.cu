@@ -10,10 +10,10 @@
 // Sums are float32: four products in order per lane, then a tree over the lanes.
 // Measured (cat_transform_quantize_act_split, k = 128): 1 x 4096 8.3 -> 5.6 us, 16 x 4096 8.9 -> 5.9.
 #include <cstring>
-#include <mutex>
 
 #include "common.cuh"
 #include "gemm_pair.cuh"
+#include "per_device.h"
 
 namespace cat {
 namespace {
@@ -192,15 +192,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// Clusters of 1, 2, 4, 8 and 16 CTAs that are resident at once (asked once per process and kernel; 16 is opt-in).
+// Clusters of 1, 2, 4, 8 and 16 CTAs that are resident at once (asked once per device and kernel; 16 is opt-in).
 struct Resident {
   int of[5];
 };
 template <typename Tin, int K>
-const Resident& resident() {
-  static std::once_flag once;
-  static Resident r = {{0, 0, 0, 0, 0}};
-  std::call_once(once, [] {
+Resident resident() {
+  static PerDevice<Resident> asked;
+  return asked.get([] {
+    Resident r = {{0, 0, 0, 0, 0}};
     auto kernel = transform_quant_few_kernel<Tin, K>;
     const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     for (int i = 0; i < (wide ? 5 : 4); ++i) {
@@ -215,8 +215,8 @@ const Resident& resident() {
       if (cudaOccupancyMaxActiveClusters(&r.of[i], kernel, &cfg) != cudaSuccess) r.of[i] = 0;
     }
     cudaGetLastError();
+    return r;
   });
-  return r;
 }
 
 // The largest cluster that leaves each CTA 128 outputs and takes the rows in one wave, while streaming T through it
@@ -226,7 +226,7 @@ template <typename Tin, int K>
 cudaError_t launch_k(const Tin* x, int64_t n, int64_t d, const float* T, uint8_t* codes, int e8, float* scale,
                      uint32_t* status, cudaStream_t stream) {
   auto kernel = transform_quant_few_kernel<Tin, K>;
-  const Resident& res = resident<Tin, K>();
+  const Resident res = resident<Tin, K>();
   int i = 4;
   while (i > 0 && d < 128 << i) --i;
   const int64_t most[5] = {kMaxT8, kMaxT8, kMaxT8, kMaxT8, kMaxT16};

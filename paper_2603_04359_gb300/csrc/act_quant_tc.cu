@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "dp_codes.cuh"
+#include "per_device.h"
 
 namespace cat {
 namespace {
@@ -1307,11 +1308,10 @@ cudaError_t launch_k(const __nv_bfloat16* x, int64_t n, int64_t d, int kb, const
     return cudaErrorInvalidValue;
   auto k0 = transform_quant_tc_kernel<K, 0>;
   auto k1 = transform_quant_tc_kernel<K, 1>;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [&] {
-    attr = cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    if (attr == cudaSuccess) attr = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  static PerDevice<cudaError_t> allowed;
+  const cudaError_t attr = allowed.get([&] {
+    const cudaError_t e = allow_smem(k0, C::SMEM);
+    return e == cudaSuccess ? allow_smem(k1, C::SMEM) : e;
   });
   if (attr != cudaSuccess) return attr;
   const int64_t units = (d / K) * ((n + TM - 1) / TM);
@@ -1411,14 +1411,10 @@ cudaError_t launch_fused_k(const __nv_bfloat16* x, int64_t n, int64_t d, int kb,
          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(transform_quant_tc_fused_kernel<N, KD, false, MODE>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F0::SMEM);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(transform_quant_tc_fused_kernel<N, KD, true, MODE>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F1::SMEM);
+  static PerDevice<cudaError_t> allowed;
+  const cudaError_t attr = allowed.get([] {
+    const cudaError_t e = allow_smem(transform_quant_tc_fused_kernel<N, KD, false, MODE>, F0::SMEM);
+    return e == cudaSuccess ? allow_smem(transform_quant_tc_fused_kernel<N, KD, true, MODE>, F1::SMEM) : e;
   });
   if (attr != cudaSuccess) return attr;
   cudaLaunchConfig_t cfg;

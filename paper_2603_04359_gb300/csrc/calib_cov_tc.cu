@@ -31,6 +31,7 @@
 
 #include "common.cuh"
 #include "gemm_pair.cuh"
+#include "per_device.h"
 
 namespace cat {
 namespace {
@@ -503,13 +504,15 @@ cudaLaunchAttribute cluster_of(int ctas) {
   return a;
 }
 
-// Clusters of 2, 4 and 8 CTAs of the wide kernel that are resident at once (asked once per process).
+// Clusters of 2, 4 and 8 CTAs of the wide kernel that are resident at once (asked once per device).
+struct WideResident {
+  int of[4];
+};
 int wide_resident(int S) {
-  static std::once_flag once;
-  static int found[4];
-  std::call_once(once, [] {
-    const bool ok = cudaFuncSetAttribute(calib_cov_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kWideSmem) == cudaSuccess;
+  static PerDevice<WideResident> asked;
+  const WideResident r = asked.get([] {
+    WideResident found = {{0, 0, 0, 0}};
+    const bool ok = allow_smem(calib_cov_wide_kernel, kWideSmem) == cudaSuccess;
     for (int i = 1; i < 4; ++i) {
       cudaLaunchConfig_t cfg;
       memset(&cfg, 0, sizeof(cfg));
@@ -519,11 +522,12 @@ int wide_resident(int S) {
       cudaLaunchAttribute attr = cluster_of(1 << i);
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
-      if (!ok || cudaOccupancyMaxActiveClusters(&found[i], calib_cov_wide_kernel, &cfg) != cudaSuccess) found[i] = 0;
+      if (!ok || cudaOccupancyMaxActiveClusters(&found.of[i], calib_cov_wide_kernel, &cfg) != cudaSuccess) found.of[i] = 0;
     }
     cudaGetLastError();
+    return found;
   });
-  return S == 2 ? found[1] : (S == 4 ? found[2] : found[3]);
+  return S == 2 ? r.of[1] : (S == 4 ? r.of[2] : r.of[3]);
 }
 
 // The wide kernel's token splits for a run the sliced kernel would cut into `sliced` (0: not for it): the first
@@ -563,12 +567,10 @@ cudaError_t launch_g(const void* x, int64_t n, int64_t d, int k, double* sigma, 
          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(calib_cov_tc_kernel<G2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM0);
-    if (attr == cudaSuccess)
-      attr = cudaFuncSetAttribute(calib_cov_tc_kernel<G2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM1);
+  static PerDevice<cudaError_t> allowed;
+  const cudaError_t attr = allowed.get([] {
+    const cudaError_t e = allow_smem(calib_cov_tc_kernel<G2, false>, C::SMEM0);
+    return e == cudaSuccess ? allow_smem(calib_cov_tc_kernel<G2, true>, C::SMEM1) : e;
   });
   if (attr != cudaSuccess) return attr;
   if (wide) {

@@ -12,9 +12,9 @@
 // 10 log10(sum ||v'||^2 / sum r^2) = C in dB.
 #include <cmath>
 #include <cstring>
-#include <mutex>
 
 #include "common.cuh"
+#include "per_device.h"
 #include "sqnr_slot.cuh"
 
 namespace cat {
@@ -147,11 +147,8 @@ template <int K>
 cudaError_t launch_k(const void* V, int dtype, int64_t rows, int64_t d, const float* M, int transpose,
                      float* row_sumsq, float* row_amax, float* Vt, cudaStream_t stream) {
   using C = DiagCfg<K>;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(block_row_stats_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-  });
+  static PerDevice<cudaError_t> allowed;
+  const cudaError_t attr = allowed.get([] { return allow_smem(block_row_stats_kernel<K>, C::SMEM); });
   if (attr != cudaSuccess) return attr;
   dim3 grid((unsigned)((rows + kRows - 1) / kRows), (unsigned)(d / K), 1);
   note_launch();
@@ -345,11 +342,8 @@ __global__ void __launch_bounds__(256) gram_f32_kernel(const Tin* __restrict__ X
 cudaError_t launch_fwht_rows(float* V, int64_t rows, int64_t d, cudaStream_t stream) {
   if (rows == 0) return cudaSuccess;
   const size_t smem = (size_t)d * sizeof(float);
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(fwht_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
-  });
+  static PerDevice<cudaError_t> allowed;
+  const cudaError_t attr = allowed.get([] { return allow_smem(fwht_rows_kernel, 32768 * 4); });
   if (attr != cudaSuccess) return attr;
   const int threads = d / 2 < 512 ? (int)(d / 2 < 32 ? 32 : d / 2) : 512;
   note_launch();

@@ -46,6 +46,7 @@
 
 #include "common.cuh"
 #include "gemm_pair.cuh"
+#include "per_device.h"
 #include "sqnr_slot.cuh"
 
 namespace cat {
@@ -617,33 +618,45 @@ cudaLaunchAttribute cluster_of(int ctas) {
   return a;
 }
 
-// CTAs that are resident at once as clusters of 1, 2, 4 and 8 (asked once per process and token count; clusters
+// All the shared memory the kernels may be launched with, allowed once per device.
+constexpr size_t kSmemMost = kSmemBudget + 4096;
+template <int NTOK>
+cudaError_t allow_decode_smem() {
+  static PerDevice<cudaError_t> allowed;
+  return allowed.get([] {
+    const cudaError_t e = allow_smem(w4a4_gemm_decode_tc_kernel<NTOK, false>, kSmemMost);
+    return e == cudaSuccess ? allow_smem(w4a4_gemm_decode_tc_kernel<NTOK, true>, kSmemMost) : e;
+  });
+}
+
+// CTAs that are resident at once as clusters of 1, 2, 4 and 8 (asked once per device and token count; clusters
 // stay within a group of SMs: 8s fill 120 of 152 here, 4s 144).
+struct ResidentCtas {
+  int of[4];
+};
 template <int NTOK>
 int resident_ctas(int log2_parts) {
-  static std::once_flag once;
-  static int ctas[4];
-  std::call_once(once, [] {
-    for (int i = 0; i < 4; ++i) {
-      ctas[i] = i == 0 ? num_sms() : 0;
+  static PerDevice<ResidentCtas> asked;
+  const ResidentCtas r = asked.get([] {
+    ResidentCtas ctas = {{num_sms(), 0, 0, 0}};
+    const bool ok = allow_decode_smem<NTOK>() == cudaSuccess;
+    for (int i = 1; i < 4; ++i) {
       cudaLaunchConfig_t cfg;
       memset(&cfg, 0, sizeof(cfg));
       cfg.gridDim = dim3(1u << i, 1, 1);
       cfg.blockDim = dim3(kThreads, 1, 1);
-      cfg.dynamicSmemBytes = kSmemBudget + 4096;
+      cfg.dynamicSmemBytes = kSmemMost;
       cudaLaunchAttribute attr = cluster_of(1 << i);
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
       int found = 0;
-      if (i > 0 &&
-          cudaFuncSetAttribute(w4a4_gemm_decode_tc_kernel<NTOK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kSmemBudget + 4096) == cudaSuccess &&
-          cudaOccupancyMaxActiveClusters(&found, w4a4_gemm_decode_tc_kernel<NTOK, false>, &cfg) == cudaSuccess)
-        ctas[i] = found << i;
+      if (ok && cudaOccupancyMaxActiveClusters(&found, w4a4_gemm_decode_tc_kernel<NTOK, false>, &cfg) == cudaSuccess)
+        ctas.of[i] = found << i;
     }
     cudaGetLastError();
+    return ctas;
   });
-  return ctas[log2_parts];
+  return r.of[log2_parts];
 }
 
 // CTAs per unit (the cluster's size; 1: whole units or stream-K), 0 when the tokens fit in no form.  A CTA
@@ -672,25 +685,21 @@ int pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms) {
 }
 
 // Whether one CTA per SM of the kernel is resident at once on this device under a cooperative launch
-// (checked once per token count; the grid never exceeds the SM count).
+// (checked once per device and token count; the grid never exceeds the SM count).
 template <int NTOK>
-bool coop_fits(size_t smem) {
-  static int ok = -1;
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
-  if (ok < 0) {
+bool coop_fits() {
+  static PerDevice<bool> asked;
+  return asked.get([] {
     int dev = 0, coop = 0, blocks = 0;
-    ok = cudaGetDevice(&dev) == cudaSuccess &&
-         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-         cudaFuncSetAttribute(w4a4_gemm_decode_tc_kernel<NTOK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kSmemBudget + 4096) == cudaSuccess &&
-         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, w4a4_gemm_decode_tc_kernel<NTOK, true>, kThreads,
-                                                       kSmemBudget + 4096) == cudaSuccess &&
-         blocks >= 1;
+    const bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+                    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+                    allow_decode_smem<NTOK>() == cudaSuccess &&
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, w4a4_gemm_decode_tc_kernel<NTOK, true>, kThreads,
+                                                                  kSmemMost) == cudaSuccess &&
+                    blocks >= 1;
     cudaGetLastError();
-  }
-  (void)smem;
-  return ok == 1;
+    return ok;
+  });
 }
 
 // One turn for both token counts: they share the slots.
@@ -720,20 +729,8 @@ cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, c
   const int nk = (num_ks + parts - 1) / parts, sp = stages_for(NTOK, nk, parts);
   if (sp == 0) return cudaErrorInvalidValue;
   const size_t smem = smem_bytes(NTOK, nk, sp, parts);
-  static std::mutex mu;
-  static size_t configured = 0;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (smem > configured) {
-      cudaError_t e = cudaFuncSetAttribute(w4a4_gemm_decode_tc_kernel<NTOK, false>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(w4a4_gemm_decode_tc_kernel<NTOK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-      if (e != cudaSuccess) return e;
-      configured = smem;
-    }
-  }
+  const cudaError_t allowed = allow_decode_smem<NTOK>();
+  if (allowed != cudaSuccess) return allowed;
   const int64_t units = (d_out + UM - 1) / UM;
   const int64_t sms = num_sms() < kDecMaxGrid ? num_sms() : kDecMaxGrid;
   // Stream-K over all (unit, K step) steps when there are more units than SMs: every CTA's range is
@@ -742,7 +739,7 @@ cudaError_t launch_ntok(const uint8_t* xq, const float* sx, const uint8_t* wq, c
   // would be shorter than a unit; CTAs inside a unit finish together with the unit's owner, and the
   // exchange through global memory then sits on the tail (measured at 16 tokens, 4096 -> 14336:
   // 15.8 us on 152 CTAs against 12.8 us for whole units on 112).
-  const int split = parts == 1 && units > sms && units <= kDecMaxUnits && coop_fits<NTOK>(smem) ? 1 : 0;
+  const int split = parts == 1 && units > sms && units <= kDecMaxUnits && coop_fits<NTOK>() ? 1 : 0;
   const int64_t ctas = parts > 1 ? units * parts : (units < sms ? units : sms);
   if (ctas > 0x7FFFFFFF || (y_ref && ctas > kSqnrMaxCtas)) return cudaErrorInvalidConfiguration;
   const unsigned grid = (unsigned)ctas;

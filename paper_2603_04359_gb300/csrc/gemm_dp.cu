@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "gemm_pair.cuh"
+#include "per_device.h"
 
 namespace cat {
 namespace {
@@ -579,33 +580,29 @@ struct DpCall {
   cudaStream_t stream;
 };
 
-// Whether a cooperative launch of `pairs` CTA pairs fits on this device (checked once per process, on the first
-// device asked).
+// Whether a cooperative launch of `pairs` CTA pairs, all that the device has, fits on it (checked once per device).
 template <int DX, int DW, int NB>
 bool stream_launch_ok(int64_t pairs) {
   using C = DpGemmCfg<DX, DW, NB>;
   constexpr bool STREAM = true;
-  static int ok = -1;
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
-  if (ok < 0) {
+  static PerDevice<bool> asked;
+  return asked.get([&] {
     int dev = 0, coop = 0, clusters = 0;
-    ok = 0;
+    bool ok = false;
     if (2 * pairs <= kStreamCtas && cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-        cudaFuncSetAttribute(dp_gemm_kernel<DX, DW, NB, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM) ==
-            cudaSuccess) {
+        allow_smem(dp_gemm_kernel<DX, DW, NB, STREAM>, C::SMEM) == cudaSuccess) {
       cudaLaunchConfig_t cfg;
       memset(&cfg, 0, sizeof(cfg));
       cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
       cfg.blockDim = dim3(kThreads, 1, 1);
       cfg.dynamicSmemBytes = C::SMEM;
       if (cudaOccupancyMaxActiveClusters(&clusters, dp_gemm_kernel<DX, DW, NB, STREAM>, &cfg) == cudaSuccess && clusters >= pairs)
-        ok = 1;
+        ok = true;
     }
     cudaGetLastError();
-  }
-  return ok == 1;
+    return ok;
+  });
 }
 
 // One turn for every kind of this kernel: they share the slots.
@@ -623,11 +620,8 @@ cudaError_t launch_nb(const DpCall& c) {
   if (!plane_map(&mx, c.x_planes, c.n, c.d_in, DX, BM) || !plane_map(&mw, c.w_planes, c.d_out, c.d_in, DW, NB / 2))
     return cudaErrorInvalidValue;
   const int use_tma = (c.d_out % 4 == 0 && output_map(&my, c.y, c.n, c.d_out)) ? 1 : 0;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(dp_gemm_kernel<DX, DW, NB, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-  });
+  static PerDevice<cudaError_t> allowed;
+  const cudaError_t attr = allowed.get([] { return allow_smem(dp_gemm_kernel<DX, DW, NB, STREAM>, C::SMEM); });
   if (attr != cudaSuccess) return attr;
   const int64_t tiles = ((c.n + 2 * BM - 1) / (2 * BM)) * ((c.d_out + NB - 1) / NB);
   if (tiles > 0x3FFFFFFF) return cudaErrorInvalidValue;

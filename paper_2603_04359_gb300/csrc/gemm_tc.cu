@@ -54,6 +54,7 @@
 
 #include "common.cuh"
 #include "gemm_pair.cuh"
+#include "per_device.h"
 #include "sqnr_slot.cuh"
 
 namespace cat {
@@ -844,20 +845,17 @@ int num_sms() {
 }
 
 // Whether a cooperative launch of `pairs` CTA pairs of the GEMM kernel fits on this device (checked
-// once per process and operand format, on the first device asked).
+// once per device, operand format and tile width).
 template <bool E8, int NB>
 bool split_launch_ok(int64_t pairs) {
   using L = GemmLayout<E8, NB>;
-  static int ok = -1;
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
-  if (ok < 0) {
+  static PerDevice<bool> asked;
+  return asked.get([&] {
     int dev = 0, coop = 0, clusters = 0;
-    ok = 0;
+    bool ok = false;
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-        cudaFuncSetAttribute(w4a4_gemm_tc_kernel<E8, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)L::kSmemBytes) == cudaSuccess) {
+        allow_smem(w4a4_gemm_tc_kernel<E8, NB>, L::kSmemBytes) == cudaSuccess) {
       cudaLaunchConfig_t cfg;
       memset(&cfg, 0, sizeof(cfg));
       cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
@@ -865,11 +863,11 @@ bool split_launch_ok(int64_t pairs) {
       cfg.dynamicSmemBytes = L::kSmemBytes;
       if (cudaOccupancyMaxActiveClusters(&clusters, w4a4_gemm_tc_kernel<E8, NB>, &cfg) == cudaSuccess &&
           clusters >= pairs)
-        ok = 1;
+        ok = true;
     }
     cudaGetLastError();
-  }
-  return ok == 1;
+    return ok;
+  });
 }
 
 // Parts that the tiles of the last wave (of nb channels each) are split into along K: a power of two, when that
@@ -921,12 +919,8 @@ cudaError_t launch_gemm_tc(const uint8_t* xq, const float* sx, const uint8_t* wq
   const int64_t row_bytes = E8 ? d_in : d_in / 2;
   if (!make_packed_map(&ta, xq, n, row_bytes, BM) || !make_packed_map(&tb, wq, d_out, row_bytes, NB / 2))
     return cudaErrorInvalidValue;
-  static std::once_flag attr_once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(attr_once, [] {
-    attr_err = cudaFuncSetAttribute(w4a4_gemm_tc_kernel<E8, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)L::kSmemBytes);
-  });
+  static PerDevice<cudaError_t> allowed;
+  const cudaError_t attr_err = allowed.get([] { return allow_smem(w4a4_gemm_tc_kernel<E8, NB>, L::kSmemBytes); });
   if (attr_err != cudaSuccess) return attr_err;
   const int64_t tiles = ((n + 2 * BM - 1) / (2 * BM)) * ((d_out + NB - 1) / NB);
   const int64_t num_k = (d_in + BK - 1) / BK;

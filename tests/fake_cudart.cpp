@@ -1,11 +1,12 @@
 // A CUDA runtime without a device: the library's objects link against it instead of cudart, so that its host code
 // (checks, routes, launch configurations, what it keeps per device) runs and is recorded on a machine without a GPU.
-// "Device" memory is host memory, kernels do nothing.  A launch is refused as the driver refuses it where the current
+// "Device" memory is host memory, or addresses from 2^44 on that hold nothing; kernels do nothing.  A launch is refused as the driver refuses it where the current
 // device's kernel attributes do not allow its shared memory or its cluster.
 #include <cuda.h>
 #include <cuda_runtime_api.h>
 #include <cxxabi.h>
 
+#include <cstdint>
 #include <cstdlib>
 #include <cstring>
 #include <map>
@@ -32,7 +33,6 @@ std::map<std::pair<int, const void*>, Attrs> attrs;
 std::map<std::pair<int, const void*>, void*> symbols;
 std::vector<Launch> launches;
 std::map<std::string, int> wanted;   // part of a kernel's name -> the int argument to record
-std::vector<void*> memory;
 thread_local int device = 0;
 thread_local struct {
   dim3 grid, block;
@@ -65,6 +65,8 @@ cudaError_t launch(const void* func, dim3 grid, dim3 block, size_t smem, int clu
   launches.push_back(l);
   return cudaSuccess;
 }
+
+bool backed(const void* p) { return (uintptr_t)p >> 40 != 0x10; }
 
 CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                 const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
@@ -190,11 +192,11 @@ cudaError_t cudaFreeAsync(void* p, cudaStream_t) {
   return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t bytes, enum cudaMemcpyKind, cudaStream_t) {
-  std::memcpy(dst, src, bytes);
+  if (backed(dst) && backed(src)) std::memcpy(dst, src, bytes);
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t bytes, cudaStream_t) {
-  std::memset(p, v, bytes);
+  if (backed(p)) std::memset(p, v, bytes);
   return cudaSuccess;
 }
 cudaError_t cudaMemcpyFromSymbol(void* dst, const void*, size_t bytes, size_t, enum cudaMemcpyKind) {

@@ -25,7 +25,7 @@ def ensure_built():
 
 
 class FakeRuntime:
-    """The library's entry points over the fake runtime; pointers are numpy arrays' or made up."""
+    """The library's entry points over the fake runtime."""
 
     def __init__(self, folder):
         objects = ensure_built()
@@ -55,7 +55,7 @@ class FakeRuntime:
         return (a.ctypes.data + 15) & ~15
 
     def call(self, name, *args):
-        """The launches of one call, which must succeed; None is NULL, a tuple of ints the address they would have."""
+        """The launches of one call, which must succeed; pointers are integers, None is NULL."""
         self.lib.fake_reset()
         status = getattr(self.lib, name)(*args)
         assert status == 0, (name, args, status, self.lib.cat_last_error())

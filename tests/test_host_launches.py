@@ -3,7 +3,7 @@ import pytest
 
 from fake_runtime import FakeRuntime
 
-P = 0x7F0000000000      # an address nothing on the host reads
+P = 0x10 << 40          # an address that holds nothing
 
 
 @pytest.fixture(scope="module")
@@ -49,3 +49,44 @@ def test_small_split_launches_share_no_scratch(fake):
     assert all(x.grid == 32 and x.cooperative for x in launches)
     first = sorted(x.arg for x in launches)
     assert all(b - a >= 16 for a, b in zip(first, first[1:])) and first[-1] + 16 <= 320, first
+
+
+def entry_calls(fake):
+    """One call, at least, of every kernel that needs an attribute of its own: shared memory or a wide cluster."""
+    blocks = fake.buffer(8 * 512 * 128)
+    for dtype in (0, 1):
+        for n, d, k in ((1, 64, 64), (16, 4096, 128), (32, 4096, 32), (3, 4096, 256), (100, 256, 32), (100, 4096, 128),
+                        (300, 4096, 256), (9000, 4096, 128), (2600, 192, 64), (40, 20480, 128), (9000, 8192, 256)):
+            yield "cat_transform_quantize_act", P, dtype, n, d, k, P, P, P, None
+            yield "cat_transform_quantize_act_dp", P, dtype, n, d, k, P, 8, 1, P, P, P, None
+            yield "cat_transform_quantize_act_dp", P, dtype, n, d, k, P, 8, 0, P, P, None, None
+        for n, d, k in ((512, 4096, 128), (512, 512, 256), (20000, 4096, 128), (3000, 256, 64), (9000, 512, 256)):
+            yield "cat_calib_cov", P, dtype, n, d, k, P, 0, None
+        yield "cat_block_row_stats", P, dtype, 100, 512, 128, P, 0, P, P, P, None
+        yield "cat_quantize_weights", P, dtype, 300, 512, 128, 2, blocks, 512, None, blocks, P, P, None
+        yield "cat_quantize_weights_dp", P, dtype, 300, 512, 128, 2, blocks, 512, None, 8, 1, blocks, P, P, P, None
+    yield "cat_fwht_rows", P, 10, 32768, None
+    for n, d_in, d_out in ((1, 4096, 6144), (32, 4096, 28672), (16, 4096, 28672), (27, 14336, 4096), (32, 32768, 260),
+                           (201, 4096, 6144), (200, 8192, 128), (2048, 4096, 6144)):
+        yield "cat_w4a4_linear", P, P, P, P, n, d_in, d_out, P, None, None
+    for n, d_in, d_out in ((2048, 4096, 6144), (256, 8192, 1000), (256, 8192, 3000), (200, 8192, 128), (1100, 4096, 5312)):
+        yield "cat_w4a4_linear_e8", P, P, P, P, n, d_in, d_out, P, None, None
+        yield "cat_w4a4_linear_sqnr_e8", P, P, P, P, n, d_in, d_out, P, P, P, None
+    for bits_x, bits_w in ((4, 4), (8, 4), (4, 8), (8, 8)):
+        for n, d_in, d_out in ((1, 4096, 64), (2048, 4096, 6144), (1000, 14336, 4096), (1000, 14336, 6144), (512, 8192, 9980)):
+            yield "cat_linear_dp", P, bits_x, 0, P, None, P, bits_w, P, None, n, d_in, d_out, P, None, None
+
+
+def test_every_kernel_is_allowed_its_launch_on_every_device(fake):
+    """Shared memory beyond 48 KB and clusters of 16 are allowed per device: what one device was asked does not hold for
+    another, so the same calls are launched the same way on two devices of a process."""
+    first, second = [], []
+    for found, device in ((first, 3), (second, 5)):
+        fake.device(device)
+        for name, *args in entry_calls(fake):
+            found += fake.call(name, *args)
+    fake.device(0)
+    assert {x.device for x in first} == {3} and {x.device for x in second} == {5}
+    same = [x._replace(device=0, arg=0) for x in first]
+    assert same == [x._replace(device=0, arg=0) for x in second]
+    assert any(x.cluster == 16 for x in first) and sum(x.smem > 48 * 1024 for x in first) > 50
