@@ -278,9 +278,9 @@ cat_status cat_codes_to_e4m3(const uint8_t* codes, int64_t rows, int64_t d, uint
  *   Arguments as cat_transform_quantize_act_split, except
  *   xq8  out, device [n][d_in] bytes: the codes of x' as byte codes.
  *   x_scale and the codes are those cat_transform_quantize_act_split writes (the same code decisions).
- *   bf16 rows on the fused tensor-core kernel, a few rows (n <= 32) and small fp32 transforms write the bytes
- *   directly; elsewhere the SM4x8 codes go to stream-ordered scratch (n * d_in / 2 bytes, cudaMallocAsync) and
- *   are converted.
+ *   The bytes are written directly, except for bf16 rows beyond the fused tensor-core kernel (more 128-channel groups
+ *   than SMs, or more than 131,072 rows): there the SM4x8 codes go to stream-ordered scratch (n * d_in / 2 bytes,
+ *   cudaMallocAsync) and are converted.
  */
 cat_status cat_transform_quantize_act_e8(const void* x, cat_dtype dtype, int64_t n, int64_t d_in, int32_t k,
                                          const float* T_blocks, const uint8_t* T_planes, uint8_t* xq8, float* x_scale,

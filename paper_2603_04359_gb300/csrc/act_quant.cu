@@ -16,7 +16,7 @@
 // and the 64 input rows are staged transposed in shared memory; each thread owns 4 rows x 8
 // consecutive channels (32 fp32 accumulators), which is exactly one packed word per row.
 //
-// Small transforms (transform_quant_rows_kernel): where all of T is small, a CTA takes 16 whole rows through every
+// Small transforms (transform_quant_rows_kernel): where T has few blocks, a CTA takes 16 whole rows through every
 // block, so the row maximum never leaves it: one launch and one pass instead of a memset, two passes and a
 // finalize launch, with the same sums in the same order.  512 float32 rows of 256 channels at k = 32: 19 us
 // and four launches before, 8.6 us now.
@@ -36,10 +36,22 @@ struct ActCfg {
   static constexpr size_t SMEM = (size_t)(K * AS_LD + K * XS_LD) * sizeof(float);
 };
 
+// Eight codes, element `at` of the matrix (a multiple of 8) on: bytes (e8) or one SM4x8 word.
+__device__ __forceinline__ void store_codes(uint8_t* codes, int64_t at, int e8, const int (&q)[8]) {
+  if (e8) {
+    uint2 o;
+    o.x = e4m3_code_byte(q[0]) | e4m3_code_byte(q[1]) << 8 | e4m3_code_byte(q[2]) << 16 | e4m3_code_byte(q[3]) << 24;
+    o.y = e4m3_code_byte(q[4]) | e4m3_code_byte(q[5]) << 8 | e4m3_code_byte(q[6]) << 16 | e4m3_code_byte(q[7]) << 24;
+    *reinterpret_cast<uint2*>(codes + at) = o;
+  } else {
+    *reinterpret_cast<uint32_t*>(codes + at / 2) = sm4_pack(q);
+  }
+}
+
 template <typename Tin, int K, int PASS>
 __global__ void __launch_bounds__(ActCfg<K>::THREADS) transform_quant_kernel(
     const Tin* __restrict__ x, int64_t n, int64_t d, const float* __restrict__ A, uint32_t* __restrict__ amax_bits,
-    uint32_t* __restrict__ codes, uint32_t* __restrict__ status) {
+    uint8_t* __restrict__ codes, int e8, uint32_t* __restrict__ status) {
   using C = ActCfg<K>;
   extern __shared__ __align__(16) float smem[];
   float* As = smem;                    // [K][AS_LD]: As[j][i] = A_b[c0 + i][j]
@@ -106,8 +118,7 @@ __global__ void __launch_bounds__(ActCfg<K>::THREADS) transform_quant_kernel(
     for (int r = tid; r < kRows; r += C::THREADS)
       if (t0 + r < n) atomicMax(&amax_bits[t0 + r], red[r]);
   } else {
-    const int64_t words_per_row = d / 8;
-    const int64_t word = ((int64_t)b * K + c0 + 8 * cg) / 8;
+    const int64_t col = (int64_t)b * K + c0 + 8 * cg;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int64_t t = t0 + 4 * tg + r;
@@ -116,7 +127,7 @@ __global__ void __launch_bounds__(ActCfg<K>::THREADS) transform_quant_kernel(
       int q[8];
 #pragma unroll
       for (int c = 0; c < 8; ++c) q[c] = qcode_exact(acc[r][c], qr, 7.0f);
-      codes[t * words_per_row + word] = sm4_pack(q);
+      store_codes(codes, t * d + col, e8, q);
     }
   }
 }
@@ -125,10 +136,9 @@ __global__ void __launch_bounds__(ActCfg<K>::THREADS) transform_quant_kernel(
 // Thread: output channel c of a slab, RPT rows.  The rows lie in shared memory, all loaded at the start, and a
 // block's x' replaces its x there; the transposed slabs of A arrive by cp.async one ahead (two buffers), so a
 // block costs its sums and two barriers, not a trip to L2.
-// Every CTA reads all of A (from L2), so A is bounded: kRowsMaxT elements (256 KB).
+// Every CTA reads all of A (from L2) and goes through it one block after the other: small A only (rows_pay).
 constexpr int kWholeRows = 16;
 constexpr int kRowsThreads = 256;
-constexpr int64_t kRowsMaxT = 65536;
 constexpr size_t kRowsMaxSmem = 220 * 1024;
 
 template <int K>
@@ -224,14 +234,7 @@ __global__ void __launch_bounds__(kRowsThreads) transform_quant_rows_kernel(
     int q[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) q[e] = qcode_exact(v[e], qr, 7.0f);
-    if (e8) {
-      uint2 o;
-      o.x = e4m3_code_byte(q[0]) | e4m3_code_byte(q[1]) << 8 | e4m3_code_byte(q[2]) << 16 | e4m3_code_byte(q[3]) << 24;
-      o.y = e4m3_code_byte(q[4]) | e4m3_code_byte(q[5]) << 8 | e4m3_code_byte(q[6]) << 16 | e4m3_code_byte(q[7]) << 24;
-      *reinterpret_cast<uint2*>(codes + (t0 + r) * d + 8 * i) = o;
-    } else {
-      *reinterpret_cast<uint32_t*>(codes + (t0 + r) * (d / 2) + 4 * i) = sm4_pack(q);
-    }
+    store_codes(codes, (t0 + r) * d + 8 * i, e8, q);
   }
   if (tid < kWholeRows && t0 + tid < n) {
     const float a = __uint_as_float(red[tid]);
@@ -244,12 +247,39 @@ __global__ void __launch_bounds__(kRowsThreads) transform_quant_rows_kernel(
   }
 }
 
+// Where whole rows are faster than the tiled kernels (a memset, two passes and a launch for the steps).  A CTA takes
+// ~7 us and per block 0.66, 1.0, 2.2, 6.3 us at k = 16, 32, 64, 128 (whatever the other CTAs do, while each has an SM);
+// the tiled kernels take 24, 30, 28, 40 us up to ~150 tiles of 64 rows and one block, then as their sums.  us, whole
+// rows against tiled, 304 / 2432 / 16384 rows of float32:
+//   k = 16:  384 channels 23/26 23/28 42/50,  512 28/25 28/28 54/56, 3072 132/28 137/52 669/276
+//   k = 32:  512 channels 24/34 24/36 64/73,  640 29/33 28/36 80/91,  768 33/33 33/37 103/99, 1760 65/34 66/45 411/214
+//   k = 64:  512 channels 25/30 26/34 89/98,  640 30/30 30/36 110/107, 768 34/30 35/36 149/129
+//   k = 128: every block costs a wave of CTAs (140 KB and more of shared memory, one per SM): 128 channels 14/42 15/42
+//            60/54 (7 waves), 512 33/43 34/44 185/167;  at 4864 rows (two waves) 256 channels 35/46, 512 58/54
+//   k = 256: 256 channels 30/70 30/69 162/212
+bool rows_pay(int k, int64_t blocks, int64_t ctas, int64_t sms) {
+  switch (k) {
+    case 16: return blocks <= 24;
+    case 32: return blocks <= 18 || (blocks <= 24 && ctas <= sms);
+    case 64: return blocks <= 8 || (blocks <= 10 && ctas <= sms);
+    case 128: return (ctas + sms - 1) / sms * blocks <= 6 && blocks <= 4;
+    default: return blocks == 1;
+  }
+}
+
+int num_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 148;
+  return sms;
+}
+
 template <typename Tin, int K>
 cudaError_t launch_rows_k(const Tin* x, int64_t n, int64_t d, const float* A, uint8_t* codes, int e8, float* scale,
                           uint32_t* status, cudaStream_t stream) {
   const size_t smem = RowsCfg<K>::smem(d);
   const int64_t ctas = (n + kWholeRows - 1) / kWholeRows;
-  if (d * K > kRowsMaxT || smem > kRowsMaxSmem || ctas > 0x7FFFFFFF) return cudaErrorNotSupported;
+  if (!rows_pay(K, d / K, ctas, num_sms()) || smem > kRowsMaxSmem || ctas > 0x7FFFFFFF) return cudaErrorNotSupported;
   // always the same limit: calls from other threads may set it in between
   cudaError_t e = cudaFuncSetAttribute(transform_quant_rows_kernel<Tin, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kRowsMaxSmem);
@@ -288,7 +318,7 @@ __global__ void finalize_scale_kernel(uint32_t* __restrict__ amax_bits, int64_t 
 }
 
 template <typename Tin, int K>
-cudaError_t launch_k(const Tin* x, int64_t n, int64_t d, const float* A, uint8_t* codes, float* scale,
+cudaError_t launch_k(const Tin* x, int64_t n, int64_t d, const float* A, uint8_t* codes, int e8, float* scale,
                      uint32_t* status, cudaStream_t stream) {
   using C = ActCfg<K>;
   cudaError_t e = cudaMemsetAsync(scale, 0, (size_t)n * sizeof(float), stream);
@@ -303,12 +333,11 @@ cudaError_t launch_k(const Tin* x, int64_t n, int64_t d, const float* A, uint8_t
   if (ny > 65535) return cudaErrorInvalidValue;
   dim3 grid((unsigned)row_tiles, (unsigned)ny);
   uint32_t* amax = reinterpret_cast<uint32_t*>(scale);
-  uint32_t* words = reinterpret_cast<uint32_t*>(codes);
   note_launch();
-  k0<<<grid, C::THREADS, C::SMEM, stream>>>(x, n, d, A, amax, words, status);
+  k0<<<grid, C::THREADS, C::SMEM, stream>>>(x, n, d, A, amax, codes, e8, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   note_launch();
-  k1<<<grid, C::THREADS, C::SMEM, stream>>>(x, n, d, A, amax, words, status);
+  k1<<<grid, C::THREADS, C::SMEM, stream>>>(x, n, d, A, amax, codes, e8, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   note_launch();
   finalize_scale_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(amax, n, status);
@@ -316,16 +345,24 @@ cudaError_t launch_k(const Tin* x, int64_t n, int64_t d, const float* A, uint8_t
 }
 
 template <typename Tin>
-cudaError_t launch_t(const Tin* x, int64_t n, int64_t d, int k, const float* A, uint8_t* codes, float* scale,
+cudaError_t launch_t(const Tin* x, int64_t n, int64_t d, int k, const float* A, uint8_t* codes, int e8, float* scale,
                      uint32_t* status, cudaStream_t stream) {
   switch (k) {
-    case 16: return launch_k<Tin, 16>(x, n, d, A, codes, scale, status, stream);
-    case 32: return launch_k<Tin, 32>(x, n, d, A, codes, scale, status, stream);
-    case 64: return launch_k<Tin, 64>(x, n, d, A, codes, scale, status, stream);
-    case 128: return launch_k<Tin, 128>(x, n, d, A, codes, scale, status, stream);
-    case 256: return launch_k<Tin, 256>(x, n, d, A, codes, scale, status, stream);
+    case 16: return launch_k<Tin, 16>(x, n, d, A, codes, e8, scale, status, stream);
+    case 32: return launch_k<Tin, 32>(x, n, d, A, codes, e8, scale, status, stream);
+    case 64: return launch_k<Tin, 64>(x, n, d, A, codes, e8, scale, status, stream);
+    case 128: return launch_k<Tin, 128>(x, n, d, A, codes, e8, scale, status, stream);
+    case 256: return launch_k<Tin, 256>(x, n, d, A, codes, e8, scale, status, stream);
     default: return cudaErrorInvalidValue;
   }
+}
+
+// Float32 units: whole rows where they pay, else the tiled kernels.
+template <typename Tin>
+cudaError_t launch_simt(const Tin* x, int64_t n, int64_t d, int k, const float* A, uint8_t* codes, int e8, float* scale,
+                        uint32_t* status, cudaStream_t stream) {
+  const cudaError_t e = launch_rows(x, n, d, k, A, codes, e8, scale, status, stream);
+  return e != cudaErrorNotSupported ? e : launch_t(x, n, d, k, A, codes, e8, scale, status, stream);
 }
 
 }  // namespace
@@ -371,27 +408,26 @@ cudaError_t launch_transform_quantize(const void* x, int dtype, int64_t n, int64
     // k = 256 beyond the fused kernel (more 64-output groups than SMs, more rows than its scratch):
     // the SIMT kernel below
   }
-  const cudaError_t er =
-      dtype == 0 ? launch_rows(static_cast<const float*>(x), n, d, k, A, codes, 0, scale, status, stream)
-                 : launch_rows(static_cast<const __nv_bfloat16*>(x), n, d, k, A, codes, 0, scale, status, stream);
-  if (er != cudaErrorNotSupported) return er;
-  if (dtype == 0) return launch_t(static_cast<const float*>(x), n, d, k, A, codes, scale, status, stream);
-  return launch_t(static_cast<const __nv_bfloat16*>(x), n, d, k, A, codes, scale, status, stream);
+  if (dtype == 0) return launch_simt(static_cast<const float*>(x), n, d, k, A, codes, 0, scale, status, stream);
+  return launch_simt(static_cast<const __nv_bfloat16*>(x), n, d, k, A, codes, 0, scale, status, stream);
 }
 
-// The same codes as byte codes ([n][d], one E4M3 byte per code), written by the fused tensor-core
-// kernel or the whole-row kernel; cudaErrorNotSupported (nothing launched) where neither applies.
+// The same codes as byte codes ([n][d], one E4M3 byte per code); cudaErrorNotSupported (nothing launched) where packed
+// ones come from the two-pass tensor-core kernel, which has no byte form.
 cudaError_t launch_transform_quantize_e8(const void* x, int dtype, int64_t n, int64_t d, int k, const float* A,
                                          uint8_t* codes8, float* scale, uint32_t* status, cudaStream_t stream,
                                          const uint8_t* planes) {
   if (n == 0) return cudaSuccess;
   const cudaError_t e1 = launch_transform_quantize_few(x, dtype, n, d, k, A, codes8, 1, scale, status, stream);
   if (e1 != cudaErrorNotSupported) return e1;
-  if (transform_quantize_tc_supported(dtype, k, n, d))
-    return launch_transform_quantize_tc_fused(x, n, d, k, A, planes, reinterpret_cast<uint32_t*>(scale),
-                                              reinterpret_cast<uint32_t*>(codes8), 1, status, stream);
-  if (dtype == 0) return launch_rows(static_cast<const float*>(x), n, d, k, A, codes8, 1, scale, status, stream);
-  return launch_rows(static_cast<const __nv_bfloat16*>(x), n, d, k, A, codes8, 1, scale, status, stream);
+  if (transform_quantize_tc_supported(dtype, k, n, d)) {
+    const cudaError_t ef = launch_transform_quantize_tc_fused(x, n, d, k, A, planes, reinterpret_cast<uint32_t*>(scale),
+                                                              reinterpret_cast<uint32_t*>(codes8), 1, status, stream);
+    if (ef != cudaErrorNotSupported || transform_tc_group(k, d) != 256) return ef;
+    // k = 256 beyond the fused kernel: the SIMT kernels, as for packed codes
+  }
+  if (dtype == 0) return launch_simt(static_cast<const float*>(x), n, d, k, A, codes8, 1, scale, status, stream);
+  return launch_simt(static_cast<const __nv_bfloat16*>(x), n, d, k, A, codes8, 1, scale, status, stream);
 }
 
 }  // namespace cat

@@ -705,7 +705,7 @@ cat_status cat_transform_quantize_act_e8(const void* x, cat_dtype dtype, int64_t
   const uint8_t* planes = cat::transform_tc_group(k, d_in) != 0 ? T_planes : nullptr;
   e = cat::launch_transform_quantize_e8(x, (int)dtype, n, d_in, k, T_blocks, xq8, x_scale, status, s, planes);
   if (e == cudaErrorNotSupported) {
-    // no kernel writes byte codes here: SM4x8 codes into stream-ordered scratch, then converted
+    // the two-pass kernel has no byte form: SM4x8 codes into stream-ordered scratch, then converted
     uint8_t* tmp = nullptr;
     if ((e = cudaMallocAsync((void**)&tmp, (size_t)n * (size_t)(d_in / 2), s)) != cudaSuccess)
       return cuda_fail(e, "cudaMallocAsync");

@@ -124,8 +124,9 @@ def test_w4a4_linear_sqnr_e8(n, d_in, d_out):
                                          (300, 512, 32, "bf16"), (300, 192, 64, "bf16"),        # embedded, 64-wide
                                          (2560, 4096, 256, "bf16"), (200, 512, 256, "bf16"),    # k = 256 quarters
                                          (1100, 9920, 64, "bf16"), (520, 20480, 128, "bf16"),   # two passes + convert
-                                         (1300, 10240, 256, "bf16"),                             # SIMT + convert
-                                         (130, 256, 32, "f32"), (5, 64, 16, "bf16")])            # SIMT + convert
+                                         (1300, 10240, 256, "bf16"), (130, 1024, 16, "f32"),     # SIMT, tiled
+                                         (300, 1024, 128, "f32"), (70, 1760, 32, "bf16"),
+                                         (130, 256, 32, "f32"), (5, 64, 16, "bf16")])            # SIMT, whole rows
 def test_transform_quantize_act_e8(n, d, k, dtype):
     """The byte codes are the byte form of cat_transform_quantize_act_split's SM4x8 codes and the steps
     are the same, bit for bit; on the first shape also checked against the oracle directly."""

@@ -90,3 +90,27 @@ def test_every_kernel_is_allowed_its_launch_on_every_device(fake):
     same = [x._replace(device=0, arg=0) for x in first]
     assert same == [x._replace(device=0, arg=0) for x in second]
     assert any(x.cluster == 16 for x in first) and sum(x.smem > 48 * 1024 for x in first) > 50
+
+
+def transform_kernel(fake, n, d, k, dtype, code_bytes):
+    name, planes = ("cat_transform_quantize_act_e8", (None,)) if code_bytes else ("cat_transform_quantize_act", ())
+    launches = fake.call(name, P, dtype, n, d, k, P, *planes, P, P, None)
+    return next(name for name in ("few", "rows", "tc_fused", "tc", "") if f"transform_quant_{name}_kernel".replace("__", "_")
+                in launches[0].kernel)
+
+
+@pytest.mark.parametrize("code_bytes", [False, True])
+@pytest.mark.parametrize("k,whole,tiled", [
+    (16, [(5, 64), (512, 384), (65536, 384)], [(33, 416), (512, 3072), (65536, 1024), (5, 3072)]),
+    (32, [(100, 32), (512, 256), (65536, 576), (2432, 768)], [(2433, 768), (100, 800), (512, 2048)]),
+    (64, [(40, 64), (65536, 512), (2432, 640)], [(2433, 640), (100, 704), (512, 1024)]),
+    (128, [(40, 128), (512, 512), (14592, 128), (7296, 256), (4864, 384), (2432, 512)],
+     [(14593, 128), (7297, 256), (4865, 384), (2433, 512), (33, 640)]),
+    (256, [(33, 256), (65536, 256)], [(33, 512)]),
+])
+def test_small_transforms_take_whole_rows_where_that_is_faster(fake, k, whole, tiled, code_bytes):
+    """float32 rows (few rows of k >= 32 have a kernel of their own): blocks and rows at the rule's lines, both code forms."""
+    for n, d in whole:
+        assert transform_kernel(fake, n, d, k, 0, code_bytes) == "rows", (n, d)
+    for n, d in tiled:
+        assert transform_kernel(fake, n, d, k, 0, code_bytes) == "", (n, d)
