@@ -245,9 +245,10 @@ cat_status cat_w4a4_linear(const uint8_t* xq, const float* x_scale, const uint8_
  *   y_ref  device [n][d_out] float32: the full-precision output y = W x;
  *   out3   out, device [3] float64: { sum y_ref^2, sum (y_ref - y)^2, 10 log10(ratio) dB }, as cat_sqnr.
  * y is written exactly as cat_w4a4_linear writes it.  The sums are formed in the GEMM's epilogue while
- * y is produced (y is not read back) -- for n > 32 when d_out % 4 == 0, for n <= 32 when the decoded
- * tokens fit in the weight-streaming kernel's shared memory (a cluster of up to eight CTAs shares a row: d_in to
- * ~80,000 at n <= 16, ~39,000 above); otherwise the GEMM is followed by the cat_sqnr reduction.  Squares are summed in fp32 over runs of at most 32 outputs, the runs as float pairs
+ * y is produced (y is not read back) -- for n > 32 when d_out % 4 == 0, for n <= 32 on the tcgen05
+ * weight-streaming kernel (a cluster of up to eight CTAs shares a row: d_in to ~80,000 at n <= 16, ~39,000
+ * above; some rows of 10,000 channels and more are faster on the mma.sync kernel); otherwise the GEMM is followed
+ * by the cat_sqnr reduction.  Squares are summed in fp32 over runs of at most 32 outputs, the runs as float pairs
  * (hi + lo, ~48 significant bits); the result does not depend on CTA timing.
  */
 cat_status cat_w4a4_linear_sqnr(const uint8_t* xq, const float* x_scale, const uint8_t* Wq, const float* w_scale,

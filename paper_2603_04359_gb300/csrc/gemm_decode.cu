@@ -1,6 +1,7 @@
-// W4A4 GEMM for a few tokens (decode) on the legacy mma.sync path: the fallback of the tcgen05
-// weight-streaming kernel (gemm_decode_tc.cu) for token operands too large for its shared memory
-// (d_in beyond ~82k codes at 16 tokens, ~39k at 32).  The packed weight stream is read once from HBM.
+// W4A4 GEMM for a few tokens (decode) on the legacy mma.sync path, beside the tcgen05 weight-streaming kernel
+// (gemm_decode_tc.cu): token operands too large for that one's shared memory (d_in beyond ~82k codes at 16 tokens,
+// ~39k at 32), and long rows where this one is faster (its pick_form).  The packed weight stream is read once
+// from HBM.
 //
 //   acc[t, o] = sum_i q_x[t, i] q_w[o, i],   y[t, o] = acc * s_x[t] * s_w[o]   (Sec. 3, Eq. 5)
 //
@@ -128,8 +129,7 @@ cudaError_t launch_w4a4_gemm_decode_tc(const uint8_t* xq, const float* sx, const
                                        int64_t n, int64_t d_in, int64_t d_out, float* y, int32_t* acc_out,
                                        const float* y_ref, double* sums3, uint32_t* status, cudaStream_t stream);
 
-// n <= 32: tcgen05 weight streaming when the decoded tokens fit in shared memory, else mma.sync
-// weight streaming with registers.
+// n <= 32: tcgen05 weight streaming, or mma.sync weight streaming with registers where decode_tc_applies says no.
 // y_ref != nullptr: also the SQNR sums of y against y_ref into sums3 (in the tcgen05 kernel's
 // epilogue, else by the separate reduction after the GEMM).
 cudaError_t launch_w4a4_gemm_decode(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw, int64_t n,

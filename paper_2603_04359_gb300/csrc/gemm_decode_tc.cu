@@ -20,7 +20,7 @@
 //     kernel's time at 4096 channels);
 //   * four epilogue warps read the double-buffered accumulators (thread = output channel) and write
 //     y[t][o] with consecutive o across a warp; y_ref, when given, is loaded while the MMAs run.
-// Work split, three forms, chosen by pick_parts:
+// Work split, three forms, chosen by pick_form:
 //   * whole 128-row units, one contiguous range of units per CTA (parts = 1);
 //   * fewer units than SMs, or rows too long for a CTA's shared memory: a unit's K steps are cut over a
 //     cluster of 2, 4 or 8 CTAs, which exchange their accumulators through distributed shared memory;
@@ -659,29 +659,71 @@ int resident_ctas(int log2_parts) {
   return r.of[log2_parts];
 }
 
-// CTAs per unit (the cluster's size; 1: whole units or stream-K), 0 when the tokens fit in no form.  A CTA
-// takes about kStart + its K steps, in units of one K step (start-up, token staging and the last outputs
-// ~4.5 us against ~0.28 us a step), a cluster kExchange more; clusters beyond what is resident run in waves,
-// stream-K does not.
-constexpr int kStart = 16, kExchange = 2;
-int pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms) {
-  const int ntok = n <= 16 ? 16 : 32;
+// How a call is best run: CTAs per unit (the cluster's size; 1: whole units or stream-K) and its time in us.  parts = 0: on the
+// mma.sync kernel, or with the SQNR sums in a launch of their own.
+//
+// The times are those of calls with cold weights, from fits over 2800 measured ones (1 to 32 tokens, 256 to 49152 -> 64 to
+// 28672 channels, every form that fits, with and without the sums; 3 to 5 % rms): a wave of CTAs takes kWaveUs
+// (start-up, token staging, the last outputs) and a K step kStepUs, more where the resident tokens leave room for three
+// packed stages only.  A cluster adds its exchange and, for every kThreads outputs that a CTA finishes, a pass over
+// them, with the sums another load of y_ref; more units than SMs in one piece (stream-K) add what the cut units wait
+// for.  The sums in a launch of their own take kSumsUs: less than in a cluster's epilogue where that runs in waves
+// (8 tokens, 14336 -> 16384: 49 us against 57) or finishes many outputs.  Without the passes and the sums, 16 tokens,
+// 2048 -> 7530 with the sums went to clusters of 2: 21.6 us, on whole units 17.6.
+//
+// The mma.sync kernel has no token operand to stage and takes rows of any length, but its time grows with the tokens:
+// at up to 8 of them it is the faster one for rows that a CTA cannot hold here and many units
+// (2 tokens, 14336 -> 22016: 52 us against 61 in clusters of 2; 14336 -> 4096: 21 against 20), at 17 to 24 for rows that only a
+// cluster of 8 holds (20480 -> 28672: 165 against 179) and for few units of rows just
+// past a CTA (24 tokens, 5120 -> 2048: 13.5 against 17.6).  Elsewhere it is not asked.
+struct DecodeForm {
+  int parts;
+  double us;
+};
+constexpr double kWaveUs[2][2] = {{4.4, 5.0}, {6.3, 6.7}};      // [SQNR sums][32 tokens]
+constexpr double kStepUs[2][2] = {{0.44, 0.51}, {0.52, 0.57}};  // [three stages][32 tokens]
+constexpr double kFixedUs = 6.3, kStreamUs = 7.0, kSumsUs = 7.0;
+
+double mma_sync_us(int64_t n, int64_t d_in, int64_t d_out) {
+  const bool few = n <= 8, more = n > 24;
+  const double least = few ? 0.81e-3 : (more ? 1.5e-3 : 1.2e-3), slope = few ? 1.1e-7 : (more ? 3.3e-7 : 2.55e-7);
+  const double rate = 0.4e-3 + slope * d_out;                   // us a channel of d_in
+  return 8.0 + d_in * (rate > least ? rate : least);
+}
+
+// The best form of the tcgen05 kernel alone, with the sums in its epilogue if there are any.
+DecodeForm pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms, bool sums) {
+  const int ntok = n <= 16 ? 16 : 32, wide = ntok == 32;
   const int64_t num_ks = (d_in / 2 + KSB - 1) / KSB, units = (d_out + UM - 1) / UM;
-  int best = 0;
-  int64_t least = 0;
+  DecodeForm best = {0, 0.0};
   for (int i = 0, parts = 1; parts <= kMaxParts && parts <= num_ks; ++i, parts *= 2) {
     const int64_t nk = (num_ks + parts - 1) / parts;
     const int64_t resident = ntok == 16 ? resident_ctas<16>(i) : resident_ctas<32>(i);
-    if (stages_for(ntok, (int)nk, parts) == 0 || resident < parts) continue;
-    const int64_t cost = parts == 1 && units > sms
-                             ? kStart + (units * num_ks + sms - 1) / sms
-                             : ((units * parts + resident - 1) / resident) * (kStart + nk + (parts > 1 ? kExchange : 0));
-    if (best == 0 || cost < least) {
-      best = parts;
-      least = cost;
-    }
+    const int stages = stages_for(ntok, (int)nk, parts);
+    if (stages == 0 || resident < parts || (sums && parts > 1 && units * parts > kSqnrMaxCtas)) continue;
+    const double step = kStepUs[stages == kDecGroups][wide], wave = kWaveUs[sums][wide];
+    const int64_t passes = (n * UM / parts + kThreads - 1) / kThreads;
+    const double part = parts == 1 ? 0.0 : (sums ? 2.6 + 1.2 * passes : 0.9 + 0.65 * passes);
+    const double us = kFixedUs + (sums ? 1.5 : 0.0) +
+                      (parts == 1 && units > sms
+                           ? wave + kStreamUs + step * units * num_ks / sms
+                           : ((units * parts + resident - 1) / resident) * (wave + part + step * nk));
+    if (best.parts == 0 || us < best.us) best = {parts, us};
   }
   return best;
+}
+
+DecodeForm pick_form(int64_t n, int64_t d_in, int64_t d_out, int64_t sms, bool sums) {
+  const int64_t num_ks = (d_in / 2 + KSB - 1) / KSB, units = (d_out + UM - 1) / UM;
+  DecodeForm plain = pick_parts(n, d_in, d_out, sms, false);
+  const bool ask = n <= 8 ? num_ks > 36 : n > 16 && (num_ks > 72 || (n <= 24 && num_ks > 18 && units <= 32));
+  if (plain.parts == 0 || ask) {
+    const double us = mma_sync_us(n, d_in, d_out);
+    if (plain.parts == 0 || us < plain.us) plain = {0, us};
+  }
+  if (!sums) return plain;
+  const DecodeForm fused = pick_parts(n, d_in, d_out, sms, true);
+  return fused.parts != 0 && fused.us <= plain.us + kSumsUs ? fused : DecodeForm{0, plain.us + kSumsUs};
 }
 
 // Whether one CTA per SM of the kernel is resident at once on this device under a cooperative launch
@@ -774,13 +816,9 @@ cudaError_t set_decode_wait_limit(uint64_t ns) {
   return cudaMemcpyToSymbol(g_dec_wait_limit, &ns, sizeof(ns));
 }
 
-// Whether this kernel takes n tokens of d_in codes (else the mma.sync kernel does): clusters may not be many
-// enough to overflow the SQNR slot's rows.
+// Whether this kernel takes the call (else the mma.sync kernel does, or the sums are not formed with y).
 bool decode_tc_applies(int64_t n, int64_t d_in, int64_t d_out, bool with_sqnr) {
-  if (n < 1 || n > 32) return false;
-  const int parts = pick_parts(n, d_in, d_out, num_sms());
-  if (parts == 0) return false;
-  return !with_sqnr || parts == 1 || (d_out + UM - 1) / UM * parts <= kSqnrMaxCtas;
+  return n >= 1 && n <= 32 && pick_form(n, d_in, d_out, num_sms(), with_sqnr).parts > 0;
 }
 
 // y_ref != nullptr: the epilogue also forms the SQNR sums of y against y_ref and writes
@@ -788,7 +826,7 @@ bool decode_tc_applies(int64_t n, int64_t d_in, int64_t d_out, bool with_sqnr) {
 cudaError_t launch_w4a4_gemm_decode_tc(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw,
                                        int64_t n, int64_t d_in, int64_t d_out, float* y, int32_t* acc_out,
                                        const float* y_ref, double* sums3, uint32_t* status, cudaStream_t stream) {
-  const int parts = pick_parts(n, d_in, d_out, num_sms());
+  const int parts = pick_form(n, d_in, d_out, num_sms(), y_ref != nullptr).parts;
   if (parts == 0) return cudaErrorInvalidValue;
   if (n <= 16) return launch_ntok<16>(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, parts, stream);
   return launch_ntok<32>(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, parts, stream);

@@ -39,16 +39,13 @@ thread_local struct {
   size_t smem;
   cudaStream_t stream;
 } pushed;
-int sms = 152;
+const int sms = 152;
 
-// Clusters of one-CTA-per-SM kernels that are resident at once: SMs come in groups of 18 and 20, a cluster stays in one.
+// Clusters of one-CTA-per-SM kernels that are resident at once: a cluster stays in a group of SMs (76 of two CTAs, 36 of
+// four, 15 of eight and 7 of sixteen, as a GB300 answers).
 int clusters(int size) {
-  int n = 0, left = sms;
-  for (int i = 0; left > 0; ++i) {
-    const int group = left < 20 ? left : (i % 2 ? 20 : 18);
-    n += group / size;
-    left -= group;
-  }
+  int n = 0;
+  for (int group : {18, 18, 20, 20, 20, 20, 22, 14}) n += group / size;
   return n;
 }
 

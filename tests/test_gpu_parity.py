@@ -545,12 +545,12 @@ def test_device_transform_refuses_singular_blocks():
 
 
 # ------------------------------------------------------------------------------------------
-# Decode GEMM: the work splits (whole units, clusters of 2, 4 and 8, stream-K)
+# Decode GEMM: the work splits (whole units, clusters of 2, 4 and 8, stream-K), mma.sync, the sums with y and apart
 # ------------------------------------------------------------------------------------------
 
 @pytest.mark.parametrize("n,d_in,d_out", [(1, 32, 1), (1, 4096, 6144), (16, 4096, 14336), (17, 544, 130), (27, 14336, 4096),
                                           (32, 4064, 1000), (5, 20000, 129), (32, 32768, 260), (16, 1024, 24001),
-                                          (32, 8192, 20480), (9, 262144, 128)])
+                                          (32, 8192, 20480), (9, 262144, 128), (3, 12288, 16416), (16, 12288, 16400)])
 def test_decode_gemm_splits(n, d_in, d_out):
     """Accumulators equal to float64 products of the codes (exact), y = acc s_x s_w, and the SQNR sums."""
     rng = np.random.default_rng(n + d_in + d_out)

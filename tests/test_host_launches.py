@@ -114,3 +114,27 @@ def test_small_transforms_take_whole_rows_where_that_is_faster(fake, k, whole, t
         assert transform_kernel(fake, n, d, k, 0, code_bytes) == "rows", (n, d)
     for n, d in tiled:
         assert transform_kernel(fake, n, d, k, 0, code_bytes) == "", (n, d)
+
+
+def decode_route(fake, n, d_in, d_out, sums):
+    """What n <= 32 tokens run on: whole units, a cluster of 2, 4 or 8 a unit, equal cuts, or mma.sync ("+": and the
+    SQNR sums in a launch of their own)."""
+    launches = (fake.call("cat_w4a4_linear_sqnr", P, P, P, P, n, d_in, d_out, P, P, P, None) if sums else
+                linear(fake, n, d_in, d_out))
+    first = launches[0]
+    form = "mma" if "gemm_decode_kernel" in first.kernel else "cut" if first.cooperative else str(first.cluster)
+    return form + "+" * (len(launches) - 1)
+
+
+@pytest.mark.parametrize("n,d_in,d_out,plain,sums", [
+    (1, 4096, 6144, "2", "1"), (16, 4096, 14336, "1", "1"), (27, 14336, 4096, "4", "4"), (16, 1024, 24001, "cut", "cut"),
+    (16, 2048, 7530, "1", "1"), (30, 864, 4096, "1", "1"), (16, 4096, 1024, "8", "8"), (32, 256, 64, "1", "1"),
+    (9, 32, 20000, "cut", "cut"), (16, 14336, 16384, "2", "2+"),
+    # rows too long for one CTA: mma.sync for up to 8 tokens and many units, for 17 to 24 past a cluster of 4
+    (2, 14336, 22016, "mma", "mma+"), (8, 10240, 28672, "mma", "mma+"), (9, 14336, 22016, "2", "2+"), (2, 14336, 1024, "8", "8"),
+    (32, 20480, 28672, "8", "8+"), (24, 20480, 8192, "mma", "mma+"), (32, 28672, 4096, "8", "8+"), (24, 5120, 2048, "mma", "mma+"),
+    (16, 100000, 4096, "mma", "mma+"), (32, 49152, 1024, "mma", "mma+"),
+])
+def test_decode_gemm_takes_the_fastest_form(fake, n, d_in, d_out, plain, sums):
+    """The split that was measured fastest, on 152 SMs with 76, 36 and 15 clusters of 2, 4 and 8 resident."""
+    assert (decode_route(fake, n, d_in, d_out, False), decode_route(fake, n, d_in, d_out, True)) == (plain, sums)
