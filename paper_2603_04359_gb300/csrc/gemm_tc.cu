@@ -873,7 +873,9 @@ bool split_launch_ok(int64_t pairs) {
 // Parts that the tiles of the last wave (of nb channels each) are split into along K: a power of two, when that
 // wave is at most half full; 1: not split.  More than kFreeSplitUnits parts (128 channels each) only where that saves
 // kMinSaved K steps: many wide parts take 6 to 12 us to exchange (26 tail tiles of 256 in two: 454 x 4096 -> 22560 with the
-// SQNR sums 57.5 -> 63.7 us, 28 of them over 56 K steps, 4096 x 14336 -> 4096, 159.6 -> 147.8).
+// SQNR sums 57.5 -> 63.7 us, 28 of them over 56 K steps, 4096 x 14336 -> 4096, 159.6 -> 147.8).  With no whole tiles to
+// hide that exchange behind, cutting in two is never worth it (3000 x 12640 -> 768, 36 tiles of 256 in two 45.6 us, 72
+// of 128 uncut 38.0), cutting in four is (1000 x 14336 -> 768, 16 tiles of 192 in four 28.8, 24 of 128 in two 31.3).
 constexpr int kFreeSplitUnits = 80, kMinSaved = 20;
 int split_parts(int64_t tiles, int64_t num_k, int nb, int64_t pairs) {
   const int64_t tail = tiles >= pairs ? tiles % pairs : tiles;
@@ -881,7 +883,8 @@ int split_parts(int64_t tiles, int64_t num_k, int nb, int64_t pairs) {
   if (tail > 0 && tail <= kMaxSplitTiles && 2 * tail <= pairs)
     while (2 * split <= max_parts(nb) && 2 * split * tail <= pairs && 2 * split <= num_k &&
            2 * split * tail * nb <= (int64_t)kMaxSplitUnits * BN &&
-           (2 * split * tail * nb <= (int64_t)kFreeSplitUnits * BN || num_k - num_k / (2 * split) >= kMinSaved))
+           (2 * split * tail * nb <= (int64_t)kFreeSplitUnits * BN ||
+            (num_k - num_k / (2 * split) >= kMinSaved && (tiles >= pairs || split >= 2))))
       split *= 2;
   // a single partial wave has no whole tiles to hide the parts' exchange behind: split it only
   // when that saves ten K steps or more
@@ -962,8 +965,9 @@ cudaError_t launch_gemm_tc(const uint8_t* xq, const float* sx, const uint8_t* wq
 // empty (2048 tokens, 4096 -> 6144: 2.53 waves of 256, 2.95 of 224: 41.5 -> 39.8 us,
 // with the SQNR sums 57.0 -> 52.2).
 // A split adds its exchange, ~3 us or kSplitSteps K steps of a 128-wide tile: 600 x 4096 -> 15000 on 192 wide with a split
-// tail 42.1 us (53.4 with the SQNR sums), on 224 without 39.9 (49.7).
-constexpr double kTileBase = 0.44, kSplitSteps = 6.4;
+// tail 42.1 us (53.4 with the SQNR sums), on 224 without 39.9 (49.7); one of many wide parts kManySteps
+// (5978 x 14336 -> 2048 on 192 wide with 72 such parts 130, on 256 without a split 123).
+constexpr double kTileBase = 0.44, kSplitSteps = 6.4, kManySteps = 12.0;
 int e8_tile_width(int64_t n, int64_t d_in, int64_t d_out) {
   const int64_t pairs = num_sms() / 2, m_tiles = (n + 2 * BM - 1) / (2 * BM), num_k = (d_in + BK - 1) / BK;
   int best = 0;
@@ -972,7 +976,9 @@ int e8_tile_width(int64_t n, int64_t d_in, int64_t d_out) {
     const int64_t tiles = m_tiles * ((d_out + nb - 1) / nb);
     const int split = split_parts(tiles, num_k, nb, pairs);   // a tail of split tiles takes 1 / split of a wave
     const double waves = (double)(tiles / pairs) + (tiles % pairs == 0 ? 0.0 : 1.0 / split);
-    const double cost = waves * (kTileBase + (1.0 - kTileBase) * nb / 128.0) + (split > 1 ? kSplitSteps / num_k : 0.0);
+    const int64_t units = (tiles >= pairs ? tiles % pairs : tiles) * split * nb;
+    const double exchange = split == 1 ? 0.0 : (units > (int64_t)kFreeSplitUnits * BN ? kManySteps : kSplitSteps);
+    const double cost = waves * (kTileBase + (1.0 - kTileBase) * nb / 128.0) + exchange / num_k;
     if (best == 0 || cost < least) {
       best = nb;
       least = cost;

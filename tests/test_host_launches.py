@@ -138,3 +138,17 @@ def decode_route(fake, n, d_in, d_out, sums):
 def test_decode_gemm_takes_the_fastest_form(fake, n, d_in, d_out, plain, sums):
     """The split that was measured fastest, on 152 SMs with 76, 36 and 15 clusters of 2, 4 and 8 resident."""
     assert (decode_route(fake, n, d_in, d_out, False), decode_route(fake, n, d_in, d_out, True)) == (plain, sums)
+
+
+@pytest.mark.parametrize("n,d_in,d_out,width,grid,split", [
+    (2048, 4096, 6144, 224, 152, False), (4096, 14336, 4096, 256, 152, True), (8192, 8192, 28672, 256, 152, True),
+    (256, 8192, 3000, 192, 128, True), (600, 4096, 15000, 224, 152, False),
+    # one partial wave of long rows: many wide parts in two are no use, in four they are
+    (3000, 12640, 768, 128, 144, False), (1000, 12640, 2048, 128, 128, False), (1000, 14336, 768, 192, 128, True),
+    (5978, 14336, 2048, 256, 152, False),
+])
+def test_byte_code_gemm_takes_the_fastest_tiles(fake, n, d_in, d_out, width, grid, split):
+    """The tile width and whether the last wave is split along K, as measured, on 76 pairs."""
+    launch, = linear_e8(fake, n, d_in, d_out)
+    assert f"w4a4_gemm_tc_kernel<true, {width}>" in launch.kernel
+    assert (launch.grid, launch.cooperative) == (grid, int(split))
