@@ -26,6 +26,8 @@
 // Measured (8-bit asymmetric activations x 4-bit weights, 2048 x 4096 -> 6144; 8 x 8 bits, 1000 x 14336
 // -> 4096): 230 and 185 us with one CTA per 128 x 128 tile and scalar stores, now 63 and 118 us; with one MMA
 // issuer instead of two (and whole tiles) the second took 154 us, with two 130.
+// Outputs that TMA cannot store (d_out % 4) go through the staging buffer too and out by a row's 32 channels a store: 121 x 192
+// -> 10354 at 4 x 4 bits 32 us with each lane storing its own row, 23 now (10356: 19).
 // Where whole tiles leave the last wave short, the last one to two waves are cut into equal ranges of (tile, stage) steps,
 // one per pair (the stream part below): 8 x 8 bits, 1000 x 14336 -> 4096, 128 tiles on 76 pairs, 129.6 -> 117.5 us.
 // Every wait is bounded.
@@ -439,11 +441,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tma_store_2d(&tmY, buf, o0, row0);
             bulk_commit();
           }
-        } else if (t < n) {
-          float* yrow = y + (int64_t)t * d_out;
+        } else {                                       // no TMA store (d_out % 4): a plain store per row, of its 32 channels
+          __syncwarp();
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (o0 + j < d_out) yrow[o0 + j] = v[j];
+          for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<float4*>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+                make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+          __syncwarp();
+          const int rows = min(32, n - row0);
+          float* dst = y + (int64_t)row0 * d_out + o0 + lane;
+          for (int r = 0; in && r < rows; ++r)
+            dst[(int64_t)r * d_out] =
+                *reinterpret_cast<const float*>(buf + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
         }
       };
       if constexpr (C::NACC == 2) {                    // the other copy takes the next tile meanwhile
