@@ -50,6 +50,12 @@ constexpr uint32_t kAtomA = BM * KB;                 // 16 KiB: one plane's atom
 constexpr uint32_t kEpiStage = 32 * 32 * 4;          // y staging buffer of an epilogue warp
 constexpr int kMaxStages = 8;
 
+// Token rows of a load: a CTA's tile, or as many as there are in whole swizzle atoms (the others keep what the shared
+// memory held: their sums are not stored).  128-row boxes over a handful of rows were slow, by how much depending on
+// where they lay in memory: one token, 4096 -> 14336 at 8 x 8 bits 75 to 89 us, with boxes of 8 rows 52, as from 16
+// tokens on.
+__host__ __device__ constexpr int token_rows(int64_t n) { return n >= BM ? BM : (int)((n + 7) / 8 * 8); }
+
 struct DpBars {
   uint64_t full[kMaxStages], ready[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], mma_done;
   uint32_t fwd_word[kMaxStages];                     // even CTA: targets of the odd CTA's st.async per stage
@@ -207,6 +213,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       const bool is_a = warp == 0;
       const CUtensorMap* map = is_a ? &tmX : &tmW;
+      const uint32_t a_bytes = (uint32_t)(DX * C::AT * token_rows(n)) * KB;
       prefetch_tensormap(map);
       uint32_t it = 0;
       bool ok = true;
@@ -220,7 +227,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           if (use > 0 && !(ok = mbar_wait_bounded(&bars->empty[s], (use - 1) & 1, abort_flag, __LINE__, lim))) break;
           uint8_t* dst = smem + s * C::STAGE + (is_a ? 0u : C::A_BYTES);
           uint64_t* fb = rank == 0 ? &bars->full[s] : &bars->ready[s];
-          mbar_arrive_expect_tx(fb, is_a ? C::A_BYTES + (rank == 0 ? 4u : 0u) : C::B_BYTES);
+          mbar_arrive_expect_tx(fb, (is_a ? a_bytes : C::B_BYTES) + (is_a && rank == 0 ? 4u : 0u));
           const int planes = is_a ? DX : DW;
           const uint32_t atom = is_a ? kAtomA : C::ATOM_B;
           for (int p = 0; p < planes; ++p)
@@ -626,7 +633,7 @@ cudaError_t launch_nb(const DpCall& c) {
   static_assert(C::CH * 8 * 32 <= kStreamWarpInt4, "a warp's part");
   CUtensorMap mx, mw, my;
   memset(&my, 0, sizeof(my));
-  if (!plane_map(&mx, c.x_planes, c.n, c.d_in, DX, BM) || !plane_map(&mw, c.w_planes, c.d_out, c.d_in, DW, NB / 2))
+  if (!plane_map(&mx, c.x_planes, c.n, c.d_in, DX, token_rows(c.n)) || !plane_map(&mw, c.w_planes, c.d_out, c.d_in, DW, NB / 2))
     return cudaErrorInvalidValue;
   const int use_tma = (c.d_out % 4 == 0 && output_map(&my, c.y, c.n, c.d_out)) ? 1 : 0;
   static PerDevice<cudaError_t> allowed;

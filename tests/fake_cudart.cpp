@@ -32,6 +32,7 @@ std::map<const void*, std::string> kernels;
 std::map<std::pair<int, const void*>, Attrs> attrs;
 std::map<std::pair<int, const void*>, void*> symbols;
 std::vector<Launch> launches;
+std::vector<int> boxes;              // rows of the tensor maps' boxes
 std::map<std::string, int> wanted;   // part of a kernel's name -> the int argument to record
 thread_local int device = 0;
 thread_local struct {
@@ -65,9 +66,10 @@ cudaError_t launch(const void* func, dim3 grid, dim3 block, size_t smem, int clu
 
 bool backed(const void* p) { return (uintptr_t)p >> 40 != 0x10; }
 
-CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                const cuuint32_t* box, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                 CUtensorMapFloatOOBfill) {
+  boxes.push_back((int)box[1]);
   return CUDA_SUCCESS;
 }
 
@@ -79,9 +81,12 @@ extern "C" {
 void fake_reset() {
   std::lock_guard<std::mutex> lock(mu);
   launches.clear();
+  boxes.clear();
 }
 void fake_set_device(int d) { device = d; }
 void fake_record_arg(const char* kernel, int index) { wanted[kernel] = index; }
+int fake_boxes() { return (int)boxes.size(); }
+int fake_box_rows(int i) { return boxes[i]; }
 int fake_launches() { return (int)launches.size(); }
 const char* fake_kernel(int i) { return launches[i].kernel.c_str(); }
 int fake_field(int i, int which) {

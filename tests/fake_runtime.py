@@ -54,6 +54,10 @@ class FakeRuntime:
         self.kept.append(a)
         return (a.ctypes.data + 15) & ~15
 
+    def box_rows(self):
+        """Rows of the boxes of the last call's tensor maps, in the order they were made."""
+        return [self.lib.fake_box_rows(i) for i in range(self.lib.fake_boxes())]
+
     def call(self, name, *args):
         """The launches of one call, which must succeed; pointers are integers, None is NULL."""
         self.lib.fake_reset()

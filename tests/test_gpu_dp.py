@@ -360,7 +360,7 @@ def test_dp_transform_tensor_core_edges(n, d, k, bits, asym):
 
 @pytest.mark.parametrize("n,d_in,d_out,bx,bw,asym", [
     (1, 32, 1, 8, 8, True), (255, 160, 258, 8, 4, True), (121, 192, 1034, 4, 4, True), (40, 288, 10355, 8, 8, False),
-    (256, 128, 256, 4, 8, False), (513, 416, 1028, 4, 4, True),
+    (256, 128, 256, 4, 8, False), (513, 416, 1028, 4, 4, True), (3, 4128, 260, 8, 8, True), (17, 2080, 388, 4, 8, False),
     (2300, 544, 9000, 8, 8, False), (2300, 544, 9001, 8, 4, True), (4600, 288, 9004, 4, 4, False)])
 def test_dp_linear_tile_edges(n, d_in, d_out, bx, bw, asym):
     """Pair tiles with one row or one channel over, both tile widths and several tiles per pair: accumulators

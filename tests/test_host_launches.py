@@ -152,3 +152,11 @@ def test_byte_code_gemm_takes_the_fastest_tiles(fake, n, d_in, d_out, width, gri
     launch, = linear_e8(fake, n, d_in, d_out)
     assert f"w4a4_gemm_tc_kernel<true, {width}>" in launch.kernel
     assert (launch.grid, launch.cooperative) == (grid, int(split))
+
+
+@pytest.mark.parametrize("n,rows", [(1, 8), (8, 8), (9, 16), (64, 64), (121, 128), (127, 128), (128, 128), (300, 128)])
+def test_digit_plane_gemm_loads_the_token_rows_there_are(fake, n, rows):
+    """Boxes of as many token rows as there are in whole swizzle atoms, never more than a CTA's 128."""
+    for bits_x, bits_w in ((4, 4), (8, 4), (4, 8), (8, 8)):
+        linear_dp(fake, n, 4096, 6144, bits_x, bits_w)
+        assert fake.box_rows()[0] == rows
