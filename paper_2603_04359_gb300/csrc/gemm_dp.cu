@@ -27,7 +27,8 @@
 // -> 4096): 230 and 185 us with one CTA per 128 x 128 tile and scalar stores, now 63 and 118 us; with one MMA
 // issuer instead of two (and whole tiles) the second took 154 us, with two 130.
 // Outputs that TMA cannot store (d_out % 4) go through the staging buffer too and out by a row's 32 channels a store: 121 x 192
-// -> 10354 at 4 x 4 bits 32 us with each lane storing its own row, 23 now (10356: 19).
+// -> 10354 at 4 x 4 bits 32 us with each lane storing its own row, 23 now (10356: 19); up to 32 tokens, two warps of a pair
+// that wait for each chunk's turn in the buffer, 32 x 1024 -> 10354 21.5 and 23.7, so there each lane stores its own.
 // Where whole tiles leave the last wave short, the last one to two waves are cut into equal ranges of (tile, stage) steps,
 // one per pair (the stream part below): 8 x 8 bits, 1000 x 14336 -> 4096, 128 tiles on 76 pairs, 129.6 -> 117.5 us.
 // Every wait is bounded.
@@ -448,7 +449,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tma_store_2d(&tmY, buf, o0, row0);
             bulk_commit();
           }
-        } else {                                       // no TMA store (d_out % 4): a plain store per row, of its 32 channels
+        } else if (n <= 32) {                          // no TMA store (d_out % 4), one warp's rows: every lane its own
+          float* yrow = y + (int64_t)t * d_out;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (t < n && o0 + j < d_out) yrow[o0 + j] = v[j];
+        } else {                                       // ... more: through the buffer, a store per row, of its 32 channels
           __syncwarp();
 #pragma unroll
           for (int q = 0; q < 8; ++q)
@@ -457,9 +463,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           __syncwarp();
           const int rows = min(32, n - row0);
           float* dst = y + (int64_t)row0 * d_out + o0 + lane;
-          for (int r = 0; in && r < rows; ++r)
-            dst[(int64_t)r * d_out] =
-                *reinterpret_cast<const float*>(buf + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
+#pragma unroll 1
+          for (int r0 = 0; r0 < rows; r0 += 8) {       // eight rows' loads in flight (rows past n: whatever is there)
+            float u[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+              u[r] = *reinterpret_cast<const float*>(buf + (r0 + r) * 128 + (((lane >> 2) ^ r) << 4) + (lane & 3) * 4);
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+              if (in && r0 + r < rows) dst[(int64_t)(r0 + r) * d_out] = u[r];
+          }
         }
       };
       if constexpr (C::NACC == 2) {                    // the other copy takes the next tile meanwhile
