@@ -133,7 +133,7 @@ cat_status cat_calib_cov(const void* x, cat_dtype dtype, int64_t n, int64_t d, i
  *   Wq             out, device [d_out][d_in/2] bytes: SM4x8 codes of W T^{-1}.
  *   w_scale        out, device [d_out] float32: per-output-channel step s_w = max_i |W'_{o,i}| / 7.
  * Synchronous: it returns after the outputs are written.  CAT and CAT_HD blocks of k <= 128 are built
- * on the device in float64; the other kinds, k = 256, and a layer with a block whose condition number
+ * on the device in float64; the other kinds, k = 256, fewer than 8 blocks of 16 or 5 of 32, and a layer with a block whose condition number
  * may exceed 1e11 or that is not positive definite are built on the host in float64 (per block, in
  * parallel over host threads) from the sums read back.  It allocates and frees its own temporaries.
  * Returns CAT_ERR_NUMERIC if a Sigma_x or Sigma_w block is not positive definite.

@@ -262,7 +262,7 @@ cat_status cat_build_transform_host(cat_tkind kind, int64_t d_in, int32_t k, con
 // The layer's T (to T_blocks) and A_w = (T^{-1})^T (to aw_d), both float32 [d_in/k][k][k] on the device: A_w maps
 // a weight row w to its (W T^{-1}) row.  Synchronizes the stream; on an error T_blocks is untouched.
 // CAT and CAT_HD with k <= 128 are built on the device (transform_dev.cu); the kinds without calibration, the
-// diagonal one, k = 256, and a layer with a block that the device build does not decide (not positive definite,
+// diagonal one, k = 256, a few small blocks, and a layer with a block that the device build does not decide (not positive definite,
 // or too near it) are built on the host in float64, which also gives that layer's error.
 static cat_status build_layer_transform(const void* W, cat_dtype dtype, int64_t d_out, int64_t d_in, int32_t k,
                                         cat_tkind kind, const double* sigma_x_blocks, int64_t n_calib,

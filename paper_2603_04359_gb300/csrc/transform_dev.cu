@@ -20,8 +20,8 @@
 // round takes ~3.6 us, ~1.5 of them fmas; the rest is the exchange across the cluster (four CTAs are the best: two
 // double the fmas, eight do not fit the SMs).
 //
-// The host path (transform_host.cpp) stays for what this one does not decide: k = 256, the diagonal kind,
-// and any layer with a block whose condition numbers may exceed 1e11 (a bound from the traces of a block
+// The host path (transform_host.cpp) stays for what this one does not decide: k = 256, the diagonal kind, a few
+// blocks of k = 16 and 32 (transform_dev_supported), and any layer with a block whose condition numbers may exceed 1e11 (a bound from the traces of a block
 // and its inverse) or that is not positive definite: the flags then send the whole layer there.
 #include <cmath>
 
@@ -482,7 +482,12 @@ cudaError_t build_k(int64_t nb, const double* sx, int64_t n_calib, const double*
 
 }  // namespace
 
-bool transform_dev_supported(int k, int64_t nb) { return k <= 128 && nb <= 0x0FFFFFFF; }
+// A few small blocks are built faster on the host (16 cores), where each has a core to itself: the whole preparation of a
+// layer with 2, 4, 8 and 16 blocks, us host/device: k = 16 570/770 580/770 830/790 1170/800, k = 32 1345/1450 1400/1425 1640/1500
+// 2040/1510.
+bool transform_dev_supported(int k, int64_t nb) {
+  return k <= 128 && nb <= 0x0FFFFFFF && nb >= (k == 16 ? 8 : (k == 32 ? 5 : 1));
+}
 
 // Stream-ordered scratch of one build: doubles, then ints (4 flags, two exponents per block).
 size_t transform_dev_bytes(int k, int64_t nb) {

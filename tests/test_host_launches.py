@@ -1,4 +1,7 @@
 """The library's host code on a CUDA runtime without a device: scratch slots, kernel attributes per device, routes."""
+import ctypes
+
+import numpy as np
 import pytest
 
 from fake_runtime import FakeRuntime
@@ -160,3 +163,16 @@ def test_digit_plane_gemm_loads_the_token_rows_there_are(fake, n, rows):
     for bits_x, bits_w in ((4, 4), (8, 4), (4, 8), (8, 8)):
         linear_dp(fake, n, 4096, 6144, bits_x, bits_w)
         assert fake.box_rows()[0] == rows
+
+
+@pytest.mark.parametrize("d,k,device", [(112, 16, False), (128, 16, True), (128, 32, False), (160, 32, True), (64, 64, True),
+                                        (128, 128, True), (512, 256, False)])
+def test_transforms_of_a_few_small_blocks_are_built_on_the_host(fake, d, k, device):
+    """Fewer than 8 blocks of 16 or 5 of 32 channels take longer on the device than on the host's cores."""
+    sigma = np.tile(np.eye(k), (d // k, 1, 1)).astype(np.float64)
+    sx, T = fake.buffer(sigma.nbytes), fake.buffer(d * k * 4)
+    ctypes.memmove(sx, sigma.ctypes.data, sigma.nbytes)
+    fake.lib.fake_reset()
+    fake.lib.cat_quantize_weights(P, 0, 300, d, k, 2, sx, 512, None, T, P, P, None)   # (no kernel ran: Sigma_w is 0)
+    kernels = [fake.lib.fake_kernel(i).decode() for i in range(fake.lib.fake_launches())]
+    assert any("jacobi_kernel" in name for name in kernels) == device
