@@ -28,7 +28,7 @@
 // issuer instead of two (and whole tiles) the second took 154 us, with two 130.
 // Outputs that TMA cannot store (d_out % 4) go through the staging buffer too and out by a row's 32 channels a store: 121 x 192
 // -> 10354 at 4 x 4 bits 32 us with each lane storing its own row, 23 now (10356: 19); up to 32 tokens, two warps of a pair
-// that wait for each chunk's turn in the buffer, 32 x 1024 -> 10354 21.5 and 23.7, so there each lane stores its own.
+// that wait for each chunk's rows, 32 x 1024 -> 10354 21.5 and 23.7, so there each lane stores its own.
 // Where whole tiles leave the last wave short, the last one to two waves are cut into equal ranges of (tile, stage) steps,
 // one per pair (the stream part below): 8 x 8 bits, 1000 x 14336 -> 4096, 128 tiles on 76 pairs, 129.6 -> 117.5 us.
 // Every wait is bounded.
@@ -165,6 +165,23 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
           smem_u32(smem_dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
       : "memory");
+}
+
+// A staged 32 x 32 chunk to y without TMA: `rows` x `cols` of it, a row at a time.  Out of line: inside the epilogue it
+// costs the accumulators registers (8 x 8 bits, 1000 x 14336 -> 4096 and no plain store in it 1 % longer).
+__device__ __noinline__ void plain_store(const uint8_t* buf, float* y, int d_out, int rows, int cols) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll 1
+  for (int r0 = 0; r0 < rows; r0 += 8) {               // eight rows' loads in flight (rows past the end: whatever is there)
+    float u[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      u[r] = *reinterpret_cast<const float*>(buf + (r0 + r) * 128 + (((lane >> 2) ^ r) << 4) + (lane & 3) * 4);
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (lane < cols && r0 + r < rows) y[(int64_t)(r0 + r) * d_out + lane] = u[r];
+  }
 }
 
 template <int DX, int DW, int NB, bool STREAM>
@@ -436,43 +453,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         float v[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = (float)(int32_t)acc[j] * sxt * __shfl_sync(0xFFFFFFFFu, swl, j);
-        if (use_tma_store) {
-          if (lane == 0) bulk_wait_read_all();         // the store before has read the buffer
-          __syncwarp();
+        if (!use_tma_store && n <= 32) {               // one warp's rows: every lane its own
+          if (t < n) {
+            float* yrow = y + (int64_t)t * d_out;
 #pragma unroll
-          for (int q = 0; q < 8; ++q)                  // row `lane`, 16-byte chunk q at q ^ (lane % 8)
-            *reinterpret_cast<float4*>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            for (int j = 0; j < 32; ++j)
+              if (o0 + j < d_out) yrow[o0 + j] = v[j];
+          }
+          return;
+        }
+        if (use_tma_store && lane == 0) bulk_wait_read_all();   // the store before has read the buffer
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 8; ++q)                    // row `lane`, 16-byte chunk q at q ^ (lane % 8)
+          *reinterpret_cast<float4*>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+              make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        if (use_tma_store) {
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
             tma_store_2d(&tmY, buf, o0, row0);
             bulk_commit();
           }
-        } else if (n <= 32) {                          // no TMA store (d_out % 4), one warp's rows: every lane its own
-          float* yrow = y + (int64_t)t * d_out;
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (t < n && o0 + j < d_out) yrow[o0 + j] = v[j];
-        } else {                                       // ... more: through the buffer, a store per row, of its 32 channels
-          __syncwarp();
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            *reinterpret_cast<float4*>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
-                make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-          __syncwarp();
-          const int rows = min(32, n - row0);
-          float* dst = y + (int64_t)row0 * d_out + o0 + lane;
-#pragma unroll 1
-          for (int r0 = 0; r0 < rows; r0 += 8) {       // eight rows' loads in flight (rows past n: whatever is there)
-            float u[8];
-#pragma unroll
-            for (int r = 0; r < 8; ++r)
-              u[r] = *reinterpret_cast<const float*>(buf + (r0 + r) * 128 + (((lane >> 2) ^ r) << 4) + (lane & 3) * 4);
-#pragma unroll
-            for (int r = 0; r < 8; ++r)
-              if (in && r0 + r < rows) dst[(int64_t)(r0 + r) * d_out] = u[r];
-          }
+        } else {
+          plain_store(buf, y + (int64_t)row0 * d_out + o0, d_out, min(32, n - row0), min(32, d_out - o0));
         }
       };
       if constexpr (C::NACC == 2) {                    // the other copy takes the next tile meanwhile
