@@ -665,8 +665,8 @@ int resident_ctas(int log2_parts) {
 // The times are those of calls with cold weights, from fits over 2800 measured ones (1 to 32 tokens, 256 to 49152 -> 64 to
 // 28672 channels, every form that fits, with and without the sums; 3 to 5 % rms): a wave of CTAs takes kWaveUs
 // (start-up, token staging, the last outputs) and a K step kStepUs, more where the resident tokens leave room for three
-// packed stages only.  A cluster adds its exchange and, for every kThreads outputs that a CTA finishes, a pass over
-// them, with the sums another load of y_ref; more units than SMs in one piece (stream-K) add what the cut units wait
+// packed stages only.  A cluster adds its exchange and a pass for every kThreads outputs that a CTA finishes, with the sums
+// loads of y_ref in it; more units than SMs in one piece (stream-K) add what the cut units wait
 // for.  The sums in a launch of their own take kSumsUs: less than in a cluster's epilogue where that runs in waves
 // (8 tokens, 14336 -> 16384: 49 us against 57) or finishes many outputs.  Without the passes and the sums, 16 tokens,
 // 2048 -> 7530 with the sums went to clusters of 2: 21.6 us, on whole units 17.6.
@@ -702,8 +702,8 @@ DecodeForm pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms, bool 
     const int stages = stages_for(ntok, (int)nk, parts);
     if (stages == 0 || resident < parts || (sums && parts > 1 && units * parts > kSqnrMaxCtas)) continue;
     const double step = kStepUs[stages == kDecGroups][wide], wave = kWaveUs[sums][wide];
-    const int64_t passes = (n * UM / parts + kThreads - 1) / kThreads;
-    const double part = parts == 1 ? 0.0 : (sums ? 2.6 + 1.2 * passes : 0.9 + 0.65 * passes);
+    const double passes = (double)(n * UM) / (parts * kThreads);
+    const double part = parts == 1 ? 0.0 : (sums ? 1.9 + 1.6 * passes : 0.6 + 0.9 * passes);
     const double us = kFixedUs + (sums ? 1.5 : 0.0) +
                       (parts == 1 && units > sms
                            ? wave + kStreamUs + step * units * num_ks / sms

@@ -130,12 +130,12 @@ def decode_route(fake, n, d_in, d_out, sums):
 
 
 @pytest.mark.parametrize("n,d_in,d_out,plain,sums", [
-    (1, 4096, 6144, "2", "1"), (16, 4096, 14336, "1", "1"), (27, 14336, 4096, "4", "4"), (16, 1024, 24001, "cut", "cut"),
+    (1, 4096, 6144, "2", "2"), (16, 4096, 14336, "1", "1"), (27, 14336, 4096, "4", "4"), (16, 1024, 24001, "cut", "cut"),
     (16, 2048, 7530, "1", "1"), (30, 864, 4096, "1", "1"), (16, 4096, 1024, "8", "8"), (32, 256, 64, "1", "1"),
     (9, 32, 20000, "cut", "cut"), (16, 14336, 16384, "2", "2+"),
     # rows too long for one CTA: mma.sync for up to 8 tokens and many units, for 17 to 24 past a cluster of 4
     (2, 14336, 22016, "mma", "mma+"), (8, 10240, 28672, "mma", "mma+"), (9, 14336, 22016, "2", "2+"), (2, 14336, 1024, "8", "8"),
-    (32, 20480, 28672, "8", "8+"), (24, 20480, 8192, "mma", "mma+"), (32, 28672, 4096, "8", "8+"), (24, 5120, 2048, "mma", "mma+"),
+    (32, 20480, 28672, "8", "8+"), (24, 20480, 8192, "mma", "mma+"), (32, 28672, 4096, "8", "8+"), (24, 5120, 2048, "mma", "4"),
     (16, 100000, 4096, "mma", "mma+"), (32, 49152, 1024, "mma", "mma+"),
 ])
 def test_decode_gemm_takes_the_fastest_form(fake, n, d_in, d_out, plain, sums):
