@@ -36,22 +36,18 @@ struct ActCfg {
   static constexpr size_t SMEM = (size_t)(K * AS_LD + K * XS_LD) * sizeof(float);
 };
 
-// Eight codes, element `at` of the matrix (a multiple of 8) on: bytes (e8) or one SM4x8 word.
-__device__ __forceinline__ void store_codes(uint8_t* codes, int64_t at, int e8, const int (&q)[8]) {
-  if (e8) {
-    uint2 o;
-    o.x = e4m3_code_byte(q[0]) | e4m3_code_byte(q[1]) << 8 | e4m3_code_byte(q[2]) << 16 | e4m3_code_byte(q[3]) << 24;
-    o.y = e4m3_code_byte(q[4]) | e4m3_code_byte(q[5]) << 8 | e4m3_code_byte(q[6]) << 16 | e4m3_code_byte(q[7]) << 24;
-    *reinterpret_cast<uint2*>(codes + at) = o;
-  } else {
-    *reinterpret_cast<uint32_t*>(codes + at / 2) = sm4_pack(q);
-  }
+// Eight codes as bytes.
+__device__ __forceinline__ uint2 code_bytes(const int (&q)[8]) {
+  return make_uint2(
+      e4m3_code_byte(q[0]) | e4m3_code_byte(q[1]) << 8 | e4m3_code_byte(q[2]) << 16 | e4m3_code_byte(q[3]) << 24,
+      e4m3_code_byte(q[4]) | e4m3_code_byte(q[5]) << 8 | e4m3_code_byte(q[6]) << 16 | e4m3_code_byte(q[7]) << 24);
 }
 
+// PASS 0: the maxima; 1: the codes as SM4x8 words; 2: as bytes.
 template <typename Tin, int K, int PASS>
 __global__ void __launch_bounds__(ActCfg<K>::THREADS) transform_quant_kernel(
     const Tin* __restrict__ x, int64_t n, int64_t d, const float* __restrict__ A, uint32_t* __restrict__ amax_bits,
-    uint8_t* __restrict__ codes, int e8, uint32_t* __restrict__ status) {
+    uint32_t* __restrict__ codes, uint32_t* __restrict__ status) {
   using C = ActCfg<K>;
   extern __shared__ __align__(16) float smem[];
   float* As = smem;                    // [K][AS_LD]: As[j][i] = A_b[c0 + i][j]
@@ -118,7 +114,8 @@ __global__ void __launch_bounds__(ActCfg<K>::THREADS) transform_quant_kernel(
     for (int r = tid; r < kRows; r += C::THREADS)
       if (t0 + r < n) atomicMax(&amax_bits[t0 + r], red[r]);
   } else {
-    const int64_t col = (int64_t)b * K + c0 + 8 * cg;
+    const int64_t words_per_row = d / 8;               // eight codes: one word, or two of bytes
+    const int64_t word = ((int64_t)b * K + c0 + 8 * cg) / 8;
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int64_t t = t0 + 4 * tg + r;
@@ -127,7 +124,10 @@ __global__ void __launch_bounds__(ActCfg<K>::THREADS) transform_quant_kernel(
       int q[8];
 #pragma unroll
       for (int c = 0; c < 8; ++c) q[c] = qcode_exact(acc[r][c], qr, 7.0f);
-      store_codes(codes, t * d + col, e8, q);
+      if constexpr (PASS == 1)
+        codes[t * words_per_row + word] = sm4_pack(q);
+      else
+        reinterpret_cast<uint2*>(codes)[t * words_per_row + word] = code_bytes(q);
     }
   }
 }
@@ -234,7 +234,11 @@ __global__ void __launch_bounds__(kRowsThreads) transform_quant_rows_kernel(
     int q[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) q[e] = qcode_exact(v[e], qr, 7.0f);
-    store_codes(codes, (t0 + r) * d + 8 * i, e8, q);
+    if (e8) {
+      *reinterpret_cast<uint2*>(codes + (t0 + r) * d + 8 * i) = code_bytes(q);
+    } else {
+      *reinterpret_cast<uint32_t*>(codes + (t0 + r) * (d / 2) + 4 * i) = sm4_pack(q);
+    }
   }
   if (tid < kWholeRows && t0 + tid < n) {
     const float a = __uint_as_float(red[tid]);
@@ -324,7 +328,7 @@ cudaError_t launch_k(const Tin* x, int64_t n, int64_t d, const float* A, uint8_t
   cudaError_t e = cudaMemsetAsync(scale, 0, (size_t)n * sizeof(float), stream);
   if (e != cudaSuccess) return e;
   auto k0 = transform_quant_kernel<Tin, K, 0>;
-  auto k1 = transform_quant_kernel<Tin, K, 1>;
+  auto k1 = e8 ? transform_quant_kernel<Tin, K, 2> : transform_quant_kernel<Tin, K, 1>;
   if ((e = cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM)) != cudaSuccess) return e;
   const int64_t row_tiles = (n + kRows - 1) / kRows;
@@ -333,11 +337,12 @@ cudaError_t launch_k(const Tin* x, int64_t n, int64_t d, const float* A, uint8_t
   if (ny > 65535) return cudaErrorInvalidValue;
   dim3 grid((unsigned)row_tiles, (unsigned)ny);
   uint32_t* amax = reinterpret_cast<uint32_t*>(scale);
+  uint32_t* words = reinterpret_cast<uint32_t*>(codes);
   note_launch();
-  k0<<<grid, C::THREADS, C::SMEM, stream>>>(x, n, d, A, amax, codes, e8, status);
+  k0<<<grid, C::THREADS, C::SMEM, stream>>>(x, n, d, A, amax, words, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   note_launch();
-  k1<<<grid, C::THREADS, C::SMEM, stream>>>(x, n, d, A, amax, codes, e8, status);
+  k1<<<grid, C::THREADS, C::SMEM, stream>>>(x, n, d, A, amax, words, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   note_launch();
   finalize_scale_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(amax, n, status);

@@ -34,8 +34,8 @@
 //     finished there.  A unit cut between CTAs is owned by the CTA holding its first step, where it is
 //     the last segment of the range; every other part is the first segment of its CTA's range, so it
 //     is done early: it stores its raw accumulators (integers times 2^-18, exact in fp32) to its CTA's
-//     slice of device scratch and bumps the unit's per-warp counter.  The owner waits (bounded) for the
-//     counter while its own MMAs run, loads the other slices, adds them (an exact sum in any order),
+//     slice of device scratch and bumps the unit's per-warp counter.  The owner, its own MMAs done, waits (bounded)
+//     for the counter, loads the other slices, adds them (an exact sum in any order),
 //     writes y and resets the counter.  The launch is cooperative, so all parts are resident while the
 //     owners wait.
 // Every mbarrier wait is bounded; a wait that gives up raises the device status word
@@ -412,8 +412,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         s_run += yr[t] * yr[t];
         e_run += e * e;
       };
-      // owner of a cut unit: the other parts ran first in their CTAs; wait for their counts and
-      // sum their slices while this segment's MMAs run (16 tokens), or after them (32)
+      // owner of a cut unit: the other parts ran first in their CTAs.  Wait for their counts and sum their slices
+      // before this segment's accumulators are read (16 tokens), or chunk by chunk with them (32).
       constexpr bool kEarly = SPLIT && NTOK == 16;
       float ext[kEarly ? NTOK : 1];
       auto wait_parts = [&]() -> bool {              // warp-uniform
@@ -445,9 +445,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int t = 0; t < (kEarly ? NTOK : 1); ++t) ext[t] += __ldcg(src + t * UM);  // exact in any order
         }
       }
-      if (!(ok = mbar_wait_bounded(&bars->acc_full[ab], (seg >> 1) & 1, abort_flag, __LINE__, lim))) break;
-      __syncwarp();
-      tc_fence_after();
       if (!kEarly && !whole && owner && !(ok = wait_parts())) break;
       float* my_slice = reinterpret_cast<float*>(&g_dec_part[part_slot][blockIdx.x][0][0]) + ch;
 #pragma unroll

@@ -418,7 +418,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       auto add_parts = [&](int c, uint32_t (&acc)[32]) {
         parts([&](int cta) {
           const int4* src = g_dp_part[stream_slot][cta][ew] + c * 8 * 32 + lane;
-          constexpr int B = C::NACC == 2 ? 8 : 2;      // loads in flight: the registers left beside the accumulators
+          constexpr int B = 2;                         // loads in flight: the registers left beside the accumulators
 #pragma unroll
           for (int i0 = 0; i0 < 8; i0 += B) {
             int4 v[B];
@@ -480,24 +480,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
       };
       if constexpr (C::NACC == 2) {                    // the other copy takes the next tile meanwhile
-        if constexpr (STREAM)
-          if (is_owner && !(ok = wait_parts())) break;
+        static_assert(!STREAM || C::NACC == 1, "the stream part is for the widest tiles");
 #pragma unroll 1
         for (int c = 0; c < chunks; ++c) {
           uint32_t acc[32];
           gather(c, acc);
           if (c == chunks - 1) release();
-          if constexpr (STREAM) {
-            if (is_part) {
-              put_part(c, acc);
-              continue;
-            }
-            if (is_owner) add_parts(c, acc);
-          }
           finish(c, acc);
         }
-        if constexpr (STREAM)
-          if (is_part) set_flag();
       } else {
         uint32_t acc[C::CH][32];
 #pragma unroll

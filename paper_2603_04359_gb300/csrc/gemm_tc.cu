@@ -222,7 +222,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   constexpr uint32_t kAtomBn = (uint32_t)(NB / 2) * 128;   // one 128-code K atom of B
   constexpr uint32_t kStageBn = (uint32_t)(NB / 2) * BK;   // a stage's B (two atoms)
   constexpr uint32_t kIdescN = idesc_e4m3_f32(2 * BM, NB);
-  static_assert(NB == NB || E8, "the packed-code path uses 128-channel tiles");
+  static_assert(NB == BN || E8, "the packed-code path uses 128-channel tiles");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // packed codes: SE x 2 atoms x [64 rows x 128 B] decoded B; byte codes: SE x [A 2 atoms x [128 rows x
@@ -904,7 +904,7 @@ int take_split_units(int need) {
 // y_ref != nullptr: the epilogue also forms the SQNR sums of y against y_ref and writes
 // sums3 = {sum y_ref^2, sum (y_ref - y)^2, dB} (sums3 needs no zeroing).  Needs d_out % 4 == 0
 // (TMA row pitch).  E8: xq and wq hold one code per byte, else SM4x8 (two per byte).  NB: channels per
-// pair tile (256 only with byte codes; the last wave is then not split along K).
+// pair tile (192, 224 and 256 with byte codes only); the last wave's tiles are split along K as split_parts decides.
 template <bool E8, int NB>
 cudaError_t launch_gemm_tc(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw, int64_t n,
                            int64_t d_in, int64_t d_out, float* y, int32_t* acc_out, const float* y_ref, double* sums3,

@@ -385,7 +385,8 @@ def test_dp_linear_tile_edges(n, d_in, d_out, bx, bw, asym):
 
 @pytest.mark.parametrize("n,d_in,d_out,bx,bw,asym", [
     (300, 3072, 4990, 8, 8, True), (2500, 6144, 1030, 8, 8, False), (1500, 6144, 3396, 6, 8, False),
-    (1000, 6144, 4990, 8, 6, True), (300, 6144, 9980, 8, 4, True)])
+    (1000, 6144, 4990, 8, 6, True), (300, 6144, 9980, 8, 4, True), (512, 8192, 9980, 4, 4, False), (300, 8192, 9980, 4, 4, True),
+    (512, 8192, 9980, 4, 8, True), (1000, 8192, 6144, 4, 8, False)])
 def test_dp_linear_cut_tiles(n, d_in, d_out, bx, bw, asym):
     """A little over one or two waves of tiles, the last of them cut along K between pairs (in columns of all token tiles
     or tile by tile), launches after one another and replays of a graph: accumulators equal to float64 products of the

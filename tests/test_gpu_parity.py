@@ -615,11 +615,11 @@ def test_calib_cov_long_run_beyond_float32():
 # Small transforms: 16 whole rows per CTA
 # ------------------------------------------------------------------------------------------
 
-@pytest.mark.parametrize("n,d,k,dtype", [(1, 32, 16, "f32"), (15, 96, 32, "bf16"), (16, 256, 32, "f32"), (17, 128, 128, "f32"),
-                                         (33, 256, 256, "f32"), (50, 2048, 32, "f32"), (40, 512, 128, "f32"), (65, 1024, 64, "f32"),
-                                         (20, 640, 128, "f32")])
+@pytest.mark.parametrize("n,d,k,dtype", [(1, 32, 16, "f32"), (15, 384, 16, "f32"), (33, 96, 32, "bf16"), (48, 256, 32, "f32"),
+                                         (49, 128, 128, "f32"), (33, 256, 256, "f32"), (50, 768, 32, "f32"), (40, 512, 128, "f32"),
+                                         (65, 640, 64, "f32")])
 def test_small_transform_whole_rows(n, d, k, dtype):
-    """The whole-row kernel (T up to 65536 elements; 640 x 128 is past it) against the oracle, the packed and the byte
+    """The whole-row kernel (few blocks, more than 32 rows except at k = 16) against the oracle, the packed and the byte
     form alike; float32 rows of a wider layer whose first blocks are these (the tiled kernels, with zero
     columns added) get the same codes and steps: the same sums in the same order."""
     rng = np.random.default_rng(n + d + k)

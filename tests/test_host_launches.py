@@ -176,3 +176,19 @@ def test_transforms_of_a_few_small_blocks_are_built_on_the_host(fake, d, k, devi
     fake.lib.cat_quantize_weights(P, 0, 300, d, k, 2, sx, 512, None, T, P, P, None)   # (no kernel ran: Sigma_w is 0)
     kernels = [fake.lib.fake_kernel(i).decode() for i in range(fake.lib.fake_launches())]
     assert any("jacobi_kernel" in name for name in kernels) == device
+
+
+@pytest.mark.parametrize("n,d_in,d_out,bits_x,bits_w,lanes", [
+    (300, 3072, 4990, 8, 8, 2), (2500, 6144, 1030, 8, 8, 1), (1500, 6144, 3396, 6, 8, 1), (1000, 6144, 4990, 8, 6, 4),
+    (300, 6144, 9980, 8, 4, 2), (512, 8192, 9980, 4, 4, 2), (300, 8192, 9980, 4, 4, 2), (512, 8192, 9980, 4, 8, 2),
+    (1000, 8192, 6144, 4, 8, 4),
+])
+def test_digit_plane_gemm_cuts_its_last_waves(fake, n, d_in, d_out, bits_x, bits_w, lanes):
+    """The shapes whose accumulators are checked for cut tiles take that path, with every kind of operand: in columns of
+    all token tiles or tile by tile."""
+    fake.record_arg("dp_gemm_kernel", 14)
+    launch, = linear_dp(fake, n, d_in, d_out, bits_x, bits_w)
+    fake.record_arg("dp_gemm_kernel", 15)
+    planes = tuple(1 if b <= 4 else 2 for b in (bits_x, bits_w))
+    assert f"dp_gemm_kernel<{planes[0]}, {planes[1]}, {128 if planes == (2, 2) else 256}, true>" in launch.kernel
+    assert launch.cooperative and launch.grid == 152 and launch.arg == lanes
