@@ -167,9 +167,8 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
-// A staged 32 x 32 chunk to y without TMA: `rows` x `cols` of it, a row at a time.  Out of line: inside the epilogue it
-// costs the accumulators registers (8 x 8 bits, 1000 x 14336 -> 4096 and no plain store in it 1 % longer).
-__device__ __noinline__ void plain_store(const uint8_t* buf, float* y, int d_out, int rows, int cols) {
+// A staged 32 x 32 chunk to y without TMA: `rows` x `cols` of it, a row at a time.
+__device__ __forceinline__ void plain_store(const uint8_t* buf, float* y, int d_out, int rows, int cols) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
 #pragma unroll 1
@@ -184,12 +183,14 @@ __device__ __noinline__ void plain_store(const uint8_t* buf, float* y, int d_out
   }
 }
 
-template <int DX, int DW, int NB, bool STREAM>
+// PLAIN: y without TMA (d_out % 4).  A kernel of its own: beside the TMA stores, inline or called, the plain ones cost the
+// accumulators registers (1000 x 4096 -> 6144 at 8 x 4 bits 37.4 -> 38.0 us).
+template <int DX, int DW, int NB, bool STREAM, bool PLAIN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     dp_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                    const __grid_constant__ CUtensorMap tmY, const float* __restrict__ sx, const int32_t* __restrict__ zx,
                    const float* __restrict__ sw, const int32_t* __restrict__ w_rowsum, int n, int d_in, int d_out,
-                   float* __restrict__ y, int32_t* __restrict__ acc_out, int use_tma_store, int num_full,
+                   float* __restrict__ y, int32_t* __restrict__ acc_out, int num_full,
                    int stream_lanes, int stream_slot, uint32_t* __restrict__ status) {
   using C = DpGemmCfg<DX, DW, NB>;
   extern __shared__ uint8_t smem_raw[];
@@ -453,22 +454,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         float v[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = (float)(int32_t)acc[j] * sxt * __shfl_sync(0xFFFFFFFFu, swl, j);
-        if (!use_tma_store && n <= 32) {               // one warp's rows: every lane its own
-          if (t < n) {
-            float* yrow = y + (int64_t)t * d_out;
+        if constexpr (PLAIN) {
+          if (n <= 32) {                               // one warp's rows: every lane its own
+            if (t < n) {
+              float* yrow = y + (int64_t)t * d_out;
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (o0 + j < d_out) yrow[o0 + j] = v[j];
+              for (int j = 0; j < 32; ++j)
+                if (o0 + j < d_out) yrow[o0 + j] = v[j];
+            }
+            return;
           }
-          return;
+        } else {
+          if (lane == 0) bulk_wait_read_all();         // the store before has read the buffer
         }
-        if (use_tma_store && lane == 0) bulk_wait_read_all();   // the store before has read the buffer
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < 8; ++q)                    // row `lane`, 16-byte chunk q at q ^ (lane % 8)
           *reinterpret_cast<float4*>(buf + lane * 128 + ((q ^ (lane & 7)) << 4)) =
               make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        if (use_tma_store) {
+        if constexpr (!PLAIN) {
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
@@ -607,22 +611,22 @@ struct DpCall {
 template <int DX, int DW, int NB>
 bool stream_launch_ok(int64_t pairs) {
   using C = DpGemmCfg<DX, DW, NB>;
-  constexpr bool STREAM = true;
   static PerDevice<bool> asked;
   return asked.get([&] {
-    int dev = 0, coop = 0, clusters = 0;
-    bool ok = false;
-    if (2 * pairs <= kStreamCtas && cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-        allow_smem(dp_gemm_kernel<DX, DW, NB, STREAM>, C::SMEM) == cudaSuccess) {
+    auto fits = [&](auto kernel) {
       cudaLaunchConfig_t cfg;
       memset(&cfg, 0, sizeof(cfg));
       cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
       cfg.blockDim = dim3(kThreads, 1, 1);
       cfg.dynamicSmemBytes = C::SMEM;
-      if (cudaOccupancyMaxActiveClusters(&clusters, dp_gemm_kernel<DX, DW, NB, STREAM>, &cfg) == cudaSuccess && clusters >= pairs)
-        ok = true;
-    }
+      int clusters = 0;
+      return allow_smem(kernel, C::SMEM) == cudaSuccess &&
+             cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= pairs;
+    };
+    int dev = 0, coop = 0;
+    const bool ok = 2 * pairs <= kStreamCtas && cudaGetDevice(&dev) == cudaSuccess &&
+                    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+                    fits(dp_gemm_kernel<DX, DW, NB, true, false>) && fits(dp_gemm_kernel<DX, DW, NB, true, true>);
     cudaGetLastError();
     return ok;
   });
@@ -634,17 +638,15 @@ int next_stream_slot() {
   return (int)(next.fetch_add(1, std::memory_order_relaxed) % kStreamSlots);
 }
 
-template <int DX, int DW, int NB, bool STREAM = false>
-cudaError_t launch_nb(const DpCall& c) {
+template <int DX, int DW, int NB, bool STREAM, bool PLAIN>
+cudaError_t launch_as(const DpCall& c, const CUtensorMap& my) {
   using C = DpGemmCfg<DX, DW, NB>;
   static_assert(C::CH * 8 * 32 <= kStreamWarpInt4, "a warp's part");
-  CUtensorMap mx, mw, my;
-  memset(&my, 0, sizeof(my));
+  CUtensorMap mx, mw;
   if (!plane_map(&mx, c.x_planes, c.n, c.d_in, DX, token_rows(c.n)) || !plane_map(&mw, c.w_planes, c.d_out, c.d_in, DW, NB / 2))
     return cudaErrorInvalidValue;
-  const int use_tma = (c.d_out % 4 == 0 && output_map(&my, c.y, c.n, c.d_out)) ? 1 : 0;
   static PerDevice<cudaError_t> allowed;
-  const cudaError_t attr = allowed.get([] { return allow_smem(dp_gemm_kernel<DX, DW, NB, STREAM>, C::SMEM); });
+  const cudaError_t attr = allowed.get([] { return allow_smem(dp_gemm_kernel<DX, DW, NB, STREAM, PLAIN>, C::SMEM); });
   if (attr != cudaSuccess) return attr;
   const int64_t tiles = ((c.n + 2 * BM - 1) / (2 * BM)) * ((c.d_out + NB - 1) / NB);
   if (tiles > 0x3FFFFFFF) return cudaErrorInvalidValue;
@@ -665,8 +667,16 @@ cudaError_t launch_nb(const DpCall& c) {
   cfg.attrs = attrs;
   cfg.numAttrs = STREAM ? 2 : 1;
   note_launch();
-  return cudaLaunchKernelEx(&cfg, dp_gemm_kernel<DX, DW, NB, STREAM>, mx, mw, my, c.sx, c.zx, c.sw, c.w_rowsum, (int)c.n,
-                            (int)c.d_in, (int)c.d_out, c.y, c.acc_out, use_tma, (int)num_full, lanes, slot, c.status);
+  return cudaLaunchKernelEx(&cfg, dp_gemm_kernel<DX, DW, NB, STREAM, PLAIN>, mx, mw, my, c.sx, c.zx, c.sw, c.w_rowsum, (int)c.n,
+                            (int)c.d_in, (int)c.d_out, c.y, c.acc_out, (int)num_full, lanes, slot, c.status);
+}
+
+template <int DX, int DW, int NB, bool STREAM = false>
+cudaError_t launch_nb(const DpCall& c) {
+  CUtensorMap my;
+  memset(&my, 0, sizeof(my));
+  const bool tma = c.d_out % 4 == 0 && output_map(&my, c.y, c.n, c.d_out);
+  return tma ? launch_as<DX, DW, NB, STREAM, false>(c, my) : launch_as<DX, DW, NB, STREAM, true>(c, my);
 }
 
 // The cycles a launch with NB-wide tiles should take: whole waves of tiles, each its stages (the MMAs of a

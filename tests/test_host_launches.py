@@ -12,7 +12,7 @@ P = 0x10 << 40          # an address that holds nothing
 @pytest.fixture(scope="module")
 def fake(tmp_path_factory):
     f = FakeRuntime(tmp_path_factory.mktemp("fake"))
-    f.record_arg("dp_gemm_kernel", 15)                # the slot of cut tiles' parts
+    f.record_arg("dp_gemm_kernel", 14)                # the slot of cut tiles' parts
     f.record_arg("w4a4_gemm_tc_kernel", 17)           # the first unit of split tiles' parts
     f.record_arg("w4a4_gemm_decode_tc_kernel", 15)    # the slot of cut units' parts
     return f
@@ -162,7 +162,7 @@ def test_digit_plane_gemm_loads_the_token_rows_there_are(fake, n, rows):
     """Boxes of as many token rows as there are in whole swizzle atoms, never more than a CTA's 128."""
     for bits_x, bits_w in ((4, 4), (8, 4), (4, 8), (8, 8)):
         linear_dp(fake, n, 4096, 6144, bits_x, bits_w)
-        assert fake.box_rows()[0] == rows
+        assert fake.box_rows()[:2] == [32, rows]                  # y's, then the tokens'
 
 
 @pytest.mark.parametrize("d,k,device", [(112, 16, False), (128, 16, True), (128, 32, False), (160, 32, True), (64, 64, True),
@@ -186,9 +186,9 @@ def test_transforms_of_a_few_small_blocks_are_built_on_the_host(fake, d, k, devi
 def test_digit_plane_gemm_cuts_its_last_waves(fake, n, d_in, d_out, bits_x, bits_w, lanes):
     """The shapes whose accumulators are checked for cut tiles take that path, with every kind of operand: in columns of
     all token tiles or tile by tile."""
-    fake.record_arg("dp_gemm_kernel", 14)
+    fake.record_arg("dp_gemm_kernel", 13)
     launch, = linear_dp(fake, n, d_in, d_out, bits_x, bits_w)
-    fake.record_arg("dp_gemm_kernel", 15)
+    fake.record_arg("dp_gemm_kernel", 14)
     planes = tuple(1 if b <= 4 else 2 for b in (bits_x, bits_w))
-    assert f"dp_gemm_kernel<{planes[0]}, {planes[1]}, {128 if planes == (2, 2) else 256}, true>" in launch.kernel
+    assert f"dp_gemm_kernel<{planes[0]}, {planes[1]}, {128 if planes == (2, 2) else 256}, true, {str(d_out % 4 != 0).lower()}>" in launch.kernel
     assert launch.cooperative and launch.grid == 152 and launch.arg == lanes
