@@ -191,6 +191,9 @@ cat_status cat_build_transform_host(cat_tkind kind, int64_t d_in, int32_t k, con
  *   x_scale  out, device [n] float32: per-token step s_x = max_i |x'_i| / 7 (0 for an all-zero token).
  * Codes are q = clamp(round_half_even(7 x'_i / max|x'|), -7, 7), x' accumulated in float32; the
  * rounding decision is exact for the float32 x' (ties included), not a float32 approximation of it.
+ * The order of x''s float32 sums depends on the shape of the call, n included (calls of up to 32 rows are
+ * summed by other kernels than larger ones), so a token whose 7 x'_i / max|x'| lies on a rounding boundary
+ * within float32 accuracy (about one code in 10^6) may get a neighbouring code in a call of another size.
  */
 cat_status cat_transform_quantize_act(const void* x, cat_dtype dtype, int64_t n, int64_t d_in, int32_t k,
                                       const float* T_blocks, uint8_t* xq, float* x_scale,
