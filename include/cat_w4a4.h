@@ -35,10 +35,11 @@
  *    scratch.  A call is handed its share when it is made, in turn, and keeps it: eight shares for
  *    the transforms, eight for the SQNR sums of a kernel, twice what the device can run at once for
  *    the GEMMs' partial sums.  Calls made one after another may overlap on any number of streams;
- *    but a call that is held back (behind other work of its stream, or captured in a graph, which
- *    keeps its share for every replay) must not run at the same time as a call that was handed the
- *    same share after it.  So order the replays of two graphs of these calls, or of a graph and
- *    calls beside it, rather than run them at the same time on two streams.
+ *    but a call must not run at the same time as a call that was handed the same share after it.
+ *    That takes a call that is held back (behind other work of its stream, or captured in a graph,
+ *    which keeps its share for every replay), or one that runs on beside a whole round of later calls
+ *    from other streams.  So order the replays of two graphs of these calls, or of a graph and
+ *    calls beside it, or a very long call and many short ones, rather than run them at the same time.
  *
  * INT4 code format ("SM4x8")
  * --------------------------
