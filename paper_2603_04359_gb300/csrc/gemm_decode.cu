@@ -124,19 +124,18 @@ __global__ void __launch_bounds__(kWarps * 32) w4a4_gemm_decode_kernel(
 
 }  // namespace
 
-bool decode_tc_applies(int64_t n, int64_t d_in, int64_t d_out, bool with_sqnr);
 cudaError_t launch_w4a4_gemm_decode_tc(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw,
                                        int64_t n, int64_t d_in, int64_t d_out, float* y, int32_t* acc_out,
                                        const float* y_ref, double* sums3, uint32_t* status, cudaStream_t stream);
 
-// n <= 32: tcgen05 weight streaming, or mma.sync weight streaming with registers where decode_tc_applies says no.
+// n <= 32: tcgen05 weight streaming, or mma.sync weight streaming with registers where that kernel does not take the call.
 // y_ref != nullptr: also the SQNR sums of y against y_ref into sums3 (in the tcgen05 kernel's
 // epilogue, else by the separate reduction after the GEMM).
 cudaError_t launch_w4a4_gemm_decode(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw, int64_t n,
                                     int64_t d_in, int64_t d_out, float* y, int32_t* acc_out, const float* y_ref,
                                     double* sums3, uint32_t* status, cudaStream_t stream) {
-  if (decode_tc_applies(n, d_in, d_out, y_ref != nullptr))
-    return launch_w4a4_gemm_decode_tc(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, stream);
+  const cudaError_t tc = launch_w4a4_gemm_decode_tc(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, stream);
+  if (tc != cudaErrorNotSupported) return tc;
   if (y_ref) {
     const cudaError_t e = launch_w4a4_gemm_decode(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, nullptr, nullptr, status,
                                                   stream);

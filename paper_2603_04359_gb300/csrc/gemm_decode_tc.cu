@@ -632,9 +632,9 @@ struct ResidentCtas {
   int of[4];
 };
 template <int NTOK>
-int resident_ctas(int log2_parts) {
+ResidentCtas resident_ctas() {
   static PerDevice<ResidentCtas> asked;
-  const ResidentCtas r = asked.get([] {
+  return asked.get([] {
     ResidentCtas ctas = {{num_sms(), 0, 0, 0}};
     const bool ok = allow_decode_smem<NTOK>() == cudaSuccess;
     for (int i = 1; i < 4; ++i) {
@@ -653,7 +653,6 @@ int resident_ctas(int log2_parts) {
     cudaGetLastError();
     return ctas;
   });
-  return r.of[log2_parts];
 }
 
 // How a call is best run: CTAs per unit (the cluster's size; 1: whole units or stream-K) and its time in us.  parts = 0: on the
@@ -689,13 +688,13 @@ double mma_sync_us(int64_t n, int64_t d_in, int64_t d_out) {
 }
 
 // The best form of the tcgen05 kernel alone, with the sums in its epilogue if there are any.
-DecodeForm pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms, bool sums) {
+DecodeForm pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms, const ResidentCtas& ctas, bool sums) {
   const int ntok = n <= 16 ? 16 : 32, wide = ntok == 32;
   const int64_t num_ks = (d_in / 2 + KSB - 1) / KSB, units = (d_out + UM - 1) / UM;
   DecodeForm best = {0, 0.0};
   for (int i = 0, parts = 1; parts <= kMaxParts && parts <= num_ks; ++i, parts *= 2) {
     const int64_t nk = (num_ks + parts - 1) / parts;
-    const int64_t resident = ntok == 16 ? resident_ctas<16>(i) : resident_ctas<32>(i);
+    const int64_t resident = ctas.of[i];
     const int stages = stages_for(ntok, (int)nk, parts);
     if (stages == 0 || resident < parts || (sums && parts > 1 && units * parts > kSqnrMaxCtas)) continue;
     const double step = kStepUs[stages == kDecGroups][wide], wave = kWaveUs[sums][wide];
@@ -712,14 +711,15 @@ DecodeForm pick_parts(int64_t n, int64_t d_in, int64_t d_out, int64_t sms, bool 
 
 DecodeForm pick_form(int64_t n, int64_t d_in, int64_t d_out, int64_t sms, bool sums) {
   const int64_t num_ks = (d_in / 2 + KSB - 1) / KSB, units = (d_out + UM - 1) / UM;
-  DecodeForm plain = pick_parts(n, d_in, d_out, sms, false);
+  const ResidentCtas ctas = n <= 16 ? resident_ctas<16>() : resident_ctas<32>();
+  DecodeForm plain = pick_parts(n, d_in, d_out, sms, ctas, false);
   const bool ask = n <= 8 ? num_ks > 36 : n > 16 && (num_ks > 72 || (n <= 24 && num_ks > 18 && units <= 32));
   if (plain.parts == 0 || ask) {
     const double us = mma_sync_us(n, d_in, d_out);
     if (plain.parts == 0 || us < plain.us) plain = {0, us};
   }
   if (!sums) return plain;
-  const DecodeForm fused = pick_parts(n, d_in, d_out, sms, true);
+  const DecodeForm fused = pick_parts(n, d_in, d_out, sms, ctas, true);
   return fused.parts != 0 && fused.us <= plain.us + kSumsUs ? fused : DecodeForm{0, plain.us + kSumsUs};
 }
 
@@ -813,18 +813,15 @@ cudaError_t set_decode_wait_limit(uint64_t ns) {
   return cudaMemcpyToSymbol(g_dec_wait_limit, &ns, sizeof(ns));
 }
 
-// Whether this kernel takes the call (else the mma.sync kernel does, or the sums are not formed with y).
-bool decode_tc_applies(int64_t n, int64_t d_in, int64_t d_out, bool with_sqnr) {
-  return n >= 1 && n <= 32 && pick_form(n, d_in, d_out, num_sms(), with_sqnr).parts > 0;
-}
-
 // y_ref != nullptr: the epilogue also forms the SQNR sums of y against y_ref and writes
-// sums3 = {sum y_ref^2, sum (y_ref - y)^2, dB} (sums3 needs no zeroing).
+// sums3 = {sum y_ref^2, sum (y_ref - y)^2, dB} (sums3 needs no zeroing).  cudaErrorNotSupported, nothing launched: the
+// mma.sync kernel is to take the call, or the sums a launch of their own.
 cudaError_t launch_w4a4_gemm_decode_tc(const uint8_t* xq, const float* sx, const uint8_t* wq, const float* sw,
                                        int64_t n, int64_t d_in, int64_t d_out, float* y, int32_t* acc_out,
                                        const float* y_ref, double* sums3, uint32_t* status, cudaStream_t stream) {
+  if (n < 1 || n > 32) return cudaErrorInvalidValue;
   const int parts = pick_form(n, d_in, d_out, num_sms(), y_ref != nullptr).parts;
-  if (parts == 0) return cudaErrorInvalidValue;
+  if (parts == 0) return cudaErrorNotSupported;
   if (n <= 16) return launch_ntok<16>(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, parts, stream);
   return launch_ntok<32>(xq, sx, wq, sw, n, d_in, d_out, y, acc_out, y_ref, sums3, status, parts, stream);
 }
